@@ -222,7 +222,7 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
                                                                             AttnArgs p) {
   extern __shared__ uint8_t smem_raw[];
   AttnTcSmem& sm = *reinterpret_cast<AttnTcSmem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
   const int qi = blockIdx.x, split = blockIdx.y;
   const void* const q_ptr = p.q;
   const void* const k_ptr = p.k;
@@ -244,7 +244,7 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
     tc::mbar_init(smem_u32(&sm.q_full), q_tma ? 1 : 32 * kLoadWarps);
     tc::mbar_init(smem_u32(&sm.q_tmem), kSoftmaxWarps);
     for (int b = 0; b < kKBufs; ++b) {
-      tc::mbar_init(smem_u32(&sm.k_full[b]), 32 * (kLoadWarps + (kPv == 2 ? 2 : 0)));
+      tc::mbar_init(smem_u32(&sm.k_full[b]), kLoadWarps + (kPv == 2 ? 2 : 0));
       tc::mbar_init(smem_u32(&sm.k_empty[b]), n_pv);
     }
     for (int b = 0; b < 2; ++b) {
@@ -285,7 +285,7 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
     // first of them arrives on the barrier with the byte count of all nine (a box that completes before that only
     // makes the count negative for a moment: the phase cannot end before the arrival)
     const int qw = warp - (kSoftmaxWarps + kMmaWarps);
-    if (q_tma && lane == 0 && qw >= 0) {
+    if (q_tma && qw >= 0 && tc::elect_one()) {
       const uint32_t stage = smem_u32(sm.k[kKBufs - 1]);
       if (qw == 0) tc::mbar_expect_tx(smem_u32(&sm.q_full), kH * kDQK * 2);
       for (int a = qw; a < kAtoms; a += kLoadWarps)
@@ -410,7 +410,8 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
       else cp_async_wait<0>();
       if (!q_handed) hand_over_q();
       tc::fence_proxy_async();
-      tc::mbar_arrive(smem_u32(&sm.k_full[first_pend % kKBufs]));
+      __syncwarp();   // one arrival per warp: 192 threads arriving on one barrier are 192 serialised shared-memory operations
+      if (lane == 0) tc::mbar_arrive(smem_u32(&sm.k_full[first_pend % kKBufs]));
       ++first_pend;
       --n_pend;
     };
@@ -439,7 +440,7 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
         // 64 consecutive window rows: nine boxes that complete k_full by byte count; the (empty) cp.async group
         // below keeps the hand-over bookkeeping the same for every kind of tile.  An issued TMA copy costs its thread
         // 200-300 cycles, so the nine boxes are dealt to the gather warps (each announces the bytes of its own)
-        if (lane == 0 && gw < kAtoms) {
+        if (gw < kAtoms && tc::elect_one()) {
           const int n_mine = (kAtoms - gw + kGw - 1) / kGw;
           tc::mbar_expect_tx_only(smem_u32(&sm.k_full[b]), n_mine * kAtomBytes);
           const int row0 = static_cast<int>(win0) + (tile_begin + i) * kTileKeys;
@@ -487,7 +488,7 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
   } else if (warp >= kSoftmaxWarps) {
     // ================= MMA issuers =================
     const int x = warp - kSoftmaxWarps;   // 0..3
-    if (lane == 0 && n_tiles > 0) {
+    if (tc::elect_one() && n_tiles > 0) {
       constexpr uint32_t idesc_qk = tc::idesc_bf16(kH, kTileKeys, 0, 0);
       constexpr uint32_t idesc_pv = n_pv == 4 ? tc::idesc_bf16(kH, 128, 0, 1) : tc::idesc_bf16(kH, 256, 0, 1);   // B = V read MN-major
       bool ok = tc::mbar_wait(smem_u32(&sm.q_full), 0, p.status) && tc::mbar_wait(smem_u32(&sm.q_tmem), 0, p.status);

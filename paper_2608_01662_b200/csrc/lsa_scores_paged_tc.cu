@@ -117,7 +117,7 @@ paged_scores_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
   constexpr uint32_t kPageBytes = kPageTok * Smem::kRowBytes;
   extern __shared__ uint8_t smem_raw[];
   Smem& sm = *reinterpret_cast<Smem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
   const int batch = p.n_query;
   PsShape sh;
   sh.S = p.S; sh.W = p.W; sh.flat = flat;
@@ -232,7 +232,7 @@ paged_scores_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
         const int i = base + j;
         const int f0 = __shfl_sync(0xffffffffu, ph0, j), f1 = __shfl_sync(0xffffffffu, ph1, j);
         bool ok = true;
-        if (lane == 0) {
+        if (tc::elect_one()) {
           const int s = i % kSlots;
           ok = tc::mbar_wait(smem_u32(&sm.k_empty[s]), ((i / kSlots) & 1) ^ 1, p.status);
           if (ok) {
@@ -258,13 +258,13 @@ paged_scores_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
             }
           }
         }
-        if (!__shfl_sync(0xffffffffu, ok, 0)) alive = false;
+        if (!__all_sync(0xffffffffu, ok)) alive = false;
       }
     }
   } else if (warp < 4) {
     // ================= MMA issuers: warp 2 the even tiles, warp 3 the odd ones; tile i into accumulator i % 4 =====
     const int me = warp - 2;
-    if (lane == 0) {
+    if (tc::elect_one()) {
       constexpr int kSteps = E4M3 ? 12 : 8;
       constexpr uint32_t idesc = E4M3 ? tc::idesc_e4m3_e5m2(kTile, kHI) : tc::idesc_bf16(kTile, kHI, 0, 0);
       const uint64_t da0 = tc::smem_desc_sw128(smem_u32(sm.k), 16, 1024);

@@ -98,6 +98,17 @@ __device__ __forceinline__ void tma_gather4_2d(uint32_t dst, const CUtensorMap* 
       : "memory");
 }
 
+// One thread of a fully converged warp (true in exactly one lane).  tcgen05.mma and the TMA copies take their operands
+// from uniform registers; behind `lane == 0` the compiler cannot tell that one thread is left and moves them there with a
+// loop over the active lanes.  Measured, one issuing thread, M64 N64 K16 with A in tensor memory: 49 cycles per MMA behind
+// `lane == 0`, 32 (the pipe's own rate) behind elect.sync.  Worth it where the issuing thread is what paces the kernel
+// (attention, paged token scores); the prefill fine stage got 4 % slower with it, the coarse kernels did not change.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.b32 %0, 1, 0, p;\n\t}" : "=r"(p));
+  return p != 0;
+}
+
 // ---- tensor memory ----------------------------------------------------------------------------------
 // Whole-warp calls.  The base address (lane 0, first column) is written to the shared word `slot`.
 __device__ __forceinline__ void tmem_alloc(uint32_t slot, uint32_t n_cols) {
