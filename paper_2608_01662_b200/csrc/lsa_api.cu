@@ -339,7 +339,6 @@ int run_attn(lsa_ctx* c, const lsa_params* p, const void* q, const void* k, cons
   a.q_pos0 = q_pos0; a.n_query = static_cast<int>(nq); a.ctx_len = ctx_len; a.out = out; a.lse = lse;
   a.n_split = 1; a.status = status_word(c);
   a.qk_waits_pv = c->tune[LSA_TUNE_ATTN_PV_WAIT];
-  a.pv_issuers = p->paged ? 4 : 2;   // decode waits on HBM gathers, prefill on the tensor pipe
   a.gather4 = c->tune[LSA_TUNE_ATTN_GATHER];
   a.rows_stable = rows != nullptr && c->last_attn_rows == rows;
   const bool use_tc = c->tune[LSA_TUNE_ATTN_TC] && lsa::attn_tc_supported(a);

@@ -65,8 +65,7 @@ struct AttnArgs {
   const int32_t* ctx_len;
   void* out;              // bf16 [n_query, H, DV]
   float* lse;             // optional [n_query, H]
-  int pv_issuers;         // tcgen05 kernel: 2 = an issuer owns a lane half (prefill), 4 = one P V issuer per 128 value dims
-  int qk_waits_pv;        // tcgen05 kernel, 2 issuers: Q K^T of tile i+1 waits for the completion barrier of P V of tile i-1
+  int qk_waits_pv;        // tcgen05 kernel: Q K^T of tile i+1 waits for the completion barrier of P V of tile i-1
   int gather4;            // tcgen05 kernel: scattered rows by TMA gather (cp.async.bulk.tensor tile::gather4) where the cache allows
   int rows_stable;        // tcgen05 kernel, row lists: `rows` / `n_rows` were complete before the previous kernel of the
                           // stream started, so they may be read ahead of the programmatic dependency wait
