@@ -6,36 +6,38 @@
 // as an item of its own.  Prefill blocks are persistent: when a query's last copies are out, the next query's Q and
 // first tiles follow them into the ring, so that only the softmax of one tile stands between two queries.
 //
-//   warps 6-13  gather: rows [window | sink | sparse] (or the caller's row list) -> 128B-swizzled K-major tiles, up to
-//               three items in flight.  Scattered rows are copied with coalesced 16-byte cp.async, a row by one warp
+//   warps 7-12  gather: two warps per ring slot.  They wait for the slot, copy rows [window | sink | sparse] (or those of the
+//               caller's row list) into its 128B-swizzled K-major tile with coalesced 16-byte cp.async, a row by one warp
 //               (spreading a tile's chunks over the warps was measured 1.3 x slower, a TMA gather of four rows per
-//               instruction - AttnArgs::gather4 - as well: the TMA unit takes about 26 cycles for its 512 bytes);
-//               tiles of 64 consecutive window rows and Q come as nine TMA boxes, dealt to the warps.
-//   warp 5      scheduler: one thread publishes the block's jobs (query, row count).  In prefill it takes the block index
+//               instruction - AttnArgs::gather4 - as well: the TMA unit takes about 26 cycles for its 512 bytes), and hand
+//               it over when it has landed; tiles of 64 consecutive window rows and Q come as one TMA box each.
+//   warp 6      scheduler: one thread publishes the block's jobs (query, row count).  In prefill it takes the block index
 //               of a block that has not started yet (cluster launch control), one job ahead of the one being worked on,
 //               latest query first: those attend the most rows.
-//   warp 4      one thread issues every tcgen05.mma:
-//                 S = Q K^T   M64 N64 K16, Q in tensor memory, as two accumulation chains: dims 0-255 and rope dims
-//                             0-31 in the even half of the lanes, dims 256-511 and rope dims 32-63 in the odd half (an
-//                             M = 64 accumulator and its A operand use 16 of the 32 lanes of each quarter, so both halves
-//                             of Q share their columns).  36 MMAs at the pipe's 32 cycles.
-//                 O += P V    tcgen05.mma.ws M64 N256 K16, P in shared memory; V is the key tile read MN-major, so that a
-//                             cache row is fetched once.  The .ws form spreads the 64 rows over all 128 lanes (heads in
-//                             lanes 0-63 and again in 64-127, each with half of the value dims), which is the full data
+//   warps 4, 5  one thread each issues tcgen05.mma:
+//                 S = Q K^T   warp 4, M64 N64 K16, Q in tensor memory (the rope dims in shared memory), as two accumulation
+//                             chains: dims 0-255 and rope dims 0-31 in the even half of the lanes, dims 256-511 and rope
+//                             dims 32-63 in the odd half (an M = 64 accumulator and its A operand use 16 of the 32 lanes of
+//                             each quarter, so both halves of Q share their columns).  36 MMAs at the pipe's 32 cycles.
+//                 O += P V    warp 5, tcgen05.mma.ws M64 N256 K16, P in shared memory; V is the key tile read MN-major, so
+//                             that a cache row is fetched once.  The .ws form spreads the 64 rows over all 128 lanes (heads
+//                             in lanes 0-63 and again in 64-127, each with half of the value dims), which is the full data
 //                             path: 81 cycles where the plain M64 N256 form takes 129.
-//               It takes whichever of "next P V" / "next Q K^T" is ready, P V first: its completion frees a ring slot,
-//               and the refill of that slot is the longest latency of the ring.
+//               Two threads, because one stalls for 300 to 500 cycles after each batch before it gets to the next, and
+//               two S buffers, so that Q K^T of the next tile need not wait for the softmax of this one: 2 340 cycles per
+//               tile with one of each.
 //   warps 0-3   softmax: move Q to tensor memory; per tile add the two partial sums (read as 16-lane fragments, so both
 //               land in the same registers), running max with lazy rescaling of O, exp2, fp32 row sums, P as bf16 into
-//               shared memory (A operand of P V); at the end of a query O / l to global.
+//               the tile's rope block (64 x 64 values; Q K^T was its only reader); at the end of a query O / l to global.
 //
 // What bounds it (prefill): per 64-key tile the tensor pipe needs 36 x 32 + 8 x 81 = 1 800 cycles (2 176 with the plain
 // form for P V), and shared memory is read and written for about as long: 576 (Q K^T) + 640 (P V) + 576 (the copies).
 //
 // Tensor memory columns:   0-255  O: value dims 0-255 in columns 0-127, 256-511 in 128-255; lanes 0-63 hold the first 128
 //                                 dims of each, lanes 64-127 the second, lane l (mod 64) = head l
-//                        256-399  Q as packed bf16, 128 columns of the two halves of dims 0-511, then 16 of the rope dims
-//                        448-511  S: the first chain's partial sum in lanes 0-15 of each quarter, the second's in 16-31
+//                        256-383  Q[:, 0:512] as packed bf16, dims 0-255 in lanes 0-15 of each quarter, 256-511 in 16-31
+//                        384-511  S, two buffers: the first chain's partial sum in lanes 0-15 of each quarter, the second's
+//                                 in 16-31
 #include "lsa_internal.h"
 #include "lsa_tc.cuh"
 
@@ -49,21 +51,23 @@ constexpr int kAtoms = kDQK / 64;            // 9 column blocks of 64 dims (128 
 constexpr int kAtomBytes = 64 * 128;         // 64 rows x 128 bytes
 constexpr int kSlotBytes = kAtoms * kAtomBytes;
 
-constexpr int kSoftmaxWarps = 4, kMmaWarp = 4, kSchedWarp = 5, kGatherWarp0 = 6, kGatherWarps = 8;
-constexpr int kThreadsAttnTc = 32 * (kGatherWarp0 + kGatherWarps);
-constexpr int kRowsPerWarp = kTileKeys / kGatherWarps;   // cache rows of a tile that one gather warp copies
-constexpr uint32_t kTmemColsAttn = 512;
 constexpr int kRing = 3;                     // 64-key tiles (or Q) in shared memory
-constexpr uint32_t kColQ = 256, kColS = 448;
+constexpr int kSoftmaxWarps = 4, kQkWarp = 4, kPvWarp = 5, kSchedWarp = 6, kGatherWarp0 = 7;
+constexpr int kSlotWarps = 2;                // gather warps of a ring slot
+constexpr int kGatherWarps = kRing * kSlotWarps;
+constexpr int kThreadsAttnTc = 32 * (kGatherWarp0 + kGatherWarps);
+constexpr int kRowsPerWarp = kTileKeys / kSlotWarps;   // cache rows of a tile that one gather warp copies
+constexpr uint32_t kTmemColsAttn = 512;
+constexpr uint32_t kColQ = 256, kColS = 384, kSBuf = 64;
 constexpr float kLog2eTc = 1.4426950408889634f;
 constexpr int kMaxClusterSplit = 8;          // row splits of one sequence = blocks of one cluster (portable limit)
 constexpr float kRescaleGap = 8.f;           // rescale O only when the row max grows by more than 2^8
-constexpr int kJobReaders = kSoftmaxWarps + 1 + kGatherWarps;   // warps that release a job slot
+constexpr int kJobReaders = kSoftmaxWarps + 2 + kGatherWarps;   // warps that release a job slot
 
 struct AttnTcSmem {
   alignas(1024) uint8_t k[kRing][kAtoms][kAtomBytes];       // [ring slot][column block][64 rows x 128 B]
-  alignas(1024) uint8_t p[kTileKeys * 128];                 // P: 64 heads x 64 keys bf16, 128B-swizzled K-major
-  alignas(8) uint64_t k_full[kRing], k_empty[kRing], q_tmem[2], s_full, s_free, p_ready, job_full[2], job_empty[2], clc_full;
+  alignas(1024) uint8_t q_rope[kAtomBytes];                 // Q[:, 512:576], 64 rows x 128 B
+  alignas(8) uint64_t k_full[kRing], k_empty[kRing], p_ready[kRing], q_tmem[2], s_full[2], s_free[2], job_full[2], job_empty[2], clc_full;
   alignas(8) uint64_t recv_full;          // two-split launches: the peer's rows and log-sum-exps have arrived
   alignas(16) uint4 clc;                  // answer of the cluster launch control
   alignas(8) int2 job[2];                 // {query or -1 = no more, rows it attends}
@@ -121,6 +125,18 @@ __device__ __forceinline__ float exp2_fast(float x) {
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+  float2 r;
+  asm("{\n\t.reg .b64 x, y;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\tadd.rn.f32x2 x, x, y;\n\tmov.b64 {%0, %1}, x;\n\t}"
+      : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return r;
+}
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+  float2 r;
+  asm("{\n\t.reg .b64 x, y, z;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\tmov.b64 z, {%6, %7};\n\tfma.rn.f32x2 x, x, y, z;\n\tmov.b64 {%0, %1}, x;\n\t}"
+      : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+  return r;
+}
 // Four 8x8 bf16 matrices from the fragments of a warp; lane l gives the address of row l % 8 of matrix l / 8.
 __device__ __forceinline__ void stmatrix_x4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
   asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
@@ -168,9 +184,9 @@ __device__ __forceinline__ bool clc_answer(uint32_t answer, int* block_x) {
 //   they stay in L2; after one cluster barrier the owner of a row combines its own part with the others'.  (Loads from
 //   a peer's shared memory moved the same rows at about a quarter of the L2 path's rate.)
 //
-// q_tma != 0: q_map describes q as a bf16 matrix [n_query * 64, 576] and Q arrives as nine TMA boxes; otherwise the
+// q_tma != 0: q_map describes q as a bf16 matrix [n_query * 64, 576] and Q arrives as one TMA box; otherwise the
 // gather warps copy it with cp.async.  k_tma != 0 (contiguous caches only): k_map describes the cache rows, and key
-// tiles that lie wholly inside the window, 64 consecutive rows, arrive as nine TMA boxes as well.  k_g4 != 0: g_map
+// tiles that lie wholly inside the window, 64 consecutive rows, arrive as one TMA box as well.  k_g4 != 0: g_map
 // describes the cache rows with a box one row high, and every other key tile is gathered four rows per instruction.
 //
 //   kRows       the caller's row lists are walked (else [window | sink | sparse] of a contiguous cache)
@@ -196,14 +212,14 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
   // ---- set-up
   if (tid == 0) {
     for (int b = 0; b < kRing; ++b) {
-      tc::mbar_init(smem_u32(&sm.k_full[b]), kGatherWarps);
+      tc::mbar_init(smem_u32(&sm.k_full[b]), kSlotWarps);
       tc::mbar_init(smem_u32(&sm.k_empty[b]), 1);
+      tc::mbar_init(smem_u32(&sm.p_ready[b]), 1);
     }
-    tc::mbar_init(smem_u32(&sm.s_full), 1);
-    tc::mbar_init(smem_u32(&sm.s_free), kSoftmaxWarps);
-    tc::mbar_init(smem_u32(&sm.p_ready), 1);
     for (int b = 0; b < 2; ++b) {
       tc::mbar_init(smem_u32(&sm.q_tmem[b]), kSoftmaxWarps);   // by job parity: a job without tiles may be overtaken by the next
+      tc::mbar_init(smem_u32(&sm.s_full[b]), 1);
+      tc::mbar_init(smem_u32(&sm.s_free[b]), kSoftmaxWarps);
       tc::mbar_init(smem_u32(&sm.job_full[b]), 1);
       tc::mbar_init(smem_u32(&sm.job_empty[b]), kJobReaders);
     }
@@ -216,7 +232,7 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
     tc::fence_mbar_init();
   }
   if (tid < kH) sm.alpha[tid] = 1.f;
-  if (warp == kMmaWarp) {
+  if (warp == kQkWarp) {
     tc::tmem_alloc(smem_u32(&sm.tmem_slot), kTmemColsAttn);
     tc::tmem_relinquish();
   }
@@ -313,32 +329,14 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
     if (early_rows) dependency_wait();
   } else if (warp >= kGatherWarp0) {
     // ================= gather warps =================
-    const int gw = warp - kGatherWarp0;
-    const int lt = gw * 32 + lane;
+    const int grp = (warp - kGatherWarp0) / kSlotWarps, gw = (warp - kGatherWarp0) % kSlotWarps;   // ring slot, warp of its group
     const uint8_t* kg = reinterpret_cast<const uint8_t*>(p.k);
     const bool g4 = k_g4 != 0;   // block-uniform
-    // TMA gather (k_g4): thread lt < 128 fetches row quad lt / 8 (tile rows 4 * quad .. + 3) of column block lt % 8, and
-    // the threads with lt % 8 == 0 also the rope block: 144 instructions per tile.
-    const int quad = (lt >> 3) & 15, atom0 = lt & 7;
+    const uint32_t full = smem_u32(&sm.k_full[grp]), empty = smem_u32(&sm.k_empty[grp]);
     bool waited = !early_rows;   // this thread has executed the dependency wait
     bool alive = true;
-    // Up to three items are in flight: an item is handed over (k_full) when its cp.async group has landed, which is
-    // looked at after the next item's copies are issued, or at once when no slot is free.  One arrival per warp: hundreds
-    // of threads arriving on one barrier are as many serialised shared-memory operations.
-    int first_pend = 0, n_pend = 0;   // ring positions first_pend .. first_pend + n_pend - 1 are issued but not handed over
-    auto hand_over_oldest = [&]() {
-      if (n_pend >= 3) cp_async_wait<2>();
-      else if (n_pend == 2) cp_async_wait<1>();
-      else cp_async_wait<0>();
-      tc::fence_proxy_async();
-      __syncwarp();
-      if (lane == 0) tc::mbar_arrive(smem_u32(&sm.k_full[slot_of(first_pend)]));
-      ++first_pend;
-      --n_pend;
-    };
-    int pos = 0;   // ring position of the next item
+    int base = 0, last_pos = -1;   // ring position of the job's first item; the group's last item that is on its way
     for (int n = 0; alive; ++n) {
-      while (n_pend > 0 && !__all_sync(0xffffffffu, tc::mbar_test(smem_u32(&sm.job_full[n & 1]), (n >> 1) & 1))) hand_over_oldest();
       int2 jd;
       if (!__all_sync(0xffffffffu, wait_job(n, &jd)) || jd.x < 0) break;
       const Job jb = job_of(jd);
@@ -356,194 +354,166 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
           return checked_row(sp[i - jb.n_win - jb.n_sink], p.n_key, p.status);
         }
       };
+      auto tile_of = [&](int e) -> int { return e - (e > jb.q_at ? 1 : 0); };
       auto tile_by_tma = [&](int i) -> bool {   // block-uniform
         return !kRows && k_tma && (jb.tile_begin + i + 1) * kTileKeys <= jb.n_win;
       };
-      auto my_key_row = [&](int i) -> int32_t {   // lanes 0-7 look up the cache rows of the warp's eight keys
-        return (!g4 && i < jb.n_tiles && lane < kRowsPerWarp && !tile_by_tma(i))
+      auto my_key_row = [&](int e) -> int32_t {   // each lane looks up the cache row of one of the warp's keys
+        const int i = tile_of(e);
+        return (e != jb.q_at && e <= jb.n_tiles && lane < kRowsPerWarp && !tile_by_tma(i))
                    ? row_of((jb.tile_begin + i) * kTileKeys + kRowsPerWarp * gw + lane) : -1;
       };
-      auto my_quad_rows = [&](int i) -> int4 {
-        int4 r = make_int4(0, 0, 0, 0);
-        if (g4 && lt < 128 && i < jb.n_tiles && !tile_by_tma(i)) {
-          const int i0 = (jb.tile_begin + i) * kTileKeys + 4 * quad;
-          // rows past the end of the list are masked in the softmax: any readable row will do
-          r.x = max(row_of(i0), 0); r.y = max(row_of(i0 + 1), 0); r.z = max(row_of(i0 + 2), 0); r.w = max(row_of(i0 + 3), 0);
-        }
-        return r;
-      };
-      int32_t my_row = my_key_row(0);
-      int4 my_rows4 = my_quad_rows(0);
-      for (int e = 0; e <= jb.n_tiles; ++e, ++pos) {
+      int e = (grp + kRing - base % kRing) % kRing;
+      int32_t my_row = my_key_row(e);
+      for (; e <= jb.n_tiles; e += kRing) {
+        const int pos = base + e;
         const bool is_q = e == jb.q_at;
-        const int i = e - (e > jb.q_at ? 1 : 0);   // the tile (if this is not Q)
-        const int b = slot_of(pos);
-        const uint32_t full = smem_u32(&sm.k_full[b]), empty = smem_u32(&sm.k_empty[b]);
-        int32_t next_row = my_row;
-        int4 next_rows4 = my_rows4;
-        if (!is_q) {   // fetched before the wait: off the critical path
-          next_row = my_key_row(i + 1);
-          next_rows4 = my_quad_rows(i + 1);
+        const int i = tile_of(e);   // the tile (if this is not Q)
+        const int32_t next_row = my_key_row(e + kRing);   // fetched before the wait: off the critical path
+        if (e >= jb.q_at && !waited) {   // the tiles before Q are in flight: now the previous kernel must be done
+          dependency_wait();
+          waited = true;
         }
-        // A block's first tile goes out alone: requested together with the next ones it would share the memory pipe
-        // with them, and the first Q K^T would start two tiles' worth of traffic later
-        if (n == 0 && e == (jb.q_at == 0 ? 2 : 1)) while (n_pend > 0) hand_over_oldest();
-        while (n_pend > 0 && !__all_sync(0xffffffffu, tc::mbar_test(empty, use_of(pos) ^ 1))) hand_over_oldest();
         if (!__all_sync(0xffffffffu, tc::mbar_wait(empty, use_of(pos) ^ 1, p.status))) { alive = false; break; }
-        if (is_q) {
-          if (!waited) {   // two tiles are in flight: now the previous kernel must be done, then Q goes out
-            dependency_wait();
-            waited = true;
+        // A block's first tile goes out alone: requested together with the next one it would share the memory pipe
+        // with it, and the first Q K^T would start a tile's worth of traffic later
+        if (n == 0 && e == (jb.q_at == 0 ? 2 : 1) &&
+            !__all_sync(0xffffffffu, tc::mbar_wait(smem_u32(&sm.k_full[slot_of(pos - 1)]), 0, p.status))) { alive = false; break; }
+        last_pos = pos;
+        if (is_q && q_tma) {
+          if (gw == 0 && tc::elect_one()) {
+            tc::mbar_expect_tx_only(full, kSlotBytes);
+            tc::tma_load_3d(smem_u32(sm.k[grp]), &q_map, 0, jb.qi * kH, 0, full);
           }
-          if (q_tma) {
-            if (tc::elect_one()) {
-              tc::mbar_expect_tx_only(full, (gw == 0 ? 2 : 1) * kAtomBytes);
-              for (int a = gw; a < kAtoms; a += kGatherWarps) tc::tma_load_2d(smem_u32(sm.k[b][a]), &q_map, a * 64, jb.qi * kH, full);
-            }
-          } else {
-            const uint8_t* qg = reinterpret_cast<const uint8_t*>(p.q) + static_cast<int64_t>(jb.qi) * kH * kDQK * 2;
-            for (int x = lt; x < kH * (kDQK / 8); x += 32 * kGatherWarps) {
-              const int r = x / (kDQK / 8), c = x % (kDQK / 8);
-              cp_async16(smem_u32(sm.k[b][c >> 3]) + r * 128 + (((c & 7) ^ (r & 7)) << 4), qg + r * kDQK * 2 + c * 16, 16);
-            }
+        } else if (is_q) {
+          const uint8_t* qg = reinterpret_cast<const uint8_t*>(p.q) + static_cast<int64_t>(jb.qi) * kH * kDQK * 2;
+          for (int x = gw * 32 + lane; x < kH * (kDQK / 8); x += 32 * kSlotWarps) {
+            const int r = x / (kDQK / 8), c = x % (kDQK / 8);
+            cp_async16(smem_u32(sm.k[grp][c >> 3]) + r * 128 + (((c & 7) ^ (r & 7)) << 4), qg + r * kDQK * 2 + c * 16, 16);
           }
         } else if (tile_by_tma(i)) {
-          // 64 consecutive window rows: nine boxes, one per warp (and a second one for the first), each counted on k_full
-          if (tc::elect_one()) {
-            tc::mbar_expect_tx_only(full, (gw == 0 ? 2 : 1) * kAtomBytes);
-            const int row0 = static_cast<int>(jb.win0) + (jb.tile_begin + i) * kTileKeys;
-            for (int a = gw; a < kAtoms; a += kGatherWarps) tc::tma_load_2d(smem_u32(sm.k[b][a]), &k_map, a * 64, row0, full);
+          // 64 consecutive window rows: one box, counted on k_full
+          if (gw == 0 && tc::elect_one()) {
+            tc::mbar_expect_tx_only(full, kSlotBytes);
+            tc::tma_load_3d(smem_u32(sm.k[grp]), &k_map, 0, static_cast<int>(jb.win0) + (jb.tile_begin + i) * kTileKeys, 0, full);
           }
         } else if (g4) {
           // scattered rows: four rows x 64 dims per instruction, straight into their place in the swizzled tile
-          if (lt == 0) tc::mbar_expect_tx_only(full, kSlotBytes);
-          if (lt < 128) {
-            tc::tma_gather4_2d(smem_u32(sm.k[b][atom0]) + quad * 512, &g_map, atom0 * 64, my_rows4.x, my_rows4.y, my_rows4.z,
-                               my_rows4.w, full);
-            if (atom0 == 0)
-              tc::tma_gather4_2d(smem_u32(sm.k[b][kAtoms - 1]) + quad * 512, &g_map, (kAtoms - 1) * 64, my_rows4.x, my_rows4.y,
-                                 my_rows4.z, my_rows4.w, full);
+          if (lane == 0) tc::mbar_expect_tx_only(full, kSlotBytes / kSlotWarps);
+          __syncwarp();
+          for (int u = lane; u < kRowsPerWarp / 4 * kAtoms; u += 32) {
+            const int q4 = u / kAtoms, atom = u % kAtoms;
+            int4 r;
+            // rows past the end of the list are masked in the softmax: any readable row will do
+            const int i0 = (jb.tile_begin + i) * kTileKeys + kRowsPerWarp * gw + 4 * q4;
+            r.x = max(row_of(i0), 0); r.y = max(row_of(i0 + 1), 0); r.z = max(row_of(i0 + 2), 0); r.w = max(row_of(i0 + 3), 0);
+            tc::tma_gather4_2d(smem_u32(sm.k[grp][atom]) + (kRowsPerWarp * gw + 4 * q4) * 128, &g_map, atom * 64, r.x, r.y, r.z, r.w, full);
           }
         } else {
           // the 72 16-byte chunks of a row: 64 by all lanes in two instructions; the last eight of four rows in one
-          const uint32_t dst0 = smem_u32(sm.k[b][lane >> 3]) + kRowsPerWarp * gw * 128;
-#pragma unroll
+          const uint32_t dst0 = smem_u32(sm.k[grp][lane >> 3]) + kRowsPerWarp * gw * 128;
+#pragma unroll 8
           for (int rr = 0; rr < kRowsPerWarp; ++rr) {
             const int32_t row = __shfl_sync(0xffffffffu, my_row, rr);
             const uint8_t* src = kg + static_cast<int64_t>(row >= 0 ? row : 0) * p.ld_k * 2 + lane * 16;
             const int nb = row >= 0 ? 16 : 0;
-            const uint32_t dst = dst0 + rr * 128 + (((lane & 7) ^ rr) << 4);
+            const uint32_t dst = dst0 + rr * 128 + (((lane & 7) ^ (rr & 7)) << 4);
             cp_async16(dst, src, nb);
             cp_async16(dst + 4 * kAtomBytes, src + 512, nb);
             if ((rr & 3) == 3) {
-              const int r4 = (rr & 4) + (lane >> 3);
+              const int r4 = rr - 3 + (lane >> 3);
               const int32_t row4 = __shfl_sync(0xffffffffu, my_row, r4);
-              cp_async16(smem_u32(sm.k[b][8]) + (kRowsPerWarp * gw + r4) * 128 + (((lane & 7) ^ r4) << 4),
+              cp_async16(smem_u32(sm.k[grp][8]) + (kRowsPerWarp * gw + r4) * 128 + (((lane & 7) ^ (r4 & 7)) << 4),
                          kg + static_cast<int64_t>(row4 >= 0 ? row4 : 0) * p.ld_k * 2 + 1024 + (lane & 7) * 16, row4 >= 0 ? 16 : 0);
             }
           }
         }
         cp_async_commit();
-        ++n_pend;
-        if (n_pend == kRing) hand_over_oldest();
+        cp_async_wait<0>();
+        tc::fence_proxy_async();
+        __syncwarp();   // one arrival per warp: dozens of threads on one barrier are as many serialised shared-memory operations
+        if (lane == 0) tc::mbar_arrive(full);
         my_row = next_row;
-        my_rows4 = next_rows4;
       }
+      base += jb.n_tiles + 1;
       __syncwarp();
       if (lane == 0) tc::mbar_arrive(smem_u32(&sm.job_empty[n & 1]));
     }
-    while (n_pend > 0) hand_over_oldest();
-    if (!alive && gw == 0)   // a wait ran out: boxes still on their way land before the block ends (the wait is bounded too)
-      for (int q = max(0, pos - kRing); q < pos; ++q) (void)tc::mbar_wait(smem_u32(&sm.k_full[slot_of(q)]), use_of(q), nullptr);
+    // a wait ran out: a box still on its way lands before the block ends (the wait is bounded too)
+    if (!alive && last_pos >= 0) (void)tc::mbar_wait(full, use_of(last_pos), nullptr);
     if (!waited) dependency_wait();
-  } else if (warp == kMmaWarp) {
-    // ================= MMA issuer =================
+  } else if (warp == kQkWarp) {
+    // ================= issuer of Q K^T =================
     if (tc::elect_one()) {
-      constexpr uint32_t idesc_qk = tc::idesc_bf16(kH, kTileKeys, 0, 0);
-      constexpr uint32_t idesc_pv = tc::idesc_bf16(kH, 256, 0, 1);   // B = V read MN-major
+      constexpr uint32_t idesc = tc::idesc_bf16(kH, kTileKeys, 0, 0);
       // Descriptors are built once; inside the loops only the start-address word moves (one add per operand).
-      const uint64_t dk0 = tc::smem_desc_sw128(smem_u32(sm.k), 16, 1024);           // K-major view (Q K^T)
-      const uint64_t dv0 = tc::smem_desc_sw128(smem_u32(sm.k), kAtomBytes, 1024);   // MN-major view (P V)
-      const uint64_t dp0 = tc::smem_desc_sw128(smem_u32(sm.p), 16, 1024);
+      const uint64_t dk0 = tc::smem_desc_sw128(smem_u32(sm.k), 16, 1024);           // K-major view
+      const uint64_t dqr = tc::smem_desc_sw128(smem_u32(sm.q_rope), 16, 1024);
       constexpr uint32_t kLane16 = 16u << 16;
       bool ok = true;
-      int base = 0, tiles_done = 0;   // ring position of the job's first item; tiles of the jobs before it
+      int base = 0, g = 0;   // ring position of the job's first item; tile number over all jobs
       for (int n = 0; ok; ++n) {
         int2 jd;
         if (!wait_job(n, &jd) || jd.x < 0) break;
         const Job jb = job_of(jd);
-        ok = tc::mbar_wait(smem_u32(&sm.q_tmem[n & 1]), (n >> 1) & 1, p.status);
-        if (!ok) break;
-        tc::mbar_arrive(smem_u32(&sm.k_empty[slot_of(base + jb.q_at)]));   // Q is in tensor memory: its ring slot is free
-        tc::fence_after_sync();
-        auto pos_of = [&](int i) -> int { return base + i + (i >= jb.q_at ? 1 : 0); };
-        auto issue_qk = [&](int i) {
+        if (!tc::mbar_wait(smem_u32(&sm.q_tmem[n & 1]), (n >> 1) & 1, p.status)) break;
+        tc::mbar_arrive(smem_u32(&sm.k_empty[slot_of(base + jb.q_at)]));   // Q has left its ring slot
+        for (int i = 0; i < jb.n_tiles; ++i, ++g) {
+          const int pos = base + i + (i >= jb.q_at ? 1 : 0);
+          ok = tc::mbar_wait(smem_u32(&sm.k_full[slot_of(pos)]), use_of(pos), p.status) &&
+               tc::mbar_wait(smem_u32(&sm.s_free[g & 1]), ((g >> 1) & 1) ^ 1, p.status);   // the S before last has been read
+          if (ok && p.qk_waits_pv != 0 && i >= 2) {   // (a debugging aid: no product needs it)
+            const int pp = base + i - 2 + (i - 2 >= jb.q_at ? 1 : 0);
+            ok = tc::mbar_wait(smem_u32(&sm.k_empty[slot_of(pp)]), use_of(pp), p.status);
+          }
+          if (!ok) break;
           tc::fence_after_sync();
-          const uint64_t dkb = tc::desc_advance(dk0, slot_of(pos_of(i)) * kSlotBytes);
+          const uint64_t dkb = tc::desc_advance(dk0, slot_of(pos) * kSlotBytes);
 #pragma unroll
           for (int x = 0; x < 2; ++x) {
-            const uint32_t q_src = tmem_base + x * kLane16 + kColQ, s_dst = tmem_base + x * kLane16 + kColS;
+            const uint32_t q_src = tmem_base + x * kLane16 + kColQ, s_dst = tmem_base + x * kLane16 + kColS + (g & 1) * kSBuf;
 #pragma unroll
             for (int s = 0; s < 16; ++s)   // dims 256x + 16s .. +15: column block 4x + s/4, 32-byte slice s%4
-              tc::umma_ts(s_dst, q_src + 8 * s, tc::desc_advance(dkb, (4 * x + (s >> 2)) * kAtomBytes + (s & 3) * 32), idesc_qk, s != 0);
+              tc::umma_ts(s_dst, q_src + 8 * s, tc::desc_advance(dkb, (4 * x + (s >> 2)) * kAtomBytes + (s & 3) * 32), idesc, s != 0);
 #pragma unroll
             for (int s = 0; s < 2; ++s)    // rope dims 512 + 32x + 16s .. +15
-              tc::umma_ts(s_dst, q_src + 128 + 8 * s, tc::desc_advance(dkb, 8 * kAtomBytes + (2 * x + s) * 32), idesc_qk, 1);
+              tc::umma_ss(s_dst, tc::desc_advance(dqr, (2 * x + s) * 32), tc::desc_advance(dkb, 8 * kAtomBytes + (2 * x + s) * 32), idesc, 1);
           }
-          tc::umma_commit(smem_u32(&sm.s_full));
-        };
-        auto issue_pv = [&](int j) {
+          tc::umma_commit(smem_u32(&sm.s_full[g & 1]));
+        }
+        base += jb.n_tiles + 1;
+        if (ok) tc::mbar_arrive(smem_u32(&sm.job_empty[n & 1]));
+      }
+    }
+  } else if (warp == kPvWarp) {
+    // ================= issuer of P V =================
+    if (tc::elect_one()) {
+      constexpr uint32_t idesc = tc::idesc_bf16(kH, 256, 0, 1);   // B = V read MN-major
+      const uint64_t dv0 = tc::smem_desc_sw128(smem_u32(sm.k), kAtomBytes, 1024);   // MN-major view of a tile
+      const uint64_t dp0 = tc::smem_desc_sw128(smem_u32(sm.k[0][8]), 16, 1024);     // P in its rope block
+      bool ok = true;
+      int base = 0, g = 0;
+      for (int n = 0; ok; ++n) {
+        int2 jd;
+        if (!wait_job(n, &jd) || jd.x < 0) break;
+        const Job jb = job_of(jd);
+        for (int i = 0; i < jb.n_tiles; ++i, ++g) {
+          const int slot = slot_of(base + i + (i >= jb.q_at ? 1 : 0));
+          ok = tc::mbar_wait(smem_u32(&sm.p_ready[g % kRing]), (g / kRing) & 1, p.status);
+          if (!ok) break;
           tc::fence_after_sync();
-          const uint64_t dvb = tc::desc_advance(dv0, slot_of(pos_of(j)) * kSlotBytes);
+          const uint64_t dvb = tc::desc_advance(dv0, slot * kSlotBytes), dpb = tc::desc_advance(dp0, slot * kSlotBytes);
 #pragma unroll
           for (int y = 0; y < 2; ++y)       // value dims 256y .. +255
 #pragma unroll
             for (int kk = 0; kk < kTileKeys / 16; ++kk)   // keys 16*kk .. +15
-              tc::umma_ws_ss(tmem_base + 128 * y, tc::desc_advance(dp0, kk * 32), tc::desc_advance(dvb, 4 * y * kAtomBytes + kk * 2048),
-                             idesc_pv, (j > 0) || (kk > 0));
-          // one completion signal per tile: "P V of tile j done" frees the ring slot for the gather warps and tells the
-          // softmax warps that O and P may be touched again
-          tc::umma_commit(smem_u32(&sm.k_empty[slot_of(pos_of(j))]));
-        };
-        // Two in-order queues, "next Q K^T" (one tile ahead of P V at most: S has one buffer) and "next P V".
-        int qk_next = 0, pv_next = 0;
-        long long t_idle = 0;
-        uint32_t spins = 0;
-        while (ok && pv_next < jb.n_tiles) {
-          bool did = false;
-          if (pv_next < qk_next && tc::mbar_test(smem_u32(&sm.p_ready), (tiles_done + pv_next) & 1)) {
-            issue_pv(pv_next++);
-            did = true;
-          } else if (qk_next < jb.n_tiles && qk_next <= pv_next + 1) {
-            const int g = tiles_done + qk_next;
-            // the softmax warps have read the S of the tile before; p.qk_waits_pv: and the P V before that is complete
-            if ((g == 0 || tc::mbar_test(smem_u32(&sm.s_free), (g - 1) & 1)) &&
-                tc::mbar_test(smem_u32(&sm.k_full[slot_of(pos_of(qk_next))]), use_of(pos_of(qk_next))) &&
-                (p.qk_waits_pv == 0 || qk_next < 2 ||
-                 tc::mbar_test(smem_u32(&sm.k_empty[slot_of(pos_of(qk_next - 2))]), use_of(pos_of(qk_next - 2))))) {
-              issue_qk(qk_next++);
-              did = true;
-            }
-          }
-          if (did) {
-            spins = 0;
-          } else if ((++spins & 255u) == 0) {
-            // bounded: nothing became ready for about a second (the clock is read only while spinning)
-            if (tc::status_raised(p.status)) {
-              ok = false;
-            } else {
-              const long long now = clock64();
-              if (spins == 256u) {
-                t_idle = now;
-              } else if (now - t_idle > tc::kWaitCycles) {
-                report_status(p.status, kDevTimeout);
-                ok = false;
-              }
-            }
-          }
+              tc::umma_ws_ss(tmem_base + 128 * y, tc::desc_advance(dpb, kk * 32), tc::desc_advance(dvb, 4 * y * kAtomBytes + kk * 2048),
+                             idesc, (i > 0) || (kk > 0));
+          // one completion signal per tile: "P V of the tile done" frees the ring slot for the gather warps and tells the
+          // softmax warps that O may be touched again
+          tc::umma_commit(smem_u32(&sm.k_empty[slot]));
         }
         base += jb.n_tiles + 1;
-        tiles_done += jb.n_tiles;
         if (ok) tc::mbar_arrive(smem_u32(&sm.job_empty[n & 1]));
       }
     }
@@ -572,15 +542,12 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
         }
         tc::tmem_st32(tmem_base + lane_addr + kColQ + part * 32, w);
       }
-      {
-        uint32_t w[16];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const uint4 u = *reinterpret_cast<const uint4*>(qs + 8 * kAtomBytes + (((4 * hi + j) ^ (row & 7)) << 4));
-          w[4 * j] = u.x; w[4 * j + 1] = u.y; w[4 * j + 2] = u.z; w[4 * j + 3] = u.w;
-        }
-        tc::tmem_st16(tmem_base + lane_addr + kColQ + 128, w);
+      for (int j = 0; j < 4; ++j) {   // the warp's 16 rows of the rope block, as they lie
+        const int at = 16 * warp * 128 + (32 * j + lane) * 16;
+        *reinterpret_cast<uint4*>(sm.q_rope + at) = *reinterpret_cast<const uint4*>(sm.k[slot_of(pos)][8] + at);
       }
+      tc::fence_proxy_async();
       tc::tmem_st_wait();
       tc::fence_before_sync();
       __syncwarp();
@@ -602,27 +569,30 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
       bool failed = false;
       for (int i = 0; i < jb.n_tiles; ++i) {
         const int g = tiles_done + i;
-        ok = ok && __all_sync(0xffffffffu, tc::mbar_wait(smem_u32(&sm.s_full), g & 1, p.status));
+        const int slot = slot_of(base + i + (i >= jb.q_at ? 1 : 0));
+        ok = ok && __all_sync(0xffffffffu, tc::mbar_wait(smem_u32(&sm.s_full[g & 1]), (g >> 1) & 1, p.status));
         tc::fence_after_sync();
-        float v[32];
+        float2 v[16];   // [key group j][row r] at 2j + r
         {
           uint32_t a[32], c[32];
-          tc::tmem_ld_16x256b_x8(tmem_base + lane_addr + kColS, a);
-          tc::tmem_ld_16x256b_x8(tmem_base + lane_addr + (16u << 16) + kColS, c);
+          tc::tmem_ld_16x256b_x8(tmem_base + lane_addr + kColS + (g & 1) * kSBuf, a);
+          tc::tmem_ld_16x256b_x8(tmem_base + lane_addr + (16u << 16) + kColS + (g & 1) * kSBuf, c);
           tc::tmem_ld_wait();
           tc::fence_before_sync();
           __syncwarp();
-          if (lane == 0) tc::mbar_arrive(smem_u32(&sm.s_free));
+          if (lane == 0) tc::mbar_arrive(smem_u32(&sm.s_free[g & 1]));
 #pragma unroll
-          for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(a[j]) + __uint_as_float(c[j]);
+          for (int j = 0; j < 16; ++j)
+            v[j] = add2(make_float2(__uint_as_float(a[2 * j]), __uint_as_float(a[2 * j + 1])),
+                        make_float2(__uint_as_float(c[2 * j]), __uint_as_float(c[2 * j + 1])));
         }
         const int n_valid = jb.n_tot - (jb.tile_begin + i) * kTileKeys;   // keys of this tile that exist
         if (n_valid < kTileKeys) {
           const int k0 = 2 * (lane & 3);
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
-            if (8 * j + k0 >= n_valid) v[4 * j] = v[4 * j + 2] = -INFINITY;
-            if (8 * j + k0 + 1 >= n_valid) v[4 * j + 1] = v[4 * j + 3] = -INFINITY;
+            if (8 * j + k0 >= n_valid) v[2 * j].x = v[2 * j + 1].x = -INFINITY;
+            if (8 * j + k0 + 1 >= n_valid) v[2 * j].y = v[2 * j + 1].y = -INFINITY;
           }
         }
         // running max in log2 units, moved only when it grows by more than kRescaleGap (O and l are then rescaled)
@@ -630,9 +600,9 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
         float alpha[2] = {1.f, 1.f};
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
-          float mx = fmaxf(v[2 * r], v[2 * r + 1]);
+          float mx = fmaxf(v[r].x, v[r].y);
 #pragma unroll
-          for (int j = 1; j < 8; ++j) mx = fmaxf(mx, fmaxf(v[4 * j + 2 * r], v[4 * j + 2 * r + 1]));
+          for (int j = 1; j < 8; ++j) mx = fmaxf(mx, fmaxf(v[2 * j + r].x, v[2 * j + r].y));
           mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
           mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
           mx *= zs;
@@ -648,24 +618,23 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
         uint32_t pk[8][2];
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
-          float sum = 0.f;
+          const float2 z2 = make_float2(zs, zs), m2 = make_float2(-m_used[r], -m_used[r]);
+          float2 sum2 = make_float2(0.f, 0.f);
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
-            const float p0 = exp2_fast(fmaf(v[4 * j + 2 * r], zs, -m_used[r]));
-            const float p1 = exp2_fast(fmaf(v[4 * j + 2 * r + 1], zs, -m_used[r]));
-            sum += p0 + p1;
-            pk[j][r] = pack_bf16(p0, p1);
+            float2 e = fma2(v[2 * j + r], z2, m2);
+            e.x = exp2_fast(e.x);
+            e.y = exp2_fast(e.y);
+            sum2 = add2(sum2, e);
+            pk[j][r] = pack_bf16(e.x, e.y);
           }
+          const float sum = sum2.x + sum2.y;
           l_run[r] = l_run[r] * alpha[r] + sum;
         }
-        // P (and O, below) may be touched once P V of the tile before is complete; at i = 0 the job before has seen to it
-        if (i > 0) {
-          const int pp = base + i - 1 + (i - 1 >= jb.q_at ? 1 : 0);
-          ok = ok && __all_sync(0xffffffffu, tc::mbar_wait(smem_u32(&sm.k_empty[slot_of(pp)]), use_of(pp), p.status));
-        }
+        // P takes the place of the tile's rope dims, which only Q K^T reads
         {
           const int row = 16 * warp + ((lane >> 3) & 1) * 8 + (lane & 7);
-          const uint32_t dst = smem_u32(sm.p) + row * 128;
+          const uint32_t dst = smem_u32(sm.k[slot][8]) + row * 128;
 #pragma unroll
           for (int j = 0; j < 8; j += 2)
             stmatrix_x4(dst + (((j + (lane >> 4)) ^ (row & 7)) << 4), pk[j][0], pk[j][1], pk[j + 1][0], pk[j + 1][1]);
@@ -682,7 +651,11 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
             failed = true;
             break;
           }
-          // rare: O of every head times its factor
+          // rare: O of every head times its factor, once P V of the tile before is complete
+          if (i > 0) {
+            const int pp = base + i - 1 + (i - 1 >= jb.q_at ? 1 : 0);
+            ok = ok && __all_sync(0xffffffffu, tc::mbar_wait(smem_u32(&sm.k_empty[slot_of(pp)]), use_of(pp), p.status));
+          }
           tc::fence_after_sync();
           const float al = sm.alpha[head_o];
 #pragma unroll 1
@@ -699,7 +672,7 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
           softmax_sync();
           if (need && (lane & 3) == 0) sm.alpha[16 * warp + (lane >> 2)] = sm.alpha[16 * warp + (lane >> 2) + 8] = 1.f;
         }
-        if (tid == 0) tc::mbar_arrive(smem_u32(&sm.p_ready));
+        if (tid == 0) tc::mbar_arrive(smem_u32(&sm.p_ready[g % kRing]));
       }
       if (failed) break;
       // ---- row sums and log-sum-exps of the job, for the threads that read O
@@ -848,7 +821,7 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
   }
   tc::fence_before_sync();
   __syncthreads();
-  if (warp == kMmaWarp) tc::tmem_dealloc(tmem_base, kTmemColsAttn);
+  if (warp == kQkWarp) tc::tmem_dealloc(tmem_base, kTmemColsAttn);
   if constexpr (kClustered) {
     // ---- merge of the splits (Sec. 4.1.1: online-softmax rescaling) for this block's heads: weights
     // 2^(lse_j - max) / sum, O = sum_j w_j O_j, bf16 to global.
@@ -899,7 +872,7 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
         __threadfence();
       }
       cluster_sync_all();   // every block of the cluster has written its rows
-      // Warp w finishes rows w, w + 14, ... of this block's share (at most two).  Lane 8k + j first fetches the
+      // Warp w finishes rows w, w + 13, ... of this block's share (at most two).  Lane 8k + j first fetches the
       // log-sum-exp of split j for the warp's k-th row, so that all of them are in flight together.
       constexpr int kMost = (kH / 4 + kWarps - 1) / kWarps;
       const int k_of = lane >> 3, j_of = lane & 7;
@@ -1007,10 +980,10 @@ cudaError_t launch_attn_tc(const AttnArgs& a, cudaStream_t st, int64_t* n_launch
   if (e != cudaSuccess) return e;
   CUtensorMap q_map{}, k_map{}, g_map{};
   const int q_tma = (reinterpret_cast<uintptr_t>(a.q) & 15u) == 0 &&
-                    make_map_bf16_rows(&q_map, a.q, kDQK, static_cast<uint64_t>(a.n_query) * kH, kH);
+                    make_map_bf16_tile(&q_map, a.q, kDQK, static_cast<uint64_t>(a.n_query) * kH, kH, kAtoms);
   // contiguous cache: the last query sees rows 0 .. q_pos0 + n_query - 1, so the cache holds at least that many
   const int k_tma = !a.paged && a.rows == nullptr && a.ld_k % 8 == 0 && (reinterpret_cast<uintptr_t>(a.k) & 15u) == 0 &&
-                    make_map_bf16_rows(&k_map, a.k, static_cast<uint64_t>(a.ld_k), static_cast<uint64_t>(a.q_pos0 + a.n_query), kTileKeys);
+                    make_map_bf16_tile(&k_map, a.k, static_cast<uint64_t>(a.ld_k), static_cast<uint64_t>(a.q_pos0 + a.n_query), kTileKeys, kAtoms);
   // gather of scattered rows by TMA: any cache whose base and row pitch TMA can address; a paged pool's row count is
   // not known here (every row number comes from the caller's list), so its map spans the whole coordinate range
   const uint64_t g_rows = a.paged || a.rows != nullptr ? 0x7fffffffull : static_cast<uint64_t>(a.q_pos0 + a.n_query);

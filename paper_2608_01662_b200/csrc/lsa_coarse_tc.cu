@@ -267,6 +267,17 @@ bool make_map_bf16_rows(CUtensorMap* map, const void* base, uint64_t cols, uint6
             box_rows == 1 ? CU_TENSOR_MAP_L2_PROMOTION_L2_128B : CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
+bool make_map_bf16_tile(CUtensorMap* map, const void* base, uint64_t ld, uint64_t rows, uint32_t box_rows, uint32_t n_blocks) {
+  EncodeTiledFn fn = encode_tiled_fn();
+  if (fn == nullptr) return false;
+  const cuuint64_t dims[3] = {64, rows, n_blocks};
+  const cuuint64_t strides[2] = {ld * 2, 128};
+  const cuuint32_t box[3] = {64, box_rows, n_blocks};
+  const cuuint32_t estr[3] = {1, 1, 1};
+  return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
 
 namespace {
 

@@ -86,6 +86,13 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map
       : "memory");
 }
 
+__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, int c0, int c1, int c2, uint32_t bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
+      ::"r"(dst), "l"(map), "r"(bar), "r"(c0), "r"(c1), "r"(c2)
+      : "memory");
+}
+
 // Four rows of a 2-D tensor (row numbers r0..r3, any order, this GPU's memory), columns c0 .. c0 + box width - 1 of
 // each, land as four consecutive rows at `dst`.  The tensor map's box must be one row high.  c0 * element size must
 // be a multiple of 16 bytes; with a 128-byte swizzle `dst` must be 512-byte aligned for the rows to take their place
@@ -299,5 +306,8 @@ bool make_map_bf16_128(CUtensorMap* map, const void* base, uint64_t rows, uint32
 // bytes [rows, 128] row-major (e4m3 codes of a 128-dim key per row), box = the whole row x box_rows rows, 128-byte swizzle.
 bool make_map_u8_128(CUtensorMap* map, const void* base, uint64_t rows, uint32_t box_rows);
 bool make_map_bf16_rows(CUtensorMap* map, const void* base, uint64_t cols, uint64_t rows, uint32_t box_rows);
+// A bf16 matrix [rows, ld] seen as [n_blocks of 64 columns][rows][64 columns]: one box (coordinates 0, row, 0) brings
+// box_rows rows x n_blocks column blocks, each block a 128-byte swizzled tile of its own, block after block.
+bool make_map_bf16_tile(CUtensorMap* map, const void* base, uint64_t ld, uint64_t rows, uint32_t box_rows, uint32_t n_blocks);
 
 }  // namespace lsa
