@@ -61,6 +61,7 @@ constexpr uint32_t kTmemColsAttn = 512;
 constexpr uint32_t kColQ = 256, kColS = 384, kSBuf = 64;
 constexpr float kLog2eTc = 1.4426950408889634f;
 constexpr int kMaxClusterSplit = 8;          // row splits of one sequence = blocks of one cluster (portable limit)
+constexpr int kFirstTileCycles = 8192;       // longest that a block's second tile is held back for the first
 constexpr float kRescaleGap = 8.f;           // rescale O only when the row max grows by more than 2^8
 constexpr int kJobReaders = kSoftmaxWarps + 2 + kGatherWarps;   // warps that release a job slot
 
@@ -376,9 +377,13 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
         }
         if (!__all_sync(0xffffffffu, tc::mbar_wait(empty, use_of(pos) ^ 1, p.status))) { alive = false; break; }
         // A block's first tile goes out alone: requested together with the next one it would share the memory pipe
-        // with it, and the first Q K^T would start a tile's worth of traffic later
-        if (n == 0 && e == (jb.q_at == 0 ? 2 : 1) &&
-            !__all_sync(0xffffffffu, tc::mbar_wait(smem_u32(&sm.k_full[slot_of(pos - 1)]), 0, p.status))) { alive = false; break; }
+        // with it, and the first Q K^T would start a tile's worth of traffic later.  (A look with a limit, not a wait: this
+        // group is not the barrier's own waiter.)
+        if (n == 0 && e == (jb.q_at == 0 ? 2 : 1)) {
+          const long long t0 = clock64();
+          while (!tc::mbar_test(smem_u32(&sm.k_full[slot_of(pos - 1)]), 0) && clock64() - t0 < kFirstTileCycles) {}
+          __syncwarp();
+        }
         last_pos = pos;
         if (is_q && q_tma) {
           if (gw == 0 && tc::elect_one()) {
