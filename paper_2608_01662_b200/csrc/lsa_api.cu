@@ -9,6 +9,9 @@
 
 #include "lsa_internal.h"
 
+constexpr int kMaxHostLayers = 16;
+constexpr int kHostSlots = 1 + kMaxHostLayers;
+
 struct lsa_ctx {
   int device;
   cudaStream_t stream;
@@ -17,9 +20,10 @@ struct lsa_ctx {
   int sm_count;
   int64_t launches;
   char cuda_msg[256];
-  // lsa_layer_group_host only
+  // lsa_layer_group_host only.  Per staging area: slot 0 the indexer's tensors, slot 1 + l layer l (created on first use).
   cudaStream_t copy_in, copy_out;
-  cudaEvent_t ev_in[2], ev_done[2], ev_out[2];
+  cudaEvent_t ev_in[2][kHostSlots], ev_done[2][kHostSlots], ev_out[2][kHostSlots], ev_start;
+  int n_host_slots;
   // per-kernel timing (lsa_profile_*): event pairs recorded around the launches of each kernel class
   int tune[LSA_TUNE_COUNT];
   // Row lists of the last kernel launched through this context, if that kernel was a paged attention launch: the next
@@ -384,11 +388,7 @@ int lsa_create(lsa_ctx** ctx, int device, void* cuda_stream, void* workspace, si
   e = cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, device);
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&c->copy_in, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&c->copy_out, cudaStreamNonBlocking);
-  for (int i = 0; i < 2 && e == cudaSuccess; ++i) {
-    e = cudaEventCreateWithFlags(&c->ev_in[i], cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_done[i], cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_out[i], cudaEventDisableTiming);
-  }
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_start, cudaEventDisableTiming);
   if (e == cudaSuccess && c->ws) e = cudaMemsetAsync(c->ws, 0, kStatusBytes, c->stream);
   if (e != cudaSuccess) {
     delete c;
@@ -401,11 +401,11 @@ int lsa_create(lsa_ctx** ctx, int device, void* cuda_stream, void* workspace, si
 int lsa_destroy(lsa_ctx* c) {
   if (c == nullptr) return LSA_ERR_ARG;
   cudaSetDevice(c->device);
-  for (int i = 0; i < 2; ++i) {
-    if (c->ev_in[i]) cudaEventDestroy(c->ev_in[i]);
-    if (c->ev_done[i]) cudaEventDestroy(c->ev_done[i]);
-    if (c->ev_out[i]) cudaEventDestroy(c->ev_out[i]);
-  }
+  for (int i = 0; i < 2; ++i)
+    for (int l = 0; l < kHostSlots; ++l)
+      for (cudaEvent_t ev : {c->ev_in[i][l], c->ev_done[i][l], c->ev_out[i][l]})
+        if (ev) cudaEventDestroy(ev);
+  if (c->ev_start) cudaEventDestroy(c->ev_start);
   if (c->prof_ev) {
     for (int i = 0; i < 2 * kProfPairs; ++i) cudaEventDestroy(c->prof_ev[i]);
     delete[] c->prof_ev;
@@ -708,14 +708,25 @@ int lsa_layer_group_host(lsa_ctx* c, const lsa_params* p, const void* q_idx_host
   if (stage == nullptr || stage[0] == nullptr || stage[1] == nullptr || stage_bytes < need) return LSA_ERR_WORKSPACE;
   if (q_idx_host == nullptr || w_host == nullptr || q_host == nullptr || out_host == nullptr || n_query < 0 || q_pos0 < 0) return LSA_ERR_ARG;
   const int R = p->n_layers;
-  if (R > 16) return LSA_ERR_SHAPE;
+  if (R > kMaxHostLayers) return LSA_ERR_SHAPE;
+  if (k == nullptr || v == nullptr) return LSA_ERR_ARG;
+  for (int l = 0; l < R; ++l)
+    if (q_host[l] == nullptr || k[l] == nullptr || v[l] == nullptr || out_host[l] == nullptr) return LSA_ERR_ARG;
   const size_t b_qi = static_cast<size_t>(p->n_heads_idx) * p->d_idx * 2, b_w = static_cast<size_t>(p->n_heads_idx) * 4;
   const size_t b_q = static_cast<size_t>(p->n_heads) * p->d_qk * 2, b_o = static_cast<size_t>(p->n_heads) * p->d_v * 2;
   cudaError_t e = cudaSuccess;
+  for (; c->n_host_slots < 1 + R && e == cudaSuccess; ++c->n_host_slots)
+    for (int s = 0; s < 2 && e == cudaSuccess; ++s)
+      for (cudaEvent_t* ev : {&c->ev_in[s][c->n_host_slots], &c->ev_done[s][c->n_host_slots], &c->ev_out[s][c->n_host_slots]})
+        if (e == cudaSuccess && *ev == nullptr) e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming);
+  if (e != cudaSuccess) return cuda_fail(c, e);
   const int64_t n_pass = (n_query + sq - 1) / sq;
   // the caller's earlier work on the context stream must be visible to the copy streams
-  e = cudaEventRecord(c->ev_done[0], c->stream);
-  if (e == cudaSuccess) e = cudaStreamWaitEvent(c->copy_in, c->ev_done[0], 0);
+  e = cudaEventRecord(c->ev_start, c->stream);
+  if (e == cudaSuccess) e = cudaStreamWaitEvent(c->copy_in, c->ev_start, 0);
+  // Every tensor is handed on by itself: the indexer starts when its queries are there, a layer when its q is, and an output
+  // leaves when its layer is done, so that outside the stream of copies there is one layer's time and one output's copy at
+  // the end.  (The bus bounds this call.  2048 queries of the 64-head shape, four layers, 512 a pass: 1.18 GB over it.)
   for (int64_t i = 0; i < n_pass && e == cudaSuccess; ++i) {
     const int s = static_cast<int>(i & 1);
     const int64_t q0 = i * sq, n = n_query - q0 < sq ? n_query - q0 : sq;
@@ -723,34 +734,49 @@ int lsa_layer_group_host(lsa_ctx* c, const lsa_params* p, const void* q_idx_host
     size_t off = 0;
     uint8_t* d_qi = base + off; off += align_up(static_cast<size_t>(sq) * b_qi, 256);
     uint8_t* d_w = base + off; off += align_up(static_cast<size_t>(sq) * b_w, 256);
-    const void* d_q[16]; void* d_o[16];
+    uint8_t *d_q[kMaxHostLayers], *d_o[kMaxHostLayers];
     for (int l = 0; l < R; ++l) { d_q[l] = base + off; off += align_up(static_cast<size_t>(sq) * b_q, 256); }
     for (int l = 0; l < R; ++l) { d_o[l] = base + off; off += align_up(static_cast<size_t>(sq) * b_o, 256); }
     int32_t* d_idx = reinterpret_cast<int32_t*>(base + off); off += align_up(static_cast<size_t>(sq) * p->k_sparse * 4, 256);
     int32_t* d_n = reinterpret_cast<int32_t*>(base + off);
-    // The input half of stage s is free once the kernels of pass i-2 have read it; its output half only once the
-    // copy-out of pass i-2 has drained it, which the kernels of this pass (not its copy-in) have to wait for.
-    if (i >= 2) e = cudaStreamWaitEvent(c->copy_in, c->ev_done[s], 0);
+    // An input's place in the staging area is free once the kernels of pass i - 2 have read it; an output's once the
+    // copy-out of pass i - 2 has drained it.
+    if (i >= 2) e = cudaStreamWaitEvent(c->copy_in, c->ev_done[s][0], 0);
     if (e == cudaSuccess) e = cudaMemcpyAsync(d_qi, static_cast<const uint8_t*>(q_idx_host) + q0 * b_qi, n * b_qi, cudaMemcpyHostToDevice, c->copy_in);
     if (e == cudaSuccess) e = cudaMemcpyAsync(d_w, reinterpret_cast<const uint8_t*>(w_host) + q0 * b_w, n * b_w, cudaMemcpyHostToDevice, c->copy_in);
-    for (int l = 0; l < R && e == cudaSuccess; ++l)
-      e = cudaMemcpyAsync(const_cast<void*>(d_q[l]), static_cast<const uint8_t*>(q_host[l]) + q0 * b_q, n * b_q, cudaMemcpyHostToDevice, c->copy_in);
-    if (e == cudaSuccess) e = cudaEventRecord(c->ev_in[s], c->copy_in);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(c->stream, c->ev_in[s], 0);
-    if (e == cudaSuccess && i >= 2) e = cudaStreamWaitEvent(c->stream, c->ev_out[s], 0);
+    if (e == cudaSuccess) e = cudaEventRecord(c->ev_in[s][0], c->copy_in);
+    for (int l = 0; l < R && e == cudaSuccess; ++l) {
+      if (i >= 2) e = cudaStreamWaitEvent(c->copy_in, c->ev_done[s][1 + l], 0);
+      if (e == cudaSuccess) e = cudaMemcpyAsync(d_q[l], static_cast<const uint8_t*>(q_host[l]) + q0 * b_q, n * b_q, cudaMemcpyHostToDevice, c->copy_in);
+      if (e == cudaSuccess) e = cudaEventRecord(c->ev_in[s][1 + l], c->copy_in);
+    }
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(c->stream, c->ev_in[s][0], 0);
     if (e != cudaSuccess) break;
-    r = lsa_layer_group(c, p, d_qi, reinterpret_cast<const float*>(d_w), k_idx, k_scale, kmean, q_pos0 + q0, n, n_key, nullptr,
-                        0, nullptr, 1, d_q, k, v, ld_k, ld_v, d_o, nullptr, d_idx, d_n);
-    if (r != LSA_OK) return r;
-    e = cudaEventRecord(c->ev_done[s], c->stream);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(c->copy_out, c->ev_done[s], 0);
-    for (int l = 0; l < R && e == cudaSuccess; ++l)
-      e = cudaMemcpyAsync(static_cast<uint8_t*>(out_host[l]) + q0 * b_o, d_o[l], n * b_o, cudaMemcpyDeviceToHost, c->copy_out);
-    if (e == cudaSuccess) e = cudaEventRecord(c->ev_out[s], c->copy_out);
+    r = index_checked(c, p, d_qi, reinterpret_cast<const float*>(d_w), k_idx, k_scale, kmean, q_pos0 + q0, n, n_key, nullptr, 0,
+                      nullptr, 1, d_idx, d_n, nullptr, nullptr, nullptr);
+    if (r != LSA_OK) break;
+    e = cudaEventRecord(c->ev_done[s][0], c->stream);
+    for (int l = 0; l < R && e == cudaSuccess; ++l) {
+      e = cudaStreamWaitEvent(c->stream, c->ev_in[s][1 + l], 0);
+      if (e == cudaSuccess && i >= 2) e = cudaStreamWaitEvent(c->stream, c->ev_out[s][1 + l], 0);
+      if (e != cudaSuccess) break;
+      r = lsa_sparse_attn(c, p, d_q[l], k[l], v[l], ld_k, ld_v, d_idx, d_n, nullptr, nullptr, q_pos0 + q0, n, n_key, nullptr, 1,
+                          d_o[l], nullptr);
+      if (r != LSA_OK) break;
+      e = cudaEventRecord(c->ev_done[s][1 + l], c->stream);
+      if (e == cudaSuccess) e = cudaStreamWaitEvent(c->copy_out, c->ev_done[s][1 + l], 0);
+      if (e == cudaSuccess) e = cudaMemcpyAsync(static_cast<uint8_t*>(out_host[l]) + q0 * b_o, d_o[l], n * b_o, cudaMemcpyDeviceToHost, c->copy_out);
+      if (e == cudaSuccess) e = cudaEventRecord(c->ev_out[s][1 + l], c->copy_out);
+    }
+    if (r != LSA_OK) break;
   }
-  // the context stream finishes only after every copy-out has
-  for (int s = 0; s < 2 && e == cudaSuccess; ++s)
-    if (n_pass > s) e = cudaStreamWaitEvent(c->stream, c->ev_out[(n_pass - 1 - s) & 1], 0);
+  // the context stream goes on only after every copy, also after an error: the staging areas are the caller's again then
+  cudaError_t ej = cudaEventRecord(c->ev_start, c->copy_out);
+  if (ej == cudaSuccess) ej = cudaStreamWaitEvent(c->stream, c->ev_start, 0);
+  if (ej == cudaSuccess) ej = cudaEventRecord(c->ev_start, c->copy_in);
+  if (ej == cudaSuccess) ej = cudaStreamWaitEvent(c->stream, c->ev_start, 0);
+  if (e == cudaSuccess) e = ej;
+  if (r != LSA_OK) return r;
   return e == cudaSuccess ? LSA_OK : cuda_fail(c, e);
 }
 
