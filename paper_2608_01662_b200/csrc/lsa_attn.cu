@@ -1,10 +1,10 @@
-// Sparse attention over sink U window U sparse (Eq. 3), one softmax over the whole set, for a block
-// of H heads that share every K/V row (absorbed-MQA / MLA latent).
+// Sparse attention over sink U window U sparse (Eq. 3), one softmax over the whole set, for a block of H heads that share
+// every K/V row of the MLA latent, on mma.sync (the tcgen05 kernel of lsa_attn_tc.cu serves this shape unless it is switched
+// off); and the merges of partial results.
 //
 // One thread block handles one query (or one split of one query's rows).  Rows are streamed in tiles
 // of 64 keys through a double-buffered shared tile; S = Q K^T and O += P V run on tensor cores with an
-// online softmax in fp32.  With the MLA latent the value tile is the key tile (v == k), so each cache
-// row is read once.
+// online softmax in fp32.  The value tile is the key tile (v == k), so each cache row is read once.
 #include "lsa_internal.h"
 #include "lsa_common.cuh"
 
@@ -16,29 +16,28 @@ constexpr int kAttnThreads = 256;
 constexpr int kKeys = 64;  // keys per tile
 constexpr float kLog2e = 1.4426950408889634f;
 
-template <int H, int DQK, int DV, bool SEP_V>
+template <int H, int DQK, int DV>
 struct AttnSmem {
   alignas(128) uint8_t q[H * DQK * 2];
   alignas(128) uint8_t k[2][kKeys * DQK * 2];
-  alignas(128) uint8_t v[SEP_V ? 2 : 1][SEP_V ? kKeys * DV * 2 : 128];
   alignas(128) uint8_t p[H * kKeys * 2];
   float pmax[8 / (H / 16)][H];
   float psum[8 / (H / 16)][H];
   int32_t rowid[2][kKeys];
 };
 
-template <int H, int DQK, int DV, bool SEP_V>
+template <int H, int DQK, int DV>
 __global__ void __launch_bounds__(kAttnThreads, 1) sparse_attn_kernel(AttnArgs p) {
   constexpr int MT = H / 16;        // 16-row head tiles
   constexpr int NWM = 8 / MT;       // warps per head tile
   constexpr int NTQ = 8 / NWM;      // 8-key n-tiles per warp in S = Q K^T
   constexpr int NTV = DV / 8 / NWM; // 8-dim n-tiles per warp in O += P V
   constexpr int KSQ = DQK / 16;
-  constexpr int QROW = DQK * 2, VROW = DV * 2;
-  static_assert(NTQ >= 1 && NTV >= 2 && NTV % 2 == 0, "shape");
+  constexpr int QROW = DQK * 2;
+  static_assert(NTQ >= 2 && NTQ % 2 == 0 && NTV >= 2 && NTV % 2 == 0, "shape");
 
   extern __shared__ __align__(128) uint8_t smem_raw[];
-  auto& sm = *reinterpret_cast<AttnSmem<H, DQK, DV, SEP_V>*>(smem_raw);
+  auto& sm = *reinterpret_cast<AttnSmem<H, DQK, DV>*>(smem_raw);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int mt = warp % MT, grp = warp / MT;
   const int g = lane >> 2, c2 = (lane & 3) * 2;
@@ -75,21 +74,12 @@ __global__ void __launch_bounds__(kAttnThreads, 1) sparse_attn_kernel(AttnArgs p
   const int n_tiles = max(0, tile_end - tile_begin);
 
   const uint8_t* kg = reinterpret_cast<const uint8_t*>(p.k);
-  const uint8_t* vg = reinterpret_cast<const uint8_t*>(p.v);
   auto issue_tile = [&](int tile, int buf) {
     constexpr int UK = DQK / 8;
     for (int e = tid; e < kKeys * UK; e += kAttnThreads) {
       const int r = e / UK, u = e % UK;
       const int32_t row = sm.rowid[buf][r];
       cp_async16(smem_u32(sm.k[buf]) + swz<QROW>(r, u), kg + (row >= 0 ? row : 0) * p.ld_k * 2 + u * 16, row >= 0 ? 16 : 0);
-    }
-    if constexpr (SEP_V) {
-      constexpr int UV = DV / 8;
-      for (int e = tid; e < kKeys * UV; e += kAttnThreads) {
-        const int r = e / UV, u = e % UV;
-        const int32_t row = sm.rowid[buf][r];
-        cp_async16(smem_u32(sm.v[buf]) + swz<VROW>(r, u), vg + (row >= 0 ? row : 0) * p.ld_v * 2 + u * 16, row >= 0 ? 16 : 0);
-      }
     }
     cp_async_commit();
   };
@@ -132,18 +122,12 @@ __global__ void __launch_bounds__(kAttnThreads, 1) sparse_attn_kernel(AttnArgs p
     for (int ks = 0; ks < KSQ; ++ks) {
       uint32_t a[4];
       ldmatrix_x4(a, q_s + swz<QROW>(a_row, 2 * ks + (lane >> 4)));
-      if constexpr (NTQ == 1) {
-        uint32_t b[2];
-        ldmatrix_x2(b, k_s + swz<QROW>(grp * 8 + (lane & 7), 2 * ks + ((lane >> 3) & 1)));
-        mma_bf16(s[0], a, b[0], b[1]);
-      } else {
 #pragma unroll
-        for (int nt = 0; nt < NTQ; nt += 2) {
-          uint32_t b[4];
-          ldmatrix_x4(b, k_s + swz<QROW>(grp * 8 * NTQ + 8 * nt + (lane & 7) + (lane >> 4) * 8, 2 * ks + ((lane >> 3) & 1)));
-          mma_bf16(s[nt], a, b[0], b[1]);
-          mma_bf16(s[nt + 1], a, b[2], b[3]);
-        }
+      for (int nt = 0; nt < NTQ; nt += 2) {
+        uint32_t b[4];
+        ldmatrix_x4(b, k_s + swz<QROW>(grp * 8 * NTQ + 8 * nt + (lane & 7) + (lane >> 4) * 8, 2 * ks + ((lane >> 3) & 1)));
+        mma_bf16(s[nt], a, b[0], b[1]);
+        mma_bf16(s[nt + 1], a, b[2], b[3]);
       }
     }
     // ---- scale, mask the ragged tail, partial row max
@@ -218,8 +202,6 @@ __global__ void __launch_bounds__(kAttnThreads, 1) sparse_attn_kernel(AttnArgs p
     }
     // ---- O += P V for head tile mt, value dims [grp*8*NTV, +8*NTV)
     const uint32_t p_s = smem_u32(sm.p);
-    const uint32_t v_s = SEP_V ? smem_u32(sm.v[buf]) : k_s;
-    constexpr int VR = SEP_V ? VROW : QROW;
 #pragma unroll
     for (int ks = 0; ks < kKeys / 16; ++ks) {
       uint32_t a[4];
@@ -228,7 +210,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1) sparse_attn_kernel(AttnArgs p
 #pragma unroll
       for (int nt = 0; nt < NTV; nt += 2) {
         uint32_t b[4];
-        ldmatrix_x4_trans(b, v_s + swz<VR>(v_row, grp * NTV + nt + (lane >> 4)));
+        ldmatrix_x4_trans(b, k_s + swz<QROW>(v_row, grp * NTV + nt + (lane >> 4)));
         mma_bf16(o[nt], a, b[0], b[1]);
         mma_bf16(o[nt + 1], a, b[2], b[3]);
       }
@@ -337,10 +319,10 @@ __global__ void merge_parts_kernel(MergeArgs a) {
   if (a.lse != nullptr && threadIdx.x == 0) a.lse[row] = den > 0.f ? m + logf(den) : -INFINITY;
 }
 
-template <int H, int DQK, int DV, bool SEP_V>
+template <int H, int DQK, int DV>
 cudaError_t launch_attn_t(const AttnArgs& a, cudaStream_t st, int64_t* n_launch) {
-  const size_t smem = sizeof(AttnSmem<H, DQK, DV, SEP_V>);
-  auto kernel = sparse_attn_kernel<H, DQK, DV, SEP_V>;
+  const size_t smem = sizeof(AttnSmem<H, DQK, DV>);
+  auto kernel = sparse_attn_kernel<H, DQK, DV>;
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (e != cudaSuccess) return e;
   dim3 grid(a.n_query, a.n_split);
@@ -372,13 +354,10 @@ cudaError_t launch_merge(const AttnArgs& a, cudaStream_t st, int64_t* n_launch) 
 
 cudaError_t launch_attn(const AttnArgs& a, cudaStream_t st, int64_t* n_launch) {
   if (a.n_query == 0) return cudaSuccess;
-  const bool sep_v = !(a.v == a.k && a.ld_v == a.ld_k);
-  if (a.H == 16) {
-    return sep_v ? launch_attn_t<16, 128, 128, true>(a, st, n_launch) : launch_attn_t<16, 128, 128, false>(a, st, n_launch);
-  }
+  if (a.H == 16) return launch_attn16(a, st, n_launch);
   // the 64-head latent shape has no room for a separate value tile: MLA layout only
-  if (sep_v) return cudaErrorInvalidValue;
-  return launch_attn_t<64, 576, 512, false>(a, st, n_launch);
+  if (!(a.v == a.k && a.ld_v == a.ld_k)) return cudaErrorInvalidValue;
+  return launch_attn_t<64, 576, 512>(a, st, n_launch);
 }
 
 }  // namespace lsa
