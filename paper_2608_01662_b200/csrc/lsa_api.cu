@@ -300,6 +300,11 @@ int run_index(lsa_ctx* c, const lsa_params* p, const void* q_idx, const float* w
       if (e != cudaSuccess) return cuda_fail(c, e);
       continue;
     }
+    if (l.big_keys == 0 && (!p->hi_enable || p->pooling == LSA_POOL_MEAN) && lsa::index8_supported(a)) {
+      e = timed(c, LSA_K_FINE_SELECT, [&] { return lsa::launch_index8(a, c->stream, &c->launches); });
+      if (e != cudaSuccess) return cuda_fail(c, e);
+      continue;
+    }
     if (p->hi_enable && p->pooling == LSA_POOL_MINMAX)
       e = timed(c, LSA_K_COARSE, [&] { return lsa::launch_coarse_minmax(a, c->stream, &c->launches); });
     else if (p->hi_enable)

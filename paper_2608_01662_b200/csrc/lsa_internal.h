@@ -102,6 +102,9 @@ cudaError_t launch_block_minmax(int DI, int key_e4m3, int B, const void* k_idx, 
 cudaError_t launch_coarse_minmax(const IndexArgs& a, cudaStream_t st, int64_t* n_launch);
 // tcgen05 version of the coarse stage (contiguous caches, H_I = 64, d_I = 128); groups = 4-query groups per block
 bool coarse_tc_supported(const IndexArgs& a);
+// a1-a4 of the 8-head, 64-dim indexer in one launch, a warp per query (contiguous bf16 caches, small budgets, mean pooling)
+bool index8_supported(const IndexArgs& a);
+cudaError_t launch_index8(const IndexArgs& a, cudaStream_t st, int64_t* n_launch);
 cudaError_t launch_coarse_tc(const IndexArgs& a, int groups, cudaStream_t st, int64_t* n_launch);
 // The coarse stage as every entry point runs it: the tcgen05 kernel where the shape allows, else the mma.sync tile.
 inline cudaError_t launch_coarse_best(const IndexArgs& a, int groups, cudaStream_t st, int64_t* n_launch) {

@@ -99,7 +99,9 @@ extern "C" int lsa_index_static(int device, void* cuda_stream, const lsa_params*
   a.fine_parts = 1;
   int64_t launches = 0;
   cudaError_t e = cudaSuccess;
-  if (p->hi_enable) e = lsa::launch_coarse_best(a, 2, st, &launches);   // the dispatch and tile grouping of lsa_index
+  // the dispatch and tile grouping of lsa_index
+  if (lsa::index8_supported(a)) return lsa::launch_index8(a, st, &launches) == cudaSuccess ? LSA_OK : LSA_ERR_CUDA;
+  if (p->hi_enable) e = lsa::launch_coarse_best(a, 2, st, &launches);
   if (e == cudaSuccess) e = lsa::launch_fine_select(a, st, &launches);
   return e == cudaSuccess ? LSA_OK : LSA_ERR_CUDA;
 }
