@@ -66,28 +66,43 @@ __global__ void block_means_kernel(const uint8_t* __restrict__ k_idx, const floa
     cnt = static_cast<int>(min64(B, n_key - row0));
   }
   float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-  for (int r = 0; r < cnt; ++r) {
-    const int64_t row = row0 + r;
-    if (E4M3) {
-      const uint2 c = *reinterpret_cast<const uint2*>(k_idx + row * DI + u * 8);
-      const float sc = k_scale[row];
-      const uint32_t w[2] = {c.x, c.y};
+  // Eight rows' loads are in flight together (a row past the last is the last once more, and is not added): one after
+  // another they were most of what a launch takes, 2 us of a short prompt's.
+  for (int r0 = 0; r0 < cnt; r0 += 8) {
+    uint4 c[8];
+    float sc[8];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        __half2_raw h = __nv_cvt_fp8x2_to_halfraw2(
-            static_cast<__nv_fp8x2_storage_t>((w[j >> 1] >> ((j & 1) * 16)) & 0xffff), __NV_E4M3);
-        const float2 f = __half22float2(*reinterpret_cast<__half2*>(&h));
-        acc[2 * j] += f.x * sc;
-        acc[2 * j + 1] += f.y * sc;
+    for (int r = 0; r < 8; ++r) {
+      const int64_t row = row0 + min(r0 + r, cnt - 1);
+      if (E4M3) {
+        const uint2 c2 = *reinterpret_cast<const uint2*>(k_idx + row * DI + u * 8);
+        c[r] = make_uint4(c2.x, c2.y, 0, 0);
+        sc[r] = k_scale[row];
+      } else {
+        c[r] = *reinterpret_cast<const uint4*>(k_idx + (row * DI + u * 8) * 2);
       }
-    } else {
-      const uint4 c = *reinterpret_cast<const uint4*>(k_idx + (row * DI + u * 8) * 2);
-      const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&c);
+    }
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const float2 f = __bfloat1622float2(h[j]);
-        acc[2 * j] += f.x;
-        acc[2 * j + 1] += f.y;
+    for (int r = 0; r < 8; ++r) {
+      if (r0 + r >= cnt) break;
+      if (E4M3) {
+        const uint32_t w[2] = {c[r].x, c[r].y};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          __half2_raw h = __nv_cvt_fp8x2_to_halfraw2(
+              static_cast<__nv_fp8x2_storage_t>((w[j >> 1] >> ((j & 1) * 16)) & 0xffff), __NV_E4M3);
+          const float2 f = __half22float2(*reinterpret_cast<__half2*>(&h));
+          acc[2 * j] += f.x * sc[r];
+          acc[2 * j + 1] += f.y * sc[r];
+        }
+      } else {
+        const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&c[r]);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const float2 f = __bfloat1622float2(h[j]);
+          acc[2 * j] += f.x;
+          acc[2 * j + 1] += f.y;
+        }
       }
     }
   }
