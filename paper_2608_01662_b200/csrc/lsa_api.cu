@@ -260,12 +260,15 @@ int run_index(lsa_ctx* c, const lsa_params* p, const void* q_idx, const float* w
       // Eq. 7 without the hierarchy over paged caches: token scores of every page of the scoring range (per-token
       // scale applied), the top-K_sparse of each sequence's row, then the cache rows.
       e = timed(c, LSA_K_COARSE, [&] { return lsa::launch_paged_scores_tc(a, 1, c->sm_count, c->stream, &c->launches); });
+      const lsa::SelectRows rows{a.rows_out, a.n_rows_out, page_table, pt_stride, p->kv_page};
+      bool rows_done = false;
       if (e == cudaSuccess)
         e = timed(c, LSA_K_SELECT, [&] {
           return lsa::launch_select(a.page_scores, a.ps_ld, nullptr, nullptr, 0, a.n_query, n_key_max, p->k_sparse, 1, p->k_sink,
-                                    p->k_swa, a.sparse_idx, a.n_sparse, c->stream, &c->launches, ctx_len);
+                                    p->k_swa, a.sparse_idx, a.n_sparse, c->stream, &c->launches, ctx_len,
+                                    a.rows_out != nullptr ? &rows : nullptr, &rows_done);
         });
-      if (e == cudaSuccess && a.rows_out != nullptr)
+      if (e == cudaSuccess && a.rows_out != nullptr && !rows_done)
         e = timed(c, LSA_K_CONVERT, [&] {
           return lsa::launch_convert(p->k_sink, p->k_swa, p->k_sparse, p->paged, p->kv_page, a.sparse_idx, a.n_sparse, a.q_pos0,
                                      a.n_query, page_table, pt_stride, ctx_len, a.rows_out, a.n_rows_out, nullptr, c->stream,

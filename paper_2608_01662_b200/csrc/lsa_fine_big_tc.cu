@@ -12,7 +12,7 @@
 //   select_keys_kernel      a4: the exact radix top-K_sparse over each query's keys; a slot's position comes from the page
 //                           list, so only the keys (4 bytes per candidate) travel through memory
 #include "lsa_internal.h"
-#include "lsa_select.cuh"
+#include "lsa_select_long.cuh"
 #include "lsa_tc.cuh"
 
 namespace lsa {
@@ -196,27 +196,36 @@ fine_scores_tc_kernel(const __grid_constant__ CUtensorMap map, IndexArgs p, cons
   if (warp == 1) tc::tmem_dealloc(tmem_base, kTmemColsBig);
 }
 
-// ---- a4 over the keys of a query's listed pages: slot c of the row is token pages[c / P] * P + c % P
+// ---- a4 over the keys of a query's listed pages: slot c of the row is token pages[c / P] * P + c % P.  Rows of kLongMinRow
+// slots or more in one pass (lsa_select_long.cuh), shorter ones, and where that does not serve, by the radix select.
 __global__ void __launch_bounds__(kSelThreads) select_keys_kernel(IndexArgs p, const int32_t* __restrict__ pages_ws,
                                                                   const int32_t* __restrict__ n_pages_ws,
-                                                                  const uint32_t* __restrict__ keys, int64_t ld) {
-  __shared__ SelectScratch sc;
-  __shared__ int32_t pages[1024];
-  const int qi = blockIdx.x, tid = threadIdx.x;
+                                                                  const uint32_t* __restrict__ keys, int64_t ld, int cap) {
+  extern __shared__ __align__(16) uint8_t smem_raw[];
+  const int qi = blockIdx.x;
   const int pshift = 31 - __clz(p.P);
-  const int nP = n_pages_ws[qi];
-  const bool cached = p.M <= 1024;
+  const int n = n_pages_ws[qi] << pshift;
   const int32_t* pg = pages_ws + static_cast<int64_t>(qi) * p.M;
-  if (cached) {
-    for (int i = tid; i < nP; i += kSelThreads) pages[i] = pg[i];
-    __syncthreads();
-    pg = pages;
-  }
   const uint32_t* krow = keys + static_cast<int64_t>(qi) * ld;
-  const int n_sel = block_select_topk([&](int i) { return krow[i]; },
-                                      [&](int i) { return (pg[i >> pshift] << pshift) + (i & (p.P - 1)); }, nP << pshift, p.Ksp,
-                                      p.sparse_idx + static_cast<int64_t>(qi) * p.Ksp, sc);
-  if (tid == 0) p.n_sparse[qi] = n_sel;
+  int32_t* out = p.sparse_idx + static_cast<int64_t>(qi) * p.Ksp;
+  struct Keys {
+    const uint32_t* row;   // 16-byte aligned: ld = M * P is a multiple of 128
+    __device__ __forceinline__ uint32_t operator()(int i) const { return row[i]; }
+    __device__ __forceinline__ void quad(int i, uint32_t (&k)[4]) const {
+      const uint4 v = *reinterpret_cast<const uint4*>(row + i);
+      k[0] = v.x; k[1] = v.y; k[2] = v.z; k[3] = v.w;
+    }
+  };
+  const Keys key{krow};
+  auto id = [&](int i) { return (pg[i >> pshift] << pshift) + (i & (p.P - 1)); };
+  int n_sel = -1;
+  if (cap > 0 && n >= kLongMinRow)
+    n_sel = long_select<false>(key, [&](int r, int i) { out[r] = id(i); }, [&](int r) { out[r] = -1; }, n, p.Ksp, cap, smem_raw);
+  if (n_sel < 0) {
+    __syncthreads();
+    n_sel = block_select_topk(key, id, n, p.Ksp, out, *reinterpret_cast<SelectScratch*>(smem_raw));
+  }
+  if (threadIdx.x == 0) p.n_sparse[qi] = n_sel;
 }
 
 }  // namespace
@@ -249,7 +258,15 @@ cudaError_t launch_fine_big(const IndexArgs& a, int32_t* pages_ws, int32_t* n_pa
   ++*n_launch;
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  select_keys_kernel<<<a.n_query, kSelThreads, 0, st>>>(a, pages_ws, n_pages_ws, keys, ld);
+  int cap = long_cap(a.Ksp);
+  size_t sel_smem = long_smem_bytes(cap, ld);
+  if (sel_smem > 226 * 1024) {   // (no room for the bits of so long a row beside so many items)
+    cap = 0;
+    sel_smem = sizeof(SelectScratch);
+  }
+  e = cudaFuncSetAttribute(select_keys_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sel_smem));
+  if (e != cudaSuccess) return e;
+  select_keys_kernel<<<a.n_query, kSelThreads, sel_smem, st>>>(a, pages_ws, n_pages_ws, keys, ld, cap);
   ++*n_launch;
   return cudaGetLastError();
 }

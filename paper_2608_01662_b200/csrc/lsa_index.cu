@@ -11,7 +11,7 @@
 // thread quad and one number per key leaves the tile.
 #include "lsa_internal.h"
 #include "lsa_select.cuh"
-#include "lsa_select_cluster.cuh"
+#include "lsa_select_long.cuh"
 #include "lsa_rows.cuh"
 
 #ifdef LSA_TIMELINE
@@ -364,8 +364,8 @@ __global__ void __launch_bounds__(kThreads, 2) coarse_score_paged_kernel(IndexAr
 // ------------------------------------------------------------------------------------------------
 // a2-a4: per query: top-M pages, fine scores on their tokens, top-K_sparse.
 // ------------------------------------------------------------------------------------------------
-constexpr int kClusterRowsMax = 256;    // rows: up to this many, a row of kClusterMinRow scores or more gets a cluster of blocks
-constexpr int kClusterMinRow = 16384;
+constexpr int kClusterRowsMax = 256;    // rows: up to this many, a row of kLongMinRow scores or more gets a cluster of blocks
+constexpr size_t kLongSmemMax = 226 * 1024;
 constexpr int kMaxSlots = 4096;  // keep_pages * page
 constexpr int kMaxPages = 64;    // keep_pages
 
@@ -685,30 +685,98 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(const float* __rest
   if (threadIdx.x == 0) n_out[qi] = n_sel;
 }
 
-// The same selection with a cluster of kClusterSel blocks per row (few long rows: the flat indexer in decode).
-__global__ void __launch_bounds__(kSelThreads) select_cluster_kernel(const float* __restrict__ scores, int64_t ld,
-                                                                    const int32_t* __restrict__ cand_pos,
-                                                                    const float* __restrict__ pos_scale, int64_t q_pos0,
-                                                                    int64_t n_cand, int k, int apply_range, int S, int W,
-                                                                    int32_t* __restrict__ idx_out, int32_t* __restrict__ n_out,
-                                                                    const int32_t* __restrict__ ctx_len) {
-  __shared__ ClusterSelScratch sc;
-  const int qi = blockIdx.y;
-  const float* row = scores + qi * ld;
-  const int32_t* pos = cand_pos ? cand_pos + qi * n_cand : nullptr;
-  const int64_t lo = S, hi = (ctx_len ? static_cast<int64_t>(ctx_len[qi]) - 1 : q_pos0 + qi) - W;
-  auto id = [&](int i) { return pos ? pos[i] : i; };
-  auto key = [&](int i) -> uint32_t {   // branch-free, as in select_kernel
-    const int64_t s = id(i);
-    const bool ok = s >= 0 && (!apply_range || (s >= lo && s <= hi));
+// The same selection over long rows: one pass over the row and the rest on what it collected (lsa_select_long.cuh), the
+// radix select where that does not serve.  CLUSTER: a cluster of kClusterSel blocks per row (few rows: the flat indexer in
+// decode), which also writes the selection's cache rows when the caller wants them.
+// Keys of a row's items.  SOURCE: the score alone, or times its position's factor, read four at a time (rows and factors
+// 16-byte aligned); or whatever the call gives, one at a time.  A template, because a test of the pointers between the loads
+// of a step keeps them from going out together.
+enum { kScoreQuads = 0, kScaledQuads = 1, kScoreAny = 2 };
+template <int SOURCE>
+struct RowKeys {
+  const float* row;
+  const int32_t* pos;      // kScoreAny: the item's position, or NULL = the item's number
+  const float* pos_scale;  // kScaledQuads; kScoreAny: or NULL
+  int lo, hi;              // positions that take part
+  __device__ __forceinline__ int id(int i) const { return SOURCE == kScoreAny && pos ? pos[i] : i; }
+  __device__ __forceinline__ uint32_t of(float v, int s) const { return s >= lo && s <= hi ? score_key(v) : 0u; }
+  __device__ __forceinline__ uint32_t operator()(int i) const {
+    const int s = id(i);
     float v = row[i];
-    if (pos_scale) v *= pos_scale[s < 0 ? 0 : s];
-    return ok ? score_key(v) : 0u;
-  };
-  int n = static_cast<int>(n_cand);
-  if (pos == nullptr && apply_range) n = static_cast<int>(max64(0, min64(n_cand, hi + 1)));
-  const int n_sel = cluster_select_topk(key, id, n, k, idx_out + static_cast<int64_t>(qi) * k, sc);
-  if (threadIdx.x == 0 && blockIdx.x == 0) n_out[qi] = n_sel;
+    if (SOURCE == kScaledQuads || (SOURCE == kScoreAny && pos_scale)) v *= pos_scale[max(s, 0)];
+    return of(v, s);
+  }
+  __device__ __forceinline__ void quad(int i, uint32_t (&k)[4]) const {
+    if constexpr (SOURCE == kScoreAny) {
+#pragma unroll
+      for (int u = 0; u < 4; ++u) k[u] = (*this)(i + u);
+    } else {
+      float4 v = *reinterpret_cast<const float4*>(row + i);
+      if constexpr (SOURCE == kScaledQuads) {
+        const float4 f = *reinterpret_cast<const float4*>(pos_scale + i);
+        v.x *= f.x; v.y *= f.y; v.z *= f.z; v.w *= f.w;
+      }
+      k[0] = of(v.x, i); k[1] = of(v.y, i + 1); k[2] = of(v.z, i + 2); k[3] = of(v.w, i + 3);
+    }
+  }
+};
+
+template <bool CLUSTER, int SOURCE>
+__global__ void __launch_bounds__(kSelThreads) select_long_kernel(const float* __restrict__ scores, int64_t ld,
+                                                                 const int32_t* __restrict__ cand_pos,
+                                                                 const float* __restrict__ pos_scale, int64_t q_pos0,
+                                                                 int64_t n_cand, int k, int apply_range, int S, int W,
+                                                                 int32_t* __restrict__ idx_out, int32_t* __restrict__ n_out,
+                                                                 const int32_t* __restrict__ ctx_len, SelectRows rows, int cap) {
+  extern __shared__ __align__(16) uint8_t smem_raw[];
+  pdl_wait();                 // the scores come from the previous kernel of the stream
+  pdl_launch_dependents();
+  const int qi = CLUSTER ? blockIdx.y : blockIdx.x;
+  const float* row = scores + qi * ld;
+  const int64_t t = ctx_len ? static_cast<int64_t>(ctx_len[qi]) - 1 : q_pos0 + qi;
+  const RowKeys<SOURCE> key{row, cand_pos ? cand_pos + qi * n_cand : nullptr, pos_scale, apply_range ? S : 0,
+                            apply_range ? static_cast<int>(max64(-1, t - W)) : 0x7fffffff};
+  auto id = [&](int i) -> int { return key.id(i); };
+  int n = static_cast<int>(n_cand);   // columns that are positions: nothing beyond the range can take part
+  if (cand_pos == nullptr) n = static_cast<int>(min64(n_cand, static_cast<int64_t>(key.hi) + 1));
+  int32_t* out = idx_out + static_cast<int64_t>(qi) * k;
+  const int32_t* pt = rows.rows_out ? rows.page_table + qi * rows.pt_stride : nullptr;
+  int32_t* row_list = rows.rows_out ? rows.rows_out + static_cast<int64_t>(qi) * (S + k + W) : nullptr;
+  const int n_sink = static_cast<int>(min64(S, t + 1)), shift = rows.rows_out ? 31 - __clz(rows.kv_page) : 0, mask = rows.kv_page - 1;
+  int n_sel = -1;
+  // (CLUSTER: also short rows, whose pieces are collected whole)
+  if (CLUSTER || n >= kLongMinRow)
+    n_sel = long_select<CLUSTER>(
+        key,
+        [&](int r, int i) {
+          const int32_t s = id(i);
+          out[r] = s;
+          if (CLUSTER && row_list) row_list[n_sink + r] = (pt[s >> shift] << shift) + (s & mask);
+        },
+        [&](int r) { out[r] = -1; }, n, k, cap, smem_raw);
+  const bool listed = n_sel >= 0;
+  if (!listed) {
+    __syncthreads();
+    if constexpr (CLUSTER) n_sel = cluster_select_topk(key, id, n, k, out, *reinterpret_cast<ClusterSelScratch*>(smem_raw));
+    else n_sel = block_select_topk<0, true>(key, id, n, k, out, *reinterpret_cast<SelectScratch*>(smem_raw));
+  }
+  if (threadIdx.x == 0 && (!CLUSTER || blockIdx.x == 0)) n_out[qi] = n_sel;
+  if constexpr (CLUSTER) {
+    if (row_list == nullptr) return;
+    const int ld_rows = S + k + W;
+    const int64_t win0 = max64(S, t - W + 1);
+    const int n_win = static_cast<int>(max64(0, t - win0 + 1)), n_tot = n_sink + n_sel + n_win;
+    // [sink | sparse | window | -1 ...]: what the selection has not written (after the radix select, all of it: its list is in
+    // global memory, ordered by the cluster barrier it ends with)
+    for (int j = blockIdx.x * kSelThreads + threadIdx.x; j < ld_rows; j += kClusterSel * kSelThreads) {
+      int64_t s = -1;
+      if (j < n_sink) s = j;
+      else if (j < n_sink + n_sel) s = listed ? -2 : out[j - n_sink];
+      else if (j < n_tot) s = win0 + (j - n_sink - n_sel);
+      if (s != -2) row_list[j] = s < 0 ? -1 : (pt[s >> shift] << shift) + static_cast<int32_t>(s & mask);
+    }
+    if (threadIdx.x == 0 && blockIdx.x == 0) rows.n_rows_out[qi] = n_tot;
+  }
 }
 
 // e4m3 codes -> the same values as bf16 (exact), for the dense scoring of the flat indexer
@@ -1175,23 +1243,50 @@ cudaError_t launch_widen_e4m3(const void* codes, void* out_bf16, int64_t n_elems
 
 cudaError_t launch_select(const float* scores, int64_t ld, const int32_t* cand_pos, const float* pos_scale,
                           int64_t q_pos0, int n_query, int64_t n_cand, int k, int apply_range, int S, int W,
-                          int32_t* idx_out, int32_t* n_out, cudaStream_t st, int64_t* n_launch, const int32_t* ctx_len) {
+                          int32_t* idx_out, int32_t* n_out, cudaStream_t st, int64_t* n_launch, const int32_t* ctx_len,
+                          const SelectRows* rows, bool* rows_done) {
   if (n_query == 0) return cudaSuccess;
-  if (n_query <= kClusterRowsMax && n_cand >= kClusterMinRow) {
+  if (rows_done) *rows_done = false;
+  const bool quads = cand_pos == nullptr && ld % 4 == 0 && ((reinterpret_cast<uintptr_t>(scores) | reinterpret_cast<uintptr_t>(pos_scale)) & 15u) == 0;
+  const int source = !quads ? kScoreAny : pos_scale ? kScaledQuads : kScoreQuads;
+  const int cap = long_cap(k);
+  const SelectRows no_rows{};
+  if (n_query <= kClusterRowsMax && n_cand >= kLongMinRow) {
     // few long rows: a cluster of blocks per row
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(kClusterSel, static_cast<unsigned>(n_query), 1);
-    cfg.blockDim = dim3(kSelThreads);
-    cfg.stream = st;
-    cudaLaunchAttribute attr{};
-    attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = kClusterSel;
-    attr.val.clusterDim.y = 1;
-    attr.val.clusterDim.z = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, select_cluster_kernel, scores, ld, cand_pos, pos_scale, q_pos0, n_cand, k,
-                                             apply_range, S, W, idx_out, n_out, ctx_len);
+    const size_t piece = long_smem_bytes(cap, long_piece(static_cast<int>(n_cand)));
+    const size_t smem = piece > sizeof(ClusterSelScratch) ? piece : sizeof(ClusterSelScratch);
+    if (smem <= kLongSmemMax) {
+      auto kernel = source == kScoreQuads ? select_long_kernel<true, kScoreQuads> : source == kScaledQuads ? select_long_kernel<true, kScaledQuads> : select_long_kernel<true, kScoreAny>;
+      cudaError_t e = set_smem(kernel, smem);
+      if (e != cudaSuccess) return e;
+      cudaLaunchConfig_t cfg{};
+      cfg.gridDim = dim3(kClusterSel, static_cast<unsigned>(n_query), 1);
+      cfg.blockDim = dim3(kSelThreads);
+      cfg.dynamicSmemBytes = smem;
+      cfg.stream = st;
+      cudaLaunchAttribute attr[2]{};
+      attr[0].id = cudaLaunchAttributeClusterDimension;
+      attr[0].val.clusterDim.x = kClusterSel;
+      attr[0].val.clusterDim.y = 1;
+      attr[0].val.clusterDim.z = 1;
+      attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+      attr[1].val.programmaticStreamSerializationAllowed = 1;
+      cfg.attrs = attr;
+      cfg.numAttrs = 2;
+      e = cudaLaunchKernelEx(&cfg, kernel, scores, ld, cand_pos, pos_scale, q_pos0, n_cand, k, apply_range, S, W,
+                             idx_out, n_out, ctx_len, rows ? *rows : no_rows, cap);
+      ++*n_launch;
+      if (rows_done) *rows_done = rows != nullptr;
+      return e;
+    }
+  }
+  const size_t smem = long_smem_bytes(cap, n_cand);
+  if (n_cand >= kLongMinRow && smem <= kLongSmemMax) {
+    auto kernel = source == kScoreQuads ? select_long_kernel<false, kScoreQuads> : source == kScaledQuads ? select_long_kernel<false, kScaledQuads> : select_long_kernel<false, kScoreAny>;
+    cudaError_t e = set_smem(kernel, smem);
+    if (e != cudaSuccess) return e;
+    e = launch_pdl(kernel, dim3(n_query), dim3(kSelThreads), smem, st, scores, ld, cand_pos, pos_scale, q_pos0,
+                   n_cand, k, apply_range, S, W, idx_out, n_out, ctx_len, no_rows, cap);
     ++*n_launch;
     return e;
   }

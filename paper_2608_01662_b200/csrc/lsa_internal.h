@@ -124,11 +124,20 @@ cudaError_t launch_fine_select_tc(const IndexArgs& a, cudaStream_t st, int64_t* 
 bool fine_big_supported(const IndexArgs& a);
 cudaError_t launch_fine_big(const IndexArgs& a, int32_t* pages_ws, int32_t* n_pages_ws, uint32_t* keys, cudaStream_t st,
                             int64_t* n_launch);
-// ctx_len != NULL (paged caches): the query of row i sits at ctx_len[i] - 1 instead of q_pos0 + i
+// ctx_len != NULL (paged caches): the query of row i sits at ctx_len[i] - 1 instead of q_pos0 + i.
+// rows (with ctx_len): the cache rows of the selections are wanted too; *rows_done says whether the kernel that served the
+// call wrote them (else launch_convert has to).
+struct SelectRows {
+  int32_t* rows_out;      // [n_query, S + k + W]
+  int32_t* n_rows_out;
+  const int32_t* page_table;
+  int64_t pt_stride;
+  int kv_page;
+};
 cudaError_t launch_select(const float* scores, int64_t ld, const int32_t* cand_pos, const float* pos_scale,
                           int64_t q_pos0, int n_query, int64_t n_cand, int k, int apply_range, int S, int W,
                           int32_t* idx_out, int32_t* n_out, cudaStream_t st, int64_t* n_launch,
-                          const int32_t* ctx_len = nullptr);
+                          const int32_t* ctx_len = nullptr, const SelectRows* rows = nullptr, bool* rows_done = nullptr);
 // Token scores over cache pages on tcgen05 (paged caches, 64-token pages, H_I = 64, d_I = 128).  flat = 0: keys of the
 // slots of the page lists a.fine_pages -> a.fine_keys; flat = 1: scores of the whole scoring range -> a.page_scores.
 bool paged_scores_tc_supported(const IndexArgs& a);
