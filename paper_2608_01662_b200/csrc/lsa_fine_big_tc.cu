@@ -198,6 +198,16 @@ fine_scores_tc_kernel(const __grid_constant__ CUtensorMap map, IndexArgs p, cons
 
 // ---- a4 over the keys of a query's listed pages: slot c of the row is token pages[c / P] * P + c % P.  Rows of kLongMinRow
 // slots or more in one pass (lsa_select_long.cuh), shorter ones, and where that does not serve, by the radix select.
+struct ListedKeys {
+  const uint32_t* row;   // 16-byte aligned: ld = M * P is a multiple of 128
+  __device__ __forceinline__ uint32_t operator()(int i) const { return row[i]; }
+  static constexpr int kQuads = 4;
+  using Raw = uint4;
+  __device__ __forceinline__ Raw load(int i) const { return load_quad(row + i); }
+  __device__ __forceinline__ void keys(const Raw& v, int, uint32_t (&k)[4]) const {
+    k[0] = v.x; k[1] = v.y; k[2] = v.z; k[3] = v.w;
+  }
+};
 __global__ void __launch_bounds__(kSelThreads) select_keys_kernel(IndexArgs p, const int32_t* __restrict__ pages_ws,
                                                                   const int32_t* __restrict__ n_pages_ws,
                                                                   const uint32_t* __restrict__ keys, int64_t ld, int cap) {
@@ -208,15 +218,7 @@ __global__ void __launch_bounds__(kSelThreads) select_keys_kernel(IndexArgs p, c
   const int32_t* pg = pages_ws + static_cast<int64_t>(qi) * p.M;
   const uint32_t* krow = keys + static_cast<int64_t>(qi) * ld;
   int32_t* out = p.sparse_idx + static_cast<int64_t>(qi) * p.Ksp;
-  struct Keys {
-    const uint32_t* row;   // 16-byte aligned: ld = M * P is a multiple of 128
-    __device__ __forceinline__ uint32_t operator()(int i) const { return row[i]; }
-    __device__ __forceinline__ void quad(int i, uint32_t (&k)[4]) const {
-      const uint4 v = *reinterpret_cast<const uint4*>(row + i);
-      k[0] = v.x; k[1] = v.y; k[2] = v.z; k[3] = v.w;
-    }
-  };
-  const Keys key{krow};
+  const ListedKeys key{krow};
   auto id = [&](int i) { return (pg[i >> pshift] << pshift) + (i & (p.P - 1)); };
   int n_sel = -1;
   if (cap > 0 && n >= kLongMinRow)
@@ -259,7 +261,7 @@ cudaError_t launch_fine_big(const IndexArgs& a, int32_t* pages_ws, int32_t* n_pa
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   int cap = long_cap(a.Ksp);
-  size_t sel_smem = long_smem_bytes(cap, ld);
+  size_t sel_smem = long_smem_bytes(false, cap, ld);
   if (sel_smem > 226 * 1024) {   // (no room for the bits of so long a row beside so many items)
     cap = 0;
     sel_smem = sizeof(SelectScratch);

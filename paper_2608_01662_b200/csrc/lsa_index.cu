@@ -706,18 +706,34 @@ struct RowKeys {
     if (SOURCE == kScaledQuads || (SOURCE == kScoreAny && pos_scale)) v *= pos_scale[max(s, 0)];
     return of(v, s);
   }
-  __device__ __forceinline__ void quad(int i, uint32_t (&k)[4]) const {
+  static constexpr int kQuads = SOURCE == kScoreQuads ? 4 : 2;
+  struct Raw {
+    uint4 v, f;   // scores; factors, or positions
+  };
+  __device__ __forceinline__ Raw load(int i) const {
+    Raw r;
+    r.f = make_uint4(i, i + 1, i + 2, i + 3);
     if constexpr (SOURCE == kScoreAny) {
+      if (pos) r.f = make_uint4(pos[i], pos[i + 1], pos[i + 2], pos[i + 3]);
+      float v[4] = {row[i], row[i + 1], row[i + 2], row[i + 3]};
+      if (pos_scale) {
+        const int s[4] = {static_cast<int>(r.f.x), static_cast<int>(r.f.y), static_cast<int>(r.f.z), static_cast<int>(r.f.w)};
 #pragma unroll
-      for (int u = 0; u < 4; ++u) k[u] = (*this)(i + u);
-    } else {
-      float4 v = *reinterpret_cast<const float4*>(row + i);
-      if constexpr (SOURCE == kScaledQuads) {
-        const float4 f = *reinterpret_cast<const float4*>(pos_scale + i);
-        v.x *= f.x; v.y *= f.y; v.z *= f.z; v.w *= f.w;
+        for (int u = 0; u < 4; ++u) v[u] *= pos_scale[max(s[u], 0)];
       }
-      k[0] = of(v.x, i); k[1] = of(v.y, i + 1); k[2] = of(v.z, i + 2); k[3] = of(v.w, i + 3);
+      r.v = make_uint4(__float_as_uint(v[0]), __float_as_uint(v[1]), __float_as_uint(v[2]), __float_as_uint(v[3]));
+    } else {
+      r.v = load_quad(row + i);
+      if constexpr (SOURCE == kScaledQuads) r.f = load_quad(pos_scale + i);
     }
+    return r;
+  }
+  __device__ __forceinline__ void keys(const Raw& r, int i, uint32_t (&k)[4]) const {
+    const uint32_t v[4] = {r.v.x, r.v.y, r.v.z, r.v.w}, f[4] = {r.f.x, r.f.y, r.f.z, r.f.w};
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      k[u] = SOURCE == kScaledQuads ? of(__uint_as_float(v[u]) * __uint_as_float(f[u]), i + u)
+                                    : of(__uint_as_float(v[u]), SOURCE == kScoreAny ? static_cast<int>(f[u]) : i + u);
   }
 };
 
@@ -1253,7 +1269,7 @@ cudaError_t launch_select(const float* scores, int64_t ld, const int32_t* cand_p
   const SelectRows no_rows{};
   if (n_query <= kClusterRowsMax && n_cand >= kLongMinRow) {
     // few long rows: a cluster of blocks per row
-    const size_t piece = long_smem_bytes(cap, long_piece(static_cast<int>(n_cand)));
+    const size_t piece = long_smem_bytes(true, cap, long_piece(static_cast<int>(n_cand)));
     const size_t smem = piece > sizeof(ClusterSelScratch) ? piece : sizeof(ClusterSelScratch);
     if (smem <= kLongSmemMax) {
       auto kernel = source == kScoreQuads ? select_long_kernel<true, kScoreQuads> : source == kScaledQuads ? select_long_kernel<true, kScaledQuads> : select_long_kernel<true, kScoreAny>;
@@ -1280,7 +1296,7 @@ cudaError_t launch_select(const float* scores, int64_t ld, const int32_t* cand_p
       return e;
     }
   }
-  const size_t smem = long_smem_bytes(cap, n_cand);
+  const size_t smem = long_smem_bytes(false, cap, n_cand);
   if (n_cand >= kLongMinRow && smem <= kLongSmemMax) {
     auto kernel = source == kScoreQuads ? select_long_kernel<false, kScoreQuads> : source == kScaledQuads ? select_long_kernel<false, kScaledQuads> : select_long_kernel<false, kScoreAny>;
     cudaError_t e = set_smem(kernel, smem);

@@ -11,6 +11,12 @@ from paper_2608_01662_b200.configs import CONFIGS
 pytestmark = pytest.mark.gpu
 
 
+def _sampled(n):
+    """The items that the kernels may sample: quads at every n / (m / 4)-th place, for each sample size m."""
+    return np.unique(np.concatenate([((np.arange(m // 4, dtype=np.int64) * n // (m // 4)) & ~3)[:, None] + np.arange(4)
+                                     for m in (4096, 8192, 16384)]).ravel())
+
+
 def _row(kind, n, rng):
     if kind == "normal":
         return rng.standard_normal(n)
@@ -20,13 +26,11 @@ def _row(kind, n, rng):
         return np.full(n, -1.25)
     if kind == "sampled_high":    # every sampled item is large, few others are: fewer than k are collected
         x = rng.standard_normal(n)
-        m = 16384 if n > 131072 else 4096
-        x[(np.arange(m, dtype=np.int64) * n) // m] += 100.0
+        x[_sampled(n)] += 100.0
         return x
     if kind == "sampled_low":     # the other way round: more than there is room for
         x = rng.standard_normal(n) + 100.0
-        m = 16384 if n > 131072 else 4096
-        x[(np.arange(m, dtype=np.int64) * n) // m] -= 100.0
+        x[_sampled(n)] -= 100.0
         return x
     x = rng.standard_normal(n)    # "piece": all of the selection in one corner of the row
     x[n // 2:n // 2 + 5000] += 50.0
