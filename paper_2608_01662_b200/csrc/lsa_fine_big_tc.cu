@@ -25,7 +25,7 @@ constexpr int kAtomA = kTile * 128;
 constexpr int kAtomQ = kHI * 128;
 constexpr int kThreadsBig = 192;           // warp 0: TMA producer, warp 1: MMA issuer, warps 2-5: epilogue
 constexpr int kStagesBig = 2;               // two blocks per SM
-constexpr int kTilesPerBlockBig = 32;
+constexpr int kTilesPerBlockBig = 64;
 constexpr uint32_t kTmemColsBig = 128;
 
 // ---- a2
@@ -61,12 +61,13 @@ struct FineBigSmem {
   alignas(1024) uint8_t a[kStagesBig][2][kAtomA];
   alignas(1024) uint8_t q[2][kAtomQ];
   float w[kHI];
+  int32_t pages[kTilesPerBlockBig * kTile / 64];   // this block's part of the page list
   alignas(8) uint64_t full[kStagesBig], empty[kStagesBig], acc_full[2], acc_empty[2];
   uint32_t tmem_slot;
 };
 
 __global__ void __launch_bounds__(kThreadsBig, 2)
-fine_scores_tc_kernel(const __grid_constant__ CUtensorMap map, IndexArgs p, const int32_t* __restrict__ pages_ws,
+fine_scores_tc_kernel(const __grid_constant__ CUtensorMap map, int one_box, IndexArgs p, const int32_t* __restrict__ pages_ws,
                       const int32_t* __restrict__ n_pages_ws, uint32_t* __restrict__ keys, int64_t ld) {
   extern __shared__ uint8_t smem_raw[];
   FineBigSmem& sm = *reinterpret_cast<FineBigSmem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
@@ -81,7 +82,6 @@ fine_scores_tc_kernel(const __grid_constant__ CUtensorMap map, IndexArgs p, cons
   const int tiles_all = static_cast<int>(ld / kTile);                   // the whole row, listed pages or not
   const int tile_end = min(tiles_all, tile_begin + kTilesPerBlockBig);
   const int tiles_live = min(tile_end, (n_slots + kTile - 1) / kTile);  // tiles that hold listed pages
-  const int32_t* pages = pages_ws + static_cast<int64_t>(qi) * p.M;
   uint32_t* krow = keys + static_cast<int64_t>(qi) * ld;
   // slots past the listed pages: marked absent for the top-K
   for (int c = max(tile_begin, tiles_live) * kTile + tid; c < tile_end * kTile; c += kThreadsBig) krow[c] = 0u;
@@ -114,12 +114,15 @@ fine_scores_tc_kernel(const __grid_constant__ CUtensorMap map, IndexArgs p, cons
     cp_async_commit();
     cp_async_wait<0>();
   }
+  const int page_begin = (tile_begin * kTile) >> pshift;
+  for (int i = tid; i < (n_tiles * kTile + p.P - 1) >> pshift; i += kThreadsBig)
+    sm.pages[i] = page_begin + i < nP ? pages_ws[static_cast<int64_t>(qi) * p.M + page_begin + i] : 0;
   tc::fence_proxy_async();
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
   const uint32_t tmem_base = sm.tmem_slot;
-  auto slot_pos = [&](int c) -> int64_t { return (static_cast<int64_t>(pages[c >> pshift]) << pshift) + (c & (p.P - 1)); };
+  auto slot_pos = [&](int c) -> int64_t { return (static_cast<int64_t>(sm.pages[(c >> pshift) - page_begin]) << pshift) + (c & (p.P - 1)); };
 
   if (warp == 0) {
     // ================= TMA producer =================
@@ -128,6 +131,10 @@ fine_scores_tc_kernel(const __grid_constant__ CUtensorMap map, IndexArgs p, cons
         const int s = i % kStagesBig;
         if (!tc::mbar_wait(smem_u32(&sm.empty[s]), ((i / kStagesBig) & 1) ^ 1, p.status)) break;
         tc::mbar_expect_tx(smem_u32(&sm.full[s]), 2 * kAtomA);
+        if (one_box) {   // 128 consecutive slots lie in one page: both column blocks of the tile at once
+          tc::tma_load_3d(smem_u32(sm.a[s][0]), &map, 0, static_cast<int>(slot_pos((tile_begin + i) * kTile)), 0, smem_u32(&sm.full[s]));
+          continue;
+        }
 #pragma unroll
         for (int h = 0; h < 2; ++h) {   // 64 consecutive slots lie in one page; rows past the cache read as zero
           const int c = (tile_begin + i) * kTile + 64 * h;
@@ -163,13 +170,23 @@ fine_scores_tc_kernel(const __grid_constant__ CUtensorMap map, IndexArgs p, cons
     // ================= epilogue warps =================
     const int quarter = warp & 3;          // warps 2-5 own TMEM lanes 32*quarter .. +31
     const int r = 32 * quarter + lane;
+    // A tile's scales are fetched a tile ahead: asked for when its MMAs are already running they were what the epilogue
+    // waited for (two dependent loads with the page list in global memory: 781 cycles per tile and SM, 677 now).
+    auto pos_of = [&](int i) -> int64_t {
+      const int c = (tile_begin + i) * kTile + r;
+      return i < n_tiles && c < n_slots ? slot_pos(c) : -1;
+    };
+    auto scale_of = [&](int64_t pos) -> float { return p.key_e4m3 && pos >= lo && pos <= hi ? p.k_scale[pos] : 1.f; };
+    int64_t pos_next = pos_of(0);
+    float sc_next = scale_of(pos_next);
     for (int i = 0; i < n_tiles; ++i) {
       const int b = i & 1;
       const int c = (tile_begin + i) * kTile + r;
-      const int64_t pos = c < n_slots ? slot_pos(c) : -1;
+      const int64_t pos = pos_next;
+      const float sc = sc_next;
       const bool cand = pos >= lo && pos <= hi;
-      float sc = 1.f;
-      if (p.key_e4m3 && cand) sc = p.k_scale[pos];   // in flight while the tile's MMAs run
+      pos_next = pos_of(i + 1);
+      sc_next = scale_of(pos_next);
       if (!__all_sync(0xffffffffu, tc::mbar_wait(smem_u32(&sm.acc_full[b]), (i >> 1) & 1, p.status))) break;
       tc::fence_after_sync();
       uint32_t v[64];
@@ -250,13 +267,16 @@ cudaError_t launch_fine_big(const IndexArgs& a, int32_t* pages_ws, int32_t* n_pa
   if (e != cudaSuccess) return e;
   CUtensorMap map;
   const void* rows = a.key_e4m3 ? a.k_wide : a.k_idx;
-  if (!make_map_bf16_128(&map, rows, static_cast<uint64_t>(a.n_key), 64)) return cudaErrorInvalidValue;
+  const int one_box = a.P >= kTile;
+  if (!(one_box ? make_map_bf16_tile(&map, rows, kDI, static_cast<uint64_t>(a.n_key), kTile, 2)
+                : make_map_bf16_128(&map, rows, static_cast<uint64_t>(a.n_key), 64)))
+    return cudaErrorInvalidValue;
   const size_t smem = sizeof(FineBigSmem) + 1024;
   e = cudaFuncSetAttribute(fine_scores_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (e != cudaSuccess) return e;
   const int64_t ld = static_cast<int64_t>(a.M) * a.P;
   const unsigned parts = static_cast<unsigned>((ld / kTile + kTilesPerBlockBig - 1) / kTilesPerBlockBig);
-  fine_scores_tc_kernel<<<dim3(a.n_query, parts), kThreadsBig, smem, st>>>(map, a, pages_ws, n_pages_ws, keys, ld);
+  fine_scores_tc_kernel<<<dim3(a.n_query, parts), kThreadsBig, smem, st>>>(map, one_box, a, pages_ws, n_pages_ws, keys, ld);
   ++*n_launch;
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
