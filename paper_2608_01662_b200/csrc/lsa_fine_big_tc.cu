@@ -23,7 +23,7 @@ constexpr int kHI = 64, kDI = 128;
 constexpr int kTile = 128;
 constexpr int kAtomA = kTile * 128;
 constexpr int kAtomQ = kHI * 128;
-constexpr int kThreadsBig = 192;           // warp 0: TMA producer, warp 1: MMA issuer, warps 2-5: epilogue
+constexpr int kThreadsBig = 320;           // warp 0: TMA producer, warp 1: MMA issuer, warps 2-9: epilogue
 constexpr int kStagesBig = 2;               // two blocks per SM
 constexpr int kTilesPerBlockBig = 64;
 constexpr uint32_t kTmemColsBig = 128;
@@ -168,7 +168,11 @@ fine_scores_tc_kernel(const __grid_constant__ CUtensorMap map, int one_box, Inde
     }
   } else {
     // ================= epilogue warps =================
-    const int quarter = warp & 3;          // warps 2-5 own TMEM lanes 32*quarter .. +31
+    // Two sets of 4 warps: set 0 drains accumulator 0 (even tiles), set 1 accumulator 1 (odd tiles).  One tile's wait, TMEM
+    // load, 64-head chain and store follow one another, 1350 cycles in all: one set made a block's tile that long: 2048 queries x 262144 keys, 1024 pages,
+    // whole selection 6.45 ms, 6.09 with two sets (a tile is then 640 cycles of shared-memory traffic: 384 MMA operands, 256 the copy).
+    const int set = (warp - 2) >> 2;
+    const int quarter = warp & 3;          // a set's warps own TMEM lanes 32*quarter .. +31
     const int r = 32 * quarter + lane;
     // A tile's scales are fetched a tile ahead: asked for when its MMAs are already running they were what the epilogue
     // waited for (two dependent loads with the page list in global memory: 781 cycles per tile and SM, 677 now).
@@ -177,24 +181,23 @@ fine_scores_tc_kernel(const __grid_constant__ CUtensorMap map, int one_box, Inde
       return i < n_tiles && c < n_slots ? slot_pos(c) : -1;
     };
     auto scale_of = [&](int64_t pos) -> float { return p.key_e4m3 && pos >= lo && pos <= hi ? p.k_scale[pos] : 1.f; };
-    int64_t pos_next = pos_of(0);
+    int64_t pos_next = pos_of(set);
     float sc_next = scale_of(pos_next);
-    for (int i = 0; i < n_tiles; ++i) {
-      const int b = i & 1;
+    for (int i = set; i < n_tiles; i += 2) {
       const int c = (tile_begin + i) * kTile + r;
       const int64_t pos = pos_next;
       const float sc = sc_next;
       const bool cand = pos >= lo && pos <= hi;
-      pos_next = pos_of(i + 1);
+      pos_next = pos_of(i + 2);
       sc_next = scale_of(pos_next);
-      if (!__all_sync(0xffffffffu, tc::mbar_wait(smem_u32(&sm.acc_full[b]), (i >> 1) & 1, p.status))) break;
+      if (!__all_sync(0xffffffffu, tc::mbar_wait(smem_u32(&sm.acc_full[set]), (i >> 1) & 1, p.status))) break;
       tc::fence_after_sync();
       uint32_t v[64];
-      tc::tmem_ld64(tmem_base + (static_cast<uint32_t>(32 * quarter) << 16) + b * kHI, v);
+      tc::tmem_ld64(tmem_base + (static_cast<uint32_t>(32 * quarter) << 16) + set * kHI, v);
       tc::tmem_ld_wait();
       tc::fence_before_sync();
       __syncwarp();
-      if (lane == 0) tc::mbar_arrive(smem_u32(&sm.acc_empty[b]));
+      if (lane == 0) tc::mbar_arrive(smem_u32(&sm.acc_empty[set]));
       float a0 = 0.f, a1 = 0.f;
       const float4* w4 = reinterpret_cast<const float4*>(sm.w);
 #pragma unroll
