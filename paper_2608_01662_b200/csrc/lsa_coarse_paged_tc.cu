@@ -237,7 +237,8 @@ coarse_score_paged_tc_kernel(const __grid_constant__ CUtensorMap map_km, const _
   } else if (warp < 6) {
     // ================= epilogue warps =================
     const int quarter = warp & 3;          // warps 2-5 own TMEM lanes 32*quarter .. +31
-    const int r = 32 * quarter + lane;     // sub-block row of the tile
+    const int row = tc::head_sum_row(lane), r = 32 * quarter + row;   // sub-block row of the tile
+    tc::HeadWeights hw;
     int n_q = 0;
     bool new_seq = true;
     for (int i = 0; i < n_tiles; ++i) {
@@ -246,28 +247,20 @@ coarse_score_paged_tc_kernel(const __grid_constant__ CUtensorMap map_km, const _
         // the head weights of the slot were stored before the arrival on q_full
         if (!__all_sync(0xffffffffu, tc::mbar_wait(smem_u32(&sm.q_full[n_q & 1]), (n_q >> 1) & 1, p.status))) break;
         ++n_q;
+        hw.load(sm.w[(n_q - 1) & 1], lane);
       }
       const int slot = (n_q - 1) & 1;
       const int seq = wk.seq, tile = wk.tile;
       new_seq = wk.next(sm.ctx, sh, batch);
       if (!__all_sync(0xffffffffu, tc::mbar_wait(smem_u32(&sm.acc_full[b]), (i >> 1) & 1, p.status))) break;
       tc::fence_after_sync();
-      uint32_t v[64];
-      tc::tmem_ld64(tmem_base + (static_cast<uint32_t>(32 * quarter) << 16) + b * kHI, v);
+      tc::HeadScores v;
+      v.load(tmem_base + (static_cast<uint32_t>(32 * quarter) << 16) + b * kHI);
       tc::tmem_ld_wait();
       tc::fence_before_sync();
       __syncwarp();
       if (lane == 0) tc::mbar_arrive(smem_u32(&sm.acc_empty[b]));
-      float a0 = 0.f, a1 = 0.f;
-      const float4* w4 = reinterpret_cast<const float4*>(sm.w[slot]);
-#pragma unroll
-      for (int j = 0; j < 16; ++j) {
-        const float4 ww = w4[j];
-        a0 = fmaf(ww.x, fmaxf(__uint_as_float(v[4 * j + 0]), 0.f), a0);
-        a1 = fmaf(ww.y, fmaxf(__uint_as_float(v[4 * j + 1]), 0.f), a1);
-        a0 = fmaf(ww.z, fmaxf(__uint_as_float(v[4 * j + 2]), 0.f), a0);
-        a1 = fmaf(ww.w, fmaxf(__uint_as_float(v[4 * j + 3]), 0.f), a1);
-      }
+      const float dot = tc::head_sum(v, hw, lane);
       if (new_seq || i + 1 == n_tiles) {   // done with this sequence's head weights
         __syncwarp();
         if (lane == 0) tc::mbar_arrive(smem_u32(&sm.q_empty[slot]));
@@ -276,9 +269,9 @@ coarse_score_paged_tc_kernel(const __grid_constant__ CUtensorMap map_km, const _
       const int n_sub = (ctx + sh.B - 1) / sh.B;
       const int hi = ctx - 1 - sh.W;
       const int sub = tile * kTile + r;
-      float sc = sub < n_sub ? a0 + a1 : 0.f;   // rows past the cache hold whatever the pool had there
-      for (int d = 1; d < spp; d <<= 1) sc += __shfl_xor_sync(0xffffffffu, sc, d);
-      if ((lane & (spp - 1)) == 0) {
+      float sc = sub < n_sub ? dot : 0.f;   // rows past the cache hold whatever the pool had there
+      for (int d = 1; d < spp; d <<= 1) sc += __shfl_xor_sync(0xffffffffu, sc, tc::head_sum_xor(d));
+      if ((row & (spp - 1)) == 0) {
         const int page = sub >> sh.spp_shift;
         if ((page << sh.p_shift) <= hi) p.page_scores[static_cast<int64_t>(seq) * p.ps_ld + page] = sc;
       }

@@ -173,7 +173,9 @@ fine_scores_tc_kernel(const __grid_constant__ CUtensorMap map, int one_box, Inde
     // whole selection 6.45 ms, 6.09 with two sets (a tile is then 640 cycles of shared-memory traffic: 384 MMA operands, 256 the copy).
     const int set = (warp - 2) >> 2;
     const int quarter = warp & 3;          // a set's warps own TMEM lanes 32*quarter .. +31
-    const int r = 32 * quarter + lane;
+    const int r = 32 * quarter + tc::head_sum_row(lane);
+    tc::HeadWeights hw;
+    hw.load(sm.w, lane);
     // A tile's scales are fetched a tile ahead: asked for when its MMAs are already running they were what the epilogue
     // waited for (two dependent loads with the page list in global memory: 781 cycles per tile and SM, 677 now).
     auto pos_of = [&](int i) -> int64_t {
@@ -192,23 +194,14 @@ fine_scores_tc_kernel(const __grid_constant__ CUtensorMap map, int one_box, Inde
       sc_next = scale_of(pos_next);
       if (!__all_sync(0xffffffffu, tc::mbar_wait(smem_u32(&sm.acc_full[set]), (i >> 1) & 1, p.status))) break;
       tc::fence_after_sync();
-      uint32_t v[64];
-      tc::tmem_ld64(tmem_base + (static_cast<uint32_t>(32 * quarter) << 16) + set * kHI, v);
+      tc::HeadScores v;
+      v.load(tmem_base + (static_cast<uint32_t>(32 * quarter) << 16) + set * kHI);
       tc::tmem_ld_wait();
       tc::fence_before_sync();
       __syncwarp();
       if (lane == 0) tc::mbar_arrive(smem_u32(&sm.acc_empty[set]));
-      float a0 = 0.f, a1 = 0.f;
-      const float4* w4 = reinterpret_cast<const float4*>(sm.w);
-#pragma unroll
-      for (int j = 0; j < 16; ++j) {
-        const float4 ww = w4[j];
-        a0 = fmaf(ww.x, fmaxf(__uint_as_float(v[4 * j + 0]), 0.f), a0);
-        a1 = fmaf(ww.y, fmaxf(__uint_as_float(v[4 * j + 1]), 0.f), a1);
-        a0 = fmaf(ww.z, fmaxf(__uint_as_float(v[4 * j + 2]), 0.f), a0);
-        a1 = fmaf(ww.w, fmaxf(__uint_as_float(v[4 * j + 3]), 0.f), a1);
-      }
-      krow[c] = cand ? score_key((a0 + a1) * sc) : 0u;   // order-preserving key; outside the scoring range: absent
+      const float dot = tc::head_sum(v, hw, lane);
+      krow[c] = cand ? score_key(dot * sc) : 0u;   // order-preserving key; outside the scoring range: absent
     }
   }
   tc::fence_before_sync();

@@ -347,7 +347,9 @@ fine_paged_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
     // ================= epilogue: warps 4-7 the even tiles, warps 8-11 the odd ones =================
     const int b = (warp >> 2) - 1;
     const int quarter = warp & 3;          // TMEM lanes 32*quarter .. +31
-    const int r = 32 * quarter + lane;     // token row of the tile
+    const int r = 32 * quarter + tc::head_sum_row(lane);   // token row of the tile
+    tc::HeadWeights hw;
+    hw.load(sm.w, lane);
     const uint32_t keys0 = smem_of_rank(smem_u32(sm.keys), 0);
     if constexpr (E4M3) {
       // the scales of this thread's tokens, straight from the pool (an issued TMA or bulk copy costs its thread some
@@ -373,8 +375,8 @@ fine_paged_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
       const bool cand = pos >= lo && pos <= hi;
       if (!__all_sync(0xffffffffu, tc::mbar_wait(smem_u32(&sm.acc_full[acc]), acc_use_parity(i), p.status))) break;
       tc::fence_after_sync();
-      uint32_t v[64];
-      tc::tmem_ld64(tmem_base + (static_cast<uint32_t>(32 * quarter) << 16) + acc * kHI, v);
+      tc::HeadScores v;
+      v.load(tmem_base + (static_cast<uint32_t>(32 * quarter) << 16) + acc * kHI);
       tc::tmem_ld_wait();
       const float sc = E4M3 ? sm.k_scale[i][r] : 1.f;
       tc::fence_before_sync();
@@ -382,17 +384,8 @@ fine_paged_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
       if (lane == 0) {
         tc::mbar_arrive(smem_u32(&sm.acc_empty[acc]));
       }
-      float a0 = 0.f, a1 = 0.f;
-      const float4* w4 = reinterpret_cast<const float4*>(sm.w);
-#pragma unroll
-      for (int j = 0; j < 16; ++j) {
-        const float4 ww = w4[j];
-        a0 = fmaf(ww.x, fmaxf(__uint_as_float(v[4 * j + 0]), 0.f), a0);
-        a1 = fmaf(ww.y, fmaxf(__uint_as_float(v[4 * j + 1]), 0.f), a1);
-        a0 = fmaf(ww.z, fmaxf(__uint_as_float(v[4 * j + 2]), 0.f), a0);
-        a1 = fmaf(ww.w, fmaxf(__uint_as_float(v[4 * j + 3]), 0.f), a1);
-      }
-      if (c < n_slots) store_cluster_u32(keys0 + static_cast<uint32_t>(c) * 4u, cand ? score_key((a0 + a1) * sc) : 0u);
+      const float dot = tc::head_sum(v, hw, lane);
+      if (c < n_slots) store_cluster_u32(keys0 + static_cast<uint32_t>(c) * 4u, cand ? score_key(dot * sc) : 0u);
     }
   }
   tc::fence_before_sync();

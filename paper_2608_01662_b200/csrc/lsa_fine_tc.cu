@@ -228,7 +228,9 @@ __global__ void __launch_bounds__(kFineThreads, 2) fine_select_tc_kernel(const _
   } else {
     // ================= epilogue warps =================
     const int quarter = warp & 3;          // warps 4-7 own TMEM lanes 32*quarter .. +31
-    const int r = 32 * quarter + lane;     // key row of the tile
+    const int r = 32 * quarter + tc::head_sum_row(lane);   // key row of the tile
+    tc::HeadWeights hw;
+    hw.load(sm.w, lane);
     bool ok = true;
     for (int i = 0; i < n_tiles && ok; ++i) {
       const int b = i & 1;
@@ -240,24 +242,15 @@ __global__ void __launch_bounds__(kFineThreads, 2) fine_select_tc_kernel(const _
       ok = __all_sync(0xffffffffu, tc::mbar_wait(smem_u32(&sm.acc_full[b]), (i >> 1) & 1, p.status));
       if (!ok) break;
       tc::fence_after_sync();
-      uint32_t v[64];
-      tc::tmem_ld64(tmem_base + (static_cast<uint32_t>(32 * quarter) << 16) + b * kHI, v);
+      tc::HeadScores v;
+      v.load(tmem_base + (static_cast<uint32_t>(32 * quarter) << 16) + b * kHI);
       tc::tmem_ld_wait();
       if (!TMA) sc = sm.scale[i & 3][r];   // read before the accumulator is handed back
       tc::fence_before_sync();
       __syncwarp();
       if (lane == 0) tc::mbar_arrive(smem_u32(&sm.acc_empty[b]));
-      float a0 = 0.f, a1 = 0.f;
-      const float4* w4 = reinterpret_cast<const float4*>(sm.w);
-#pragma unroll
-      for (int j = 0; j < 16; ++j) {
-        const float4 ww = w4[j];
-        a0 = fmaf(ww.x, fmaxf(__uint_as_float(v[4 * j + 0]), 0.f), a0);
-        a1 = fmaf(ww.y, fmaxf(__uint_as_float(v[4 * j + 1]), 0.f), a1);
-        a0 = fmaf(ww.z, fmaxf(__uint_as_float(v[4 * j + 2]), 0.f), a0);
-        a1 = fmaf(ww.w, fmaxf(__uint_as_float(v[4 * j + 3]), 0.f), a1);
-      }
-      if (c < n_slots) sm.keys[c] = cand ? score_key((a0 + a1) * sc) : 0u;
+      const float dot = tc::head_sum(v, hw, lane);
+      if (c < n_slots) sm.keys[c] = cand ? score_key(dot * sc) : 0u;
     }
   }
   tc::fence_before_sync();

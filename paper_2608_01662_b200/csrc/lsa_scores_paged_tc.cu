@@ -317,7 +317,8 @@ paged_scores_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
     // ================= epilogue: warps 4-7 the even tiles, warps 8-11 the odd ones =================
     const int me = (warp >> 2) - 1;
     const int quarter = warp & 3;          // TMEM lanes 32*quarter .. +31
-    const int r = 32 * quarter + lane;     // token row of the tile
+    const int r = 32 * quarter + tc::head_sum_row(lane);   // token row of the tile
+    tc::HeadWeights hw;
     int n_q = 0;
     bool new_seq = true, ok = true;
     auto leave_slot = [&](int slot) {
@@ -331,8 +332,8 @@ paged_scores_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
         // (every sequence's slot is waited for: see the issuers); the head weights were stored before the arrival
         ok = __all_sync(0xffffffffu, tc::mbar_wait(smem_u32(&sm.q_full[(n_q - 1) & 1]), ((n_q - 1) >> 1) & 1, p.status));
         if (!ok) break;
+        hw.load(sm.w[(n_q - 1) & 1], lane);
       }
-      const int slot = (n_q - 1) & 1;
       const int seq = wk.seq, tile = wk.tile;
       new_seq = wk.next(sm.ntile, batch);
       if ((i & 1) != me) continue;
@@ -349,8 +350,8 @@ paged_scores_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
       ok = __all_sync(0xffffffffu, tc::mbar_wait(smem_u32(&sm.acc_full[acc]), (i >> 2) & 1, p.status));
       if (!ok) break;
       tc::fence_after_sync();
-      uint32_t v[64];
-      tc::tmem_ld64(tmem_base + (static_cast<uint32_t>(32 * quarter) << 16) + acc * kHI, v);
+      tc::HeadScores v;
+      v.load(tmem_base + (static_cast<uint32_t>(32 * quarter) << 16) + acc * kHI);
       tc::tmem_ld_wait();
       const float sc = E4M3 ? sm.k_scale[i & 15][r] : 1.f;   // read before the accumulator is handed back (see k_scale)
       tc::fence_before_sync();
@@ -358,17 +359,8 @@ paged_scores_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
       if (lane == 0) {
         tc::mbar_arrive(smem_u32(&sm.acc_empty[acc]));
       }
-      float a0 = 0.f, a1 = 0.f;
-      const float4* w4 = reinterpret_cast<const float4*>(sm.w[slot]);
-#pragma unroll
-      for (int j = 0; j < 16; ++j) {
-        const float4 ww = w4[j];
-        a0 = fmaf(ww.x, fmaxf(__uint_as_float(v[4 * j + 0]), 0.f), a0);
-        a1 = fmaf(ww.y, fmaxf(__uint_as_float(v[4 * j + 1]), 0.f), a1);
-        a0 = fmaf(ww.z, fmaxf(__uint_as_float(v[4 * j + 2]), 0.f), a0);
-        a1 = fmaf(ww.w, fmaxf(__uint_as_float(v[4 * j + 3]), 0.f), a1);
-      }
-      const float score = (a0 + a1) * sc;
+      const float dot = tc::head_sum(v, hw, lane);
+      const float score = dot * sc;
       if (flat) {
         if (cand) p.page_scores[static_cast<int64_t>(seq) * p.ps_ld + pos] = score;
       } else if (lp >= 0) {

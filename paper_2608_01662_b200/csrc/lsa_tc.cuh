@@ -212,6 +212,61 @@ __device__ __forceinline__ void tmem_ld_16x256b_x8(uint32_t taddr, uint32_t (&r)
         "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
       : "r"(taddr));
 }
+// 16 lanes x 64 columns: register 2 i + j of lane l is row (l / 4) + 8 j, column 4 i + (l % 4)
+__device__ __forceinline__ void tmem_ld_16x128b_x16(uint32_t taddr, uint32_t (&r)[32]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.16x128b.x16.b32 "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
+        "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
+        "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+      : "r"(taddr));
+}
+
+// ---- head sums of indexer scores: sum_h w[h] * max(v[row][h], 0) over the 64 heads in a warp's 32 TMEM lanes ----
+// In a 16-lane fragment layout a thread holds 4 rows of 16 heads, the same heads for every row and tile, so that its weights are
+// 16 registers.  With a row of 64 heads per thread they were 16 broadcast loads of 16 bytes per tile and warp, which write
+// back for 4 cycles each and share the shared-memory pipe with the MMAs' operand reads and the copies (it was 60 to 70 % busy):
+// token scores and selection of 16384 queries 2.72 -> 2.57 ms, of 32768 4.46 -> 4.21 ms; one flat decode step of 16 sequences
+// 240 -> 236 us.  Where N = 256 keeps the accumulators busy (lsa_coarse_tc.cu) the slower TMEM loads lose more than that.
+// (A 32 x 64 block leaves TMEM in 39 cycles as whole rows, 70 in this layout and 129 in the 16x256b one.)
+// fmaxf issues at half the rate of an add: every other head takes w/2 * (v + |v|) instead, the same number.
+struct HeadWeights {
+  float2 w[8];   // heads 8 i + (lane & 3) and, halved, 8 i + 4 + (lane & 3)
+  __device__ __forceinline__ void load(const float* smem_w, int lane) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) w[i] = make_float2(smem_w[8 * i + (lane & 3)], 0.5f * smem_w[8 * i + 4 + (lane & 3)]);
+  }
+};
+struct HeadScores {
+  uint32_t lo[32], hi[32];   // rows 0-15, rows 16-31
+  __device__ __forceinline__ void load(uint32_t taddr) {
+    tmem_ld_16x128b_x16(taddr, lo);
+    tmem_ld_16x128b_x16(taddr + (16u << 16), hi);
+  }
+};
+// the row (of 32) whose sum head_sum() returns to a lane, and the lane mask that flips bit `off` (a power of two) of that row
+__device__ __forceinline__ int head_sum_row(int lane) { return (lane >> 2) + ((lane & 1) << 4) + ((lane & 2) << 2); }
+__device__ __forceinline__ int head_sum_xor(int off) { return off < 8 ? off << 2 : 16 / off; }
+__device__ __forceinline__ float head_sum(const HeadScores& s, const HeadWeights& hw, int lane) {
+  float2 a[4] = {};
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const float x = __uint_as_float((j < 2 ? s.lo : s.hi)[4 * i + (j & 1)]), y = __uint_as_float((j < 2 ? s.lo : s.hi)[4 * i + 2 + (j & 1)]);
+      a[j] = fma2(hw.w[i], make_float2(fmaxf(x, 0.f), y + fabsf(y)), a[j]);
+    }
+  }
+  // four lanes hold the parts of the same four rows: two exchanges leave each with one row
+  const float r0 = a[0].x + a[0].y, r1 = a[1].x + a[1].y, r2 = a[2].x + a[2].y, r3 = a[3].x + a[3].y;
+  const bool up = lane & 1, odd = lane & 2;
+  const float k0 = (up ? r2 : r0) + __shfl_xor_sync(0xffffffffu, up ? r0 : r2, 1);
+  const float k1 = (up ? r3 : r1) + __shfl_xor_sync(0xffffffffu, up ? r1 : r3, 1);
+  return (odd ? k1 : k0) + __shfl_xor_sync(0xffffffffu, odd ? k0 : k1, 2);
+}
+
 __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 // Makes this thread's earlier generic-proxy writes to shared memory visible to the async proxy
 // (tcgen05.mma operand reads, TMA).
