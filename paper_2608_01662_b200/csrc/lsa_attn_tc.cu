@@ -693,18 +693,28 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
       if (softmax_any(!ok)) break;
       const Job done = jb;
       const int last = base + done.n_tiles - 1 + (done.n_tiles - 1 >= done.q_at ? 1 : 0);   // ring position of the last tile
+      auto wait_last = [&]() {   // P V of the last tile is complete
+        if (!have_o) return;
+        const bool o_ok = __all_sync(0xffffffffu, tc::mbar_wait(smem_u32(&sm.k_empty[slot_of(last)]), use_of(last), p.status));
+        have_o = o_ok;
+        ok = ok && o_ok;
+      };
       if constexpr (!kClustered) {
         base += done.n_tiles + 1;
         tiles_done += done.n_tiles;
         if (jd.x >= 0) {
           jb = job_of(jd);
+          // Behind early tiles Q may lie in the slot of the last tile, and all four warps' word that Q has moved lets its issuer
+          // release that slot once more: a warp that had not yet seen the release by the last P V would look for a phase that
+          // is two uses back, and wait for good.  (Q is there, so that P V is complete: nothing is waited for.)
+          if (jb.q_at > 0) wait_last();
           move_q(base + jb.q_at, n + 1);
+          if (jb.q_at == 0) wait_last();
+        } else {
+          wait_last();
         }
-      }
-      if (have_o) {
-        const bool o_ok = __all_sync(0xffffffffu, tc::mbar_wait(smem_u32(&sm.k_empty[slot_of(last)]), use_of(last), p.status));
-        have_o = o_ok;
-        ok = ok && o_ok;
+      } else {
+        wait_last();
       }
       tc::fence_after_sync();
       if constexpr (kClustered) break;
