@@ -31,7 +31,7 @@
 // The query heads are fetched before the dependency wait (they are an input of the call, not a product of the
 // coarse kernel that precedes this one in the stream).
 #include "lsa_internal.h"
-#include "lsa_select.cuh"
+#include "lsa_select_short.cuh"
 #include "lsa_tc.cuh"
 
 namespace lsa {
@@ -113,13 +113,16 @@ __device__ __forceinline__ void finish_sequence(const IndexArgs& p, const uint32
   int32_t* rows = p.rows_out != nullptr ? p.rows_out + static_cast<int64_t>(qi) * ld : nullptr;
   if (tid < kSelThreads) {
     int32_t* out_idx = p.sparse_idx + static_cast<int64_t>(qi) * p.Ksp;
-    const int n_sel = block_select_topk_emit<kSelBar>(
-        [&](int i) { return keys[i]; },
-        [&](int r, int i) {
-          out_idx[r] = pages[i >> 6] * kPageTok + (i & (kPageTok - 1));
-          if (rows != nullptr) rows[n_sink + r] = phys[i >> 6] * kPageTok + (i & (kPageTok - 1));
-        },
-        [&](int r) { out_idx[r] = -1; }, n_slots, p.Ksp, sel);
+    const int n_sel = short_select<kSelBar>(smem_u32(keys), n_slots, p.Ksp, smem_u32(keys), smem_u32(&sel));
+    for (int r = tid; r < p.Ksp; r += kSelThreads) {
+      if (r >= n_sel) {
+        out_idx[r] = -1;
+        continue;
+      }
+      const int i = short_item(smem_u32(keys), r);
+      out_idx[r] = pages[i >> 6] * kPageTok + (i & (kPageTok - 1));
+      if (rows != nullptr) rows[n_sink + r] = phys[i >> 6] * kPageTok + (i & (kPageTok - 1));
+    }
     if (tid == 0) {
       p.n_sparse[qi] = n_sel;
       sel.n_valid = static_cast<uint32_t>(n_sel);
@@ -246,7 +249,9 @@ fine_paged_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
               if (i0 + u * kSelThreads < nE) pk[i0 + u * kSelThreads] = score_key(v[u]);
           }
           select_sync<kSelBar>();
-          nP = block_select_topk<kSelBar>([&](int i) { return pk[i]; }, [&](int i) { return p0 + i; }, nE, p.M, sm.pages, sm.sel);
+          nP = short_select<kSelBar>(smem_u32(pk), nE, p.M, smem_u32(pk), smem_u32(&sm.sel));
+          for (int i = tid; i < nP; i += kSelThreads) sm.pages[i] = p0 + short_item(smem_u32(pk), i);
+          select_sync<kSelBar>();
           tc::fence_proxy_async();   // the ring is handed to the TMA copies
         } else {
           nP = block_select_topk<kSelBar, true>([&](int i) { return score_key(ps[i]); }, [&](int i) { return p0 + i; }, nE, p.M,

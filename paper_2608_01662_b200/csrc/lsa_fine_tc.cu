@@ -14,7 +14,7 @@
 //
 // and the candidate buffer then goes through the exact radix top-K_sparse (Eq. 12) with all eight warps.
 #include "lsa_internal.h"
-#include "lsa_select.cuh"
+#include "lsa_select_short.cuh"
 #include "lsa_tc.cuh"
 
 namespace lsa {
@@ -96,7 +96,8 @@ __global__ void __launch_bounds__(kFineThreads, 2) fine_select_tc_kernel(const _
     if (nE <= kMaxSlotsTc) {
       for (int i = tid; i < nE; i += kFineThreads) sm.keys[i] = score_key(ps[i]);
       __syncthreads();
-      nP = block_select_topk([&](int i) { return sm.keys[i]; }, [&](int i) { return p0 + i; }, nE, p.M, sm.pages, sm.sel);
+      nP = short_select<0>(smem_u32(sm.keys), nE, p.M, smem_u32(sm.keys), smem_u32(&sm.sel));
+      for (int i = tid; i < nP; i += kFineThreads) sm.pages[i] = p0 + short_item(smem_u32(sm.keys), i);
     } else {
       nP = block_select_topk<0, true>([&](int i) { return score_key(ps[i]); }, [&](int i) { return p0 + i; }, nE, p.M, sm.pages,
                              sm.sel);
@@ -264,9 +265,8 @@ __global__ void __launch_bounds__(kFineThreads, 2) fine_select_tc_kernel(const _
     for (int c = c0 + tid; c < c1; c += kFineThreads) fk[c] = sm.keys[c];
     return;
   }
-  const int n_sel = block_select_topk([&](int i) { return sm.keys[i]; },
-                                      [&](int i) { return static_cast<int>(slot_pos(i)); }, n_slots, p.Ksp, out_idx,
-                                      sm.sel);
+  const int n_sel = short_select<0>(smem_u32(sm.keys), n_slots, p.Ksp, smem_u32(sm.keys), smem_u32(&sm.sel));
+  for (int r = tid; r < p.Ksp; r += kFineThreads) out_idx[r] = r < n_sel ? static_cast<int>(slot_pos(short_item(smem_u32(sm.keys), r))) : -1;
   if (tid == 0) p.n_sparse[qi] = n_sel;
 }
 

@@ -10,7 +10,7 @@
 // one query on the N axis, so that the ReLU / head-weight / head-sum epilogue of Eq. 1 runs inside one
 // thread quad and one number per key leaves the tile.
 #include "lsa_internal.h"
-#include "lsa_select.cuh"
+#include "lsa_select_short.cuh"
 #include "lsa_select_long.cuh"
 #include "lsa_rows.cuh"
 
@@ -426,7 +426,8 @@ __global__ void __launch_bounds__(kThreads, 2) fine_select_kernel(IndexArgs p) {
       for (int i = tid; i < nE; i += kThreads) sm.keys[i] = score_key(ps[i]);
       __syncthreads();
       LSA_TLF(7);
-      nP = block_select_topk([&](int i) { return sm.keys[i]; }, [&](int i) { return p0 + i; }, nE, p.M, sm.pages, sm.sel);
+      nP = short_select<0>(smem_u32(sm.keys), nE, p.M, smem_u32(sm.keys), smem_u32(&sm.sel));
+      for (int i = tid; i < nP; i += kThreads) sm.pages[i] = p0 + short_item(smem_u32(sm.keys), i);
     } else {
       nP = block_select_topk<0, true>([&](int i) { return score_key(ps[i]); }, [&](int i) { return p0 + i; }, nE, p.M,
                              sm.pages, sm.sel);
@@ -570,9 +571,8 @@ __global__ void __launch_bounds__(kThreads, 2) fine_select_kernel(IndexArgs p) {
     LSA_TLF(6);
     return;
   }
-  const int n_sel = block_select_topk([&](int i) { return sm.keys[i]; },
-                                      [&](int i) { return static_cast<int>(slot_pos(i)); }, n_slots, p.Ksp, out_idx,
-                                      sm.sel);
+  const int n_sel = short_select<0>(smem_u32(sm.keys), n_slots, p.Ksp, smem_u32(sm.keys), smem_u32(&sm.sel));
+  for (int r = tid; r < p.Ksp; r += kThreads) out_idx[r] = r < n_sel ? static_cast<int>(slot_pos(short_item(smem_u32(sm.keys), r))) : -1;
   if (tid == 0) p.n_sparse[qi] = n_sel;
   // (rows_out: the caller runs convert_kernel after an unsplit launch; a call to the row writer at this point of the
   // template trips an internal error of nvcc 12.9)
@@ -611,7 +611,9 @@ __global__ void __launch_bounds__(kSelThreads) page_topm_paged_kernel(IndexArgs 
     if (nE <= kMaxSlots) {
       for (int i = tid; i < nE; i += kSelThreads) keys[i] = score_key(ps[i]);
       __syncthreads();
-      nP = block_select_topk([&](int i) { return keys[i]; }, [&](int i) { return p0 + i; }, nE, p.M, pages, sc);
+      nP = short_select<0>(smem_u32(keys), nE, p.M, smem_u32(keys), smem_u32(&sc));
+      for (int i = tid; i < nP; i += kSelThreads) pages[i] = p0 + short_item(smem_u32(keys), i);
+      __syncthreads();
     } else {
       nP = block_select_topk<0, true>([&](int i) { return score_key(ps[i]); }, [&](int i) { return p0 + i; }, nE, p.M, pages, sc);
     }
@@ -642,11 +644,14 @@ __global__ void __launch_bounds__(kSelThreads) fine_topk_kernel(IndexArgs p) {
   for (int i = tid; i < nP; i += kSelThreads) pages[i] = fp[i];
   __syncthreads();
   const int pshift = 31 - __clz(p.P);
-  const int n_sel = block_select_topk([&](int i) { return keys[i]; },
-                                      [&](int i) { return pages[i >> pshift] * p.P + (i & (p.P - 1)); }, n_slots, p.Ksp,
-                                      p.sparse_idx + static_cast<int64_t>(qi) * p.Ksp, sc);
+  const int n_sel = short_select<0>(smem_u32(keys), n_slots, p.Ksp, smem_u32(keys), smem_u32(&sc));
+  int32_t* out_idx = p.sparse_idx + static_cast<int64_t>(qi) * p.Ksp;
+  for (int r = tid; r < p.Ksp; r += kSelThreads) {
+    const int i = r < n_sel ? short_item(smem_u32(keys), r) : -1;
+    out_idx[r] = i >= 0 ? pages[i >> pshift] * p.P + (i & (p.P - 1)) : -1;
+  }
   if (tid == 0) p.n_sparse[qi] = n_sel;
-  // the select ended with a barrier: the list is visible to the block
+  __syncthreads();   // the list is visible to the block
   emit_rows_of_query<kSelThreads>(p.rows_out, p.n_rows_out, p.sparse_idx, p.page_table, p.pt_stride,
                                   p.paged ? static_cast<int64_t>(p.ctx_len[qi]) - 1 : p.q_pos0 + qi, p.S, p.W, p.Ksp, p.paged,
                                   p.P, qi, tid, n_sel);

@@ -19,7 +19,7 @@ namespace lsa {
 constexpr int kSelThreads = 256;
 constexpr int kSelWarps = kSelThreads / 32;
 
-struct SelectScratch {
+struct alignas(16) SelectScratch {
   uint32_t hist[kSelWarps][256];
   uint32_t warp_gt[kSelWarps];
   uint32_t warp_eq[kSelWarps];
