@@ -180,14 +180,17 @@ int* status_word(lsa_ctx* c) { return c->ws ? reinterpret_cast<int*>(c->ws) : nu
 // Number of row splits per sequence in paged (decode) attention.  Blocks run one per SM in waves; a block costs its
 // share of the 64-key units plus a fixed part (Q load, tensor-memory set-up, fp32 partial output), taken as six
 // units' worth.  The split count with the smallest estimate wins; ties go to fewer splits (less merging).  The
-// tcgen05 kernel merges its splits inside a thread-block cluster and takes only the counts that allows.
+// tcgen05 kernel merges its splits inside a thread-block cluster and takes only the counts that allows; its waves are counted
+// in clusters that fit the chip together, not in SMs: 15 clusters of eight run at once, and a 16th sequence doubled the time
+// (decode step of 16 sequences, 4 layers: 190 us as 8 splits, 144 as 4; of 36: 255 as 4, 186 as 2).
 int pick_split(int sm_count, int batch, int max_rows, bool tc_kernel) {
   const int units = (max_rows + 63) / 64;
   int best = 1;
   long best_cost = -1;
   for (int s = 1; s <= kMaxSplit && s <= units; ++s) {
     if (tc_kernel && !lsa::attn_tc_split_ok(s)) continue;
-    const long waves = (static_cast<long>(batch) * s + sm_count - 1) / sm_count;
+    const int fit = tc_kernel && s > 1 ? lsa::attn_tc_resident(s) : 0;
+    const long waves = fit > 0 ? (batch + fit - 1) / fit : (static_cast<long>(batch) * s + sm_count - 1) / sm_count;
     const long cost = waves * ((units + s - 1) / s + 6);
     if (best_cost < 0 || cost < best_cost) {
       best_cost = cost;

@@ -970,6 +970,13 @@ bool attn_tc_split_ok(int n_split) {
   return (n_split == 2 || n_split == 4 || n_split == 8) && n_split <= max_cluster_blocks();
 }
 
+int attn_tc_resident(int n_split) {
+  static const int n[3] = {resident_clusters(reinterpret_cast<const void*>(sparse_attn_tc_kernel<true, true>), kThreadsAttnTc, sizeof(AttnTcSmem) + 1024, 2),
+                           resident_clusters(reinterpret_cast<const void*>(sparse_attn_tc_kernel<true, true>), kThreadsAttnTc, sizeof(AttnTcSmem) + 1024, 4),
+                           resident_clusters(reinterpret_cast<const void*>(sparse_attn_tc_kernel<true, true>), kThreadsAttnTc, sizeof(AttnTcSmem) + 1024, 8)};
+  return n_split == 2 ? n[0] : n_split == 4 ? n[1] : n_split == 8 ? n[2] : 0;
+}
+
 bool attn_tc_supported(const AttnArgs& a) {
   return a.H == kH && a.DQK == kDQK && a.DV == kDV && a.v == a.k && a.ld_v == a.ld_k;
 }

@@ -413,8 +413,8 @@ bool fine_paged_tc_supported(const IndexArgs& a) {
 }
 
 // One cluster per sequence, of as many blocks as all clusters can have at once: its tiles' MMAs are 49 cycles each, 12 a tile,
-// one after another.  (Clusters of eight or four do not fill every GPC: an eighth of the SMs is kept out of the count.)  One
-// sequence of 20K: the scoring part 11.8 thousand cycles on two blocks, 5.1 on eight; 23 sequences of up to 40K 11 on four.
+// one after another.  One sequence of 20K: the scoring part 11.8 thousand cycles on two blocks, 5.1 on eight; 23 sequences of up
+// to 40K: 11 on four.
 cudaError_t launch_fine_paged_tc(const IndexArgs& a, int sm_count, cudaStream_t st, int64_t* n_launch) {
   if (a.n_query == 0) return cudaSuccess;
   // The key pool belongs to the caller and its size is not part of the call: the map spans the largest row range a
@@ -424,7 +424,12 @@ cudaError_t launch_fine_paged_tc(const IndexArgs& a, int sm_count, cudaStream_t 
       !(a.key_e4m3 ? make_map_u8_128(&map_k, a.k_idx, 1ull << 31, kPageTok) : make_map_bf16_128(&map_k, a.k_idx, 1ull << 31, kPageTok)))
     return cudaErrorInvalidValue;
   const int sms = sm_count > 0 ? sm_count : 148;
-  const unsigned n_rank = 9 * a.n_query <= sms ? 8u : 9 * a.n_query <= 2 * sms ? 4u : 2 * a.n_query <= sms ? 2u : 1u;
+  static const int fit_f8[2] = {resident_clusters(reinterpret_cast<const void*>(fine_paged_tc_kernel<true>), kThreadsFp, sizeof(FpSmem<true>) + 1024, 8),
+                                resident_clusters(reinterpret_cast<const void*>(fine_paged_tc_kernel<true>), kThreadsFp, sizeof(FpSmem<true>) + 1024, 4)};
+  static const int fit_bf[2] = {resident_clusters(reinterpret_cast<const void*>(fine_paged_tc_kernel<false>), kThreadsFp, sizeof(FpSmem<false>) + 1024, 8),
+                                resident_clusters(reinterpret_cast<const void*>(fine_paged_tc_kernel<false>), kThreadsFp, sizeof(FpSmem<false>) + 1024, 4)};
+  const int* fit = a.key_e4m3 ? fit_f8 : fit_bf;
+  const unsigned n_rank = a.n_query <= fit[0] ? 8u : a.n_query <= fit[1] ? 4u : 2 * a.n_query <= sms ? 2u : 1u;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(n_rank, static_cast<unsigned>(a.n_query), 1);
   cfg.blockDim = dim3(kThreadsFp);

@@ -154,6 +154,30 @@ cudaError_t launch_attn16(const AttnArgs& a, cudaStream_t st, int64_t* n_launch)
 bool attn_tc_supported(const AttnArgs& a);
 // row splits that kernel merges itself (clusters of n_split blocks); other counts need launch_merge
 bool attn_tc_split_ok(int n_split);
+// Clusters of n_split blocks of that kernel that run at the same time.
+int attn_tc_resident(int n_split);
+
+// Clusters of `blocks` blocks of a kernel that the device can hold at the same time (0: it cannot, or cannot say).  Fewer than
+// the SMs divided by the cluster's size: a cluster lies in one GPC, and one block per SM leaves a rest in each.
+inline int resident_clusters(const void* kernel, int threads, size_t smem, int blocks) {
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) == cudaSuccess) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(static_cast<unsigned>(blocks) * 256);
+    cfg.blockDim = dim3(static_cast<unsigned>(threads));
+    cfg.dynamicSmemBytes = smem;
+    cudaLaunchAttribute attr[1]{};
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = static_cast<unsigned>(blocks);
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) == cudaSuccess) return n;
+  }
+  (void)cudaGetLastError();
+  return 0;
+}
 cudaError_t launch_attn_tc(const AttnArgs& a, cudaStream_t st, int64_t* n_launch);
 cudaError_t launch_merge(const AttnArgs& a, cudaStream_t st, int64_t* n_launch);
 
