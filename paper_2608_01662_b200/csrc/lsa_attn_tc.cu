@@ -79,17 +79,15 @@ struct AttnTcSmem {
   alignas(16) float lse_own[kH];          // its log-sum-exp per head (log2 units)
   alignas(16) float lse_peer[kH / 2];     // two-split launches: the peer's, for the heads this block finishes
 };
-constexpr int kPitchPart = kDV * 4 + 16;                  // staged fp32 row of a partial result, padded against bank conflicts
-// Two-split launches stage their rows in the order the softmax warps read them out of tensor memory: per warp (32 heads,
+// Splits stage their partial rows in the order the softmax warps read them out of tensor memory: per warp (32 heads,
 // half of the value dims) four column steps, each [head][64 floats] = 8 KB, the 16-byte chunks of a head's 256-byte piece
-// XOR-swizzled by the head (no bank conflicts either way).  A step's 8 KB is contiguous, so the rows the peer finishes
-// leave step by step, one bulk copy each, while the rest is still being read out; the peer's rows land behind the
-// staged ones in the same layout.
+// XOR-swizzled by the head (no bank conflicts either way).  A step's 8 KB is contiguous, so the rows leave step by step, one bulk
+// copy each, while the rest is still being read out, and keep that layout where they go: with two splits the rows the peer
+// finishes, behind its staged ones; with more all of them, to the global scratch.
 constexpr int kWarpStage = 32 * 256 * 4;
 constexpr int kRecvOffset = kSoftmaxWarps * kWarpStage;
 constexpr uint32_t kRecvBytes = 2 * kWarpStage + (kH / 2) * 4;
 static_assert(kRecvOffset + 2 * kWarpStage <= kRing * kSlotBytes, "staged and received rows must fit the ring");
-static_assert(kH * kPitchPart <= kRing * kSlotBytes, "staged rows must fit the ring");
 
 // ---- thread-block cluster: barrier and loads from a peer block's shared memory
 __device__ __forceinline__ void cluster_sync_all() {
@@ -169,9 +167,10 @@ __device__ __forceinline__ bool clc_answer(uint32_t answer, int* block_x) {
 //   barrier is used in halves: a thread arrives when it has left the tile loop and waits before the first copy (the
 //   peer's ring must be out of use before it receives), and once more around the end, so that no block leaves
 //   while the other may still write into it.  Nothing goes through global memory.
-//   Four or eight splits: the other rows (one bulk copy per row) and all log-sum-exps go to the global scratch, where
-//   they stay in L2; after one cluster barrier the owner of a row combines its own part with the others'.  (Loads from
-//   a peer's shared memory moved the same rows at about a quarter of the L2 path's rate.)
+//   Four or eight splits: the rows and all log-sum-exps go to the global scratch, where they stay in L2, as 16 bulk copies of
+//   8 KB; after one cluster barrier the owner of a row combines the parts.  (Loads from a peer's shared memory moved the
+//   same rows at about a quarter of the L2 path's rate; a bulk copy per row took 3 000 cycles longer to issue, stores
+//   straight from the registers 4 000.)
 //
 // q_tma != 0: q_map describes q as a bf16 matrix [n_query * 64, 576] and Q arrives as one TMA box; otherwise the
 // gather warps copy it with cp.async.  k_tma != 0 (contiguous caches only): k_map describes the cache rows, and key
@@ -763,8 +762,8 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
         bar_peer = peer_smem(smem_u32(&sm.recv_full), peer);
         dst_peer = peer_smem(smem_u32(stage + kRecvOffset + half_o * kWarpStage), peer);
       }
-      uint8_t* my_row = stage + head_o * kPitchPart;           // (four or eight splits: padded rows)
-      uint8_t* my_warp = stage + warp * kWarpStage;            // (two splits: this warp's 32 KB)
+      uint8_t* my_warp = stage + warp * kWarpStage;
+      uint8_t* dst_part = reinterpret_cast<uint8_t*>(part_out + (static_cast<int64_t>(qi) * p.n_split + split) * kH * kDV) + warp * kWarpStage;
 #pragma unroll 1
       for (int c = 0; c < 256; c += 64) {
         uint32_t o[64];
@@ -775,25 +774,20 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
 #pragma unroll
           for (int j = 0; j < 64; ++j) o[j] = 0u;
         }
-        if (pair) {
-          uint8_t* piece = my_warp + (c / 64) * 8192 + lane * 256;
+        uint8_t* piece = my_warp + (c / 64) * 8192 + lane * 256;
 #pragma unroll
-          for (int j = 0; j < 16; ++j)
-            *reinterpret_cast<float4*>(piece + ((j ^ (lane & 15)) << 4)) =
-                make_float4(__uint_as_float(o[4 * j]) * inv, __uint_as_float(o[4 * j + 1]) * inv,
-                            __uint_as_float(o[4 * j + 2]) * inv, __uint_as_float(o[4 * j + 3]) * inv);
-          if (foreign) {
-            tc::fence_proxy_async();
-            __syncwarp();
-            if (lane == 0)
-              bulk_copy_to_peer(dst_peer + (c / 64) * 8192, smem_u32(my_warp + (c / 64) * 8192), 8192, bar_peer);
+        for (int j = 0; j < 16; ++j)
+          *reinterpret_cast<float4*>(piece + ((j ^ (lane & 15)) << 4)) =
+              make_float4(__uint_as_float(o[4 * j]) * inv, __uint_as_float(o[4 * j + 1]) * inv,
+                          __uint_as_float(o[4 * j + 2]) * inv, __uint_as_float(o[4 * j + 3]) * inv);
+        if (foreign || !pair) {
+          tc::fence_proxy_async();
+          __syncwarp();
+          if (lane == 0) {
+            const uint32_t src = smem_u32(my_warp + (c / 64) * 8192);
+            if (pair) bulk_copy_to_peer(dst_peer + (c / 64) * 8192, src, 8192, bar_peer);
+            else asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst_part + (c / 64) * 8192), "r"(src), "n"(8192) : "memory");
           }
-        } else {
-#pragma unroll
-          for (int j = 0; j < 16; ++j)   // floats 256 (c / 128) + 128 half + c % 128 .. of the row
-            *reinterpret_cast<float4*>(my_row + ((c >> 7) * 256 + 128 * half_o + (c & 127) + 4 * j) * 4) =
-                make_float4(__uint_as_float(o[4 * j]) * inv, __uint_as_float(o[4 * j + 1]) * inv,
-                            __uint_as_float(o[4 * j + 2]) * inv, __uint_as_float(o[4 * j + 3]) * inv);
         }
       }
       tc::fence_proxy_async();
@@ -806,14 +800,12 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
           cluster_wait();   // (every thread passes the first half of the barrier once)
         }
       } else {
-        softmax_sync();     // a row is staged by two warps
-        const int rows_per = kH / p.n_split;
-        if (tid < kH && tid / rows_per != split) {   // one bulk copy per row (2 KB) that another block finishes
-          float* dst = part_out + ((static_cast<int64_t>(qi) * p.n_split + split) * kH + tid) * kDV;
-          asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;"
-                       :: "l"(dst), "r"(smem_u32(stage + tid * kPitchPart)), "n"(kDV * 4) : "memory");
+        if (lane == 0) {   // written, not only read out of shared memory
           asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+          asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+          __threadfence();
         }
+        __syncwarp();
       }
     }
   }
@@ -870,13 +862,9 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
       }
       cluster_wait();   // (see the arrival above)
     } else {
-      if (warp < kSoftmaxWarps) {   // the threads that sent rows wait until they are written (not only read out of shared memory)
-        asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
-        __threadfence();
-      }
       cluster_sync_all();   // every block of the cluster has written its rows
       // Warp w finishes rows w, w + 13, ... of this block's share (at most two).  Lane 8k + j first fetches the
-      // log-sum-exp of split j for the warp's k-th row, so that all of them are in flight together.
+      // log-sum-exp of split j for the warp's k-th row, and the first row's first parts are asked for with them.
       constexpr int kMost = (kH / 4 + kWarps - 1) / kWarps;
       const int k_of = lane >> 3, j_of = lane & 7;
       const int rl_mine = warp + kWarps * k_of;
@@ -884,6 +872,18 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
       if (k_of < kMost && rl_mine < rows_per && j_of < n)
         my_l = j_of == split ? sm.lse_own[row0 + rl_mine]
                              : __ldcg(part_lse + (static_cast<int64_t>(qi) * n + j_of) * kH + row0 + rl_mine);
+      float4 v[4][4];   // [split][128 dims each]
+      auto fetch = [&](int rl, int j0) {
+        const int R = row0 + rl;
+        const uint8_t* src = reinterpret_cast<const uint8_t*>(part_out + (static_cast<int64_t>(qi) * n + j0) * kH * kDV) +
+                             (R >> 5) * kWarpStage + (lane >> 4) * 8192 + (R & 31) * 256 + (((lane & 15) ^ (R & 15)) << 4);
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+          for (int u = 0; u < 4; ++u)   // dims 128u + 4 lane .. + 3: see the pair's version
+            v[j][u] = __ldcg(reinterpret_cast<const float4*>(src + j * (kH * kDV * 4) + (u & 1) * 2 * kWarpStage + (u >> 1) * 2 * 8192));
+      };
+      if (warp < rows_per) fetch(warp, 0);
       float m = my_l;
 #pragma unroll
       for (int d = 1; d < 8; d <<= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, d));
@@ -901,20 +901,15 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
           float4 acc[4];
 #pragma unroll
           for (int u = 0; u < 4; ++u) acc[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-          for (int j = 0; j < n; ++j) {
-            const float w = __shfl_sync(0xffffffffu, wgt, 8 * k + j);
-            float4 v[4];
-            if (j == split) {
+          for (int j0 = 0; j0 < n; j0 += 4) {
+            if (k > 0 || j0 > 0) fetch(rl, j0);
 #pragma unroll
-              for (int u = 0; u < 4; ++u) v[u] = *reinterpret_cast<const float4*>(stage + (row0 + rl) * kPitchPart + (lane + 32 * u) * 16);
-            } else {
-              const float4* src = reinterpret_cast<const float4*>(part_out + ((static_cast<int64_t>(qi) * n + j) * kH + row0 + rl) * kDV);
+            for (int j = 0; j < 4; ++j) {
+              const float w = __shfl_sync(0xffffffffu, wgt, 8 * k + j0 + j);
 #pragma unroll
-              for (int u = 0; u < 4; ++u) v[u] = __ldcg(src + lane + 32 * u);
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-              acc[u].x += w * v[u].x; acc[u].y += w * v[u].y; acc[u].z += w * v[u].z; acc[u].w += w * v[u].w;
+              for (int u = 0; u < 4; ++u) {
+                acc[u].x += w * v[j][u].x; acc[u].y += w * v[j][u].y; acc[u].z += w * v[j][u].z; acc[u].w += w * v[j][u].w;
+              }
             }
           }
 #pragma unroll
