@@ -182,7 +182,8 @@ int* status_word(lsa_ctx* c) { return c->ws ? reinterpret_cast<int*>(c->ws) : nu
 // units' worth.  The split count with the smallest estimate wins; ties go to fewer splits (less merging).  The
 // tcgen05 kernel merges its splits inside a thread-block cluster and takes only the counts that allows; its waves are counted
 // in clusters that fit the chip together, not in SMs: 15 clusters of eight run at once, and a 16th sequence doubled the time
-// (decode step of 16 sequences, 4 layers: 190 us as 8 splits, 144 as 4; of 36: 255 as 4, 186 as 2).
+// (decode step of 16 sequences, 4 layers: 190 us as 8 splits, 144 as 4; of 36: 255 as 4, 186 as 2; of one: 77.5 as 16, 82.7 as 8;
+// of 8: 153 and 99).
 int pick_split(int sm_count, int batch, int max_rows, bool tc_kernel) {
   const int units = (max_rows + 63) / 64;
   int best = 1;

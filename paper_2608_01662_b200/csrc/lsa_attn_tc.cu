@@ -60,7 +60,7 @@ constexpr int kRowsPerWarp = kTileKeys / kSlotWarps;   // cache rows of a tile t
 constexpr uint32_t kTmemColsAttn = 512;
 constexpr uint32_t kColQ = 256, kColS = 384, kSBuf = 64;
 constexpr float kLog2eTc = 1.4426950408889634f;
-constexpr int kMaxClusterSplit = 8;          // row splits of one sequence = blocks of one cluster (portable limit)
+constexpr int kMaxClusterSplit = 16;         // row splits of one sequence = blocks of one cluster (eight is the portable limit)
 constexpr int kFirstTileCycles = 8192;       // longest that a block's second tile is held back for the first
 constexpr float kRescaleGap = 8.f;           // rescale O only when the row max grows by more than 2^8
 constexpr int kJobReaders = kSoftmaxWarps + 2 + kGatherWarps;   // warps that release a job slot
@@ -167,7 +167,7 @@ __device__ __forceinline__ bool clc_answer(uint32_t answer, int* block_x) {
 //   barrier is used in halves: a thread arrives when it has left the tile loop and waits before the first copy (the
 //   peer's ring must be out of use before it receives), and once more around the end, so that no block leaves
 //   while the other may still write into it.  Nothing goes through global memory.
-//   Four or eight splits: the rows and all log-sum-exps go to the global scratch, where they stay in L2, as 16 bulk copies of
+//   Four, eight or 16 splits: the rows and all log-sum-exps go to the global scratch, where they stay in L2, as 16 bulk copies of
 //   8 KB; after one cluster barrier the owner of a row combines the parts.  (Loads from a peer's shared memory moved the
 //   same rows at about a quarter of the L2 path's rate; a bulk copy per row took 3 000 cycles longer to issue, stores
 //   straight from the registers 4 000.)
@@ -863,10 +863,12 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
       cluster_wait();   // (see the arrival above)
     } else {
       cluster_sync_all();   // every block of the cluster has written its rows
-      // Warp w finishes rows w, w + 13, ... of this block's share (at most two).  Lane 8k + j first fetches the
-      // log-sum-exp of split j for the warp's k-th row, and the first row's first parts are asked for with them.
+      // Warp w finishes rows w, w + 13, ... of this block's share (at most two; one of 16 splits' four).  Lane 8k + j (16k + j)
+      // first fetches the log-sum-exp of split j for the warp's k-th row, and the first row's first parts are asked for with
+      // them.
+      const int lanes = n > 8 ? 16 : 8;   // of a row
       constexpr int kMost = (kH / 4 + kWarps - 1) / kWarps;
-      const int k_of = lane >> 3, j_of = lane & 7;
+      const int k_of = lane / lanes, j_of = lane & (lanes - 1);
       const int rl_mine = warp + kWarps * k_of;
       float my_l = -INFINITY;
       if (k_of < kMost && rl_mine < rows_per && j_of < n)
@@ -886,11 +888,11 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
       if (warp < rows_per) fetch(warp, 0);
       float m = my_l;
 #pragma unroll
-      for (int d = 1; d < 8; d <<= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, d));
+      for (int d = 1; d < 16; d <<= 1) m = d < lanes ? fmaxf(m, __shfl_xor_sync(0xffffffffu, m, d)) : m;
       float wgt = m > -INFINITY ? exp2f(my_l - m) : 0.f;
       float den = wgt;
 #pragma unroll
-      for (int d = 1; d < 8; d <<= 1) den += __shfl_xor_sync(0xffffffffu, den, d);
+      for (int d = 1; d < 16; d <<= 1) den += d < lanes ? __shfl_xor_sync(0xffffffffu, den, d) : 0.f;
       wgt = den > 0.f ? wgt / den : 0.f;
       if (p.lse != nullptr && j_of == 0 && k_of < kMost && rl_mine < rows_per)
         p.lse[static_cast<int64_t>(qi) * kH + row0 + rl_mine] = den > 0.f ? (m + log2f(den)) / kLog2eTc : -INFINITY;
@@ -905,7 +907,7 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
             if (k > 0 || j0 > 0) fetch(rl, j0);
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-              const float w = __shfl_sync(0xffffffffu, wgt, 8 * k + j0 + j);
+              const float w = __shfl_sync(0xffffffffu, wgt, lanes * k + j0 + j);
 #pragma unroll
               for (int u = 0; u < 4; ++u) {
                 acc[u].x += w * v[j][u].x; acc[u].y += w * v[j][u].y; acc[u].z += w * v[j][u].z; acc[u].w += w * v[j][u].w;
@@ -927,7 +929,6 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
 
 }  // namespace
 
-// Largest cluster of full-SM blocks of this kernel the device can place (queried once per process).
 static_assert(sizeof(AttnTcSmem) + 1024 <= 227 * 1024, "shared memory of the attention kernel exceeds one SM");
 
 using AttnTcKernel = void (*)(CUtensorMap, int, CUtensorMap, int, CUtensorMap, int, AttnArgs);
@@ -938,39 +939,17 @@ static AttnTcKernel pick_kernel(const AttnArgs& a) {
   return a.n_split > 1 ? sparse_attn_tc_kernel<true, true> : sparse_attn_tc_kernel<true, false>;
 }
 
-static int max_cluster_blocks() {
-  static const int n = [] {
-    const size_t smem = sizeof(AttnTcSmem) + 1024;
-    AttnTcKernel kernel = sparse_attn_tc_kernel<true, true>;
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess) return 1;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(1, kMaxClusterSplit);
-    cfg.blockDim = dim3(kThreadsAttnTc);
-    cfg.dynamicSmemBytes = smem;
-    int size = 0;
-    const cudaError_t eq = cudaOccupancyMaxPotentialClusterSize(&size, kernel, &cfg);
-    if (eq != cudaSuccess) {
-      (void)cudaGetLastError();
-      return 1;
-    }
-    return size < 1 ? 1 : size;
-  }();
-  return n;
-}
-
-// Row splits the tcgen05 kernel can merge inside a cluster: a power of two that divides the 64 heads, at most 8 blocks
-// and at most what the device can co-schedule.
-bool attn_tc_split_ok(int n_split) {
-  if (n_split == 1) return true;
-  return (n_split == 2 || n_split == 4 || n_split == 8) && n_split <= max_cluster_blocks();
-}
-
 int attn_tc_resident(int n_split) {
-  static const int n[3] = {resident_clusters(reinterpret_cast<const void*>(sparse_attn_tc_kernel<true, true>), kThreadsAttnTc, sizeof(AttnTcSmem) + 1024, 2),
-                           resident_clusters(reinterpret_cast<const void*>(sparse_attn_tc_kernel<true, true>), kThreadsAttnTc, sizeof(AttnTcSmem) + 1024, 4),
-                           resident_clusters(reinterpret_cast<const void*>(sparse_attn_tc_kernel<true, true>), kThreadsAttnTc, sizeof(AttnTcSmem) + 1024, 8)};
-  return n_split == 2 ? n[0] : n_split == 4 ? n[1] : n_split == 8 ? n[2] : 0;
+  auto count = [](int blocks) {
+    return resident_clusters(reinterpret_cast<const void*>(sparse_attn_tc_kernel<true, true>), kThreadsAttnTc, sizeof(AttnTcSmem) + 1024, blocks);
+  };
+  static const int n[4] = {count(2), count(4), count(8), count(kMaxClusterSplit)};   // (queried once per process)
+  return n_split == 2 ? n[0] : n_split == 4 ? n[1] : n_split == 8 ? n[2] : n_split == kMaxClusterSplit ? n[3] : 0;
 }
+
+// Row splits the tcgen05 kernel can merge inside a cluster: a power of two that divides the 64 heads, as many blocks as the
+// device can co-schedule.
+bool attn_tc_split_ok(int n_split) { return n_split == 1 || attn_tc_resident(n_split) > 0; }
 
 bool attn_tc_supported(const AttnArgs& a) {
   return a.H == kH && a.DQK == kDQK && a.DV == kDV && a.v == a.k && a.ld_v == a.ld_k;
@@ -998,6 +977,7 @@ cudaError_t launch_attn_tc(const AttnArgs& a, cudaStream_t st, int64_t* n_launch
     kernel<<<dim3(a.n_query, 1, 1), kThreadsAttnTc, smem, st>>>(q_map, q_tma, k_map, k_tma, g_map, k_g4, a);
   } else {
     if (!attn_tc_split_ok(a.n_split)) return cudaErrorInvalidValue;
+    if (a.n_split > 8 && (e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess) return e;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(a.n_query, a.n_split, 1);
     cfg.blockDim = dim3(kThreadsAttnTc);

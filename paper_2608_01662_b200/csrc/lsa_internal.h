@@ -160,7 +160,8 @@ int attn_tc_resident(int n_split);
 // Clusters of `blocks` blocks of a kernel that the device can hold at the same time (0: it cannot, or cannot say).  Fewer than
 // the SMs divided by the cluster's size: a cluster lies in one GPC, and one block per SM leaves a rest in each.
 inline int resident_clusters(const void* kernel, int threads, size_t smem, int blocks) {
-  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) == cudaSuccess) {
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) == cudaSuccess &&
+      (blocks <= 8 || cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess)) {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(static_cast<unsigned>(blocks) * 256);
     cfg.blockDim = dim3(static_cast<unsigned>(threads));

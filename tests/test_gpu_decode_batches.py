@@ -6,6 +6,8 @@ import torch
 from paper_2608_01662_b200.configs import CONFIGS
 from paper_2608_01662_b200.workload import DecodeWorkload
 
+import parity_util as pu
+
 pytestmark = pytest.mark.gpu
 
 
@@ -23,3 +25,16 @@ def test_blocks_that_go_on(cuda_device, batch, lo, hi, layers):
         for a, b in zip(first, wl.out):
             differ += (a.view(torch.int16) != b.view(torch.int16)).sum()
     assert wl.ctx.status() == 0 and int(differ) == 0
+
+
+@pytest.mark.parametrize("batch,lo,hi", [(1, 20000, 20000), (3, 1, 400), (7, 900, 3000)])
+def test_sixteen_splits(cuda_device, batch, lo, hi):
+    """Sixteen row splits of a sequence, also where most of them have no rows."""
+    cfg = CONFIGS["cfg4"].replace(batch=batch, ctx_lo=lo, ctx_hi=hi, R=2, seed=batch)
+    wl = DecodeWorkload(cfg, cuda_device)
+    wl.prepare()
+    wl.ctx.tune(2, 16)             # LSA_TUNE_ATTN_SPLIT
+    wl.step()
+    assert wl.ctx.status() == 0
+    m = pu.check_decode(wl, range(batch))
+    m.assert_ok(pu.TOL_BF16)
