@@ -51,7 +51,8 @@ constexpr int kIssuers = 3;                 // MMA-issuing warps 1..3
 // run two phases ahead of a barrier shared with other issuers would take an old phase for the one it waits for.)
 __device__ __forceinline__ int acc_of_tile(int i) { return i % kIssuers + kIssuers * ((i / kIssuers) & 1); }
 __device__ __forceinline__ uint32_t acc_use_parity(int i) { return static_cast<uint32_t>(i / (2 * kIssuers)) & 1u; }
-constexpr int kSelBar = 1;                  // named barrier of threads 0-255 (the selections)
+constexpr int kSelBar = 1, kWarmBar = 2;    // named barriers of threads 0-255 (the selections) and of the last warp
+constexpr int kWarmWarp = kThreadsFp / 32 - 1;   // idle until the tiles: it fetches the selection's instructions
 
 template <bool E4M3>
 struct FpSmem {
@@ -76,7 +77,8 @@ struct FpSmem {
   uint32_t tmem_slot;
 };
 static_assert(sizeof(FpSmem<true>) + 1024 <= 227 * 1024 && sizeof(FpSmem<false>) + 1024 <= 227 * 1024, "shared memory");
-static_assert(FpSmem<true>::kSlots * FpSmem<true>::kTileBytes >= kMaxSlotsFp * 4, "page keys fit the ring");
+static_assert(FpSmem<true>::kSlots * FpSmem<true>::kTileBytes >= kMaxSlotsFp * 4 + kShortWarm && FpSmem<false>::kSlots * FpSmem<false>::kTileBytes >= kMaxSlotsFp * 4 + kShortWarm,
+              "page keys and the made-up ones fit the ring");
 static_assert(FpSmem<true>::kSlots % kIssuers == 0 && FpSmem<false>::kSlots % kIssuers == 0, "a ring slot has one consumer");
 
 __device__ __forceinline__ uint32_t cluster_rank() {
@@ -189,9 +191,13 @@ fine_paged_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
     tc::tmem_alloc(smem_u32(&sm.tmem_slot), kTmemColsFp);
     tc::tmem_relinquish();
   }
+  if (warp == kWarmWarp) {
+    short_select_warm<kWarmBar>(smem_u32(sm.k) + kMaxSlotsFp * 4);   // behind the page scores' keys
+    tc::fence_proxy_async();   // (that part of the ring is handed to the TMA copies)
+  }
   if constexpr (E4M3) {
     // query heads -> three e5m2 planes in the swizzled K-major layout; head weights take the inverse of the head's scale
-    for (int u = tid; u < kHI * 8; u += kThreadsFp) {   // 8 threads per head, 16 dims each (a warp never straddles a head group)
+    for (int u = tid; u < kHI * 8 && warp != kWarmWarp; u += kThreadsFp - 32) {   // 8 threads per head, 16 dims each (a warp never straddles a head group)
       const int h = u >> 3, sub = u & 7;
       const uint4* src = reinterpret_cast<const uint4*>(reinterpret_cast<const uint8_t*>(p.q_idx) +
                                                         (static_cast<int64_t>(qi) * kHI + h) * kDI * 2 + sub * 32);

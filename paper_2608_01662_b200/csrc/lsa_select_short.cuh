@@ -46,10 +46,10 @@ static_assert(kShortScratch <= sizeof(SelectScratch), "the scratch of the radix 
 // keys: shared address of n <= kShortMax keys.  list: shared address where the selected indices go, ascending, 16 bits each (it
 // may be `keys`: they are in registers by then).  scratch: shared address of kShortScratch bytes, 16-byte aligned.  Every one of
 // the 256 threads calls it, converged; the keys must be visible to all of them.  Returns the number selected, min(k, #present),
-// with the list visible.
-template <int BAR>
-__device__ __noinline__ int short_select(uint32_t keys, int n, int k, uint32_t list, uint32_t scratch) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+// with the list visible.  They are threads 0-255 of the block and meet on barrier `bar`; short_select_warm calls it otherwise.
+static __device__ __noinline__ int short_select(uint32_t keys, int n, int k, uint32_t list, uint32_t scratch, int bar, int tid, int n_threads) {
+  const int lane = tid & 31, warp = tid >> 5;
+  auto sync = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(bar), "r"(n_threads) : "memory"); };
   constexpr uint32_t kAll = 0xffffffffu;
   const int base = tid * kShortPer;   // the thread holds items base .. base + 15
   const uint32_t of_warp = scratch + kShortWarp + 4u * (lane & 7), my_warp = scratch + kShortWarp + 4u * warp;
@@ -100,7 +100,7 @@ __device__ __noinline__ int short_select(uint32_t keys, int n, int k, uint32_t l
       short_sts(my_warp + 32u, mn);
       short_sts(my_warp + 64u, cnt);
     }
-    select_sync<BAR>();   // (every key has been read: `list` may be written from the next barrier on)
+    sync();   // (every key has been read: `list` may be written from the next barrier on)
     mx = __reduce_max_sync(kAll, short_lds(of_warp));
     mn = __reduce_min_sync(kAll, short_lds(of_warp + 32u));
     if (pass == 0) {
@@ -125,7 +125,7 @@ __device__ __noinline__ int short_select(uint32_t keys, int n, int k, uint32_t l
       part[j] = bin0 - 4u * __float_as_uint(fminf((key_value(v[j]) - lo) * scale, kShortBins - 1.f) + 8388608.f);   // (rounded to a whole number)
 #pragma unroll
     for (int j = 0; j < kShortPer; ++j) red_if((act >> j) & 1u, part[j]);
-    select_sync<BAR>();
+    sync();
     uint32_t h[4];
     asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(h[0]), "=r"(h[1]), "=r"(h[2]), "=r"(h[3]) : "r"(my_bins) : "memory");
     clear_bins();
@@ -137,7 +137,7 @@ __device__ __noinline__ int short_select(uint32_t keys, int n, int k, uint32_t l
       if (lane >= d) incl += x;
     }
     if (lane == 31) short_sts(my_warp + 96u, incl);
-    select_sync<BAR>();
+    sync();
     incl += __reduce_add_sync(kAll, lane < warp ? short_lds(of_warp + 96u) : 0u);
     uint32_t before = incl - sum;
     if (before < static_cast<uint32_t>(rem) && static_cast<uint32_t>(rem) <= incl) {   // exactly one thread
@@ -152,7 +152,7 @@ __device__ __noinline__ int short_select(uint32_t keys, int n, int k, uint32_t l
       short_sts(found + 4u, before);
       short_sts(found + 8u, b == 0 ? h[0] : b == 1 ? h[1] : b == 2 ? h[2] : h[3]);
     }
-    select_sync<BAR>();
+    sync();
     const uint32_t bin = scratch + kShortHist + 4u * short_lds(found);
     rem -= static_cast<int>(short_lds(found + 4u));
     const int members = static_cast<int>(short_lds(found + 8u));
@@ -167,7 +167,7 @@ __device__ __noinline__ int short_select(uint32_t keys, int n, int k, uint32_t l
       short_sts(scratch + kShortMembers + 4u * at, key);
       act &= act - 1u;
     }
-    select_sync<BAR>();
+    sync();
     const uint32_t m = lane < members ? short_lds(scratch + kShortMembers + 4u * lane) : 0u;
     int larger = 0, same = 0;
 #pragma unroll 1
@@ -197,7 +197,7 @@ __device__ __noinline__ int short_select(uint32_t keys, int n, int k, uint32_t l
       for (int j = 0; j < kShortPer; ++j) c += v[j] >= cand;
       c = __reduce_add_sync(kAll, c);
       if (lane == 0) short_sts(my_warp + 96u + 32u * (b & 1), c);
-      select_sync<BAR>();
+      sync();
       c = __reduce_add_sync(kAll, lane < 8 ? short_lds(of_warp + 96u + 32u * (b & 1)) : 0u);
       if (static_cast<int>(c) >= k) {
         T = cand;
@@ -222,7 +222,7 @@ __device__ __noinline__ int short_select(uint32_t keys, int n, int k, uint32_t l
     if (lane >= d) upto += x;
   }
   if (lane == 31) short_sts(my_warp + 160u, upto);
-  select_sync<BAR>();
+  sync();
   const uint32_t one = lane < 8 ? short_lds(of_warp + 160u) : 0u;
   const uint32_t all = __reduce_add_sync(kAll, one);
   upto += __reduce_add_sync(kAll, lane < warp ? one : 0u) - mine;   // what lies before this thread
@@ -237,8 +237,27 @@ __device__ __noinline__ int short_select(uint32_t keys, int n, int k, uint32_t l
     sts16_if(take, out, static_cast<uint32_t>(base + j));
     out += take ? 2u : 0u;
   }
-  select_sync<BAR>();
+  sync();
   return min(k, n_valid);
+}
+template <int BAR>
+__device__ __forceinline__ int short_select(uint32_t keys, int n, int k, uint32_t list, uint32_t scratch) {
+  return short_select(keys, n, k, list, scratch, BAR, static_cast<int>(threadIdx.x), kSelThreads);
+}
+// A selection of 64 made-up keys by one otherwise idle warp, on barrier BAR and in shared memory that nobody uses
+// (kShortWarm bytes, 16-byte aligned): its instructions are then at hand when the block needs them.  The first selection of a
+// decode kernel spent 6 to 8 of its 11 to 13 thousand cycles on their fetch.
+constexpr uint32_t kShortWarm = 2048 + ((kShortScratch + 15u) & ~15u);
+template <int BAR>
+__device__ __forceinline__ void short_select_warm(uint32_t area) {
+  const int lane = threadIdx.x & 31;
+  const uint32_t scratch = area + 2048u;
+  for (uint32_t a = 4u * lane; a < 2048u; a += 128u) short_sts(area + a, score_key(1.f + static_cast<float>(a)));
+  for (uint32_t a = 4u * lane; a < kShortScratch; a += 128u) short_sts(scratch + a, 0u);
+  __syncwarp();
+  if (lane < 8) short_sts(scratch + kShortWarp + 32u + 4u * lane, 0xffffffffu);   // seven warps without keys
+  __syncwarp();
+  (void)short_select(area, 64, 8, area, scratch, BAR, lane, 32);
 }
 // r-th item of the list
 __device__ __forceinline__ int short_item(uint32_t list, int r) {
