@@ -835,28 +835,51 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
       // copies still read this block's shared memory).  A thread arrives as soon as it has seen this block's own
       // bytes complete and waits at the very end, by when the peer has normally long arrived.
       cluster_arrive();
-#pragma unroll
-      for (int rl = warp; rl < kH / 2; rl += kWarps) {   // a warp finishes a row: lane l the chunks l, l + 32, ...
-        const int R = row0 + rl;
-        const float l_own = sm.lse_own[R], l_peer = sm.lse_peer[rl];
-        const float m = fmaxf(l_own, l_peer);
-        float w_own = m > -INFINITY ? exp2f(l_own - m) : 0.f, w_peer = m > -INFINITY ? exp2f(l_peer - m) : 0.f;
-        const float den = w_own + w_peer;
-        const float r_den = den > 0.f ? 1.f / den : 0.f;
-        w_own *= r_den;
-        w_peer *= r_den;
-        if (lane == 0 && p.lse != nullptr)
-          p.lse[static_cast<int64_t>(qi) * kH + R] = den > 0.f ? (m + log2f(den)) / kLog2eTc : -INFINITY;
+      // A warp finishes rows w, w + 13, w + 26 of this block's 32: lane k works out the k-th row's weights, and a row's parts
+      // (lane l: the 16-byte chunks l, l + 32, ...) are read while the row before is written.
+      constexpr int kRowsOfWarp = (kH / 2 + kWarps - 1) / kWarps;
+      float4 a[2][4], b[2][4];
+      auto fetch = [&](int k) {
+        const int rl = min(warp + kWarps * k, kH / 2 - 1);
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-          // 16-byte chunk (four dims) lane + 32u of the row: dims 128u .. of it are half u & 1, column steps 2 (u >> 1) and
-          // one more; the warp that staged them is split + 2 * half here, and sent from half * kWarpStage there
+          // chunk lane + 32u (four dims) of the row: dims 128u .. of it are half u & 1, column steps 2 (u >> 1) and one
+          // more; the warp that staged them is split + 2 * half here, and sent from half * kWarpStage there
           const int ch = (2 * (u >> 1) + (lane >> 4)) * 8192 + rl * 256 + (((lane & 15) ^ (rl & 15)) << 4);
-          const float4 a = *reinterpret_cast<const float4*>(stage + (split + 2 * (u & 1)) * kWarpStage + ch);
-          const float4 b = *reinterpret_cast<const float4*>(stage + kRecvOffset + (u & 1) * kWarpStage + ch);
+          a[k & 1][u] = *reinterpret_cast<const float4*>(stage + (split + 2 * (u & 1)) * kWarpStage + ch);
+          b[k & 1][u] = *reinterpret_cast<const float4*>(stage + kRecvOffset + (u & 1) * kWarpStage + ch);
+        }
+      };
+      fetch(0);
+      float my_own = 0.f, my_peer = 0.f;
+      {
+        const int rl = warp + kWarps * lane;
+        if (lane < kRowsOfWarp && rl < kH / 2) {
+          const int R = row0 + rl;
+          const float l_own = sm.lse_own[R], l_peer = sm.lse_peer[rl];
+          const float m = fmaxf(l_own, l_peer);
+          my_own = m > -INFINITY ? exp2f(l_own - m) : 0.f;
+          my_peer = m > -INFINITY ? exp2f(l_peer - m) : 0.f;
+          const float den = my_own + my_peer;
+          const float r_den = den > 0.f ? 1.f / den : 0.f;
+          my_own *= r_den;
+          my_peer *= r_den;
+          if (p.lse != nullptr) p.lse[static_cast<int64_t>(qi) * kH + R] = den > 0.f ? (m + log2f(den)) / kLog2eTc : -INFINITY;
+        }
+        __syncwarp();
+      }
+#pragma unroll
+      for (int k = 0; k < kRowsOfWarp; ++k) {
+        if (k + 1 < kRowsOfWarp) fetch(k + 1);
+        const float w_own = __shfl_sync(0xffffffffu, my_own, k), w_peer = __shfl_sync(0xffffffffu, my_peer, k);
+        const int rl = warp + kWarps * k;
+        if (rl >= kH / 2) break;   // warp-uniform
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const float4 x = a[k & 1][u], y = b[k & 1][u];
           uint2 o;
-          o.x = pack_bf16(w_own * a.x + w_peer * b.x, w_own * a.y + w_peer * b.y);
-          o.y = pack_bf16(w_own * a.z + w_peer * b.z, w_own * a.w + w_peer * b.w);
+          o.x = pack_bf16(w_own * x.x + w_peer * y.x, w_own * x.y + w_peer * y.y);
+          o.y = pack_bf16(w_own * x.z + w_peer * y.z, w_own * x.w + w_peer * y.w);
           *reinterpret_cast<uint2*>(out + static_cast<int64_t>(rl) * kDV + (lane + 32 * u) * 4) = o;
         }
       }
