@@ -4,31 +4,36 @@
 // A block works on one query at a time (or on one row split of one sequence in decode).  Its 64 heads are the M = 64
 // rows of every MMA; the attended cache rows stream through a ring of three 64-key shared tiles, into which Q goes
 // as an item of its own.  Prefill blocks are persistent: when a query's last copies are out, the next query's Q and
-// first tiles follow them into the ring, so that only the softmax of one tile stands between two queries.
+// first tiles follow them into the ring, and warps of their own move that Q and write this O, so that the tensor pipe
+// waits between two queries only for O to leave tensor memory.
 //
-//   warps 7-12  gather: two warps per ring slot.  They wait for the slot, copy rows [window | sink | sparse] (or those of the
+//   warps 10-15 gather: two warps per ring slot.  They wait for the slot, copy rows [window | sink | sparse] (or those of the
 //               caller's row list) into its 128B-swizzled K-major tile with coalesced 16-byte cp.async, a row by one warp
 //               (spreading a tile's chunks over the warps was measured 1.3 x slower, a TMA gather of four rows per
 //               instruction - AttnArgs::gather4 - as well: the TMA unit takes about 26 cycles for its 512 bytes), and hand
 //               it over when it has landed; tiles of 64 consecutive window rows and Q come as one TMA box each.
-//   warp 6      scheduler: one thread publishes the block's jobs (query, row count).  In prefill it takes the block index
-//               of a block that has not started yet (cluster launch control), one job ahead of the one being worked on,
-//               latest query first: those attend the most rows.
-//   warps 4, 5  one thread each issues tcgen05.mma:
-//                 S = Q K^T   warp 4, M64 N64 K16, Q in tensor memory (the rope dims in shared memory), as two accumulation
+//   warps 4-7   the ends of a job: they move Q to tensor memory (as soon as the last Q K^T of the job before is complete: the
+//               softmax and P V of its last tile run meanwhile) and, once its last P V is, write O / l to global; only the
+//               next job's P V waits for them.  With both done by the softmax warps a query cost 7.2 thousand cycles beside
+//               its tiles: 1000 queries of up to 1000 rows 625 -> 597 us, a prompt of 32768 30.4 -> 30.0 ms.
+//               One thread of warp 4 is the scheduler and publishes the block's jobs (query, row count).  In prefill it takes
+//               the block index of a block that has not started yet (cluster launch control), one job ahead of the one being
+//               worked on, latest query first: those attend the most rows.
+//   warps 8, 9  one thread each issues tcgen05.mma:
+//                 S = Q K^T   warp 8, M64 N64 K16, Q in tensor memory (the rope dims in shared memory), as two accumulation
 //                             chains: dims 0-255 and rope dims 0-31 in the even half of the lanes, dims 256-511 and rope
 //                             dims 32-63 in the odd half (an M = 64 accumulator and its A operand use 16 of the 32 lanes of
 //                             each quarter, so both halves of Q share their columns).  36 MMAs at the pipe's 32 cycles.
-//                 O += P V    warp 5, tcgen05.mma.ws M64 N256 K16, P in shared memory; V is the key tile read MN-major, so
+//                 O += P V    warp 9, tcgen05.mma.ws M64 N256 K16, P in shared memory; V is the key tile read MN-major, so
 //                             that a cache row is fetched once.  The .ws form spreads the 64 rows over all 128 lanes (heads
 //                             in lanes 0-63 and again in 64-127, each with half of the value dims), which is the full data
 //                             path: 81 cycles where the plain M64 N256 form takes 129.
 //               Two threads, because one stalls for 300 to 500 cycles after each batch before it gets to the next, and
 //               two S buffers, so that Q K^T of the next tile need not wait for the softmax of this one: 2 340 cycles per
 //               tile with one of each.
-//   warps 0-3   softmax: move Q to tensor memory; per tile add the two partial sums (read as 16-lane fragments, so both
+//   warps 0-3   softmax: per tile add the two partial sums (read as 16-lane fragments, so both
 //               land in the same registers), running max with lazy rescaling of O, exp2, fp32 row sums, P as bf16 into
-//               the tile's rope block (64 x 64 values; Q K^T was its only reader); at the end of a query O / l to global.
+//               the tile's rope block (64 x 64 values; Q K^T was its only reader); a split's partial O to the merge.
 //
 // What bounds it (prefill): per 64-key tile the tensor pipe needs 36 x 32 + 8 x 81 = 1 800 cycles (2 176 with the plain
 // form for P V), and shared memory is read and written for about as long: 576 (Q K^T) + 640 (P V) + 576 (the copies).
@@ -52,7 +57,7 @@ constexpr int kAtomBytes = 64 * 128;         // 64 rows x 128 bytes
 constexpr int kSlotBytes = kAtoms * kAtomBytes;
 
 constexpr int kRing = 3;                     // 64-key tiles (or Q) in shared memory
-constexpr int kSoftmaxWarps = 4, kQkWarp = 4, kPvWarp = 5, kSchedWarp = 6, kGatherWarp0 = 7;
+constexpr int kSoftmaxWarps = 4, kDrainWarp0 = 4, kDrainWarps = 4, kQkWarp = 8, kPvWarp = 9, kGatherWarp0 = 10;
 constexpr int kSlotWarps = 2;                // gather warps of a ring slot
 constexpr int kGatherWarps = kRing * kSlotWarps;
 constexpr int kThreadsAttnTc = 32 * (kGatherWarp0 + kGatherWarps);
@@ -63,12 +68,14 @@ constexpr float kLog2eTc = 1.4426950408889634f;
 constexpr int kMaxClusterSplit = 16;         // row splits of one sequence = blocks of one cluster (eight is the portable limit)
 constexpr int kFirstTileCycles = 8192;       // longest that a block's second tile is held back for the first
 constexpr float kRescaleGap = 8.f;           // rescale O only when the row max grows by more than 2^8
-constexpr int kJobReaders = kSoftmaxWarps + 2 + kGatherWarps;   // warps that release a job slot
+constexpr int kJobReaders = kSoftmaxWarps + kDrainWarps + 2 + kGatherWarps;   // warps that release a job slot
 
 struct AttnTcSmem {
   alignas(1024) uint8_t k[kRing][kAtoms][kAtomBytes];       // [ring slot][column block][64 rows x 128 B]
   alignas(1024) uint8_t q_rope[kAtomBytes];                 // Q[:, 512:576], 64 rows x 128 B
-  alignas(8) uint64_t k_full[kRing], k_empty[kRing], p_ready[kRing], q_tmem[2], s_full[2], s_free[2], job_full[2], job_empty[2], clc_full;
+  alignas(8) uint64_t k_full[kRing], k_empty[kRing], p_ready[kRing], pv_done[kRing], q_tmem[2], s_full[2], s_free[2], job_full[2], job_empty[2], clc_full;
+  alignas(8) uint64_t q_free;             // every Q K^T of a job is complete
+  alignas(8) uint64_t o_full[2], o_free;  // a job's O and row sums are complete (by job parity); O has been read out
   alignas(8) uint64_t recv_full;          // two-split launches: the peer's rows and log-sum-exps have arrived
   alignas(16) uint4 clc;                  // answer of the cluster launch control
   alignas(8) int2 job[2];                 // {query or -1 = no more, rows it attends}
@@ -203,15 +210,19 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
       tc::mbar_init(smem_u32(&sm.k_full[b]), kSlotWarps);
       tc::mbar_init(smem_u32(&sm.k_empty[b]), 1);
       tc::mbar_init(smem_u32(&sm.p_ready[b]), 1);
+      tc::mbar_init(smem_u32(&sm.pv_done[b]), 1);
     }
     for (int b = 0; b < 2; ++b) {
-      tc::mbar_init(smem_u32(&sm.q_tmem[b]), kSoftmaxWarps);   // by job parity: a job without tiles may be overtaken by the next
+      tc::mbar_init(smem_u32(&sm.o_full[b]), 1 + kSoftmaxWarps);
+      tc::mbar_init(smem_u32(&sm.q_tmem[b]), kDrainWarps);     // by job parity: a job without tiles may be overtaken by the next
       tc::mbar_init(smem_u32(&sm.s_full[b]), 1);
       tc::mbar_init(smem_u32(&sm.s_free[b]), kSoftmaxWarps);
       tc::mbar_init(smem_u32(&sm.job_full[b]), 1);
       tc::mbar_init(smem_u32(&sm.job_empty[b]), kJobReaders);
     }
     tc::mbar_init(smem_u32(&sm.clc_full), 1);
+    tc::mbar_init(smem_u32(&sm.q_free), 1);
+    tc::mbar_init(smem_u32(&sm.o_free), kDrainWarps);
     if constexpr (kClustered) {
       tc::mbar_init(smem_u32(&sm.recv_full), 1);
       if (p.n_split == 2) tc::mbar_expect_tx(smem_u32(&sm.recv_full), kRecvBytes);   // armed once; used once per launch
@@ -239,7 +250,8 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   };
-  if (!(early_rows && warp >= kSchedWarp)) dependency_wait();
+  const bool reads_early = warp >= kGatherWarp0 || (warp >= kDrainWarp0 && warp < kDrainWarp0 + kDrainWarps);
+  if (!(early_rows && reads_early)) dependency_wait();
 
   // ---- the parts of a job that every role derives for itself
   struct Job {
@@ -276,45 +288,133 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
   auto slot_of = [](int pos) -> int { return pos % kRing; };
   auto use_of = [](int pos) -> uint32_t { return static_cast<uint32_t>(pos / kRing) & 1u; };   // parity of the slot's use
 
-  if (warp == kSchedWarp) {
-    // ================= scheduler =================
-    if (tc::elect_one()) {
+  if (warp >= kDrainWarp0 && warp < kDrainWarp0 + kDrainWarps) {
+    // ================= scheduler, Q and O =================
+    const int dw = warp - kDrainWarp0;   // TMEM lanes 32 dw .. +31
+    const uint32_t lane_addr = static_cast<uint32_t>(32 * dw) << 16;
+    // n-th job of this block, by one thread; false: there are no more.  (Its slot is free once every role is through with the
+    // job before the previous one, so at most one job beyond the one being worked on is taken from the other blocks.)
+    auto publish = [&](int n) -> bool {
+      if (!tc::mbar_wait(smem_u32(&sm.job_empty[n & 1]), ((n >> 1) & 1) ^ 1, p.status)) return false;
       int qi = kClustered ? static_cast<int>(blockIdx.x) : p.n_query - 1 - static_cast<int>(blockIdx.x);
-      for (int n = 0;; ++n) {
-        // (the slot is free once every role is through with the job before the previous one, so at most one job beyond
-        // the one being worked on is taken from the other blocks)
-        if (!tc::mbar_wait(smem_u32(&sm.job_empty[n & 1]), ((n >> 1) & 1) ^ 1, p.status)) break;
-        if (n > 0) {
-          qi = -1;
-          if constexpr (!kClustered) {
-            tc::mbar_expect_tx(smem_u32(&sm.clc_full), 16);
-            clc_request(smem_u32(&sm.clc), smem_u32(&sm.clc_full));
-            if (!tc::mbar_wait(smem_u32(&sm.clc_full), (n - 1) & 1, nullptr)) {   // (an answer on its way is waited for in any case)
-              report_status(p.status, kDevTimeout);
-              break;
-            }
-            int x;
-            if (clc_answer(smem_u32(&sm.clc), &x)) qi = p.n_query - 1 - x;
-            tc::fence_proxy_async();   // the answer has been read: the next one may overwrite it
+      if (n > 0) {
+        qi = -1;
+        if constexpr (!kClustered) {
+          tc::mbar_expect_tx(smem_u32(&sm.clc_full), 16);
+          clc_request(smem_u32(&sm.clc), smem_u32(&sm.clc_full));
+          if (!tc::mbar_wait(smem_u32(&sm.clc_full), (n - 1) & 1, nullptr)) {   // (an answer on its way is waited for in any case)
+            report_status(p.status, kDevTimeout);
+            return false;
           }
+          int x;
+          if (clc_answer(smem_u32(&sm.clc), &x)) qi = p.n_query - 1 - x;
+          tc::fence_proxy_async();   // the answer has been read: the next one may overwrite it
         }
-        int n_tot = 0;
-        if (qi >= 0) {
-          if constexpr (kRows) {
-            n_tot = p.n_rows[qi];
-          } else {
-            const int64_t t = p.q_pos0 + qi;
-            const int64_t win0 = max64(p.S, t - p.W + 1);
-            n_tot = static_cast<int>(min64(p.S, t + 1) + max64(0, t - win0 + 1)) + p.n_sparse[qi];
-          }
-        }
-        sm.job[n & 1] = make_int2(qi, n_tot);
-        tc::mbar_arrive(smem_u32(&sm.job_full[n & 1]));
-        if (qi < 0) break;
       }
-    }
+      int n_tot = 0;
+      if (qi >= 0) {
+        if constexpr (kRows) {
+          n_tot = p.n_rows[qi];
+        } else {
+          const int64_t t = p.q_pos0 + qi;
+          const int64_t win0 = max64(p.S, t - p.W + 1);
+          n_tot = static_cast<int>(min64(p.S, t + 1) + max64(0, t - win0 + 1)) + p.n_sparse[qi];
+        }
+      }
+      sm.job[n & 1] = make_int2(qi, n_tot);
+      tc::mbar_arrive(smem_u32(&sm.job_full[n & 1]));
+      return qi >= 0;
+    };
+    bool more = dw == 0 && lane == 0;   // this thread publishes, and there may be more jobs
+    if (more) more = publish(0);
+    if (more) more = publish(1);
     __syncwarp();
     if (early_rows) dependency_wait();
+    // Q of a job from its ring slot to tensor memory, in the order the tensor core reads an A operand (two dims per column)
+    auto move_q = [&](int pos, int n_job) -> bool {
+      if (!__all_sync(0xffffffffu, tc::mbar_wait(smem_u32(&sm.k_full[slot_of(pos)]), use_of(pos), p.status))) return false;
+      const int row = 16 * dw + (lane & 15), hi = lane >> 4;
+      const uint8_t* qs = sm.k[slot_of(pos)][0] + row * 128;
+#pragma unroll 1
+      for (int part = 0; part < 4; ++part) {
+        uint32_t w[32];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          const int c = 32 * hi + 8 * part + j;
+          const uint4 u = *reinterpret_cast<const uint4*>(qs + (c >> 3) * kAtomBytes + (((c & 7) ^ (row & 7)) << 4));
+          w[4 * j] = u.x; w[4 * j + 1] = u.y; w[4 * j + 2] = u.z; w[4 * j + 3] = u.w;
+        }
+        tc::tmem_st32(tmem_base + lane_addr + kColQ + part * 32, w);
+      }
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {   // the warp's 16 rows of the rope block, as they lie
+        const int at = 16 * dw * 128 + (32 * j + lane) * 16;
+        *reinterpret_cast<uint4*>(sm.q_rope + at) = *reinterpret_cast<const uint4*>(sm.k[slot_of(pos)][8] + at);
+      }
+      tc::fence_proxy_async();
+      tc::tmem_st_wait();
+      tc::fence_before_sync();
+      __syncwarp();
+      if (lane == 0) tc::mbar_arrive(smem_u32(&sm.q_tmem[n_job & 1]));
+      return true;
+    };
+    int2 jd;
+    int base = 0;
+    bool ok = __all_sync(0xffffffffu, wait_job(0, &jd));
+    Job jb = job_of(jd);
+    ok = ok && move_q(base + jb.q_at, 0);
+    if constexpr (!kClustered) {
+      // Of O a warp reads its TMEM lanes: heads 32 (dw & 1) + lane, half dw >> 1 of the value dims of each 256.
+      const int head_o = 32 * (dw & 1) + lane, half_o = dw >> 1;
+      for (int n = 0; ok; ++n) {
+        const Job done = jb;
+        base += done.n_tiles + 1;
+        ok = __all_sync(0xffffffffu, wait_job(n + 1, &jd));
+        if (!ok) break;
+        if (jd.x >= 0) {   // the next Q follows the last Q K^T of this job, whose softmax and P V are still to come
+          jb = job_of(jd);
+          ok = __all_sync(0xffffffffu, tc::mbar_wait(smem_u32(&sm.q_free), n & 1, p.status));
+          if (!ok) break;
+          tc::fence_after_sync();
+          ok = move_q(base + jb.q_at, n + 1);
+          if (!ok) break;
+        }
+        ok = __all_sync(0xffffffffu, tc::mbar_wait(smem_u32(&sm.o_full[n & 1]), (n >> 1) & 1, p.status));
+        if (!ok) break;
+        tc::fence_after_sync();
+        // ---- O / l: a thread owns half of the value dims of a head, in two runs of 128
+        const float inv = sm.inv[n & 1][head_o];
+        uint8_t* dst = reinterpret_cast<uint8_t*>(reinterpret_cast<__nv_bfloat16*>(p.out) + (static_cast<int64_t>(done.qi) * kH + head_o) * kDV + 128 * half_o);
+        const bool by32 = (reinterpret_cast<uintptr_t>(p.out) & 31u) == 0;
+#pragma unroll 1
+        for (int c = 0; c < 256; c += 64) {
+          uint32_t o[64];
+          if (done.n_tiles > 0) {
+            tc::tmem_ld64(tmem_base + lane_addr + c, o);
+            tc::tmem_ld_wait();
+          } else {
+#pragma unroll
+            for (int j = 0; j < 64; ++j) o[j] = 0u;
+          }
+          if (c == 192) {   // all of O is in registers: the next job's P V may begin
+            tc::fence_before_sync();
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive(smem_u32(&sm.o_free));
+          }
+          uint32_t w[32];
+#pragma unroll
+          for (int j = 0; j < 32; ++j) w[j] = pack_bf16(__uint_as_float(o[2 * j]) * inv, __uint_as_float(o[2 * j + 1]) * inv);
+          uint8_t* d = dst + ((c >> 7) * 256 + (c & 127)) * 2;
+#pragma unroll
+          for (int j = 0; j < 32; j += 8) store_words8(d + j * 4, w + j, by32);
+        }
+        __syncwarp();
+        if (lane == 0) tc::mbar_arrive(smem_u32(&sm.job_empty[n & 1]));
+        if (more) more = publish(n + 2);
+        __syncwarp();
+        if (jd.x < 0) break;
+      }
+    }
   } else if (warp >= kGatherWarp0) {
     // ================= gather warps =================
     const int grp = (warp - kGatherWarp0) / kSlotWarps, gw = (warp - kGatherWarp0) % kSlotWarps;   // ring slot, warp of its group
@@ -474,7 +574,12 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
           tc::umma_commit(smem_u32(&sm.s_full[g & 1]));
         }
         base += jb.n_tiles + 1;
-        if (ok) tc::mbar_arrive(smem_u32(&sm.job_empty[n & 1]));
+        if (!ok) break;
+        if constexpr (!kClustered) {
+          if (jb.n_tiles > 0) tc::umma_commit(smem_u32(&sm.q_free));
+          else tc::mbar_arrive(smem_u32(&sm.q_free));
+        }
+        tc::mbar_arrive(smem_u32(&sm.job_empty[n & 1]));
       }
     }
   } else if (warp == kPvWarp) {
@@ -489,7 +594,8 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
         int2 jd;
         if (!wait_job(n, &jd) || jd.x < 0) break;
         const Job jb = job_of(jd);
-        for (int i = 0; i < jb.n_tiles; ++i, ++g) {
+        if (!kClustered && n > 0) ok = tc::mbar_wait(smem_u32(&sm.o_free), (n - 1) & 1, p.status);   // the last job's O has been read out
+        for (int i = 0; i < jb.n_tiles && ok; ++i, ++g) {
           const int slot = slot_of(base + i + (i >= jb.q_at ? 1 : 0));
           ok = tc::mbar_wait(smem_u32(&sm.p_ready[g % kRing]), (g / kRing) & 1, p.status);
           if (!ok) break;
@@ -501,12 +607,19 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
             for (int kk = 0; kk < kTileKeys / 16; ++kk)   // keys 16*kk .. +15
               tc::umma_ws_ss(tmem_base + 128 * y, tc::desc_advance(dpb, kk * 32), tc::desc_advance(dvb, 4 * y * kAtomBytes + kk * 2048),
                              idesc, (i > 0) || (kk > 0));
-          // one completion signal per tile: "P V of the tile done" frees the ring slot for the gather warps and tells the
-          // softmax warps that O may be touched again
+          // "P V of the tile done" frees the ring slot for the gather warps, and tells the softmax warps that O may be touched
+          // again: where a block goes on to another job by a barrier of its own, since the slot's may go on with the next
+          // query (which only its issuer waits for) before they look, and a barrier two uses on looks like an unused one
           tc::umma_commit(smem_u32(&sm.k_empty[slot]));
+          if constexpr (!kClustered) tc::umma_commit(smem_u32(&sm.pv_done[g % kRing]));
         }
         base += jb.n_tiles + 1;
-        if (ok) tc::mbar_arrive(smem_u32(&sm.job_empty[n & 1]));
+        if (!ok) break;
+        if constexpr (!kClustered) {
+          if (jb.n_tiles > 0) tc::umma_commit(smem_u32(&sm.o_full[n & 1]));
+          else tc::mbar_arrive(smem_u32(&sm.o_full[n & 1]));
+        }
+        tc::mbar_arrive(smem_u32(&sm.job_empty[n & 1]));
       }
     }
   } else {
@@ -518,38 +631,15 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
     const int head_o = 32 * (warp & 1) + lane, half_o = warp >> 1;
     const float zs = p.sm_scale * kLog2eTc;
     bool ok = true;
-    // Q of a job from its ring slot to tensor memory, in the order the tensor core reads an A operand (two dims per column)
-    auto move_q = [&](int pos, int n_job) {
-      ok = __all_sync(0xffffffffu, tc::mbar_wait(smem_u32(&sm.k_full[slot_of(pos)]), use_of(pos), p.status)) && ok;
-      const int row = 16 * warp + (lane & 15), hi = lane >> 4;
-      const uint8_t* qs = sm.k[slot_of(pos)][0] + row * 128;
-#pragma unroll 1
-      for (int part = 0; part < 4; ++part) {
-        uint32_t w[32];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const int c = 32 * hi + 8 * part + j;
-          const uint4 u = *reinterpret_cast<const uint4*>(qs + (c >> 3) * kAtomBytes + (((c & 7) ^ (row & 7)) << 4));
-          w[4 * j] = u.x; w[4 * j + 1] = u.y; w[4 * j + 2] = u.z; w[4 * j + 3] = u.w;
-        }
-        tc::tmem_st32(tmem_base + lane_addr + kColQ + part * 32, w);
-      }
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {   // the warp's 16 rows of the rope block, as they lie
-        const int at = 16 * warp * 128 + (32 * j + lane) * 16;
-        *reinterpret_cast<uint4*>(sm.q_rope + at) = *reinterpret_cast<const uint4*>(sm.k[slot_of(pos)][8] + at);
-      }
-      tc::fence_proxy_async();
-      tc::tmem_st_wait();
-      tc::fence_before_sync();
-      __syncwarp();
-      if (lane == 0) tc::mbar_arrive(smem_u32(&sm.q_tmem[n_job & 1]));
+    // P V of tile g (over all jobs), which lies at ring position `pos`, is complete; whole warp
+    auto wait_pv = [&](int g, int pos) -> bool {
+      const uint32_t bar = kClustered ? smem_u32(&sm.k_empty[slot_of(pos)]) : smem_u32(&sm.pv_done[g % kRing]);
+      return __all_sync(0xffffffffu, tc::mbar_wait(bar, kClustered ? use_of(pos) : static_cast<uint32_t>(g / kRing) & 1u, p.status));
     };
     int base = 0, tiles_done = 0, n = 0;
     int2 jd;
     ok = __all_sync(0xffffffffu, wait_job(0, &jd));
     Job jb = job_of(jd);
-    if (ok) move_q(base + jb.q_at, 0);
     bool have_o = false;
     float m_used[2] = {0.f, 0.f}, l_run[2] = {0.f, 0.f};   // rows lane / 4 and lane / 4 + 8; l_run is this thread's share
     // A warp whose wait ran out goes on to the next vote, where all four learn of it and leave together: the named barrier
@@ -644,10 +734,7 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
             break;
           }
           // rare: O of every head times its factor, once P V of the tile before is complete
-          if (i > 0) {
-            const int pp = base + i - 1 + (i - 1 >= jb.q_at ? 1 : 0);
-            ok = ok && __all_sync(0xffffffffu, tc::mbar_wait(smem_u32(&sm.k_empty[slot_of(pp)]), use_of(pp), p.status));
-          }
+          if (i > 0) ok = ok && wait_pv(g - 1, base + i - 1 + (i - 1 >= jb.q_at ? 1 : 0));
           tc::fence_after_sync();
           const float al = sm.alpha[head_o];
 #pragma unroll 1
@@ -686,65 +773,24 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
           }
         }
       }
-      // the next job's Q goes to tensor memory before O is written out, so that its first Q K^T runs meanwhile
-      if constexpr (!kClustered) ok = __all_sync(0xffffffffu, wait_job(n + 1, &jd)) && ok;
+      if constexpr (!kClustered) {
+        __syncwarp();
+        if (lane == 0) tc::mbar_arrive(smem_u32(&sm.o_full[n & 1]));
+        ok = __all_sync(0xffffffffu, wait_job(n + 1, &jd)) && ok;
+      }
       if (!ok) sm.fail = 1;
       if (softmax_any(!ok)) break;
-      const Job done = jb;
-      const int last = base + done.n_tiles - 1 + (done.n_tiles - 1 >= done.q_at ? 1 : 0);   // ring position of the last tile
-      auto wait_last = [&]() {   // P V of the last tile is complete
-        if (!have_o) return;
-        const bool o_ok = __all_sync(0xffffffffu, tc::mbar_wait(smem_u32(&sm.k_empty[slot_of(last)]), use_of(last), p.status));
-        have_o = o_ok;
-        ok = ok && o_ok;
-      };
-      if constexpr (!kClustered) {
-        base += done.n_tiles + 1;
-        tiles_done += done.n_tiles;
-        if (jd.x >= 0) {
-          jb = job_of(jd);
-          // Behind early tiles Q may lie in the slot of the last tile, and all four warps' word that Q has moved lets its issuer
-          // release that slot once more: a warp that had not yet seen the release by the last P V would look for a phase that
-          // is two uses back, and wait for good.  (Q is there, so that P V is complete: nothing is waited for.)
-          if (jb.q_at > 0) wait_last();
-          move_q(base + jb.q_at, n + 1);
-          if (jb.q_at == 0) wait_last();
-        } else {
-          wait_last();
-        }
-      } else {
-        wait_last();
+      if constexpr (kClustered) {
+        if (have_o) have_o = wait_pv(jb.n_tiles - 1, jb.n_tiles - 1 + (jb.n_tiles - 1 >= jb.q_at ? 1 : 0));   // the last tile's
+        tc::fence_after_sync();
+        break;
       }
-      tc::fence_after_sync();
-      if constexpr (kClustered) break;
-      // ---- O / l: a thread owns half of the value dims of a head, in two runs of 128
-      {
-        const float inv = sm.inv[n & 1][head_o];
-        uint8_t* dst = reinterpret_cast<uint8_t*>(reinterpret_cast<__nv_bfloat16*>(p.out) + (static_cast<int64_t>(done.qi) * kH + head_o) * kDV + 128 * half_o);
-        const bool by32 = (reinterpret_cast<uintptr_t>(p.out) & 31u) == 0;
-#pragma unroll 1
-        for (int c = 0; c < 256; c += 64) {
-          uint32_t o[64];
-          if (have_o) {
-            tc::tmem_ld64(tmem_base + lane_addr + c, o);
-            tc::tmem_ld_wait();
-          } else {
-#pragma unroll
-            for (int j = 0; j < 64; ++j) o[j] = 0u;
-          }
-          uint32_t w[32];
-#pragma unroll
-          for (int j = 0; j < 32; ++j) w[j] = pack_bf16(__uint_as_float(o[2 * j]) * inv, __uint_as_float(o[2 * j + 1]) * inv);
-          uint8_t* d = dst + ((c >> 7) * 256 + (c & 127)) * 2;
-#pragma unroll
-          for (int j = 0; j < 32; j += 8) store_words8(d + j * 4, w + j, by32);
-        }
-        tc::fence_before_sync();   // (the next job's first P V waits for a p_ready that comes after this)
-      }
-      __syncwarp();
       if (lane == 0) tc::mbar_arrive(smem_u32(&sm.job_empty[n & 1]));
+      base += jb.n_tiles + 1;
+      tiles_done += jb.n_tiles;
       ++n;
       if (jd.x < 0) break;
+      jb = job_of(jd);
     }
     if constexpr (kClustered) {
       // ---- partial result of a split: normalised fp32 rows in the ring
