@@ -1034,7 +1034,7 @@ cudaError_t launch_attn_tc(const AttnArgs& a, cudaStream_t st, int64_t* n_launch
   const int k_g4 = a.gather4 && a.ld_k % 8 == 0 && (reinterpret_cast<uintptr_t>(a.k) & 15u) == 0 &&
                    make_map_bf16_rows(&g_map, a.k, static_cast<uint64_t>(a.ld_k), g_rows, 1);
   if (a.n_split <= 1) {
-    kernel<<<dim3(a.n_query, 1, 1), kThreadsAttnTc, smem, st>>>(q_map, q_tma, k_map, k_tma, g_map, k_g4, a);
+    if ((e = launch_pdl(kernel, dim3(a.n_query, 1, 1), dim3(kThreadsAttnTc), smem, st, q_map, q_tma, k_map, k_tma, g_map, k_g4, a)) != cudaSuccess) return e;
   } else {
     if (!attn_tc_split_ok(a.n_split)) return cudaErrorInvalidValue;
     if (a.n_split > 8 && (e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess) return e;

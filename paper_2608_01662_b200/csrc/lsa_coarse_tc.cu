@@ -68,6 +68,8 @@ coarse_score_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
   extern __shared__ uint8_t smem_raw[];
   Smem& sm = *reinterpret_cast<Smem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  pdl_wait();
+  pdl_launch_dependents();
 
   // heavy blocks first: the first blocks take the last queries.  A query block's tiles are dealt to `parts` blocks.
   const int qb = (gridDim.x - 1 - blockIdx.x) / parts, part = static_cast<int>(blockIdx.x) % parts;
@@ -303,9 +305,9 @@ cudaError_t launch_tc(const IndexArgs& a, cudaStream_t st, int64_t* n_launch) {
   const int64_t tiles = (a.q_pos0 + a.n_query - a.W) / (static_cast<int64_t>(kTileM) * a.B) + 1;
   int parts = 1;
   while (parts < 8 && static_cast<int64_t>(blocks) * parts < kFullWaves * kSmCount && tiles / (2 * parts) >= kMinTilesOfPart) parts *= 2;
-  kernel<<<blocks * parts, kThreadsTc, smem, st>>>(map_q, map_km, parts, a);
+  e = launch_pdl(kernel, dim3(blocks * parts), dim3(kThreadsTc), smem, st, map_q, map_km, parts, a);
   ++*n_launch;
-  return cudaGetLastError();
+  return e;
 }
 
 }  // namespace

@@ -52,6 +52,8 @@ __global__ void __launch_bounds__(kFineThreads, 2) fine_select_tc_kernel(const _
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int qi = blockIdx.x;
   const int part = blockIdx.y, n_parts = gridDim.y;
+  pdl_wait();
+  pdl_launch_dependents();
   int64_t t, n_key;
   const int32_t* pt = nullptr;
   if (p.paged) {
@@ -276,9 +278,9 @@ cudaError_t launch_t(const IndexArgs& a, const CUtensorMap& map, cudaStream_t st
   cudaError_t e = cudaFuncSetAttribute(fine_select_tc_kernel<TMA>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (e != cudaSuccess) return e;
   const int parts = a.fine_parts > 1 ? a.fine_parts : 1;
-  fine_select_tc_kernel<TMA><<<dim3(a.n_query, parts), kFineThreads, smem, st>>>(map, a);
+  e = launch_pdl(fine_select_tc_kernel<TMA>, dim3(a.n_query, parts), dim3(kFineThreads), smem, st, map, a);
   ++*n_launch;
-  return cudaGetLastError();
+  return e;
 }
 
 // bf16 key rows the TMA path can read: the cache itself, or the widened copy of an e4m3 cache
