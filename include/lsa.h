@@ -137,9 +137,8 @@ LSA_API int64_t lsa_launch_count(lsa_ctx* ctx);
  *   LSA_TUNE_ATTN_SPLIT     row splits per sequence in paged attention: 0 (default) = chosen by the wave cost model,
  *                           1..16 = fixed (the tcgen05 kernel merges its splits inside a thread-block cluster and
  *                           accepts 1, 2, 4, 8 or 16; other values make lsa_sparse_attn return LSA_ERR_ARG there)
- *   LSA_TUNE_ATTN_PV_WAIT   prefill on the tcgen05 attention kernel.  0 (default): the Q K^T of a tile follows the P V that
- *                           frees its accumulator in the issuing thread's program order; 1: it waits for that P V's
- *                           completion barrier (slower, same bits).  Paged calls always wait.
+ *   LSA_TUNE_ATTN_PV_WAIT   tcgen05 attention kernel.  0 (default): the Q K^T of a tile waits for its rows and a free S buffer only;
+ *                           1: also for the completion of the P V two tiles before (slower, same bits).
  *   LSA_TUNE_ATTN_GATHER    tcgen05 attention kernel, scattered cache rows.  0 (default): coalesced 16-byte cp.async
  *                           copies; 1: TMA gather, four rows per cp.async.bulk.tensor tile::gather4 instruction (needs a
  *                           16-byte aligned cache whose row pitch is a multiple of 16 bytes, else the other path is
