@@ -52,6 +52,7 @@ constexpr int kIssuers = 3;                 // MMA-issuing warps 1..3
 __device__ __forceinline__ int acc_of_tile(int i) { return i % kIssuers + kIssuers * ((i / kIssuers) & 1); }
 __device__ __forceinline__ uint32_t acc_use_parity(int i) { return static_cast<uint32_t>(i / (2 * kIssuers)) & 1u; }
 constexpr int kSelBar = 1, kWarmBar = 2;    // named barriers of threads 0-255 (the selections) and of the last warp
+constexpr int kMaxTailRows = 16384;         // sink and window rows that the ring holds at the end
 constexpr int kWarmWarp = kThreadsFp / 32 - 1;   // idle until the tiles: it fetches the selection's instructions
 
 template <bool E4M3>
@@ -77,8 +78,12 @@ struct FpSmem {
   uint32_t tmem_slot;
 };
 static_assert(sizeof(FpSmem<true>) + 1024 <= 227 * 1024 && sizeof(FpSmem<false>) + 1024 <= 227 * 1024, "shared memory");
-static_assert(FpSmem<true>::kSlots * FpSmem<true>::kTileBytes >= kMaxSlotsFp * 4 + kShortWarm && FpSmem<false>::kSlots * FpSmem<false>::kTileBytes >= kMaxSlotsFp * 4 + kShortWarm,
-              "page keys and the made-up ones fit the ring");
+template <bool E4M3>
+constexpr bool ring_holds() {   // the keys of the page scores and the made-up ones; the sink and window rows
+  constexpr int bytes = FpSmem<E4M3>::kSlots * FpSmem<E4M3>::kTileBytes;
+  return bytes >= kMaxSlotsFp * 4 + static_cast<int>(kShortWarm) && bytes >= kMaxTailRows * 4;
+}
+static_assert(ring_holds<true>() && ring_holds<false>(), "the ring holds what lies there before and after the tiles");
 static_assert(FpSmem<true>::kSlots % kIssuers == 0 && FpSmem<false>::kSlots % kIssuers == 0, "a ring slot has one consumer");
 
 __device__ __forceinline__ uint32_t cluster_rank() {
@@ -108,22 +113,38 @@ __device__ __forceinline__ void store_cluster_u32(uint32_t addr, uint32_t v) {
 // padding of the row list by everybody.  Row list: [sink | sparse | window | -1 ...], S + Ksp + W entries.
 // Inlined: the selection's scratch and the key array must be known to be shared memory (generic atomics are slow).
 __device__ __forceinline__ void finish_sequence(const IndexArgs& p, const uint32_t* keys, const int32_t* pages, const int32_t* phys,
-                                             SelectScratch& sel, int n_slots, int qi, int64_t t) {
+                                             SelectScratch& sel, int32_t* tail, int n_slots, int qi, int64_t t) {
   const int tid = threadIdx.x;
   const int ld = p.S + p.Ksp + p.W;
   const int n_sink = static_cast<int>(min64(p.S, t + 1));
   int32_t* rows = p.rows_out != nullptr ? p.rows_out + static_cast<int64_t>(qi) * ld : nullptr;
+  const int64_t win0 = max64(p.S, t - p.W + 1);
+  const int n_win = static_cast<int>(max64(0, t - win0 + 1));
+  const int32_t* pt = p.page_table + static_cast<int64_t>(qi) * p.pt_stride;
+  auto tail_row = [&](int j) -> int32_t {   // j-th of the sink and window rows
+    const int64_t pos = j < n_sink ? j : win0 + (j - n_sink);
+    return static_cast<int32_t>(static_cast<int64_t>(pt[pos >> 6]) * kPageTok + (pos & (kPageTok - 1)));
+  };
+  const bool staged = n_sink + n_win <= kMaxTailRows;
+  if (tid >= kSelThreads && rows != nullptr && staged)   // looked up by the other warps meanwhile
+    for (int j = tid - kSelThreads; j < n_sink + n_win; j += kThreadsFp - kSelThreads) tail[j] = tail_row(j);
   if (tid < kSelThreads) {
     int32_t* out_idx = p.sparse_idx + static_cast<int64_t>(qi) * p.Ksp;
     const int n_sel = short_select<kSelBar>(smem_u32(keys), n_slots, p.Ksp, smem_u32(keys), smem_u32(&sel));
-    for (int r = tid; r < p.Ksp; r += kSelThreads) {
-      if (r >= n_sel) {
-        out_idx[r] = -1;
-        continue;
+    for (int r0 = tid; r0 < p.Ksp; r0 += 4 * kSelThreads) {   // four rows in flight per thread
+      int pos[4], row[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int i = short_item(smem_u32(keys), min(r0 + u * kSelThreads, max(n_sel - 1, 0))) & (kMaxSlotsFp - 1);
+        pos[u] = pages[i >> 6] * kPageTok + (i & (kPageTok - 1));
+        row[u] = phys[i >> 6] * kPageTok + (i & (kPageTok - 1));
       }
-      const int i = short_item(smem_u32(keys), r);
-      out_idx[r] = pages[i >> 6] * kPageTok + (i & (kPageTok - 1));
-      if (rows != nullptr) rows[n_sink + r] = phys[i >> 6] * kPageTok + (i & (kPageTok - 1));
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int r = r0 + u * kSelThreads;
+        if (r < p.Ksp) out_idx[r] = r < n_sel ? pos[u] : -1;
+        if (r < n_sel && rows != nullptr) rows[n_sink + r] = row[u];
+      }
     }
     if (tid == 0) {
       p.n_sparse[qi] = n_sel;
@@ -133,24 +154,9 @@ __device__ __forceinline__ void finish_sequence(const IndexArgs& p, const uint32
   __syncthreads();
   if (rows == nullptr) return;
   const int n_sel = static_cast<int>(sel.n_valid);
-  const int64_t win0 = max64(p.S, t - p.W + 1);
-  const int n_win = static_cast<int>(max64(0, t - win0 + 1));
-  const int32_t* pt = p.page_table + static_cast<int64_t>(qi) * p.pt_stride;
   // everything but the sparse part: ld - n_sel entries
-  for (int j = tid; j < ld - n_sel; j += kThreadsFp) {
-    int32_t r = -1;
-    int at = j;
-    if (j < n_sink) {
-      r = static_cast<int32_t>(static_cast<int64_t>(pt[j >> 6]) * kPageTok + (j & (kPageTok - 1)));
-    } else {
-      at = j + n_sel;
-      if (j - n_sink < n_win) {
-        const int64_t pos = win0 + (j - n_sink);
-        r = static_cast<int32_t>(static_cast<int64_t>(pt[pos >> 6]) * kPageTok + (pos & (kPageTok - 1)));
-      }
-    }
-    rows[at] = r;
-  }
+  for (int j = tid; j < ld - n_sel; j += kThreadsFp)
+    rows[j < n_sink ? j : j + n_sel] = j >= n_sink + n_win ? -1 : staged ? tail[j] : tail_row(j);
   if (tid == 0) p.n_rows_out[qi] = n_sink + n_sel + n_win;
 }
 
@@ -168,7 +174,7 @@ fine_paged_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
   const uint32_t rank = cluster_rank(), n_rank = cluster_size();
   // The cluster barrier has no time limit: every path below reaches both of its phases, also after a failed wait.
   cluster_arrive();   // phase 1: "this block runs" (its shared memory may be written from now on)
-  const bool live = !tc::status_raised(p.status);
+  const bool live = !__syncthreads_or(tc::status_raised(p.status));   // the same in all threads: they meet on barriers below
 
   if (tid == 0) {
     for (int s = 0; s < kSlots; ++s) {
@@ -405,7 +411,7 @@ fine_paged_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
   cluster_arrive();   // phase 2: this block's keys are in the first block's shared memory
   cluster_wait();
   if (rank != 0) return;
-  finish_sequence(p, sm.keys, sm.pages, sm.phys, sm.sel, tc::status_raised(p.status) ? 0 : n_slots, qi, t);
+  finish_sequence(p, sm.keys, sm.pages, sm.phys, sm.sel, reinterpret_cast<int32_t*>(sm.k), tc::status_raised(p.status) ? 0 : n_slots, qi, t);
 }
 
 }  // namespace
