@@ -353,7 +353,7 @@ int run_attn(lsa_ctx* c, const lsa_params* p, const void* q, const void* k, cons
   a.rows_ld = p->k_sink + p->k_sparse + p->k_swa;
   a.n_key = p->paged ? 0 : n_key;   // (the checking build validates caller-given row numbers against it)
   a.q_pos0 = q_pos0; a.n_query = static_cast<int>(nq); a.ctx_len = ctx_len; a.out = out; a.lse = lse;
-  a.n_split = 1; a.status = status_word(c);
+  a.n_split = 1; a.sm_count = c->sm_count; a.status = status_word(c);
   a.qk_waits_pv = c->tune[LSA_TUNE_ATTN_PV_WAIT];
   a.gather4 = c->tune[LSA_TUNE_ATTN_GATHER];
   a.rows_stable = rows != nullptr && c->last_attn_rows == rows;

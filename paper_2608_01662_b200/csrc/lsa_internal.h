@@ -69,6 +69,7 @@ struct AttnArgs {
   int gather4;            // tcgen05 kernel: scattered rows by TMA gather (cp.async.bulk.tensor tile::gather4) where the cache allows
   int rows_stable;        // tcgen05 kernel, row lists: `rows` / `n_rows` were complete before the previous kernel of the
                           // stream started, so they may be read ahead of the programmatic dependency wait
+  int sm_count;           // tcgen05 kernel: blocks that run at the same time
   int n_split;            // >1: partial results in part_out / part_lse, merged afterwards
   float* part_out;        // fp32 [n_query, n_split, H, DV]
   float* part_lse;        // fp32 [n_query, n_split, H]
