@@ -198,8 +198,8 @@ __global__ void __launch_bounds__(32 * kWarps8) index8_kernel(IndexArgs p) {
     for (int r = 0; r < R; ++r) key[r] = 32 * r < n_slots ? sk[32 * r + lane] : 0u;
     // ---- a4
     n_sel = warp_topk<R>(key, p.Ksp, [&](int rank, int, int r) { out_idx[rank] = static_cast<int32_t>(group_pos(32 * r)) + lane; });
-    if (out_pages)
-      for (int i = lane; i < n_pages; i += 32) out_pages[i] = pages[i];
+    if (out_pages)   // (without the hierarchy a query has every eligible page, which may be more than the list holds)
+      for (int i = lane; i < min(n_pages, p.M); i += 32) out_pages[i] = pages[i];
   }
   for (int i = n_sel + lane; i < p.Ksp; i += 32) out_idx[i] = -1;
   if (out_pages)
