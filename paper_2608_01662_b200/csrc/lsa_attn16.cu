@@ -95,7 +95,7 @@ __global__ void __launch_bounds__(32 * kWarps16, 2) sparse_attn16_kernel(AttnArg
   auto load_k = [&](int32_t row) {
 #pragma unroll
     for (int nt = 0; nt < 2; ++nt) {
-      const int32_t r = max(__shfl_sync(0xffffffffu, row, 8 * nt + g), 0);   // absent keys are masked: any row will do
+      const int32_t r = max(__shfl_sync(0xffffffffu, row, 8 * nt + g), 0);   // an absent key's score is masked: any row will do
       const uint8_t* src = kg + static_cast<int64_t>(r) * p.ld_k * 2;
 #pragma unroll
       for (int j = 0; j < 4; ++j) kf[nt][j] = *reinterpret_cast<const uint4*>(src + j * 64);
@@ -104,10 +104,12 @@ __global__ void __launch_bounds__(32 * kWarps16, 2) sparse_attn16_kernel(AttnArg
   auto load_v = [&](int32_t row) {
 #pragma unroll
     for (int s = 0; s < 4; ++s) {
-      const int32_t r = max(__shfl_sync(0xffffffffu, row, 2 * t + (s & 1) + 8 * (s >> 1)), 0);
+      // An absent key's values are zero, not some other row's: its weight is 0, but 0 x NaN is not (in a pool, row 0 may be
+      // another sequence's, or nobody's).
+      const int32_t r = __shfl_sync(0xffffffffu, row, 2 * t + (s & 1) + 8 * (s >> 1));
       const uint8_t* src = vg + static_cast<int64_t>(r) * p.ld_v * 2;
-      vf[s][0] = *reinterpret_cast<const uint4*>(src);
-      vf[s][1] = *reinterpret_cast<const uint4*>(src + 128);
+      vf[s][0] = r >= 0 ? *reinterpret_cast<const uint4*>(src) : make_uint4(0u, 0u, 0u, 0u);
+      vf[s][1] = r >= 0 ? *reinterpret_cast<const uint4*>(src + 128) : make_uint4(0u, 0u, 0u, 0u);
     }
   };
 
