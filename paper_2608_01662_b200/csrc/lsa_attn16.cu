@@ -166,9 +166,10 @@ __global__ void __launch_bounds__(32 * kWarps16, 2) sparse_attn16_kernel(AttnArg
     uint32_t pa[4];
 #pragma unroll
     for (int nt = 0; nt < 2; ++nt) {
-      // (a row of padding only, possible in the checking build, has no maximum yet: its weights are zero)
-      const float p0 = m_run[0] > -INFINITY ? exp2f(s[nt][0] - m_run[0]) : 0.f, p1 = m_run[0] > -INFINITY ? exp2f(s[nt][1] - m_run[0]) : 0.f;
-      const float p2 = m_run[1] > -INFINITY ? exp2f(s[nt][2] - m_run[1]) : 0.f, p3 = m_run[1] > -INFINITY ? exp2f(s[nt][3] - m_run[1]) : 0.f;
+      // (absent keys by their bits, not by the maximum: a head whose scores are all NaN has none, and its weights are NaN)
+      const unsigned there = live >> (8 * nt + 2 * t);
+      const float p0 = there & 1u ? exp2f(s[nt][0] - m_run[0]) : 0.f, p1 = there & 2u ? exp2f(s[nt][1] - m_run[0]) : 0.f;
+      const float p2 = there & 1u ? exp2f(s[nt][2] - m_run[1]) : 0.f, p3 = there & 2u ? exp2f(s[nt][3] - m_run[1]) : 0.f;
       l_run[0] += p0 + p1;   // fp32 sums of the unrounded weights
       l_run[1] += p2 + p3;
       pa[2 * nt] = pack_bf16(p0, p1);
@@ -217,7 +218,7 @@ __global__ void __launch_bounds__(32 * kWarps16, 2) sparse_attn16_kernel(AttnArg
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
       const float inv = l_run[r] > 0.f ? 1.f / l_run[r] : 0.f;
-      const float lse2 = l_run[r] > 0.f ? m_run[r] + log2f(l_run[r]) : -INFINITY;
+      const float lse2 = l_run[r] != 0.f ? m_run[r] + log2f(l_run[r]) : -INFINITY;
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         float x[16];
@@ -266,7 +267,7 @@ __global__ void __launch_bounds__(32 * kWarps16, 2) sparse_attn16_kernel(AttnArg
         x[4 * i] += wgt * v.x; x[4 * i + 1] += wgt * v.y; x[4 * i + 2] += wgt * v.z; x[4 * i + 3] += wgt * v.w;
       }
     }
-    finish(head, dim, x, den > 0.f ? 1.f / den : 0.f, den > 0.f ? m + log2f(den) : -INFINITY, (tid & 7) == 0);
+    finish(head, dim, x, den > 0.f ? 1.f / den : 0.f, den != 0.f ? m + log2f(den) : -INFINITY, (tid & 7) == 0);
   }
 }
 

@@ -1,5 +1,5 @@
 """Attention reads nothing but the listed cache rows into its results (needs a B200): every other row is NaN, and the row counts are
-no multiples of a tile."""
+no multiples of a tile.  And what is not finite in the listed rows or the queries shows in the results."""
 import numpy as np
 import pytest
 import torch
@@ -71,3 +71,39 @@ def test_rows_that_no_query_attends(cuda_device, base, n_query):
                                           sm_scale=cfg.sm_scale, d_v=cfg.d_v)
         m.add_out(pu.to_np(out[i]), want[0], pu.to_np(lse[i]), want_lse[0])
     m.assert_ok(pu.TOL_BF16)
+
+
+@pytest.mark.parametrize("base,n_query", [("cfg1", 40), ("cfg1", 1300), ("cfg3", 40)])
+def test_what_is_not_finite_shows(cuda_device, base, n_query):
+    """A NaN in one head of a query: that head's output is NaN and no other changes.  A NaN in a cache row: every head of the queries
+    that attend it."""
+    n_key, W, K = 2000, 50, 4
+    cfg = CONFIGS[base].replace(L=n_key, S=0, W=W, Ksp=K, R=1)
+    ctx = binding.Context(binding.make_params(cfg), n_query, n_key, 1, device=cuda_device)
+    g = torch.Generator(device=cuda_device).manual_seed(n_query)
+    draw = lambda *shape: torch.randn(shape, generator=g, device=cuda_device).to(torch.bfloat16)  # noqa: E731
+    q, k = draw(n_query, cfg.H, cfg.d_qk), draw(n_key, cfg.d_qk)
+    v = k[:, :cfg.d_v] if cfg.mla else draw(n_key, cfg.d_v)
+    idx = torch.full((n_query, K), -1, dtype=torch.int32, device=cuda_device)
+    n_sparse = torch.zeros(n_query, dtype=torch.int32, device=cuda_device)
+    q_pos0 = n_key - n_query
+
+    def run():
+        out = torch.empty((n_query, cfg.H, cfg.d_v), dtype=torch.bfloat16, device=cuda_device)
+        ctx.sparse_attn(q, k, v, idx, n_sparse, q_pos0, n_query, n_key, out)
+        assert ctx.status() == 0
+        return out
+
+    plain = run()
+    assert torch.isfinite(plain).all()
+    q[7, 3, 5] = float("nan")
+    got = run()
+    assert torch.isnan(got[7, 3]).all()
+    got[7, 3] = plain[7, 3]
+    assert torch.equal(got, plain)
+    q[7, 3, 5] = 0.5
+    row = q_pos0 + 20
+    k[row, 0] = float("nan")
+    got = run()
+    attends = (torch.arange(n_query, device=cuda_device) >= 20) & (torch.arange(n_query, device=cuda_device) < 20 + W)
+    assert torch.isnan(got[attends]).all() and torch.isfinite(got[~attends]).all()
