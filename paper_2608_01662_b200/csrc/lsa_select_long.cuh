@@ -84,6 +84,7 @@ __device__ __forceinline__ uint32_t block_exclusive_sum(uint32_t v, uint32_t* wa
 template <bool CLUSTER, class KeyF, class EmitF, class AbsentF>
 __device__ int long_select(KeyF key, EmitF emit, AbsentF absent, int n, int k, int cap, uint8_t* smem) {
   namespace cs = cluster_sel;
+  if (k <= 0) return 0;   // (the same in every block; no key is the k-th largest)
   LongScratch& sc = *reinterpret_cast<LongScratch*>(smem);
   LongAll& all = *reinterpret_cast<LongAll*>(smem + sizeof(LongScratch));
   uint32_t* ck = reinterpret_cast<uint32_t*>(smem + sizeof(LongScratch) + (CLUSTER ? sizeof(LongAll) : 0));

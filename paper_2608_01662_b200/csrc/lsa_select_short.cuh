@@ -50,6 +50,10 @@ static_assert(kShortScratch <= sizeof(SelectScratch), "the scratch of the radix 
 static __device__ __noinline__ int short_select(uint32_t keys, int n, int k, uint32_t list, uint32_t scratch, int bar, int tid, int n_threads) {
   const int lane = tid & 31, warp = tid >> 5;
   auto sync = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(bar), "r"(n_threads) : "memory"); };
+  if (k <= 0) {   // (no key is the k-th largest: the search below would find nothing and go by what it finds in the scratch)
+    sync();
+    return 0;
+  }
   constexpr uint32_t kAll = 0xffffffffu;
   const int base = tid * kShortPer;   // the thread holds items base .. base + 15
   const uint32_t of_warp = scratch + kShortWarp + 4u * (lane & 7), my_warp = scratch + kShortWarp + 4u * warp;
