@@ -204,8 +204,7 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
 
   constexpr bool clustered = kClustered;
   const bool pair = kClustered && p.n_split == 2;   // two splits exchange their rows through shared memory
-  const bool dead = tc::status_raised(p.status);   // an earlier block of this launch (or an earlier launch) gave up on a wait
-  if (dead && !clustered) return;
+  const bool raised = tc::status_raised(p.status);   // an earlier block of this launch (or an earlier launch) gave up on a wait
 
   // ---- set-up
   if (tid == 0) {
@@ -239,9 +238,13 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
     tc::tmem_relinquish();
   }
   tc::fence_before_sync();
-  __syncthreads();
+  const bool dead = __syncthreads_or(raised) != 0;   // the same in all threads (see block_gives_up); the set-up ran meanwhile
   tc::fence_after_sync();
   const uint32_t tmem_base = sm.tmem_slot;
+  if (dead && !clustered) {
+    if (warp == kQkWarp) tc::tmem_dealloc(tmem_base, kTmemColsAttn);
+    return;
+  }
   // Programmatic dependent launch: this block may have been placed while the previous kernel of the stream was still
   // draining; what that kernel wrote is read, and what it may still read is overwritten, only after
   // griddepcontrol.wait.  The next kernel's blocks may be placed from then on.

@@ -85,7 +85,7 @@ coarse_score_paged_tc_kernel(const __grid_constant__ CUtensorMap map_km, const _
   sh.p_shift = 31 - __clz(p.P);
   const int spp = p.P / p.B;                       // sub-blocks per page: 8, 16 or 32
   sh.spp_shift = 31 - __clz(spp);
-  if (tc::status_raised(p.status)) return;
+  if (tc::block_gives_up(p.status)) return;
   pdl_wait();                 // the cached lengths may come from the previous kernel of the stream (lsa_append)
   pdl_launch_dependents();
 

@@ -87,7 +87,7 @@ fine_scores_tc_kernel(const __grid_constant__ CUtensorMap map, int one_box, Inde
   for (int c = max(tile_begin, tiles_live) * kTile + tid; c < tile_end * kTile; c += kThreadsBig) krow[c] = 0u;
   const int n_tiles = tiles_live - tile_begin;
   if (n_tiles <= 0) return;
-  if (tc::status_raised(p.status)) return;
+  if (tc::block_gives_up(p.status)) return;
 
   if (tid == 0) {
     for (int s = 0; s < kStagesBig; ++s) {

@@ -174,7 +174,7 @@ fine_paged_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
   const uint32_t rank = cluster_rank(), n_rank = cluster_size();
   // The cluster barrier has no time limit: every path below reaches both of its phases, also after a failed wait.
   cluster_arrive();   // phase 1: "this block runs" (its shared memory may be written from now on)
-  const bool live = !__syncthreads_or(tc::status_raised(p.status));   // the same in all threads: they meet on barriers below
+  const bool live = !tc::block_gives_up(p.status);
 
   if (tid == 0) {
     for (int s = 0; s < kSlots; ++s) {
@@ -411,7 +411,7 @@ fine_paged_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
   cluster_arrive();   // phase 2: this block's keys are in the first block's shared memory
   cluster_wait();
   if (rank != 0) return;
-  finish_sequence(p, sm.keys, sm.pages, sm.phys, sm.sel, reinterpret_cast<int32_t*>(sm.k), tc::status_raised(p.status) ? 0 : n_slots, qi, t);
+  finish_sequence(p, sm.keys, sm.pages, sm.phys, sm.sel, reinterpret_cast<int32_t*>(sm.k), tc::block_gives_up(p.status) ? 0 : n_slots, qi, t);
 }
 
 }  // namespace

@@ -75,7 +75,7 @@ __global__ void __launch_bounds__(kFineThreads, 2) fine_select_tc_kernel(const _
     if (tid == 0) p.n_sparse[qi] = 0;
     return;
   }
-  if (tc::status_raised(p.status)) return;   // an earlier block of this launch gave up on a wait
+  if (tc::block_gives_up(p.status)) return;   // an earlier block of this launch gave up on a wait
 
   // query heads (K-major, 128B swizzle) and head weights: asynchronous copies that land during the page selection
   {

@@ -121,7 +121,7 @@ paged_scores_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
   const int batch = p.n_query;
   PsShape sh;
   sh.S = p.S; sh.W = p.W; sh.flat = flat;
-  if (tc::status_raised(p.status)) return;
+  if (tc::block_gives_up(p.status)) return;
   pdl_wait();                 // page lists and cached lengths come from earlier kernels of the stream
   pdl_launch_dependents();
 
@@ -379,7 +379,8 @@ paged_scores_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
       new_seq = wk.next(sm.ntile, batch);
       if (!fresh) continue;
       const int slot = n_q & 1;
-      ok = tc::mbar_wait(smem_u32(&sm.q_empty[slot]), ((n_q >> 1) & 1) ^ 1, p.status);   // (every thread waits: no hand-over needed)
+      // every thread waits (no hand-over needed), and they agree on the outcome: the barrier below counts all of them
+      ok = tc::all_of<kQBar, kQThreads>(tc::mbar_wait(smem_u32(&sm.q_empty[slot]), ((n_q >> 1) & 1) ^ 1, p.status));
       if (!ok) break;
       ++n_q;
       if constexpr (E4M3) {

@@ -55,6 +55,18 @@ constexpr long long kWaitCycles = 1ll << 31;
 __device__ __forceinline__ bool status_raised(const int* status) {
   return status != nullptr && *reinterpret_cast<const volatile int*>(status) != 0;
 }
+// Whether the block gives up at its start, the same answer in all of its threads: the word may be raised between two threads'
+// looks at it, and threads that went different ways would wait for one another for ever on a barrier that counts them
+// (bar.sync with a number of threads; the aligned instructions of a warp).  Every thread of the block calls it.
+__device__ __forceinline__ bool block_gives_up(const int* status) { return __syncthreads_or(status_raised(status)) != 0; }
+// Whether all THREADS threads that meet on barrier BAR said yes; each learns it, and they leave together.
+template <int BAR, int THREADS>
+__device__ __forceinline__ bool all_of(bool v) {
+  uint32_t r;
+  asm volatile("{\n\t.reg .pred a, b;\n\tsetp.ne.b32 a, %1, 0;\n\tbar.red.and.pred b, %2, %3, a;\n\tselp.b32 %0, 1, 0, b;\n\t}"
+               : "=r"(r) : "r"(static_cast<uint32_t>(v)), "n"(BAR), "n"(THREADS) : "memory");
+  return r != 0;
+}
 // The wait with its cycle budget as an argument (the production kernels use kWaitCycles; the self-test a short one).
 __device__ __forceinline__ bool mbar_wait_budget(uint32_t bar, uint32_t parity, int* status, long long budget) {
   if (mbar_try_wait(bar, parity)) return true;
