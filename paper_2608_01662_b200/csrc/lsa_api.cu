@@ -184,21 +184,25 @@ int* status_word(lsa_ctx* c) { return c->ws ? reinterpret_cast<int*>(c->ws) : nu
 // in clusters that fit the chip together, not in SMs: 15 clusters of eight run at once, and a 16th sequence doubled the time
 // (decode step of 16 sequences, 4 layers: 190 us as 8 splits, 144 as 4; of 36: 255 as 4, 186 as 2; of one: 77.5 as 16, 82.7 as 8;
 // of 8: 153 and 99).
-int pick_split(int sm_count, int batch, int max_rows, bool tc_kernel) {
+cudaError_t pick_split(int sm_count, int batch, int max_rows, bool tc_kernel, int* split) {
   const int units = (max_rows + 63) / 64;
-  int best = 1;
+  *split = 1;
   long best_cost = -1;
   for (int s = 1; s <= kMaxSplit && s <= units; ++s) {
-    if (tc_kernel && !lsa::attn_tc_split_ok(s)) continue;
-    const int fit = tc_kernel && s > 1 ? lsa::attn_tc_resident(s) : 0;
+    int fit = 0;
+    if (tc_kernel && s > 1) {
+      const cudaError_t e = lsa::attn_tc_resident(s, &fit);
+      if (e != cudaSuccess) return e;
+      if (fit == 0) continue;
+    }
     const long waves = fit > 0 ? (batch + fit - 1) / fit : (static_cast<long>(batch) * s + sm_count - 1) / sm_count;
     const long cost = waves * ((units + s - 1) / s + 6);
     if (best_cost < 0 || cost < best_cost) {
       best_cost = cost;
-      best = s;
+      *split = s;
     }
   }
-  return best;
+  return cudaSuccess;
 }
 
 int run_index(lsa_ctx* c, const lsa_params* p, const void* q_idx, const float* w, const void* k_idx,
@@ -361,9 +365,13 @@ int run_attn(lsa_ctx* c, const lsa_params* p, const void* q, const void* k, cons
   if (p->paged) {
     const WsLayout l = ws_layout(p, nq, 0, batch);
     if (c->ws == nullptr || l.total > c->ws_bytes) return LSA_ERR_WORKSPACE;
-    a.n_split = c->tune[LSA_TUNE_ATTN_SPLIT] > 0 ? c->tune[LSA_TUNE_ATTN_SPLIT]
-                                                 : pick_split(c->sm_count, batch, a.rows_ld, use_tc);
-    if (use_tc && !lsa::attn_tc_split_ok(a.n_split)) return LSA_ERR_ARG;
+    bool split_ok = true;
+    cudaError_t es = cudaSuccess;
+    a.n_split = c->tune[LSA_TUNE_ATTN_SPLIT];
+    if (a.n_split <= 0) es = pick_split(c->sm_count, batch, a.rows_ld, use_tc, &a.n_split);
+    else if (use_tc) es = lsa::attn_tc_split_ok(a.n_split, &split_ok);
+    if (es != cudaSuccess) return cuda_fail(c, es);
+    if (!split_ok) return LSA_ERR_ARG;
     a.part_out = reinterpret_cast<float*>(c->ws + l.part_out);
     a.part_lse = reinterpret_cast<float*>(c->ws + l.part_lse);
   }

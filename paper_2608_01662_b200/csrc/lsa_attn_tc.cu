@@ -1004,17 +1004,24 @@ static AttnTcKernel pick_kernel(const AttnArgs& a) {
   return a.n_split > 1 ? sparse_attn_tc_kernel<true, true> : sparse_attn_tc_kernel<true, false>;
 }
 
-int attn_tc_resident(int n_split) {
-  auto count = [](int blocks) {
-    return resident_clusters(reinterpret_cast<const void*>(sparse_attn_tc_kernel<true, true>), kThreadsAttnTc, sizeof(AttnTcSmem) + 1024, blocks);
-  };
-  static const int n[4] = {count(2), count(4), count(8), count(kMaxClusterSplit)};   // (queried once per process)
-  return n_split == 2 ? n[0] : n_split == 4 ? n[1] : n_split == 8 ? n[2] : n_split == kMaxClusterSplit ? n[3] : 0;
+cudaError_t attn_tc_resident(int n_split, int* clusters) {
+  static DeviceCount n[4];
+  const int at = n_split == 2 ? 0 : n_split == 4 ? 1 : n_split == 8 ? 2 : n_split == kMaxClusterSplit ? 3 : -1;
+  *clusters = 0;
+  if (at < 0) return cudaSuccess;
+  return n[at].get(clusters, [&](int* c) {
+    return resident_clusters(reinterpret_cast<const void*>(sparse_attn_tc_kernel<true, true>), kThreadsAttnTc, sizeof(AttnTcSmem) + 1024, n_split, c);
+  });
 }
 
 // Row splits the tcgen05 kernel can merge inside a cluster: a power of two that divides the 64 heads, as many blocks as the
 // device can co-schedule.
-bool attn_tc_split_ok(int n_split) { return n_split == 1 || attn_tc_resident(n_split) > 0; }
+cudaError_t attn_tc_split_ok(int n_split, bool* ok) {
+  int n = 0;
+  const cudaError_t e = attn_tc_resident(n_split, &n);
+  *ok = n_split == 1 || n > 0;
+  return e;
+}
 
 bool attn_tc_supported(const AttnArgs& a) {
   return a.H == kH && a.DQK == kDQK && a.DV == kDV && a.v == a.k && a.ld_v == a.ld_k;
@@ -1041,7 +1048,9 @@ cudaError_t launch_attn_tc(const AttnArgs& a, cudaStream_t st, int64_t* n_launch
   if (a.n_split <= 1) {
     if ((e = launch_pdl(kernel, dim3(a.n_query, 1, 1), dim3(kThreadsAttnTc), smem, st, q_map, q_tma, k_map, k_tma, g_map, k_g4, a)) != cudaSuccess) return e;
   } else {
-    if (!attn_tc_split_ok(a.n_split)) return cudaErrorInvalidValue;
+    bool ok = false;
+    if ((e = attn_tc_split_ok(a.n_split, &ok)) != cudaSuccess) return e;
+    if (!ok) return cudaErrorInvalidValue;
     if (a.n_split > 8 && (e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess) return e;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(a.n_query, a.n_split, 1);

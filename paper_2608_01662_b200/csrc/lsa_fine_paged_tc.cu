@@ -436,11 +436,15 @@ cudaError_t launch_fine_paged_tc(const IndexArgs& a, int sm_count, cudaStream_t 
       !(a.key_e4m3 ? make_map_u8_128(&map_k, a.k_idx, 1ull << 31, kPageTok) : make_map_bf16_128(&map_k, a.k_idx, 1ull << 31, kPageTok)))
     return cudaErrorInvalidValue;
   const int sms = sm_count > 0 ? sm_count : 148;
-  static const int fit_f8[2] = {resident_clusters(reinterpret_cast<const void*>(fine_paged_tc_kernel<true>), kThreadsFp, sizeof(FpSmem<true>) + 1024, 8),
-                                resident_clusters(reinterpret_cast<const void*>(fine_paged_tc_kernel<true>), kThreadsFp, sizeof(FpSmem<true>) + 1024, 4)};
-  static const int fit_bf[2] = {resident_clusters(reinterpret_cast<const void*>(fine_paged_tc_kernel<false>), kThreadsFp, sizeof(FpSmem<false>) + 1024, 8),
-                                resident_clusters(reinterpret_cast<const void*>(fine_paged_tc_kernel<false>), kThreadsFp, sizeof(FpSmem<false>) + 1024, 4)};
-  const int* fit = a.key_e4m3 ? fit_f8 : fit_bf;
+  static DeviceCount counts[2][2];   // [key type][clusters of eight, of four]
+  int fit[2];
+  for (int i = 0; i < 2; ++i) {
+    const cudaError_t ec = counts[a.key_e4m3 ? 1 : 0][i].get(&fit[i], [&](int* n) {
+      return a.key_e4m3 ? resident_clusters(reinterpret_cast<const void*>(fine_paged_tc_kernel<true>), kThreadsFp, sizeof(FpSmem<true>) + 1024, i == 0 ? 8 : 4, n)
+                        : resident_clusters(reinterpret_cast<const void*>(fine_paged_tc_kernel<false>), kThreadsFp, sizeof(FpSmem<false>) + 1024, i == 0 ? 8 : 4, n);
+    });
+    if (ec != cudaSuccess) return ec;
+  }
   const unsigned n_rank = a.n_query <= fit[0] ? 8u : a.n_query <= fit[1] ? 4u : 2 * a.n_query <= sms ? 2u : 1u;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(n_rank, static_cast<unsigned>(a.n_query), 1);

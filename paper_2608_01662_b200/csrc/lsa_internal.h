@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "../../include/lsa.h"
 
 namespace lsa {
@@ -154,31 +156,58 @@ cudaError_t launch_attn16(const AttnArgs& a, cudaStream_t st, int64_t* n_launch)
 // tcgen05 version of the attention kernel (MLA latent shape only)
 bool attn_tc_supported(const AttnArgs& a);
 // row splits that kernel merges itself (clusters of n_split blocks); other counts need launch_merge
-bool attn_tc_split_ok(int n_split);
-// Clusters of n_split blocks of that kernel that run at the same time.
-int attn_tc_resident(int n_split);
+cudaError_t attn_tc_split_ok(int n_split, bool* ok);
+// Clusters of n_split blocks of that kernel that the current device runs at the same time (0: none, or no such count).
+cudaError_t attn_tc_resident(int n_split, int* clusters);
 
-// Clusters of `blocks` blocks of a kernel that the device can hold at the same time (0: it cannot, or cannot say).  Fewer than
-// the SMs divided by the cluster's size: a cluster lies in one GPC, and one block per SM leaves a rest in each.
-inline int resident_clusters(const void* kernel, int threads, size_t smem, int blocks) {
-  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) == cudaSuccess &&
-      (blocks <= 8 || cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess)) {
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(static_cast<unsigned>(blocks) * 256);
-    cfg.blockDim = dim3(static_cast<unsigned>(threads));
-    cfg.dynamicSmemBytes = smem;
-    cudaLaunchAttribute attr[1]{};
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = static_cast<unsigned>(blocks);
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) == cudaSuccess) return n;
+// A count that depends on the device, asked for once per device and kept (an error is not: the next call asks again).
+class DeviceCount {
+ public:
+  template <class Ask>   // cudaError_t ask(int* n)
+  cudaError_t get(int* n, Ask ask) {
+    int device = 0;
+    cudaError_t e = cudaGetDevice(&device);
+    if (e != cudaSuccess) return e;
+    const bool kept = device >= 0 && device < kDevices;
+    const int known = kept ? n_plus_1_[device].load(std::memory_order_relaxed) : 0;
+    if (known != 0) {
+      *n = known - 1;
+      return cudaSuccess;
+    }
+    e = ask(n);
+    if (e == cudaSuccess && kept) n_plus_1_[device].store(*n + 1, std::memory_order_relaxed);   // (threads that ask at once store the same)
+    return e;
   }
-  (void)cudaGetLastError();
-  return 0;
+
+ private:
+  static constexpr int kDevices = 64;
+  std::atomic<int> n_plus_1_[kDevices]{};
+};
+
+// Clusters of `blocks` blocks of a kernel that the current device can hold at the same time.  Fewer than the SMs divided by the
+// cluster's size: a cluster lies in one GPC, and one block per SM leaves a rest in each.
+inline cudaError_t resident_clusters(const void* kernel, int threads, size_t smem, int blocks, int* n) {
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  if (e == cudaSuccess && blocks > 8) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(static_cast<unsigned>(blocks) * 256);
+  cfg.blockDim = dim3(static_cast<unsigned>(threads));
+  cfg.dynamicSmemBytes = smem;
+  cudaLaunchAttribute attr[1]{};
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = static_cast<unsigned>(blocks);
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  e = cudaOccupancyMaxActiveClusters(n, kernel, &cfg);
+  if (e == cudaErrorInvalidClusterSize) {   // (an answer, not a failure: a slice of a device may not have so many SMs together)
+    (void)cudaGetLastError();
+    *n = 0;
+    e = cudaSuccess;
+  }
+  return e;
 }
 cudaError_t launch_attn_tc(const AttnArgs& a, cudaStream_t st, int64_t* n_launch);
 cudaError_t launch_merge(const AttnArgs& a, cudaStream_t st, int64_t* n_launch);
