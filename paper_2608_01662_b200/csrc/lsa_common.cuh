@@ -125,7 +125,7 @@ __device__ __forceinline__ int e5m2_head_shift(float head_max_abs) {
   if (!(head_max_abs > 0.f)) return 0;
   const int e = static_cast<int>((__float_as_uint(head_max_abs) >> 23) & 0xffu) - 127;
   const int s = 14 - e;
-  return s > 100 ? 100 : (s < -100 ? -100 : s);
+  return s > 100 ? 100 : s;   // (-113 at least: 2^s and 2^-s are both normal numbers)
 }
 // 16 consecutive elements of a query head, scaled, as three e5m2 planes (16 bytes each): x = p1 + p2 + p3.
 __device__ __forceinline__ void split_e5m2x16(const float (&x)[16], uint4& p1, uint4& p2, uint4& p3) {
