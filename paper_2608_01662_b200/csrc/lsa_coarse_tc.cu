@@ -41,11 +41,14 @@ struct CoarseTcSmem {
   float w[NG * kGroupQ][kHI];
   alignas(8) uint64_t full[kStages], empty[kStages], q_full, acc_full[2], acc_empty[2];
   uint32_t tmem_slot;
+  int again;   // a score is not finite
 };
 
-// sum_h w[h] * max(v[h], 0) of one row, odd heads as w/2 * (v + |v|): the same number, and fmaxf issues at half the rate of an add.
-// (Weights of odd heads are staged halved.)  16 broadcast loads of the weights per row: with the MMAs' operands they are what
-// fills the shared-memory pipe here; without them 4096 queries against a million keys would take 7.0 ms, not 7.6.
+// sum_h w[h] * max(v[h], 0) of one row, odd heads as w/2 * (v + |v|): fmaxf issues at half the rate of an add (4096 queries
+// against a million keys: 7.83 ms with fmaxf alone, 7.47 so, at one clock).  It is the same number as long as 2 v is finite; where it is not the
+// sum comes out infinite or NaN, and score_again() has the last word.  (Weights of odd heads are staged halved.)  16 broadcast
+// loads of the weights per row: with the MMAs' operands they are what fills the shared-memory pipe here; without them it would
+// be 7.0 ms.
 __device__ __forceinline__ float head_sum_row64(const uint32_t (&v)[64], const float* w) {
   const float4* w4 = reinterpret_cast<const float4*>(w);
   float2 a = make_float2(0.f, 0.f);
@@ -59,9 +62,35 @@ __device__ __forceinline__ float head_sum_row64(const uint32_t (&v)[64], const f
   return a.x + a.y;
 }
 
+// The scores of pages page0 .. page1 - 1 and queries q0 .. q0 + nq - 1 once more where they are not finite in the form above (a
+// head's dot product beyond fp32: below it the head counts as 0).  By the whole block, behind its loop: hardly ever, and inside
+// the loop there is no register for it.
+__device__ __noinline__ void score_again(const IndexArgs& p, int q0, int nq, int64_t page0, int64_t page1) {
+  const int spp = p.P / p.B;
+  const int64_t n_sub = (p.n_key + p.B - 1) / p.B, n_pages = page1 - page0;
+  for (int64_t i = threadIdx.x; i < n_pages * nq; i += kThreadsTc) {
+    const int q = q0 + static_cast<int>(i / n_pages);
+    const int64_t page = page0 + i % n_pages;
+    if (page * p.P > p.q_pos0 + q - p.W) continue;   // (not scored)
+    float* score = p.page_scores + static_cast<int64_t>(q) * p.ps_ld + page;
+    if (fabsf(*score) < INFINITY) continue;
+    double sum = 0.0;
+    for (int64_t sub = page * spp; sub < min64((page + 1) * spp, n_sub); ++sub) {
+      const __nv_bfloat16* k = reinterpret_cast<const __nv_bfloat16*>(p.kmean) + sub * kDI;
+      const __nv_bfloat16* qh = reinterpret_cast<const __nv_bfloat16*>(p.q_idx) + static_cast<int64_t>(q) * kHI * kDI;
+      for (int h = 0; h < kHI; ++h, qh += kDI) {
+        double dot = 0.0;
+        for (int d = 0; d < kDI; ++d) dot += static_cast<double>(__bfloat162float(qh[d])) * static_cast<double>(__bfloat162float(k[d]));
+        if (dot > 0.0) sum += static_cast<double>(p.w[static_cast<int64_t>(q) * kHI + h]) * dot;
+      }
+    }
+    *score = static_cast<float>(sum);
+  }
+}
+
 template <int NG>
 __global__ void __launch_bounds__(kThreadsTc, 1)
-coarse_score_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_km, int parts, IndexArgs p) {
+coarse_score_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_km, int parts, const __grid_constant__ IndexArgs p) {
   using Smem = CoarseTcSmem<NG>;
   constexpr int NS = Smem::kStages;
   constexpr int QB = NG * kGroupQ;  // queries per block
@@ -99,6 +128,7 @@ coarse_score_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
       tc::mbar_init(smem_u32(&sm.empty[s]), 1);
     }
     tc::mbar_init(smem_u32(&sm.q_full), 1);
+    sm.again = 0;
     for (int b = 0; b < 2; ++b) {
       tc::mbar_init(smem_u32(&sm.acc_full[b]), 1);
       tc::mbar_init(smem_u32(&sm.acc_empty[b]), kEpiWarps / 2);
@@ -203,8 +233,11 @@ coarse_score_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
         for (int qq = 0; qq < 2; ++qq) {
           const int ql = ql0 + qq;
           const int64_t t = p.q_pos0 + q0 + ql;
-          if (ql < nq && page * p.P <= t - p.W)
-            p.page_scores[static_cast<int64_t>(q0 + ql) * p.ps_ld + page] = qq ? acc1 : acc0;
+          if (ql < nq && page * p.P <= t - p.W) {
+            const float score = qq ? acc1 : acc0;
+            p.page_scores[static_cast<int64_t>(q0 + ql) * p.ps_ld + page] = score;
+            if (!(fabsf(score) < INFINITY)) sm.again = 1;
+          }
         }
       }
     }
@@ -212,6 +245,8 @@ coarse_score_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
   tc::fence_before_sync();
   __syncthreads();
   if (warp == 1) tc::tmem_dealloc(tmem_base, kTmemCols);
+  if (sm.again)
+    score_again(p, q0, nq, static_cast<int64_t>(tile0) * kTileM >> spp_shift, static_cast<int64_t>(tile0 + n_tiles) * kTileM >> spp_shift);
 }
 
 }  // namespace

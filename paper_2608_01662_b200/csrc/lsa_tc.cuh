@@ -243,12 +243,11 @@ __device__ __forceinline__ void tmem_ld_16x128b_x16(uint32_t taddr, uint32_t (&r
 // token scores and selection of 16384 queries 2.72 -> 2.57 ms, of 32768 4.46 -> 4.21 ms; one flat decode step of 16 sequences
 // 240 -> 236 us.  Where N = 256 keeps the accumulators busy (lsa_coarse_tc.cu) the slower TMEM loads lose more than that.
 // (A 32 x 64 block leaves TMEM in 39 cycles as whole rows, 70 in this layout and 129 in the 16x256b one.)
-// fmaxf issues at half the rate of an add: every other head takes w/2 * (v + |v|) instead, the same number.
 struct HeadWeights {
-  float2 w[8];   // heads 8 i + (lane & 3) and, halved, 8 i + 4 + (lane & 3)
+  float2 w[8];   // heads 8 i + (lane & 3) and 8 i + 4 + (lane & 3)
   __device__ __forceinline__ void load(const float* smem_w, int lane) {
 #pragma unroll
-    for (int i = 0; i < 8; ++i) w[i] = make_float2(smem_w[8 * i + (lane & 3)], 0.5f * smem_w[8 * i + 4 + (lane & 3)]);
+    for (int i = 0; i < 8; ++i) w[i] = make_float2(smem_w[8 * i + (lane & 3)], smem_w[8 * i + 4 + (lane & 3)]);
   }
 };
 struct HeadScores {
@@ -268,7 +267,7 @@ __device__ __forceinline__ float head_sum(const HeadScores& s, const HeadWeights
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       const float x = __uint_as_float((j < 2 ? s.lo : s.hi)[4 * i + (j & 1)]), y = __uint_as_float((j < 2 ? s.lo : s.hi)[4 * i + 2 + (j & 1)]);
-      a[j] = fma2(hw.w[i], make_float2(fmaxf(x, 0.f), y + fabsf(y)), a[j]);
+      a[j] = fma2(hw.w[i], make_float2(fmaxf(x, 0.f), fmaxf(y, 0.f)), a[j]);
     }
   }
   // four lanes hold the parts of the same four rows: two exchanges leave each with one row

@@ -4,7 +4,7 @@ import pytest
 import torch
 
 from paper_2608_01662_b200.configs import CONFIGS
-from paper_2608_01662_b200.workload import DecodeWorkload
+from paper_2608_01662_b200.workload import DecodeWorkload, PrefillWorkload
 
 import parity_util as pu
 
@@ -33,8 +33,25 @@ def _far_heads(wl):
         wl.w[:, h] = wl.w[:, h] * 1.0e-38
 
 
-@pytest.mark.parametrize("key_dtype", ["e4m3"])
-@pytest.mark.parametrize("change", [dict(hi_enable=False)])
+# prompt; the same with many queries; flat; large budget
+@pytest.mark.parametrize("base,change,n_query", [("cfg2", dict(L=9000, M=16), 40), ("cfg3", dict(L=9000, M=16), 40), ("cfg2", dict(L=3000, M=8), 3000),
+                                                 ("cfg2", dict(L=6000, hi_enable=False), 20), ("cfg3", dict(L=20000, hi_enable=False), 20),
+                                                 ("cfg2", dict(L=20000, M=80), 20), ("cfg3", dict(L=20000, M=80), 20)])
+def test_prompt(cuda_device, base, change, n_query):
+    cfg = CONFIGS[base].replace(**{"R": 1, "Ksp": 256, "W": 130, "seed": 9, **change})
+    wl = PrefillWorkload(cfg, cuda_device, q_pos0=cfg.L - n_query, n_query=n_query)
+    _far_heads(wl)
+    wl.prepare()
+    pages = torch.empty((n_query, cfg.M), dtype=torch.int32, device=cuda_device)
+    wl.index(pages_out=pages)
+    assert wl.ctx.status() == 0
+    m = pu.check_prefill(wl, range(wl.q_pos0, wl.q_pos0 + n_query, max(1, n_query // 12)), check_attention=False, pages=pages if cfg.hi_enable else None)
+    print(base, change, m.summary())
+    m.assert_ok(pu.TOL_BF16)
+
+
+@pytest.mark.parametrize("key_dtype", ["e4m3", "bf16"])
+@pytest.mark.parametrize("change", [dict(), dict(P=128, kv_page=128, M=8), dict(hi_enable=False)])
 def test_decode(cuda_device, key_dtype, change):
     cfg = CONFIGS["cfg4"].replace(**{"batch": 6, "ctx_lo": 3000, "ctx_hi": 9000, "M": 16, "Ksp": 256, "R": 1, "W": 130, "seed": 9, "key_dtype": key_dtype, **change})
     wl = DecodeWorkload(cfg, cuda_device)
