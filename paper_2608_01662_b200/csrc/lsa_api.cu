@@ -729,17 +729,20 @@ int lsa_layer_group_host(lsa_ctx* c, const lsa_params* p, const void* q_idx_host
   if (q_idx_host == nullptr || w_host == nullptr || q_host == nullptr || out_host == nullptr || n_query < 0 || q_pos0 < 0) return LSA_ERR_ARG;
   const int R = p->n_layers;
   if (R > kMaxHostLayers) return LSA_ERR_SHAPE;
+  if (n_query == 0) return LSA_OK;   // (nothing to copy, compute or wait for)
   if (k == nullptr || v == nullptr) return LSA_ERR_ARG;
   for (int l = 0; l < R; ++l)
     if (q_host[l] == nullptr || k[l] == nullptr || v[l] == nullptr || out_host[l] == nullptr) return LSA_ERR_ARG;
   const size_t b_qi = static_cast<size_t>(p->n_heads_idx) * p->d_idx * 2, b_w = static_cast<size_t>(p->n_heads_idx) * 4;
   const size_t b_q = static_cast<size_t>(p->n_heads) * p->d_qk * 2, b_o = static_cast<size_t>(p->n_heads) * p->d_v * 2;
   cudaError_t e = cudaSuccess;
-  for (; c->n_host_slots < 1 + R && e == cudaSuccess; ++c->n_host_slots)
+  while (c->n_host_slots < 1 + R) {
     for (int s = 0; s < 2 && e == cudaSuccess; ++s)
       for (cudaEvent_t* ev : {&c->ev_in[s][c->n_host_slots], &c->ev_done[s][c->n_host_slots], &c->ev_out[s][c->n_host_slots]})
         if (e == cudaSuccess && *ev == nullptr) e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming);
-  if (e != cudaSuccess) return cuda_fail(c, e);
+    if (e != cudaSuccess) return cuda_fail(c, e);
+    ++c->n_host_slots;   // (only when all of its events are there: the next call goes on where this one failed)
+  }
   const int64_t n_pass = (n_query + sq - 1) / sq;
   // the caller's earlier work on the context stream must be visible to the copy streams
   e = cudaEventRecord(c->ev_start, c->stream);
