@@ -756,7 +756,7 @@ __global__ void __launch_bounds__(kSelThreads) select_long_kernel(const float* _
   const float* row = scores + qi * ld;
   const int64_t t = ctx_len ? static_cast<int64_t>(ctx_len[qi]) - 1 : q_pos0 + qi;
   const RowKeys<SOURCE> key{row, cand_pos ? cand_pos + qi * n_cand : nullptr, pos_scale, apply_range ? S : 0,
-                            apply_range ? static_cast<int>(max64(-1, t - W)) : 0x7fffffff};
+                            apply_range ? static_cast<int>(max64(-1, min64(t - W, 0x7fffffff))) : 0x7fffffff};
   auto id = [&](int i) -> int { return key.id(i); };
   int n = static_cast<int>(n_cand);   // columns that are positions: nothing beyond the range can take part
   if (cand_pos == nullptr) n = static_cast<int>(min64(n_cand, static_cast<int64_t>(key.hi) + 1));

@@ -58,3 +58,21 @@ def test_select_long_rows(cuda_device, n_cand, k, n_query):
             want = orc.select_fp32(rows[i % len(KINDS)], None, q_pos0 + i, k, apply_range=in_range, S=5, W=77)
             got = idx[i].cpu().numpy()
             assert int(cnt[i]) == len(want) and np.array_equal(got[:len(want)], want) and (got[len(want):] == -1).all(), (i, in_range)
+
+
+# the last columns of the scoring range at the query's position, and positions past 2^31
+@pytest.mark.parametrize("n_cand,n_query", [(1000, 5), (20000, 5), (20000, 300)])
+@pytest.mark.parametrize("q_pos0", [(1 << 31) - 1 - 80, (1 << 31) + 70, 1 << 40])
+def test_queries_at_far_positions(cuda_device, n_cand, n_query, q_pos0):
+    """apply_range with positions that do not fit 32 bits: every candidate from the sink on is in range."""
+    rng = np.random.default_rng(n_cand)
+    rows = rng.standard_normal((n_query, n_cand)).astype(np.float32)
+    k = 500
+    ctx = binding.Context(binding.make_params(CONFIGS["cfg1"].replace(S=5, W=77)), n_query, n_cand, device=cuda_device)
+    idx = torch.empty((n_query, k), dtype=torch.int32, device=cuda_device)
+    cnt = torch.empty((n_query,), dtype=torch.int32, device=cuda_device)
+    ctx.select(torch.from_numpy(rows).to(cuda_device), None, q_pos0, k, True, idx, cnt)
+    assert ctx.status() == 0
+    for i in (0, n_query - 1):
+        want = orc.select_fp32(rows[i], None, q_pos0 + i, k, apply_range=True, S=5, W=77)
+        assert int(cnt[i]) == len(want) == k and np.array_equal(idx[i].cpu().numpy(), want)
