@@ -273,7 +273,7 @@ int run_index(lsa_ctx* c, const lsa_params* p, const void* q_idx, const float* w
       if (e == cudaSuccess)
         e = timed(c, LSA_K_SELECT, [&] {
           return lsa::launch_select(a.page_scores, a.ps_ld, nullptr, nullptr, 0, a.n_query, n_key_max, p->k_sparse, 1, p->k_sink,
-                                    p->k_swa, a.sparse_idx, a.n_sparse, c->stream, &c->launches, ctx_len,
+                                    p->k_swa, a.sparse_idx, a.n_sparse, c->stream, &c->launches, c->sm_count, ctx_len,
                                     a.rows_out != nullptr ? &rows : nullptr, &rows_done);
         });
       if (e == cudaSuccess && a.rows_out != nullptr && !rows_done)
@@ -304,7 +304,7 @@ int run_index(lsa_ctx* c, const lsa_params* p, const void* q_idx, const float* w
         e = timed(c, LSA_K_SELECT, [&] {
           return lsa::launch_select(a.page_scores, a.ps_ld, nullptr, a.key_e4m3 ? k_scale : nullptr, a.q_pos0, a.n_query,
                                     n_key, p->k_sparse, 1, p->k_sink, p->k_swa, a.sparse_idx, a.n_sparse, c->stream,
-                                    &c->launches);
+                                    &c->launches, c->sm_count);
         });
       if (e == cudaSuccess && a.pages_out != nullptr)
         e = cudaMemsetAsync(a.pages_out, 0xff, static_cast<size_t>(a.n_query) * p->keep_pages * sizeof(int32_t), c->stream);
@@ -612,7 +612,7 @@ int lsa_select(lsa_ctx* c, const lsa_params* p, const float* scores, int64_t ld_
   if (n_query == 0 || k == 0) return LSA_OK;
   cudaError_t e = timed(c, LSA_K_SELECT, [&] {
     return lsa::launch_select(scores, ld_scores, cand_pos, nullptr, q_pos0, static_cast<int>(n_query), n_cand, k, apply_range,
-                              p->k_sink, p->k_swa, idx_out, n_out, c->stream, &c->launches);
+                              p->k_sink, p->k_swa, idx_out, n_out, c->stream, &c->launches, c->sm_count);
   });
   return e == cudaSuccess ? LSA_OK : cuda_fail(c, e);
 }

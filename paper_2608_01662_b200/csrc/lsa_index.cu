@@ -364,8 +364,8 @@ __global__ void __launch_bounds__(kThreads, 2) coarse_score_paged_kernel(IndexAr
 // ------------------------------------------------------------------------------------------------
 // a2-a4: per query: top-M pages, fine scores on their tokens, top-K_sparse.
 // ------------------------------------------------------------------------------------------------
-constexpr int kClusterRowsMax = 256;    // rows: up to this many, a row of kLongMinRow scores or more gets a cluster of blocks
-constexpr size_t kLongSmemMax = 226 * 1024;
+constexpr int kClusterRowsMax = 256;    // rows: up to this many may get a cluster of blocks each (see select_form)
+constexpr size_t kLongSmemMax = 226 * 1024, kSmSmem = 228 * 1024;   // of a block; of an SM
 constexpr int kMaxSlots = 4096;  // keep_pages * page
 constexpr int kMaxPages = 64;    // keep_pages
 
@@ -691,8 +691,8 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(const float* __rest
 }
 
 // The same selection over long rows: one pass over the row and the rest on what it collected (lsa_select_long.cuh), the
-// radix select where that does not serve.  CLUSTER: a cluster of kClusterSel blocks per row (few rows: the flat indexer in
-// decode), which also writes the selection's cache rows when the caller wants them.
+// radix select where that does not serve (cap = 0: at once).  CLUSTER: a cluster of kClusterSel blocks per row, which also
+// writes the selection's cache rows when the caller wants them (flat indexer in decode).
 // Keys of a row's items.  SOURCE: the score alone, or times its position's factor, read four at a time (rows and factors
 // 16-byte aligned); or whatever the call gives, one at a time.  A template, because a test of the pointers between the loads
 // of a step keeps them from going out together.
@@ -766,7 +766,7 @@ __global__ void __launch_bounds__(kSelThreads) select_long_kernel(const float* _
   const int n_sink = static_cast<int>(min64(S, t + 1)), shift = rows.rows_out ? 31 - __clz(rows.kv_page) : 0, mask = rows.kv_page - 1;
   int n_sel = -1;
   // (CLUSTER: also short rows, whose pieces are collected whole)
-  if (CLUSTER || n >= kLongMinRow)
+  if (cap > 0 && (CLUSTER || n >= kLongMinRow))
     n_sel = long_select<CLUSTER>(
         key,
         [&](int r, int i) {
@@ -1262,53 +1262,71 @@ cudaError_t launch_widen_e4m3(const void* codes, void* out_bf16, int64_t n_elems
   return cudaGetLastError();
 }
 
+// How launch_select serves rows of n_cand scores (any: not read four at a time).  Measured (us, k = 2048 unless said; one pass by
+// a block per row / one pass by clusters / radix select by clusters / radix select by a block):
+//   rows x scores      16 x 32768   64 x 65536   64 x 131072   128 x 131072   256 x 16384   400 x 131072
+//                      29/29/29/96  41/41/59/192 61/45/104/363 72/76/186/375  27/121/83/66  109/190/497/666
+//   any, odd pitch                  66/49/64/193 113/59/107/363 117/109/190/373 31/114/88/68
+// A block per row is the rule.  Clusters serve rows so few and long that a block's read of one is what the call waits for, as
+// long as all of them are resident: a second wave doubles the time, and the lists of a large k leave room for one or two
+// blocks on an SM (16 rows of 131072, k = 8192: 76 us by blocks, 82 by clusters, of which 15 fit).  Few rows of a large k that
+// miss that are the radix clusters' (32 x 65536, k = 8192: 51/84/43/198; 64 x 16384: 39/74/27/45), and many rows that the lists
+// of one pass would hold whole the radix blocks' (400 x 16384, k = 8192: 98/363/120/84).  Where the cache rows are wanted too,
+// clusters serve up to kClusterRowsMax rows (flat decode step of 33 sequences 147 us, 168 by a block per row; of 64 and 128 the same).
+enum SelectForm { kRadixBlock, kRadixCluster, kOnePassBlock, kOnePassCluster };
+SelectForm select_form(int n_query, int64_t n_cand, int k, bool any, bool rows, int sm_count) {
+  if (n_cand < kLongMinRow) return kRadixBlock;
+  const bool few = n_query <= kClusterRowsMax;
+  const size_t by_block = long_smem_bytes(false, long_cap(k), n_cand), by_cluster = long_smem_bytes(true, long_cap(k), long_piece(static_cast<int>(n_cand)));
+  const bool cluster_fits = by_cluster <= kLongSmemMax;
+  if (rows && few) return cluster_fits ? kOnePassCluster : kRadixCluster;
+  const int per_sm = static_cast<int>(kSmSmem / (by_cluster + 1024)), blocks = sm_count * (per_sm < 8 ? per_sm : 8);
+  const int resident = blocks / kClusterSel - 3;   // (a cluster lies in one GPC: what is left over in each)
+  if (cluster_fits && n_query <= resident && n_query * static_cast<int64_t>(any ? 1024 : 2048) <= n_cand) return kOnePassCluster;
+  if (k >= 4096 && (any || n_cand < 32768 ? 2 : 4) * n_query <= sm_count && n_cand <= 262144) return kRadixCluster;
+  if (!few && n_cand <= long_cap(k)) return kRadixBlock;
+  if (by_block <= kLongSmemMax) return kOnePassBlock;
+  if (few) return cluster_fits ? kOnePassCluster : kRadixCluster;   // (rows of more than about 1.5 and 12 million)
+  return kRadixBlock;
+}
+
 cudaError_t launch_select(const float* scores, int64_t ld, const int32_t* cand_pos, const float* pos_scale,
                           int64_t q_pos0, int n_query, int64_t n_cand, int k, int apply_range, int S, int W,
-                          int32_t* idx_out, int32_t* n_out, cudaStream_t st, int64_t* n_launch, const int32_t* ctx_len,
+                          int32_t* idx_out, int32_t* n_out, cudaStream_t st, int64_t* n_launch, int sm_count, const int32_t* ctx_len,
                           const SelectRows* rows, bool* rows_done) {
   if (n_query == 0) return cudaSuccess;
   if (rows_done) *rows_done = false;
   const bool quads = cand_pos == nullptr && ld % 4 == 0 && ((reinterpret_cast<uintptr_t>(scores) | reinterpret_cast<uintptr_t>(pos_scale)) & 15u) == 0;
-  const int source = !quads ? kScoreAny : pos_scale ? kScaledQuads : kScoreQuads;
-  const int cap = long_cap(k);
-  const SelectRows no_rows{};
-  if (n_query <= kClusterRowsMax && n_cand >= kLongMinRow) {
-    // few long rows: a cluster of blocks per row
-    const size_t piece = long_smem_bytes(true, cap, long_piece(static_cast<int>(n_cand)));
-    const size_t smem = piece > sizeof(ClusterSelScratch) ? piece : sizeof(ClusterSelScratch);
-    if (smem <= kLongSmemMax) {
-      auto kernel = source == kScoreQuads ? select_long_kernel<true, kScoreQuads> : source == kScaledQuads ? select_long_kernel<true, kScaledQuads> : select_long_kernel<true, kScoreAny>;
-      cudaError_t e = set_smem(kernel, smem);
-      if (e != cudaSuccess) return e;
-      cudaLaunchConfig_t cfg{};
-      cfg.gridDim = dim3(kClusterSel, static_cast<unsigned>(n_query), 1);
-      cfg.blockDim = dim3(kSelThreads);
-      cfg.dynamicSmemBytes = smem;
-      cfg.stream = st;
-      cudaLaunchAttribute attr[2]{};
-      attr[0].id = cudaLaunchAttributeClusterDimension;
-      attr[0].val.clusterDim.x = kClusterSel;
-      attr[0].val.clusterDim.y = 1;
-      attr[0].val.clusterDim.z = 1;
-      attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-      attr[1].val.programmaticStreamSerializationAllowed = 1;
-      cfg.attrs = attr;
-      cfg.numAttrs = 2;
-      e = cudaLaunchKernelEx(&cfg, kernel, scores, ld, cand_pos, pos_scale, q_pos0, n_cand, k, apply_range, S, W,
-                             idx_out, n_out, ctx_len, rows ? *rows : no_rows, cap);
-      ++*n_launch;
-      if (rows_done) *rows_done = rows != nullptr;
-      return e;
-    }
-  }
-  const size_t smem = long_smem_bytes(false, cap, n_cand);
-  if (n_cand >= kLongMinRow && smem <= kLongSmemMax) {
-    auto kernel = source == kScoreQuads ? select_long_kernel<false, kScoreQuads> : source == kScaledQuads ? select_long_kernel<false, kScaledQuads> : select_long_kernel<false, kScoreAny>;
+  const SelectForm form = select_form(n_query, n_cand, k, !quads, rows != nullptr, sm_count > 0 ? sm_count : 148);
+  if (form != kRadixBlock) {
+    const int source = !quads ? kScoreAny : pos_scale ? kScaledQuads : kScoreQuads;
+    const bool cluster = form != kOnePassBlock;
+    const int cap = form == kRadixCluster ? 0 : long_cap(k);
+    size_t smem = cap == 0 ? 0 : long_smem_bytes(cluster, cap, cluster ? long_piece(static_cast<int>(n_cand)) : n_cand);
+    const size_t radix = cluster ? sizeof(ClusterSelScratch) : sizeof(SelectScratch);
+    if (smem < radix) smem = radix;
+    auto kernel = cluster ? (source == kScoreQuads ? select_long_kernel<true, kScoreQuads> : source == kScaledQuads ? select_long_kernel<true, kScaledQuads> : select_long_kernel<true, kScoreAny>)
+                          : (source == kScoreQuads ? select_long_kernel<false, kScoreQuads> : source == kScaledQuads ? select_long_kernel<false, kScaledQuads> : select_long_kernel<false, kScoreAny>);
     cudaError_t e = set_smem(kernel, smem);
     if (e != cudaSuccess) return e;
-    e = launch_pdl(kernel, dim3(n_query), dim3(kSelThreads), smem, st, scores, ld, cand_pos, pos_scale, q_pos0,
-                   n_cand, k, apply_range, S, W, idx_out, n_out, ctx_len, no_rows, cap);
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = cluster ? dim3(kClusterSel, static_cast<unsigned>(n_query), 1) : dim3(static_cast<unsigned>(n_query), 1, 1);
+    cfg.blockDim = dim3(kSelThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2]{};
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = kClusterSel;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = cluster ? 2 : 1;
+    e = cudaLaunchKernelEx(&cfg, kernel, scores, ld, cand_pos, pos_scale, q_pos0, n_cand, k, apply_range, S, W,
+                           idx_out, n_out, ctx_len, rows && cluster ? *rows : SelectRows{}, cap);
     ++*n_launch;
+    if (rows_done) *rows_done = rows != nullptr && cluster;
     return e;
   }
   select_kernel<<<n_query, kSelThreads, 0, st>>>(scores, ld, cand_pos, pos_scale, q_pos0, n_cand, k, apply_range, S, W,

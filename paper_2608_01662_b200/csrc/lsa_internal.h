@@ -139,7 +139,7 @@ struct SelectRows {
 };
 cudaError_t launch_select(const float* scores, int64_t ld, const int32_t* cand_pos, const float* pos_scale,
                           int64_t q_pos0, int n_query, int64_t n_cand, int k, int apply_range, int S, int W,
-                          int32_t* idx_out, int32_t* n_out, cudaStream_t st, int64_t* n_launch,
+                          int32_t* idx_out, int32_t* n_out, cudaStream_t st, int64_t* n_launch, int sm_count,
                           const int32_t* ctx_len = nullptr, const SelectRows* rows = nullptr, bool* rows_done = nullptr);
 // Token scores over cache pages on tcgen05 (paged caches, 64-token pages, H_I = 64, d_I = 128).  flat = 0: keys of the
 // slots of the page lists a.fine_pages -> a.fine_keys; flat = 1: scores of the whole scoring range -> a.page_scores.

@@ -7,6 +7,9 @@ import torch
 from oracle import lsa_oracle as orc
 from paper_2608_01662_b200 import binding
 from paper_2608_01662_b200.configs import CONFIGS
+from paper_2608_01662_b200.workload import DecodeWorkload
+
+import parity_util as pu
 
 pytestmark = pytest.mark.gpu
 
@@ -41,7 +44,9 @@ KINDS = ("normal", "ties", "equal", "sampled_high", "sampled_low", "piece")
 
 
 @pytest.mark.parametrize("n_cand,k,n_query", [(16384, 1, 300), (16640, 700, 9), (16385, 2048, 257), (65537, 2048, 260), (40000, 4100, 258), (140001, 300, 257),
-                                              (16384, 2048, 6), (49153, 8192, 6), (131073, 2048, 12), (600001, 2048, 6)])
+                                              (16384, 2048, 6), (49153, 8192, 6), (131073, 2048, 12), (600001, 2048, 6),
+                                              # a block per row although few; the radix select by clusters, and by blocks
+                                              (20001, 2048, 40), (70000, 8192, 20), (16385, 8192, 9), (16384, 8192, 258)])
 def test_select_long_rows(cuda_device, n_cand, k, n_query):
     rng = np.random.default_rng(n_cand + k)
     rows = np.stack([_row(kind, n_cand, rng) for kind in KINDS]).astype(np.float32)
@@ -76,3 +81,16 @@ def test_queries_at_far_positions(cuda_device, n_cand, n_query, q_pos0):
     for i in (0, n_query - 1):
         want = orc.select_fp32(rows[i], None, q_pos0 + i, k, apply_range=True, S=5, W=77)
         assert int(cnt[i]) == len(want) == k and np.array_equal(idx[i].cpu().numpy(), want)
+
+
+@pytest.mark.parametrize("batch", [2, 40, 257])
+def test_flat_decode_lists_its_rows(cuda_device, batch):
+    """The selection of long rows by clusters writes the cache rows as well; for more rows than get a cluster a kernel of its own does."""
+    cfg = CONFIGS["cfg4"].replace(batch=batch, ctx_lo=300, ctx_hi=20000, hi_enable=False, R=1, Ksp=1024, seed=batch)
+    wl = DecodeWorkload(cfg, cuda_device)
+    wl.prepare()
+    wl.step()
+    assert wl.ctx.status() == 0
+    m = pu.check_decode(wl, range(0, batch, max(1, batch // 12)))
+    print(batch, m.summary())
+    m.assert_ok(pu.TOL_FP8)
