@@ -1,10 +1,10 @@
 // a1-a4 for the 8-head, 64-dim indexer on contiguous bf16 caches with a recall budget of at most 1024 tokens: coarse page
 // scores (Eq. 9), top-M pages (Eq. 10), token scores on them (Eq. 11) and the top-K_sparse outside sink and window
-// (Eq. 12), one warp per query, in one launch.
+// (Eq. 12), one warp per query (4 or 16 where there are few), in one launch.
 //
-// Nothing is shared between warps: key rows go from global memory (L1 or L2: the caches of this shape are small, and the
-// warps of a block hold neighbouring queries) straight to the A operands of m16n8k16 MMAs, whose eight columns are the
-// eight heads.  The sum over dims may run in any order, so a thread takes the 16-byte chunks t and 4 + t (t = lane % 4) of
+// Nothing is shared between the warps of different queries: key rows go from global memory (L1 or L2: the caches of this shape
+// are small, and the warps of a block hold neighbouring queries) straight to the A operands of m16n8k16 MMAs, whose eight
+// columns are the eight heads.  The sum over dims may run in any order, so a thread takes the 16-byte chunks t and 4 + t (t = lane % 4) of
 // a row, and the query heads are fetched in the same order.  A group of 32 rows ends as one score per lane, and the keys of
 // all candidates stay in registers (32 per lane at most), where the K-th largest is found bit by bit: a count of the keys
 // above a trial value is one compare per register and one warp-wide add.
@@ -23,6 +23,7 @@ constexpr int kHI8 = 8, kDI8 = 64, kRow8 = kDI8 * 2;
 constexpr int kWarps8 = 4;
 constexpr int kMaxSlots8 = 1024;             // candidate tokens of a query
 constexpr int kMaxPages8 = 1024;             // eligible pages of a query
+constexpr int kMaxMeans8 = 8192;             // mean keys of the cache
 constexpr int kMaxKept8 = kMaxSlots8 / 64;
 static_assert(kMaxPages8 <= kMaxSlots8, "page keys and candidate keys share their place");
 
@@ -108,12 +109,22 @@ __device__ __forceinline__ int warp_topk(const uint32_t (&key)[R], int k, Emit e
   return base;
 }
 
-template <int R>
-__global__ void __launch_bounds__(32 * kWarps8) index8_kernel(IndexArgs p) {
-  __shared__ uint32_t keys[kWarps8][kMaxSlots8];   // of the pages, then of the candidates
-  __shared__ int32_t kept[kWarps8][kMaxKept8];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, t = lane & 3;
-  const int slot = static_cast<int>(blockIdx.x) * kWarps8 + warp;
+// kWpq warps share a query (1: four queries per block).  They deal the groups of 32 mean keys and of 64 tokens among them and
+// meet before each selection, which is the first one's; a row's score does not depend on the warp that takes it, so every
+// kWpq gives the same lists.
+template <int R, int kWpq>
+__global__ void __launch_bounds__(32 * (kWpq > kWarps8 ? kWpq : kWarps8)) index8_kernel(IndexArgs p) {
+  constexpr int kQueries = kWpq > 1 ? 1 : kWarps8;
+  __shared__ uint32_t keys[kQueries][kMaxSlots8];   // of the pages, then of the candidates
+  __shared__ int32_t kept[kQueries][kMaxKept8];
+  __shared__ int n_kept;
+  const int lane = threadIdx.x & 31, t = lane & 3;
+  const int part = kWpq > 1 ? threadIdx.x >> 5 : 0, own = kWpq > 1 ? 0 : threadIdx.x >> 5;   // the warp's part of the query, its query
+  auto meet = [&]() {
+    if constexpr (kWpq > 1) __syncthreads();
+    else __syncwarp();
+  };
+  const int slot = static_cast<int>(blockIdx.x) * kQueries + own;
   const int qi = p.n_query - 1 - slot;   // late queries have the most pages: they go first
   if (qi < 0) return;
   pdl_wait();                 // the mean keys may come from the previous kernel of the stream
@@ -135,64 +146,73 @@ __global__ void __launch_bounds__(32 * kWarps8) index8_kernel(IndexArgs p) {
     const int p_shift = 31 - __clz(p.P);
     const int p0 = static_cast<int>(lo >> p_shift), p1 = static_cast<int>(hi >> p_shift);
     const int n_elig = p1 - p0 + 1;
-    int32_t* pages = kept[warp];
+    int32_t* pages = kept[own];
     if (p.hi_enable && n_elig > p.M) {
       const int spp = p.P / p.B, spp_shift = 31 - __clz(spp);   // sub-blocks per page: 8, 16 or 32
       const int n_sub = static_cast<int>((p.n_key + p.B - 1) / p.B);
       const int sub0 = p0 << spp_shift, sub1 = min(n_sub, (p1 + 1) << spp_shift);
       const uint8_t* km = reinterpret_cast<const uint8_t*>(p.kmean);
-      uint32_t* pk = keys[warp];
+      uint32_t* pk = keys[own];
+      constexpr int kStep = 32 * kWpq;
       uint4 a[2][4][2];   // the next group is on its way while one is scored
-      load_32rows(a[0], km + static_cast<int64_t>(sub0) * kRow8, sub1 - 1 - sub0);
+      auto load_means = [&](uint4 (&to)[4][2], int s) {
+        if (s < sub1) load_32rows(to, km + static_cast<int64_t>(s) * kRow8, sub1 - 1 - s);
+      };
+      load_means(a[0], sub0 + 32 * part);
       auto score_group = [&](int s, const uint4 (&now)[4][2], uint4 (&next)[4][2]) {
-        if (s + 32 < sub1) load_32rows(next, km + static_cast<int64_t>(s + 32) * kRow8, sub1 - 1 - (s + 32));
+        load_means(next, s + kStep);
         float v = score_32rows(h, now);
         if (s + lane >= sub1) v = 0.f;
         for (int d = 1; d < spp; d <<= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
         if ((lane & (spp - 1)) == 0 && s + lane < sub1) pk[(s + lane - sub0) >> spp_shift] = score_key(v);
       };
-      for (int s = sub0; s < sub1; s += 64) {
+      for (int s = sub0 + 32 * part; s < sub1; s += 2 * kStep) {
         score_group(s, a[0], a[1]);
-        if (s + 32 < sub1) score_group(s + 32, a[1], a[0]);
+        if (s + kStep < sub1) score_group(s + kStep, a[1], a[0]);
       }
-      __syncwarp();
+      meet();
       auto keep = [&](int rank, int item, int) { pages[rank] = p0 + item; };
       auto page_key = [&](int i) -> uint32_t { return i < n_elig ? pk[i] : 0u; };
-      if (n_elig <= 256) {
-        uint32_t key[8];
+      if (part == 0) {
+        if (n_elig <= 256) {
+          uint32_t key[8];
 #pragma unroll
-        for (int r = 0; r < 8; ++r) key[r] = page_key(32 * r + lane);
-        n_pages = warp_topk<8>(key, p.M, keep);
-      } else {
-        uint32_t key[kMaxPages8 / 32];
+          for (int r = 0; r < 8; ++r) key[r] = page_key(32 * r + lane);
+          n_pages = warp_topk<8>(key, p.M, keep);
+        } else {
+          uint32_t key[kMaxPages8 / 32];
 #pragma unroll
-        for (int r = 0; r < kMaxPages8 / 32; ++r) key[r] = page_key(32 * r + lane);
-        n_pages = warp_topk<kMaxPages8 / 32>(key, p.M, keep);
+          for (int r = 0; r < kMaxPages8 / 32; ++r) key[r] = page_key(32 * r + lane);
+          n_pages = warp_topk<kMaxPages8 / 32>(key, p.M, keep);
+        }
       }
     } else {
       n_pages = n_elig;   // the host guarantees that they fit
-      if (lane < n_pages) pages[lane] = p0 + lane;
+      if (part == 0 && lane < n_pages) pages[lane] = p0 + lane;
     }
-    __syncwarp();
+    if (kWpq > 1 && threadIdx.x == 0) n_kept = n_pages;
+    meet();
+    if constexpr (kWpq > 1) n_pages = n_kept;
 
     // ---- a3: tokens of the kept pages; a group of 32 slots lies in one page
     const int n_slots = n_pages << p_shift;
     const uint8_t* kg = reinterpret_cast<const uint8_t*>(p.k_idx);
     auto group_pos = [&](int c) -> int64_t { return (static_cast<int64_t>(pages[c >> p_shift]) << p_shift) + (c & (p.P - 1)); };
-    uint32_t* sk = keys[warp];   // (a rolled loop cannot index registers: the keys pass through shared memory)
+    uint32_t* sk = keys[own];   // (a rolled loop cannot index registers: the keys pass through shared memory)
     uint4 a[2][4][2];
     auto load_group = [&](uint4 (&to)[4][2], int64_t pos) { load_32rows(to, kg + pos * kRow8, static_cast<int>(min64(31, p.n_key - 1 - pos))); };
-    load_group(a[0], group_pos(0));
-    for (int c = 0; c < n_slots; c += 64) {   // (a page has 64 tokens at least)
+    if (64 * part < n_slots) load_group(a[0], group_pos(64 * part));
+    for (int c = 64 * part; c < n_slots; c += 64 * kWpq) {   // (a page has 64 tokens at least)
       const int64_t pos = group_pos(c);
       load_group(a[1], pos + 32);
       float v = score_32rows(h, a[0]);
       sk[c + lane] = pos + lane >= lo && pos + lane <= hi ? score_key(v) : 0u;
-      if (c + 64 < n_slots) load_group(a[0], group_pos(c + 64));
+      if (c + 64 * kWpq < n_slots) load_group(a[0], group_pos(c + 64 * kWpq));
       v = score_32rows(h, a[1]);
       sk[c + 32 + lane] = pos + 32 + lane >= lo && pos + 32 + lane <= hi ? score_key(v) : 0u;
     }
-    __syncwarp();
+    meet();
+    if (part != 0) return;   // (nothing below waits for other warps)
     uint32_t key[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) key[r] = 32 * r < n_slots ? sk[32 * r + lane] : 0u;
@@ -201,6 +221,7 @@ __global__ void __launch_bounds__(32 * kWarps8) index8_kernel(IndexArgs p) {
     if (out_pages)   // (without the hierarchy a query has every eligible page, which may be more than the list holds)
       for (int i = lane; i < min(n_pages, p.M); i += 32) out_pages[i] = pages[i];
   }
+  if (part != 0) return;
   for (int i = n_sel + lane; i < p.Ksp; i += 32) out_idx[i] = -1;
   if (out_pages)
     for (int i = n_pages + lane; i < p.M; i += 32) out_pages[i] = -1;
@@ -209,21 +230,49 @@ __global__ void __launch_bounds__(32 * kWarps8) index8_kernel(IndexArgs p) {
 
 }  // namespace
 
-// Contiguous bf16 caches, mean pooling, at most 1024 candidates and 1024 pages a query, and sub-blocks few enough that a
-// warp that scores all of its query's is not what the launch waits for.  Longer caches: the coarse stage as a kernel of its
-// own, whose blocks score a tile of mean keys against 32 queries.
+// Contiguous bf16 caches, mean pooling, at most 1024 candidates, 1024 pages and 8192 mean keys a query.  Longer caches: the
+// coarse stage as a kernel of its own, whose blocks score a tile of mean keys against 32 queries (4096 queries, 16384 mean
+// keys: 812 us so, 850 here; 8192: 486 and 431).  Not a matter of the number of queries: a chunk gives the rows of the whole run.
 bool index8_supported(const IndexArgs& a) {
   if (a.HI != kHI8 || a.DI != kDI8 || a.paged || a.key_e4m3) return false;
   const int64_t pages = (a.n_key + a.P - 1) / a.P, slots = a.hi_enable ? static_cast<int64_t>(a.M) * a.P : pages * a.P;
-  return slots <= kMaxSlots8 && pages <= kMaxPages8;
+  return slots <= kMaxSlots8 && pages <= kMaxPages8 && (!a.hi_enable || a.n_key <= static_cast<int64_t>(kMaxMeans8) * a.B);
 }
+
+namespace {
+
+// Warps per query: the count with the smallest estimate, in hundredths of a microsecond: a selection's 9 us and 0.019 us per
+// mean key and token of a warp's share, in waves of 16 warps per SM.
+int warps_per_query(const IndexArgs& a) {
+  const int64_t pages = (a.n_key + a.P - 1) / a.P, slots = a.hi_enable ? static_cast<int64_t>(a.M) * a.P : pages * a.P;
+  const int64_t rows = slots + (a.hi_enable && pages > a.M ? min64(a.n_key, a.q_pos0 + a.n_query) / a.B : 0);
+  const int64_t at_once = 16 * static_cast<int64_t>(a.sm_count > 0 ? a.sm_count : 148);
+  int best = 1;
+  int64_t best_cost = 0;
+  for (int w : {1, 4, 16}) {
+    const int64_t cost = (a.n_query * static_cast<int64_t>(w) + at_once - 1) / at_once * (900 + 2 * rows / w);
+    if (w == 1 || cost < best_cost) {
+      best = w;
+      best_cost = cost;
+    }
+  }
+  return best;
+}
+
+template <int kWpq>
+cudaError_t launch8(const IndexArgs& a, cudaStream_t st) {
+  const int64_t slots = a.hi_enable ? static_cast<int64_t>(a.M) * a.P : (a.n_key + a.P - 1) / a.P * a.P;
+  const int queries = kWpq > 1 ? 1 : kWarps8, warps = kWpq > 1 ? kWpq : kWarps8;
+  return launch_pdl(slots <= kMaxSlots8 / 2 ? index8_kernel<kMaxSlots8 / 64, kWpq> : index8_kernel<kMaxSlots8 / 32, kWpq>,
+                    dim3(static_cast<unsigned>((a.n_query + queries - 1) / queries)), dim3(32 * warps), 0, st, a);
+}
+
+}  // namespace
 
 cudaError_t launch_index8(const IndexArgs& a, cudaStream_t st, int64_t* n_launch) {
   if (a.n_query == 0) return cudaSuccess;
-  const int64_t pages = (a.n_key + a.P - 1) / a.P, slots = a.hi_enable ? static_cast<int64_t>(a.M) * a.P : pages * a.P;
-  const unsigned blocks = static_cast<unsigned>((a.n_query + kWarps8 - 1) / kWarps8);
-  const cudaError_t e = launch_pdl(slots <= kMaxSlots8 / 2 ? index8_kernel<kMaxSlots8 / 64> : index8_kernel<kMaxSlots8 / 32>, dim3(blocks),
-                                   dim3(32 * kWarps8), 0, st, a);
+  const int w = warps_per_query(a);
+  const cudaError_t e = w == 1 ? launch8<1>(a, st) : w == 4 ? launch8<4>(a, st) : launch8<16>(a, st);
   ++*n_launch;
   return e;
 }

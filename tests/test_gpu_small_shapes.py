@@ -38,6 +38,26 @@ def test_small_prefill(cuda_device, change):
     m.assert_ok(pu.TOL_BF16)
 
 
+@pytest.mark.parametrize("change", [dict(L=6000), dict(L=6000, M=16, Ksp=700), dict(L=20000, P=128, M=8), dict(L=9000, P=256, M=4, B=8),
+                                    dict(L=1000, hi_enable=False, Ksp=400), dict(L=40, W=4)])
+def test_chunks_give_the_lists_of_the_whole_run(cuda_device, change):
+    """The indexer's lists do not depend on how many queries a call has (one, four or sixteen warps per query)."""
+    cfg = SMALL.replace(**{"name": "chunks", "seed": 8, "R": 1, **change})
+
+    def lists(n_query):
+        wl = PrefillWorkload(cfg, cuda_device, q_pos0=cfg.L - n_query, n_query=n_query)
+        wl.prepare()
+        pages = torch.empty((n_query, cfg.M), dtype=torch.int32, device=cuda_device)
+        wl.index(pages_out=pages)
+        assert wl.ctx.status() == 0
+        return wl.sparse_idx, wl.n_sparse, pages
+
+    whole = lists(cfg.L)
+    for n_query in (1, 17, 140, 149, 500, 600, 1300):
+        if n_query < cfg.L:
+            assert all(torch.equal(a, b[-n_query:]) for a, b in zip(lists(n_query), whole)), n_query
+
+
 @pytest.mark.parametrize("batch,split", [(1, 0), (3, 2), (5, 3), (130, 1)])
 def test_small_paged_decode(cuda_device, batch, split):
     cfg = SMALL.replace(name="small_dec", mode="decode", batch=batch, ctx_lo=1, ctx_hi=3000, kv_page=64, R=1, seed=batch)
