@@ -68,3 +68,23 @@ def test_prompt(cuda_device, kind, L, P, M, Ksp):
         got, n, gp = pu.to_np(wl.sparse_idx[t]), int(wl.n_sparse[t]), pu.to_np(pages[t])
         assert list(gp[gp >= 0]) == list(want_pages), t
         assert n == len(want) and list(got[:n]) == list(want) and (got[n:] == -1).all(), t
+
+
+@pytest.mark.parametrize("kind", ["few", "plain"])
+@pytest.mark.parametrize("pages", [1023, 1024, 1025, 1100])
+def test_pages_of_long_contexts(cuda_device, kind, pages):
+    """Pages of 128 tokens on either side of the count where their selection changes hands (page 0 holds the sink, the last one the window)."""
+    cfg = CONFIGS["cfg4"].replace(batch=2, ctx_lo=pages * 128 + 130, ctx_hi=pages * 128 + 130, key_dtype="bf16", R=1, M=8, P=128, kv_page=128, W=130,
+                                  Ksp=256, seed=pages, H=16, d_qk=128, d_v=128, mla=False)
+    wl = DecodeWorkload(cfg, cuda_device)
+    _whole_numbers(wl, kind, pages)
+    wl.prepare()
+    listed = torch.empty((cfg.batch, cfg.M), dtype=torch.int32, device=cuda_device)
+    for knob in (0, 2):
+        wl.ctx.tune(5, knob)       # LSA_TUNE_FINE_PAGED_TC
+        wl.index(pages_out=listed)
+        assert wl.ctx.status() == 0
+        caches, t = pu.decode_caches(wl, 1)
+        want, want_pages = ref.select_query(t, pu.to_np(wl.q_idx[1]), pu.to_np(wl.w[1]), caches, P=cfg.P, B=cfg.B, M=cfg.M, Ksp=cfg.Ksp, S=cfg.S, W=cfg.W)
+        assert list(pu.to_np(listed[1])) == list(want_pages)
+        assert list(pu.to_np(wl.sparse_idx[1]))[:len(want)] == list(want)
