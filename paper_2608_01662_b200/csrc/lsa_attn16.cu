@@ -1,8 +1,9 @@
 // a6 for the 16-head, 128-dim shape (separate K and V rows): sparse attention (Eq. 3) without shared-memory tiles.
 //
 // A warp walks 16 keys at a time: S = Q K^T and O += P V as m16n8k16 MMAs (the 16 heads are the M rows) with an online
-// softmax of its own, so warps never wait for one another; 4 warps share a query (every fourth tile each) and merge their
-// parts once at the end, or, when there are enough queries to fill the GPU twice over, each has a query to itself.
+// softmax of its own, so warps never wait for one another; 8 or 4 warps share a query (every eighth or fourth tile each) and merge
+// their parts once at the end, or, when there are enough queries, each has a query to itself.  (A query's result depends on that
+// split as far as bf16 weights against another running maximum do: 2e-3 of its norm between a chunk and the whole run.)
 //
 // Cache rows go from global memory straight to MMA operands.  The sum over dims may run in any order, so a thread takes
 // the 16-byte chunks that suit its loads: dims 32 j + 8 t .. + 7 (t = lane % 4) of a key are its B operands of k-steps
@@ -12,7 +13,7 @@
 //
 // What bounds it: the rows from L2 (512 bytes per attended key) and their latency; the next tile's K and V are in flight
 // while this one is worked on (64 registers).  The form before, one block of 8 warps per query around shared 64-key tiles,
-// spent its time on four block barriers per tile: 2048 queries x 388 rows took 100 us there and 69 us here, 16384 queries
+// spent its time on four block barriers per tile: 2048 queries x 388 rows took 100 us there and 65 us here, 16384 queries
 // 836 and 510 us (a limit of 168 registers, for half as many warps again, spills: 89 and 676 us).
 #include "lsa_internal.h"
 #include "lsa_common.cuh"
@@ -22,28 +23,31 @@ namespace lsa {
 namespace {
 
 constexpr int kH16 = 16, kD16 = 128;
-constexpr int kWarps16 = 4;
+constexpr int kWarps16 = 4, kManyWarps16 = 8;
 constexpr int kKeys16 = 16;                  // keys of a tile
 constexpr int kPitch16 = kD16 + 4;           // floats of a staged row
 constexpr float kLog2e16 = 1.4426950408889634f;
 
-struct Attn16Smem {
-  float o[kWarps16][kH16][kPitch16];
-  float m[kWarps16][kH16], l[kWarps16][kH16];
-};
-
-// kWpq: warps that share a query (1 or 4).  Grid: (ceil(n_query / (4 / kWpq)), n_split).
 template <int kWpq>
-__global__ void __launch_bounds__(32 * kWarps16, 2) sparse_attn16_kernel(AttnArgs p) {
-  constexpr int kQueries = kWarps16 / kWpq;
-  __shared__ __align__(16) uint8_t smem_raw[kWpq > 1 ? sizeof(Attn16Smem) : 16];
+struct Attn16Smem {
+  float o[kWpq][kH16][kPitch16];
+  float m[kWpq][kH16], l[kWpq][kH16];
+};
+template <>
+struct Attn16Smem<1> {};
+
+// kWpq: warps that share a query (1, 4 or 8).  Grid: (ceil(n_query / (kWpq > 1 ? 1 : 4)), n_split).
+template <int kWpq>
+__global__ void __launch_bounds__(32 * (kWpq > 1 ? kWpq : kWarps16), kWpq > kWarps16 ? 1 : 2) sparse_attn16_kernel(AttnArgs p) {
+  constexpr int kQueries = kWpq > 1 ? 1 : kWarps16;
+  extern __shared__ __align__(16) uint8_t smem_raw[];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int g = lane >> 2, t = lane & 3;
   // late queries attend the most rows: they go first
-  const int slot = static_cast<int>(blockIdx.x) * kQueries + warp / kWpq, split = blockIdx.y;
+  const int slot = static_cast<int>(blockIdx.x) * kQueries + (kWpq > 1 ? 0 : warp), split = blockIdx.y;
   const int qi = p.n_query - 1 - slot;
   if (qi < 0) return;   // (kWpq = 1 only: whole warps, and nothing below waits for other warps then)
-  const int part = warp % kWpq;
+  const int part = kWpq > 1 ? warp : 0;
 
   pdl_wait();                 // the index set may come from the previous kernel of the stream
   pdl_launch_dependents();
@@ -195,22 +199,21 @@ __global__ void __launch_bounds__(32 * kWarps16, 2) sparse_attn16_kernel(AttnArg
     l_run[r] += __shfl_xor_sync(0xffffffffu, l_run[r], 2);
   }
 
-  // ---- results: 16 consecutive dims of a head, or of a part that launch_merge puts together (normalised fp32, log2 lse)
-  auto finish = [&](int head, int dim, const float (&x)[16], float inv, float lse2, bool writes_lse) {
+  // ---- results: kDims consecutive dims of a head, or of a part that launch_merge puts together (normalised fp32, log2 lse)
+  constexpr int kDims = kWpq > 1 ? kH16 * kD16 / (32 * kWpq) : 16;
+  auto finish = [&](int head, int dim, const float (&x)[kDims], float inv, float lse2, bool writes_lse) {
     if (p.n_split == 1) {
-      uint4 w[2];
-      uint32_t* u = reinterpret_cast<uint32_t*>(w);
-#pragma unroll
-      for (int i = 0; i < 8; ++i) u[i] = pack_bf16(x[2 * i] * inv, x[2 * i + 1] * inv);
       uint4* dst = reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(p.out) + (static_cast<int64_t>(qi) * kH16 + head) * kD16 + dim);
-      dst[0] = w[0];
-      dst[1] = w[1];
+#pragma unroll
+      for (int i = 0; i < kDims; i += 8)
+        dst[i / 8] = make_uint4(pack_bf16(x[i] * inv, x[i + 1] * inv), pack_bf16(x[i + 2] * inv, x[i + 3] * inv),
+                                pack_bf16(x[i + 4] * inv, x[i + 5] * inv), pack_bf16(x[i + 6] * inv, x[i + 7] * inv));
       if (writes_lse && p.lse != nullptr) p.lse[static_cast<int64_t>(qi) * kH16 + head] = lse2 / kLog2e16;
     } else {
       const int64_t row = (static_cast<int64_t>(qi) * p.n_split + split) * kH16 + head;
       float4* dst = reinterpret_cast<float4*>(p.part_out + row * kD16 + dim);
 #pragma unroll
-      for (int i = 0; i < 4; ++i) dst[i] = make_float4(x[4 * i] * inv, x[4 * i + 1] * inv, x[4 * i + 2] * inv, x[4 * i + 3] * inv);
+      for (int i = 0; i < kDims / 4; ++i) dst[i] = make_float4(x[4 * i] * inv, x[4 * i + 1] * inv, x[4 * i + 2] * inv, x[4 * i + 3] * inv);
       if (writes_lse) p.part_lse[row] = lse2;
     }
   };
@@ -231,7 +234,7 @@ __global__ void __launch_bounds__(32 * kWarps16, 2) sparse_attn16_kernel(AttnArg
       }
     }
   } else {
-    Attn16Smem& sm = *reinterpret_cast<Attn16Smem*>(smem_raw);
+    auto& sm = *reinterpret_cast<Attn16Smem<kWpq>*>(smem_raw);
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
       const int head = g + 8 * r;
@@ -250,40 +253,50 @@ __global__ void __launch_bounds__(32 * kWarps16, 2) sparse_attn16_kernel(AttnArg
       }
     }
     __syncthreads();
-    const int head = tid >> 3, dim = (tid & 7) * 16;
-    float m = -INFINITY, den = 0.f, x[16];
+    constexpr int kPerHead = kD16 / kDims;   // threads
+    const int head = tid / kPerHead, dim = (tid % kPerHead) * kDims;
+    float m = -INFINITY, den = 0.f, x[kDims];
 #pragma unroll
-    for (int i = 0; i < 16; ++i) x[i] = 0.f;
+    for (int i = 0; i < kDims; ++i) x[i] = 0.f;
 #pragma unroll
-    for (int w = 0; w < kWarps16; ++w) m = fmaxf(m, sm.m[w][head]);
+    for (int w = 0; w < kWpq; ++w) m = fmaxf(m, sm.m[w][head]);
 #pragma unroll
-    for (int w = 0; w < kWarps16; ++w) {
+    for (int w = 0; w < kWpq; ++w) {
       const float wgt = sm.m[w][head] > -INFINITY ? exp2f(sm.m[w][head] - m) : 0.f;   // (a warp without a tile)
       den += wgt * sm.l[w][head];
       const float4* src = reinterpret_cast<const float4*>(&sm.o[w][head][dim]);
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
+      for (int i = 0; i < kDims / 4; ++i) {
         const float4 v = src[i];
         x[4 * i] += wgt * v.x; x[4 * i + 1] += wgt * v.y; x[4 * i + 2] += wgt * v.z; x[4 * i + 3] += wgt * v.w;
       }
     }
-    finish(head, dim, x, den > 0.f ? 1.f / den : 0.f, den != 0.f ? m + log2f(den) : -INFINITY, (tid & 7) == 0);
+    finish(head, dim, x, den > 0.f ? 1.f / den : 0.f, den != 0.f ? m + log2f(den) : -INFINITY, tid % kPerHead == 0);
   }
 }
 
-// From this many queries (times row splits) on a warp takes a query to itself: two blocks on each of 148 SMs.  (2048
-// queries: 69 us so, 86 us with four warps a query; 64 queries take 12.6 us with four.)
-constexpr int kWholeWarpQueries = 1184;
+template <int kWpq>
+cudaError_t launch_t(const AttnArgs& a, cudaStream_t st) {
+  const size_t smem = kWpq > 1 ? sizeof(Attn16Smem<kWpq>) : 0;
+  if (smem > 48 * 1024) {
+    const cudaError_t e = cudaFuncSetAttribute(sparse_attn16_kernel<kWpq>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    if (e != cudaSuccess) return e;
+  }
+  const int queries = kWpq > 1 ? 1 : kWarps16, warps = kWpq > 1 ? kWpq : kWarps16;
+  return launch_pdl(sparse_attn16_kernel<kWpq>, dim3((a.n_query + queries - 1) / queries, a.n_split), dim3(32 * warps), smem, st, a);
+}
 
 }  // namespace
 
+// Warps per query: eight while every query (times row splits) has an SM to itself; one from the count on where four would take a
+// third wave of two blocks per SM, a fourth where there are more rows.  (us with a cold L2, one / four / eight warps: 388 rows, 148
+// queries 43/21/16, 296 43/21/25, 592 41/35/43, 700 43/47/50, 2048 78/100/127; 1540 rows, 148 queries 123/49/31, 592 121/90/96, 800
+// 127/123/135, 1000 131/158/158, 2048 242/277/303.)
 cudaError_t launch_attn16(const AttnArgs& a, cudaStream_t st, int64_t* n_launch) {
   if (a.n_query == 0) return cudaSuccess;
-  cudaError_t e;
-  if (static_cast<int64_t>(a.n_query) * a.n_split >= kWholeWarpQueries)
-    e = launch_pdl(sparse_attn16_kernel<1>, dim3((a.n_query + kWarps16 - 1) / kWarps16, a.n_split), dim3(32 * kWarps16), 0, st, a);
-  else
-    e = launch_pdl(sparse_attn16_kernel<kWarps16>, dim3(a.n_query, a.n_split), dim3(32 * kWarps16), 0, st, a);
+  const int64_t jobs = static_cast<int64_t>(a.n_query) * a.n_split, sms = a.sm_count > 0 ? a.sm_count : 148;
+  const int rows = a.rows_ld / a.n_split;
+  const cudaError_t e = jobs <= sms ? launch_t<kManyWarps16>(a, st) : jobs <= (rows <= 1024 ? 4 : 6) * sms ? launch_t<kWarps16>(a, st) : launch_t<1>(a, st);
   ++*n_launch;
   return e;
 }

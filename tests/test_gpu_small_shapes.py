@@ -69,3 +69,17 @@ def test_small_paged_decode(cuda_device, batch, split):
     m = pu.check_decode(wl, range(min(batch, 12)))
     print(batch, split, m.summary())
     m.assert_ok(pu.TOL_BF16)
+
+
+@pytest.mark.parametrize("W,Ksp,M", [(64, 64, 4), (1024, 512, 16)])
+@pytest.mark.parametrize("n_query", [1, 148, 149, 592, 593, 889])
+def test_attention_of_few_queries(cuda_device, n_query, W, Ksp, M):
+    """One, four and eight warps per query, at the counts where they change hands on 148 SMs (592 and 888 with few and many rows)."""
+    cfg = SMALL.replace(name="few", L=3000, W=W, Ksp=Ksp, M=M, seed=n_query)
+    wl = PrefillWorkload(cfg, cuda_device, q_pos0=cfg.L - n_query, n_query=n_query)
+    wl.prepare()
+    wl.step()
+    assert wl.ctx.status() == 0
+    m = pu.check_prefill(wl, range(wl.q_pos0, cfg.L, max(1, n_query // 10)))
+    print(n_query, W, m.summary())
+    m.assert_ok(pu.TOL_BF16)
