@@ -30,7 +30,7 @@ constexpr int kGroupBytesB = 2 * kAtomBytesB;
 constexpr int kEpiWarps = 16;               // 4 per TMEM lane quarter: one per query of the group
 constexpr int kThreadsTc = 32 * (2 + kEpiWarps);
 constexpr uint32_t kTmemCols = 512;
-constexpr int kSmCount = 148, kFullWaves = 10;   // launches of fewer waves are cut into more blocks ...
+constexpr int kFullWaves = 10;                    // launches of fewer waves are cut into more blocks ...
 constexpr int kMinTilesOfPart = 16;               // ... of this many tiles at least
 
 template <int NG>
@@ -338,8 +338,9 @@ cudaError_t launch_tc(const IndexArgs& a, cudaStream_t st, int64_t* n_launch) {
   // One block per SM, and a block's time is its tiles': with few query blocks the last wave is mostly empty (512 blocks of
   // 4096 queries against a million keys: 3.5 waves, 8.4 ms; in four parts each 13.8 waves, 7.7 ms).
   const int64_t tiles = (a.q_pos0 + a.n_query - a.W) / (static_cast<int64_t>(kTileM) * a.B) + 1;
+  const int sms = a.sm_count > 0 ? a.sm_count : 148;
   int parts = 1;
-  while (parts < 8 && static_cast<int64_t>(blocks) * parts < kFullWaves * kSmCount && tiles / (2 * parts) >= kMinTilesOfPart) parts *= 2;
+  while (parts < 8 && static_cast<int64_t>(blocks) * parts < kFullWaves * sms && tiles / (2 * parts) >= kMinTilesOfPart) parts *= 2;
   e = launch_pdl(kernel, dim3(blocks * parts), dim3(kThreadsTc), smem, st, map_q, map_km, parts, a);
   ++*n_launch;
   return e;

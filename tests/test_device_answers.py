@@ -18,3 +18,13 @@ def test_no_answer_about_a_device_is_kept_in_a_static():
         for m in re.finditer(r"\bstatic\b[^;{(]*(?:=|\{|\[)[^;]*;", text):   # a static with an initialiser
             assert not re.search(ASKS, m.group(0)), (name, m.group(0)[:120])
     assert asked >= 4
+
+
+def test_no_rule_names_the_sms_of_one_chip():
+    """148 stands only where a call has no device's count to go by."""
+    for name in sorted(os.listdir(CSRC)):
+        if name.endswith((".cu", ".cuh", ".h")):
+            with open(os.path.join(CSRC, name)) as f:
+                code = re.sub(r"//[^\n]*", "", f.read())
+            for line in code.split("\n"):
+                assert not re.search(r"\b(148|1184|296)\b", line) or re.search(r"\? [\w.]+ : 148\b|return 148;|n = 148;", line), (name, line)
