@@ -504,9 +504,11 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
           for (int u = lane; u < kRowsPerWarp / 4 * kAtoms; u += 32) {
             const int q4 = u / kAtoms, atom = u % kAtoms;
             int4 r;
-            // rows past the end of the list are masked in the softmax: any readable row will do
+            // past the end of the list its last row once more: masked in the softmax, and as a value of weight 0 it must not be
+            // somebody else's (0 x NaN)
             const int i0 = (jb.tile_begin + i) * kTileKeys + kRowsPerWarp * gw + 4 * q4;
-            r.x = max(row_of(i0), 0); r.y = max(row_of(i0 + 1), 0); r.z = max(row_of(i0 + 2), 0); r.w = max(row_of(i0 + 3), 0);
+            auto listed = [&](int k) -> int32_t { return max(row_of(min(k, jb.n_tot - 1)), 0); };
+            r.x = listed(i0); r.y = listed(i0 + 1); r.z = listed(i0 + 2); r.w = listed(i0 + 3);
             tc::tma_gather4_2d(smem_u32(sm.k[grp][atom]) + (kRowsPerWarp * gw + 4 * q4) * 128, &g_map, atom * 64, r.x, r.y, r.z, r.w, full);
           }
         } else {

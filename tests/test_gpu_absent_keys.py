@@ -14,12 +14,14 @@ import parity_util as pu
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("base,batch,split", [("cfg1", 1, 0), ("cfg1", 9, 0), ("cfg1", 9, 1), ("cfg1", 200, 0), ("cfg4", 1, 0), ("cfg4", 9, 0), ("cfg4", 160, 0)])
-def test_rows_of_nobody_in_a_pool(cuda_device, base, batch, split):
+@pytest.mark.parametrize("base,batch,split,gather", [("cfg1", 1, 0, 0), ("cfg1", 9, 0, 0), ("cfg1", 9, 1, 0), ("cfg1", 200, 0, 0), ("cfg4", 1, 0, 0),
+                                                     ("cfg4", 9, 0, 0), ("cfg4", 160, 0, 0), ("cfg4", 9, 0, 1), ("cfg4", 160, 0, 1)])
+def test_rows_of_nobody_in_a_pool(cuda_device, base, batch, split, gather):
     cfg = CONFIGS[base].replace(name="nobody", mode="decode", batch=batch, ctx_lo=1, ctx_hi=700, kv_page=64, R=1, M=4, Ksp=64, W=100, seed=batch)
     wl = DecodeWorkload(cfg, cuda_device)
     wl.prepare()
     wl.ctx.tune(2, split)          # LSA_TUNE_ATTN_SPLIT
+    wl.ctx.tune(4, gather)         # LSA_TUNE_ATTN_GATHER
     # a page of nobody in front of the pool: no sequence has row 0
     front = lambda t, rows: torch.cat([torch.zeros_like(t[:rows]), t])  # noqa: E731
     wl.page_table = torch.where(wl.page_table >= 0, wl.page_table + 1, -1)
