@@ -70,7 +70,7 @@ struct FpSmem {
   alignas(1024) uint8_t q[kQBytes];
   float k_scale[E4M3 ? kMaxPagesFp / 2 : 1][kTile];   // per-token scales of the block's tiles (e4m3); a thread reads what it wrote
   float w[kHI];
-  uint32_t keys[kMaxSlotsFp];   // candidate keys of the whole cluster (used in the first block only)
+  alignas(16) uint32_t keys[kMaxSlotsFp];   // candidate keys of the whole cluster (used in the first block only)
   int32_t pages[kMaxPagesFp];   // kept pages, ascending
   int32_t phys[kMaxPagesFp];    // their places in the pool
   SelectScratch sel;

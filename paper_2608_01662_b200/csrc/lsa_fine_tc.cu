@@ -36,7 +36,7 @@ struct FineTcSmem {
   alignas(1024) uint8_t q[2][kAtomQ];      // [column block][64 rows x 128 B]
   float w[kHI];
   float scale[4][kTile];   // four deep: a tile's scales are read by the epilogue after its key buffer is already free
-  uint32_t keys[kMaxSlotsTc];
+  alignas(16) uint32_t keys[kMaxSlotsTc];
   int32_t pages[kMaxPagesTc];
   SelectScratch sel;
   alignas(8) uint64_t k_full[2], k_empty[2], acc_full[2], acc_empty[2];

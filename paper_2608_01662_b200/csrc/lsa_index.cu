@@ -378,7 +378,7 @@ struct FineSmem {
   alignas(128) uint8_t a[2][kTileRows * DI * 2];
   alignas(128) uint8_t q[HI * DI * 2];
   float w[HI];
-  uint32_t keys[kMaxSlots];
+  alignas(16) uint32_t keys[kMaxSlots];
   float scale[2][kTileRows];   // per-token key scales of the tile in flight (e4m3 keys)
   int32_t pages[kMaxPages];
   int32_t phys[kMaxPages];     // where each selected page lives in the cache (page-table entry; the page itself when contiguous)
@@ -590,7 +590,7 @@ __global__ void __launch_bounds__(kThreads, 2) fine_select_kernel(IndexArgs p) {
 // the pages of sequence qi that survive the coarse stage (Eq. 10), ascending, into fine_pages[qi], their count last.
 // A sequence without candidates gets its (empty) results here.
 __global__ void __launch_bounds__(kSelThreads) page_topm_paged_kernel(IndexArgs p) {
-  __shared__ uint32_t keys[kMaxSlots];
+  __shared__ alignas(16) uint32_t keys[kMaxSlots];
   __shared__ int32_t pages[kMaxPages];
   __shared__ SelectScratch sc;
   const int qi = blockIdx.x, tid = threadIdx.x;
@@ -641,7 +641,7 @@ __global__ void __launch_bounds__(kSelThreads) page_topm_paged_kernel(IndexArgs 
 
 // Second half of the split fine stage: top-K_sparse over the keys the scoring blocks left in global memory.
 __global__ void __launch_bounds__(kSelThreads) fine_topk_kernel(IndexArgs p) {
-  __shared__ uint32_t keys[kMaxSlots];
+  __shared__ alignas(16) uint32_t keys[kMaxSlots];
   __shared__ int32_t pages[kMaxPages];
   __shared__ SelectScratch sc;
   const int qi = blockIdx.x, tid = threadIdx.x;

@@ -43,7 +43,7 @@ constexpr uint32_t kShortHist = 0, kShortWarp = 4 * kShortBins, kShortFound = kS
 constexpr uint32_t kShortScratch = kShortMembers + 128;
 static_assert(kShortScratch <= sizeof(SelectScratch), "the scratch of the radix select serves this one too");
 
-// keys: shared address of n <= kShortMax keys.  list: shared address where the selected indices go, ascending, 16 bits each (it
+// keys: shared address of n <= kShortMax keys, 16-byte aligned, with room for 16 per thread (all of it is read).  list: shared address where the selected indices go, ascending, 16 bits each (it
 // may be `keys`: they are in registers by then).  scratch: shared address of kShortScratch bytes, 16-byte aligned.  Every one of
 // the 256 threads calls it, converged; the keys must be visible to all of them.  Returns the number selected, min(k, #present),
 // with the list visible.  They are threads 0-255 of the block and meet on barrier `bar`; short_select_warm calls it otherwise.
