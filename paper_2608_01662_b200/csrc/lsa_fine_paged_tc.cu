@@ -130,7 +130,7 @@ __device__ __forceinline__ void finish_sequence(const IndexArgs& p, const uint32
     for (int j = tid - kSelThreads; j < n_sink + n_win; j += kThreadsFp - kSelThreads) tail[j] = tail_row(j);
   if (tid < kSelThreads) {
     int32_t* out_idx = p.sparse_idx + static_cast<int64_t>(qi) * p.Ksp;
-    const int n_sel = short_select<kSelBar>(smem_u32(keys), n_slots, p.Ksp, smem_u32(keys), smem_u32(&sel));
+    const int n_sel = n_slots > 0 ? short_select<kSelBar>(smem_u32(keys), n_slots, p.Ksp, smem_u32(keys), smem_u32(&sel)) : 0;
     for (int r0 = tid; r0 < p.Ksp; r0 += 4 * kSelThreads) {   // four rows in flight per thread
       int pos[4], row[4];
 #pragma unroll
@@ -174,6 +174,10 @@ fine_paged_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
   const uint32_t rank = cluster_rank(), n_rank = cluster_size();
   // The cluster barrier has no time limit: every path below reaches both of its phases, also after a failed wait.
   cluster_arrive();   // phase 1: "this block runs" (its shared memory may be written from now on)
+  // Whether the sequence is likely to be longer than its window (the kernel before may still add a token: this decides nothing but
+  // whether the selection's instructions are fetched ahead).
+  bool selects = false;
+  if (warp == kWarmWarp) selects = __any_sync(0xffffffffu, *reinterpret_cast<const volatile int32_t*>(p.ctx_len + qi) > p.S + p.W);
   const bool live = !tc::block_gives_up(p.status);
 
   if (tid == 0) {
@@ -197,7 +201,7 @@ fine_paged_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
     tc::tmem_alloc(smem_u32(&sm.tmem_slot), kTmemColsFp);
     tc::tmem_relinquish();
   }
-  if (warp == kWarmWarp) {
+  if (selects) {
     short_select_warm<kWarmBar>(smem_u32(sm.k) + kMaxSlotsFp * 4);   // behind the page scores' keys
     tc::fence_proxy_async();   // (that part of the ring is handed to the TMA copies)
   }

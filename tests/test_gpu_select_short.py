@@ -88,3 +88,24 @@ def test_pages_of_long_contexts(cuda_device, kind, pages):
         want, want_pages = ref.select_query(t, pu.to_np(wl.q_idx[1]), pu.to_np(wl.w[1]), caches, P=cfg.P, B=cfg.B, M=cfg.M, Ksp=cfg.Ksp, S=cfg.S, W=cfg.W)
         assert list(pu.to_np(listed[1])) == list(want_pages)
         assert list(pu.to_np(wl.sparse_idx[1]))[:len(want)] == list(want)
+
+
+@pytest.mark.parametrize("kind", ["few", "plain"])
+@pytest.mark.parametrize("M,Ksp", [(3, 100), (9, 4), (64, 612)])
+def test_contexts_about_the_window(cuda_device, kind, M, Ksp):
+    """Sequences inside their window, which select nothing, beside some that do."""
+    cfg = CONFIGS["cfg4"].replace(batch=33, ctx_lo=255, ctx_hi=900, key_dtype="bf16", R=1, M=M, Ksp=Ksp, seed=M + Ksp)
+    wl = DecodeWorkload(cfg, cuda_device)
+    edge = [1, 255, 256, 259, 260, 261, 262, 323, 324]
+    wl.ctx_len[:len(edge)] = torch.minimum(torch.tensor(edge, dtype=torch.int32, device=cuda_device), (wl.page_table[:len(edge)] >= 0).sum(1).int() * 64)
+    _whole_numbers(wl, kind, M)
+    wl.prepare()
+    pages = torch.empty((cfg.batch, M), dtype=torch.int32, device=cuda_device)
+    wl.index(pages_out=pages)
+    assert wl.ctx.status() == 0
+    for b in range(cfg.batch):
+        caches, t = pu.decode_caches(wl, b)
+        want, want_pages = ref.select_query(t, pu.to_np(wl.q_idx[b]), pu.to_np(wl.w[b]), caches, P=cfg.P, B=cfg.B, M=M, Ksp=Ksp, S=cfg.S, W=cfg.W)
+        got, gp, n = pu.to_np(wl.sparse_idx[b]), pu.to_np(pages[b]), int(wl.n_sparse[b])
+        assert list(gp[gp >= 0]) == list(want_pages), (b, t)
+        assert n == len(want) and list(got[:n]) == list(want) and (got[n:] == -1).all(), (b, t)
