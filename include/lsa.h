@@ -216,7 +216,8 @@ LSA_API int lsa_append(lsa_ctx* ctx, const lsa_params* p, const void* k_new, voi
  *                      [batch, page_table_stride] maps logical page -> physical page
  *   sparse_idx  int32 [n_query, Ksp]  ascending positions (logical), padded with -1
  *   n_sparse    int32 [n_query]
- *   pages_out   optional int32 [n_query, M] kept pages ascending, -1 padded (NULL to skip)
+ *   pages_out   optional int32 [n_query, M] kept pages ascending, -1 padded (NULL to skip); with hi_enable = 0 the first M
+ *               eligible ones where the caches are short (<= 4096 tokens), else -1
  * Scratch: the page-score matrix fp32 [n_query, ceil(n_key_max/P)] in the workspace; for e4m3 caches with the
  * 64-head, 128-dim indexer also a bf16 copy of the codes [n_key_max, d_idx] (exact, unscaled), rewritten by every call,
  * from which the fine stage fetches key tiles. */
@@ -280,7 +281,7 @@ LSA_API int lsa_index_static_status(int device, void* cuda_stream, int* device_s
  *   cand_pos  NULL: candidate c is position c;  else int32 [n_query, n_cand] positions, -1 = absent
  *   apply_range 1: only positions inside C(q_pos0+i) (from k_sink, k_swa) take part; 0: all present
  *   idx_out   int32 [n_query, k] ascending positions, -1 padded;  n_out int32 [n_query]
- * n_cand is unlimited (scores are re-read from memory on every radix pass); k <= 8192. */
+ * n_cand < 2^31; k <= 8192. */
 LSA_API int lsa_select(lsa_ctx* ctx, const lsa_params* p, const float* scores, int64_t ld_scores,
                const int32_t* cand_pos, int64_t q_pos0, int64_t n_query, int64_t n_cand, int32_t k,
                int32_t apply_range, int32_t* idx_out, int32_t* n_out);

@@ -891,7 +891,7 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
       // copies still read this block's shared memory).  A thread arrives as soon as it has seen this block's own
       // bytes complete and waits at the very end, by when the peer has normally long arrived.
       cluster_arrive();
-      // A warp finishes rows w, w + 13, w + 26 of this block's 32: lane k works out the k-th row's weights, and a row's parts
+      // A warp finishes rows w and w + 16 of this block's 32: lane k works out the k-th row's weights, and a row's parts
       // (lane l: the 16-byte chunks l, l + 32, ...) are read while the row before is written.
       constexpr int kRowsOfWarp = (kH / 2 + kWarps - 1) / kWarps;
       float4 a[2][4], b[2][4];

@@ -12,7 +12,7 @@
 //               32 boxes of a tile are spread over four warps.  When the block's share crosses into the next sequence,
 //               warp 0 fetches that sequence's query heads (TMA) and head weights into the other of two query slots
 //   warp 1      one thread issues 8 x tcgen05.mma (M128 N64 K16) per tile into one of two TMEM accumulators
-//   warps 2-5   epilogue: one thread = one sub-block row: sum_j w_j relu(acc_j), then the sum over the page's
+//   warps 2-5   epilogue, four threads to four sub-block rows: sum_j w_j relu(acc_j), then the sum over the page's
 //               sub-blocks (Eq. 9) with warp shuffles, page score to global
 #include "lsa_internal.h"
 #include "lsa_tc.cuh"

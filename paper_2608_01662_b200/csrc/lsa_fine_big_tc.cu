@@ -9,8 +9,8 @@
 //                           but the scores go to global memory as order-preserving keys (0 = not a candidate): a block
 //                           covers a run of a query's tiles, several blocks share a query
 //
-//   select_keys_kernel      a4: the exact radix top-K_sparse over each query's keys; a slot's position comes from the page
-//                           list, so only the keys (4 bytes per candidate) travel through memory
+//   select_keys_kernel      a4: the exact top-K_sparse over each query's keys (lsa_select_long.cuh); a slot's position comes
+//                           from the page list, so only the keys (4 bytes per candidate) travel through memory
 #include "lsa_internal.h"
 #include "lsa_select_long.cuh"
 #include "lsa_tc.cuh"

@@ -3,7 +3,7 @@
 // the sequence's cache rows for the attention kernels (streaming-aware conversion).  64-head / 128-dim indexer,
 // 64-token cache pages (a cache page is a selection page), up to 64 kept pages.
 //
-// A sequence is owned by a thread-block cluster of one or two blocks.  Every block of the cluster selects the pages
+// A sequence is owned by a thread-block cluster of up to eight blocks.  Every block of the cluster selects the pages
 // (the same list in each: no exchange needed), takes its share of the list's tiles (two pages = the M = 128 rows of an
 // MMA; the 64 heads are N, d_I = 128 is K) and scores them; the candidate keys of all blocks land in the shared memory
 // of the cluster's first block (remote stores of 4 bytes per token), which takes the top-K and writes the results.
@@ -26,8 +26,8 @@
 //   warps 1-3    one thread of each issues the MMAs of every third tile, alternating between two TMEM accumulators of
 //                its own (one thread issues an MMA about every 95 cycles, the pipe needs 48: three issuers keep it
 //                busy, and nobody waits for the epilogue of a recent tile)
-//   warps 4-7 / 8-11   epilogue of the even / odd tiles: one thread = one token: sum_j w_j relu(acc_j), times the
-//                token's scale, as an order-preserving key into the first block's candidate array
+//   warps 4-7 / 8-11   epilogue of the even / odd tiles: four threads share four tokens, one ends with each: sum_j w_j
+//                relu(acc_j), times the token's scale, as an order-preserving key into the first block's candidate array
 // The query heads are fetched before the dependency wait (they are an input of the call, not a product of the
 // coarse kernel that precedes this one in the stream).
 #include "lsa_internal.h"

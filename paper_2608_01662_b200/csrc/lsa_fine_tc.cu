@@ -9,10 +9,10 @@
 //               tile issued by one thread; without a widened copy the warps gather e4m3 codes and widen them in
 //               registers (exact), the per-token scales riding along
 //   warp 3      one thread issues the MMAs into one of two 64-column TMEM accumulators
-//   warps 4-7   epilogue: tcgen05.ld, sum_j w_j * relu(acc_j) in-thread (one thread = one key), times the key's
-//               scale, range check, order-preserving key into the candidate buffer
+//   warps 4-7   epilogue: tcgen05.ld, sum_j w_j * relu(acc_j) (four threads share four keys, one ends with each), times
+//               the key's scale, range check, order-preserving key into the candidate buffer
 //
-// and the candidate buffer then goes through the exact radix top-K_sparse (Eq. 12) with all eight warps.
+// and the exact top-K_sparse (Eq. 12) of the candidate buffer follows with all eight warps (lsa_select_short.cuh).
 #include "lsa_internal.h"
 #include "lsa_select_short.cuh"
 #include "lsa_tc.cuh"

@@ -426,7 +426,7 @@ __global__ void __launch_bounds__(kThreads, 2) fine_select_kernel(IndexArgs p) {
     const float* ps = p.page_scores + static_cast<int64_t>(qi) * p.ps_ld + p0;
     if (nE <= kMaxSlots) {
       // one pass over the page scores (L2) into the candidate buffer, which is idle until the fine stage;
-      // the six passes of the radix select then run out of shared memory
+      // the passes of the selection then run out of shared memory
       for (int i = tid; i < nE; i += kThreads) sm.keys[i] = score_key(ps[i]);
       __syncthreads();
       LSA_TLF(7);

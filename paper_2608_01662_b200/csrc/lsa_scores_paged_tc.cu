@@ -21,7 +21,7 @@
 //                256-byte bulk copy of the page's per-token scales (e4m3).  An issued copy costs its thread 200-300
 //                cycles, hence two producers
 //   warps 2, 3   one thread of each issues the MMAs of its tiles into accumulator i % 4 of TMEM
-//   warps 4-7 / 8-11   epilogue of the even / odd tiles: one thread = one token: sum_j w_j relu(acc_j), times the
+//   warps 4-7 / 8-11   epilogue of the even / odd tiles, four threads to four tokens: sum_j w_j relu(acc_j), times the
 //                token's scale, out
 //   warps 12-15  the query heads of the share's next sequence into the other of two slots: e5m2 planes built from
 //                the bf16 heads (e4m3 cache) or a TMA load (bf16 cache), and the head weights
