@@ -54,6 +54,7 @@ __global__ void __launch_bounds__(kFineThreads, 2) fine_select_tc_kernel(const _
   const int part = blockIdx.y, n_parts = gridDim.y;
   pdl_wait();
   pdl_launch_dependents();
+  const bool raised = tc::status_raised(p.status);   // an earlier block of this launch gave up on a wait
   int64_t t, n_key;
   const int32_t* pt = nullptr;
   if (p.paged) {
@@ -75,7 +76,6 @@ __global__ void __launch_bounds__(kFineThreads, 2) fine_select_tc_kernel(const _
     if (tid == 0) p.n_sparse[qi] = 0;
     return;
   }
-  if (tc::block_gives_up(p.status)) return;   // an earlier block of this launch gave up on a wait
 
   // query heads (K-major, 128B swizzle) and head weights: asynchronous copies that land during the page selection
   {
@@ -93,11 +93,16 @@ __global__ void __launch_bounds__(kFineThreads, 2) fine_select_tc_kernel(const _
   const int p0 = static_cast<int>(lo / p.P), p1 = static_cast<int>(hi / p.P);
   const int nE = p1 - p0 + 1;
   int nP;
-  if (p.hi_enable && nE > p.M) {
-    const float* ps = p.page_scores + static_cast<int64_t>(qi) * p.ps_ld + p0;
+  const bool scored = p.hi_enable && nE > p.M;
+  const float* ps = p.page_scores + static_cast<int64_t>(qi) * p.ps_ld + p0;
+  if (scored && nE <= kMaxSlotsTc)
+    for (int i = tid; i < nE; i += kFineThreads) sm.keys[i] = score_key(ps[i]);
+  if (__syncthreads_or(raised)) {   // (the page keys are visible; and the block gives up by a vote: see block_gives_up)
+    cp_async_wait<0>();
+    return;
+  }
+  if (scored) {
     if (nE <= kMaxSlotsTc) {
-      for (int i = tid; i < nE; i += kFineThreads) sm.keys[i] = score_key(ps[i]);
-      __syncthreads();
       nP = short_select<0>(smem_u32(sm.keys), nE, p.M, smem_u32(sm.keys), smem_u32(&sm.sel));
       for (int i = tid; i < nP; i += kFineThreads) sm.pages[i] = p0 + short_item(smem_u32(sm.keys), i);
     } else {
