@@ -132,13 +132,13 @@ def attn_bytes_per_launch(cfg, positions):
     return float(rows * cfg.d_qk * 2 + len(positions) * cfg.H * (cfg.d_qk + cfg.d_v) * 2)
 
 
-# DRAM traffic of one attention launch, from the ncu capture of an earlier form of the kernel on cfg3 cut to 16384 queries
-# (profiles/sparse_attn_tc_cfg3_16k.md: dram__bytes_read.sum 1.344671 GB + dram__bytes_write.sum 1.047908 GB).
+# DRAM traffic of one attention launch, from the ncu capture of the same kernel on cfg3 cut to 16384 queries
+# (profiles/attention_and_small_indexer.md: dram__bytes_read.sum 1.344909 GB + dram__bytes_write.sum 1.031480 GB).
 # Traffic there is q + out (the KV latent stays in L2), so it scales with the number of queries of a launch.
-NCU_ATTN_DRAM_BYTES_PER_QUERY = (1.344671e9 + 1.047908e9) / 16384
-# Decode: DRAM bytes of one attention launch per sequence, from the ncu capture of that form at batch 16
-# (profiles/sparse_attn_tc_cfg4_decode_batch16.md: dram__bytes_read.sum 43.95 MB + dram__bytes_write.sum 0.47 MB).
-NCU_DECODE_ATTN_DRAM_BYTES_PER_SEQ = (43949568 + 472832) / 16
+NCU_ATTN_DRAM_BYTES_PER_QUERY = (1.344909e9 + 1.031480e9) / 16384
+# Decode: DRAM bytes of one attention launch per sequence, from the ncu capture at batch 16
+# (profiles/attention_and_small_indexer.md: dram__bytes_read.sum 43.94 MB + dram__bytes_write.sum 0.29 MB).
+NCU_DECODE_ATTN_DRAM_BYTES_PER_SEQ = (43939840 + 291072) / 16
 
 
 def measured_peaks():
@@ -328,7 +328,7 @@ def main():
             roofline = {"kernel": "sparse_attn_tc_kernel" if cfg.H == 64 else "sparse_attn16_kernel", "bound": "tensor", "achieved": a,
                         "peak": peaks["tensor_tflops"], "unit": "TFLOP/s", "frac": a / peaks["tensor_tflops"],
                         "traffic": NCU_ATTN_DRAM_BYTES_PER_QUERY * len(positions) if cfg.H == 64 else None,
-                        "traffic_source": "ncu capture of an earlier form of the kernel at 16384 queries, scaled by queries per launch",
+                        "traffic_source": "ncu capture at 16384 queries, scaled by queries per launch",
                         "algorithmic_bytes": float(len(positions)) * cfg.H * (cfg.d_qk + cfg.d_v) * 2,
                         "peak_source": peaks["source"], "launch_ms": attn_ms / attn_n}
     kernels = {k: {"ms_per_step": v[0] / args.steps, "launches_per_step": v[1] / args.steps}
@@ -406,7 +406,7 @@ def decode_attn_roofline(cfg, prof, launch_us, positions, peaks):
     return with_nominal({"kernel": "sparse_attn_tc_kernel", "bound": "hbm", "achieved": a, "peak": peaks["hbm_gbs"],
                          "unit": "GB/s", "frac": a / peaks["hbm_gbs"],
                          "traffic": NCU_DECODE_ATTN_DRAM_BYTES_PER_SEQ * cfg.batch,
-                         "traffic_source": "ncu capture of an earlier form of the kernel at batch 16, scaled by sequences per launch",
+                         "traffic_source": "ncu capture at batch 16, scaled by sequences per launch",
                          "algorithmic_bytes": bytes_per_launch, "peak_source": peaks["source"], "launch_us": launch_us,
                          "launch_us_in_step": attn_ms / attn_n * 1e3,
                          "timing": "one event pair around 10 x R back-to-back launches, each layer on its own cache"})

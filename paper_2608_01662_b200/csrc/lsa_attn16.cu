@@ -11,10 +11,11 @@
 // 2 t, 2 t + 1, 2 t + 8, 2 t + 9: dim j of two keys packed is its B operand of n-tile (h, j), whose column n then stands for
 // dim 64 h + 8 n + j; a thread ends with 16 consecutive dims of its rows.
 //
-// What bounds it: the rows from L2 (512 bytes per attended key) and their latency; the next tile's K and V are in flight
-// while this one is worked on (64 registers).  The form before, one block of 8 warps per query around shared 64-key tiles,
-// spent its time on four block barriers per tile: 2048 queries x 388 rows took 100 us there and 65 us here, 16384 queries
-// 836 and 510 us (a limit of 168 registers, for half as many warps again, spills: 89 and 676 us).
+// What bounds it: the latency of a warp's own chain (loads, MMAs, softmax), with 8 warps on an SM at 228 registers a thread; the next
+// tile's K and V are in flight while this one is worked on (64 registers).  2048 queries: 56 % of the rows come from L1, the path
+// from L2 is 9 % busy, the tensor pipe 19 %, one issue slot in three is used.  The form before, one block of 8 warps per query
+// around shared 64-key tiles, spent its time on four block barriers per tile: 2048 queries x 388 rows took 100 us there and 65 us
+// here, 16384 queries 836 and 510 us (a limit of 168 registers, for half as many warps again, spills: 89 and 676 us).
 #include "lsa_internal.h"
 #include "lsa_common.cuh"
 
