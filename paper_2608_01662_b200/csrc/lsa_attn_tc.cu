@@ -7,36 +7,44 @@
 // first tiles follow them into the ring, and warps of their own move that Q and write this O, so that the tensor pipe
 // waits between two queries only for O to leave tensor memory.
 //
-//   warps 10-15 gather: two warps per ring slot.  They wait for the slot, copy rows [window | sink | sparse] (or those of the
+//   (warp numbers of the prefill form; struct Warps)
+//   warps 14-22 gather: three warps per ring slot (two where row lists are walked).  They wait for the slot, copy rows [window | sink | sparse] (or those of the
 //               caller's row list) into its 128B-swizzled K-major tile with coalesced 16-byte cp.async, a row by one warp
 //               (spreading a tile's chunks over the warps was measured 1.3 x slower, a TMA gather of four rows per
 //               instruction - AttnArgs::gather4 - as well: the TMA unit takes about 26 cycles for its 512 bytes), and hand
 //               it over when it has landed; tiles of 64 consecutive window rows and Q come as one TMA box each.
-//   warps 4-7   the ends of a job: they move Q to tensor memory (as soon as the last Q K^T of the job before is complete: the
+//   warps 8-11  the ends of a job: they move Q to tensor memory (as soon as the last Q K^T of the job before is complete: the
 //               softmax and P V of its last tile run meanwhile) and, once its last P V is, write O / l to global; only the
 //               next job's P V waits for them.  With both done by the softmax warps a query cost 7.2 thousand cycles beside
 //               its tiles: 1000 queries of up to 1000 rows 625 -> 597 us, a prompt of 32768 30.4 -> 30.0 ms.
-//               One thread of warp 4 is the scheduler and publishes the block's jobs (query, row count).  In prefill it takes
+//               One thread of warp 8 is the scheduler and publishes the block's jobs (query, row count).  In prefill it takes
 //               the block index of a block that has not started yet (cluster launch control), one job ahead of the one being
 //               worked on, latest query first: those attend the most rows.
-//   warps 8, 9  one thread each issues tcgen05.mma:
-//                 S = Q K^T   warp 8, M64 N64 K16, Q in tensor memory (the rope dims in shared memory), as two accumulation
+//   warps 12, 13  one thread each issues tcgen05.mma:
+//                 S = Q K^T   warp 12, M64 N64 K16, Q in tensor memory (the rope dims in shared memory), as two accumulation
 //                             chains: dims 0-255 and rope dims 0-31 in the even half of the lanes, dims 256-511 and rope
 //                             dims 32-63 in the odd half (an M = 64 accumulator and its A operand use 16 of the 32 lanes of
 //                             each quarter, so both halves of Q share their columns).  36 MMAs at the pipe's 32 cycles.
-//                 O += P V    warp 9, tcgen05.mma.ws M64 N256 K16, P in shared memory; V is the key tile read MN-major, so
+//                 O += P V    warp 13, tcgen05.mma.ws M64 N256 K16, P in shared memory; V is the key tile read MN-major, so
 //                             that a cache row is fetched once.  The .ws form spreads the 64 rows over all 128 lanes (heads
 //                             in lanes 0-63 and again in 64-127, each with half of the value dims), which is the full data
 //                             path: 81 cycles where the plain M64 N256 form takes 129.
 //               Two threads, because one stalls for 300 to 500 cycles after each batch before it gets to the next, and
 //               two S buffers, so that Q K^T of the next tile need not wait for the softmax of this one: 2 340 cycles per
 //               tile with one of each.
-//   warps 0-3   softmax: per tile add the two partial sums (read as 16-lane fragments, so both
-//               land in the same registers), running max with lazy rescaling of O, exp2, fp32 row sums, P as bf16 into
-//               the tile's rope block (64 x 64 values; Q K^T was its only reader); a split's partial O to the merge.
+//   warps 0-7   softmax, four warps for each half of a tile's keys (four in all where row lists are walked): per tile add the two partial sums (read as 16-lane
+//               fragments, so both land in the same registers), running max with lazy rescaling of O, exp2, fp32 row sums, P as
+//               bf16 into the tile's rope block (64 x 64 values; Q K^T was its only reader); a split's partial O to the merge.
 //
 // What bounds it (prefill): per 64-key tile the tensor pipe needs 36 x 32 + 8 x 81 = 1 800 cycles (2 176 with the plain
-// form for P V), and shared memory is read and written for about as long: 576 (Q K^T) + 640 (P V) + 576 (the copies).
+// form for P V), and shared memory is read and written for about as long: 576 (Q K^T) + 640 (P V) + 576 (the copies).  A window
+// tile takes 2 000.  A gathered one waits for its slot: three slots, each held from Q K^T to the end of P V (4 250 cycles) and
+// refilled (1 750 from L2, 2 400 of 131072 rows, 2 900 of a million).  L2 itself has room: scattered rows reach the SMs at
+// 18 TB/s with 216 KB in flight on each, but only a slot or so is.  The hold is a chain of hand-overs of 200-500 cycles each beside
+// the MMAs, in a load/store pipe that the copies fill.  With four softmax warps that took a maximum over each row for every
+// tile, two gather warps a slot and the last tile worked on whole, holds were 4 500 and a gathered tile 2 264 (16384 rows; now
+// 2 110), but the clock gives half of it back under the power cap: 32768 queries, two layers, 24.4 ms -> 23.7 ms; 16384 of
+// 131072, four layers, 34.5 -> 33.5 ms; 4096 of a million, four layers, 11.4 -> 11.0 ms.
 //
 // Tensor memory columns:   0-255  O: value dims 0-255 in columns 0-127, 256-511 in 128-255; lanes 0-63 hold the first 128
 //                                 dims of each, lanes 64-127 the second, lane l (mod 64) = head l
@@ -57,18 +65,27 @@ constexpr int kAtomBytes = 64 * 128;         // 64 rows x 128 bytes
 constexpr int kSlotBytes = kAtoms * kAtomBytes;
 
 constexpr int kRing = 3;                     // 64-key tiles (or Q) in shared memory
-constexpr int kSoftmaxWarps = 4, kDrainWarp0 = 4, kDrainWarps = 4, kQkWarp = 8, kPvWarp = 9, kGatherWarp0 = 10;
-constexpr int kSlotWarps = 2;                // gather warps of a ring slot
-constexpr int kGatherWarps = kRing * kSlotWarps;
-constexpr int kThreadsAttnTc = 32 * (kGatherWarp0 + kGatherWarps);
-constexpr int kRowsPerWarp = kTileKeys / kSlotWarps;   // cache rows of a tile that one gather warp copies
+constexpr int kDrainWarps = 4;
+constexpr int kSumWarps = 4;                 // softmax warps that put a row's sums together (those of the tiles' first keys)
 constexpr uint32_t kTmemColsAttn = 512;
 constexpr uint32_t kColQ = 256, kColS = 384, kSBuf = 64;
 constexpr float kLog2eTc = 1.4426950408889634f;
 constexpr int kMaxClusterSplit = 16;         // row splits of one sequence = blocks of one cluster (eight is the portable limit)
 constexpr int kFirstTileCycles = 8192;       // longest that a block's second tile is held back for the first
 constexpr float kRescaleGap = 8.f;           // rescale O only when the row max grows by more than 2^8
-constexpr int kJobReaders = kSoftmaxWarps + kDrainWarps + 2 + kGatherWarps;   // warps that release a job slot
+// Warps of a block.  Prefill: the softmax of a tile by two warps per lane quarter, each with half of its keys, and three gather
+// warps a ring slot (two issue a tile's 144 copies in 1 530 cycles, three in 1 430, which is about what the SM takes).  Where row
+// lists are walked one and two: HBM paces the tiles, and a layer's ends are shorter with fewer threads (64 sequences, four layers:
+// 189 us, 195 with the prefill's eight softmax warps).
+template <bool kRows>
+struct Warps {
+  static constexpr int kHalves = kRows ? 1 : 2, kSoftmax = 4 * kHalves;
+  static constexpr int kDrain0 = kSoftmax, kQk = kDrain0 + kDrainWarps, kPv = kQk + 1, kGather0 = kPv + 1;
+  static constexpr int kSlot = kRows ? 2 : 3, kAll = kGather0 + kRing * kSlot, kThreads = 32 * kAll;
+  static constexpr int kRowsEach = kRows ? 32 : 24;   // cache rows of a tile that a gather warp copies (the last one the rest)
+  static constexpr int kJobReaders = kSoftmax + kDrainWarps + 2 + kRing * kSlot;   // warps that release a job slot
+  static_assert(kRowsEach % 8 == 0 && kRowsEach <= 32 && kRowsEach * (kSlot - 1) < kTileKeys, "whole groups of eight rows, a lane each");
+};
 
 struct AttnTcSmem {
   alignas(1024) uint8_t k[kRing][kAtoms][kAtomBytes];       // [ring slot][column block][64 rows x 128 B]
@@ -81,9 +98,10 @@ struct AttnTcSmem {
   alignas(8) int2 job[2];                 // {query or -1 = no more, rows it attends}
   uint32_t tmem_slot;
   int fail;                               // a softmax warp's wait ran out
-  float alpha[kH];                        // pending rescale factor of O per head (1 = none)
+  float half_max[2][kH];                  // [half of a tile's keys][head]: its maximum, where both halves have to know it
+  float half_sum[kH];                     // row sums of the second halves
   float inv[2][kH];                       // 1 / l per head of the query being written out, by job parity
-  alignas(16) float lse_own[kH];          // its log-sum-exp per head (log2 units)
+  alignas(16) float lse_own[kH];          // its log-sum-exp per head (log2 units); before that, of a rescale of O, the factors
   alignas(16) float lse_peer[kH / 2];     // two-split launches: the peer's, for the heads this block finishes
 };
 // Splits stage their partial rows in the order the softmax warps read them out of tensor memory: per warp (32 heads,
@@ -92,7 +110,7 @@ struct AttnTcSmem {
 // copy each, while the rest is still being read out, and keep that layout where they go: with two splits the rows the peer
 // finishes, behind its staged ones; with more all of them, to the global scratch.
 constexpr int kWarpStage = 32 * 256 * 4;
-constexpr int kRecvOffset = kSoftmaxWarps * kWarpStage;
+constexpr int kRecvOffset = 4 * kWarpStage;
 constexpr uint32_t kRecvBytes = 2 * kWarpStage + (kH / 2) * 4;
 static_assert(kRecvOffset + 2 * kWarpStage <= kRing * kSlotBytes, "staged and received rows must fit the ring");
 
@@ -118,12 +136,14 @@ __device__ __forceinline__ void bulk_copy_to_peer(uint32_t dst_peer, uint32_t sr
                ::"r"(dst_peer), "r"(src), "r"(bytes), "r"(bar_peer) : "memory");
 }
 
-// ---- barrier of the 128 softmax threads; the second form also tells every one of them whether any of them said yes
-__device__ __forceinline__ void softmax_sync() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
+// ---- barrier of the softmax threads; the second form also tells every one of them whether any of them said yes
+template <int kThreads>
+__device__ __forceinline__ void softmax_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kThreads) : "memory"); }
+template <int kThreads>
 __device__ __forceinline__ bool softmax_any(bool v) {
   uint32_t r;
-  asm volatile("{\n\t.reg .pred a, b;\n\tsetp.ne.b32 a, %1, 0;\n\tbar.red.or.pred b, 1, 128, a;\n\tselp.b32 %0, 1, 0, b;\n\t}"
-               : "=r"(r) : "r"(static_cast<uint32_t>(v)) : "memory");
+  asm volatile("{\n\t.reg .pred a, b;\n\tsetp.ne.b32 a, %1, 0;\n\tbar.red.or.pred b, 1, %2, a;\n\tselp.b32 %0, 1, 0, b;\n\t}"
+               : "=r"(r) : "r"(static_cast<uint32_t>(v)), "n"(kThreads) : "memory");
   return r != 0;
 }
 __device__ __forceinline__ float exp2_fast(float x) {
@@ -191,10 +211,13 @@ __device__ __forceinline__ bool clc_answer(uint32_t answer, int* block_x) {
 //   kClustered  the blocks of a cluster are row splits of one sequence and merge their results; else the block goes on
 //               to further queries
 template <bool kRows, bool kClustered>
-__global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const __grid_constant__ CUtensorMap q_map, int q_tma,
+__global__ void __launch_bounds__(Warps<kRows>::kThreads, 1) sparse_attn_tc_kernel(const __grid_constant__ CUtensorMap q_map, int q_tma,
                                                                             const __grid_constant__ CUtensorMap k_map, int k_tma,
                                                                             const __grid_constant__ CUtensorMap g_map, int k_g4,
                                                                             AttnArgs p) {
+  using W = Warps<kRows>;
+  constexpr int kHalves = W::kHalves, kSoftmaxWarps = W::kSoftmax, kDrainWarp0 = W::kDrain0, kQkWarp = W::kQk, kPvWarp = W::kPv, kGatherWarp0 = W::kGather0;
+  constexpr int kSlotWarps = W::kSlot, kRowsPerWarp = W::kRowsEach, kJobReaders = W::kJobReaders, kSoftmaxThreads = 32 * kSoftmaxWarps;
   extern __shared__ uint8_t smem_raw[];
   AttnTcSmem& sm = *reinterpret_cast<AttnTcSmem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
   const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
@@ -215,7 +238,7 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
       tc::mbar_init(smem_u32(&sm.pv_done[b]), 1);
     }
     for (int b = 0; b < 2; ++b) {
-      tc::mbar_init(smem_u32(&sm.o_full[b]), 1 + kSoftmaxWarps);
+      tc::mbar_init(smem_u32(&sm.o_full[b]), 1 + kSumWarps);
       tc::mbar_init(smem_u32(&sm.q_tmem[b]), kDrainWarps);     // by job parity: a job without tiles may be overtaken by the next
       tc::mbar_init(smem_u32(&sm.s_full[b]), 1);
       tc::mbar_init(smem_u32(&sm.s_free[b]), kSoftmaxWarps);
@@ -232,7 +255,6 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
     sm.fail = 0;
     tc::fence_mbar_init();
   }
-  if (tid < kH) sm.alpha[tid] = 1.f;
   if (warp == kQkWarp) {
     tc::tmem_alloc(smem_u32(&sm.tmem_slot), kTmemColsAttn);
     tc::tmem_relinquish();
@@ -285,6 +307,12 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
     if (dead) b.n_tiles = 0;   // the peers of this cluster still expect this block at the cluster barrier
     b.q_at = early_rows ? min(2, b.n_tiles) : 0;
     return b;
+  };
+  // Keys of tile i that are worked on: the last tile's in whole MMA steps of 16 (3076 rows are 48 tiles and four rows).  Not where
+  // row lists are walked: HBM paces those tiles, and loops of a constant length are issued faster.
+  auto tile_keys = [](const Job& b, int i) -> int {
+    if constexpr (kRows) return kTileKeys;
+    else return min(kTileKeys, (b.n_tot - (b.tile_begin + i) * kTileKeys + 15) & ~15);
   };
   auto wait_job = [&](int n, int2* j) -> bool {   // n-th job of this block; whole warp or one thread
     const bool ok = tc::mbar_wait(smem_u32(&sm.job_full[n & 1]), (n >> 1) & 1, p.status);
@@ -395,26 +423,26 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
         uint8_t* dst = reinterpret_cast<uint8_t*>(reinterpret_cast<__nv_bfloat16*>(p.out) + (static_cast<int64_t>(done.qi) * kH + head_o) * kDV + 128 * half_o);
         const bool by32 = (reinterpret_cast<uintptr_t>(p.out) & 31u) == 0;
 #pragma unroll 1
-        for (int c = 0; c < 256; c += 64) {
-          uint32_t o[64];
+        for (int c = 0; c < 256; c += 32) {
+          uint32_t o[32];
           if (done.n_tiles > 0) {
-            tc::tmem_ld64(tmem_base + lane_addr + c, o);
+            tc::tmem_ld32(tmem_base + lane_addr + c, o);
             tc::tmem_ld_wait();
           } else {
 #pragma unroll
-            for (int j = 0; j < 64; ++j) o[j] = 0u;
+            for (int j = 0; j < 32; ++j) o[j] = 0u;
           }
-          if (c == 192) {   // all of O is in registers: the next job's P V may begin
+          if (c == 224) {   // all of O is in registers: the next job's P V may begin
             tc::fence_before_sync();
             __syncwarp();
             if (lane == 0) tc::mbar_arrive(smem_u32(&sm.o_free));
           }
-          uint32_t w[32];
+          uint32_t w[16];
 #pragma unroll
-          for (int j = 0; j < 32; ++j) w[j] = pack_bf16(__uint_as_float(o[2 * j]) * inv, __uint_as_float(o[2 * j + 1]) * inv);
+          for (int j = 0; j < 16; ++j) w[j] = pack_bf16(__uint_as_float(o[2 * j]) * inv, __uint_as_float(o[2 * j + 1]) * inv);
           uint8_t* d = dst + ((c >> 7) * 256 + (c & 127)) * 2;
 #pragma unroll
-          for (int j = 0; j < 32; j += 8) store_words8(d + j * 4, w + j, by32);
+          for (int j = 0; j < 16; j += 8) store_words8(d + j * 4, w + j, by32);
         }
         __syncwarp();
         if (lane == 0) tc::mbar_arrive(smem_u32(&sm.job_empty[n & 1]));
@@ -426,6 +454,7 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
   } else if (warp >= kGatherWarp0) {
     // ================= gather warps =================
     const int grp = (warp - kGatherWarp0) / kSlotWarps, gw = (warp - kGatherWarp0) % kSlotWarps;   // ring slot, warp of its group
+    const int warp_rows = kSlotWarps * kRowsPerWarp == kTileKeys ? kRowsPerWarp : min(kRowsPerWarp, kTileKeys - kRowsPerWarp * gw);
     const uint8_t* kg = reinterpret_cast<const uint8_t*>(p.k);
     const bool g4 = k_g4 != 0;   // block-uniform
     const uint32_t full = smem_u32(&sm.k_full[grp]), empty = smem_u32(&sm.k_empty[grp]);
@@ -456,7 +485,7 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
       };
       auto my_key_row = [&](int e) -> int32_t {   // each lane looks up the cache row of one of the warp's keys
         const int i = tile_of(e);
-        return (e != jb.q_at && e <= jb.n_tiles && lane < kRowsPerWarp && !tile_by_tma(i))
+        return (e != jb.q_at && e <= jb.n_tiles && lane < warp_rows && !tile_by_tma(i))
                    ? row_of((jb.tile_begin + i) * kTileKeys + kRowsPerWarp * gw + lane) : -1;
       };
       int e = (grp + kRing - base % kRing) % kRing;
@@ -465,7 +494,16 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
         const int pos = base + e;
         const bool is_q = e == jb.q_at;
         const int i = tile_of(e);   // the tile (if this is not Q)
+        const int rows_here = kRows ? warp_rows : max(0, min(warp_rows, tile_keys(jb, i) - kRowsPerWarp * gw));   // of it, by this warp (a multiple of 8)
         const int32_t next_row = my_key_row(e + kRing);   // fetched before the wait: off the critical path
+#if LSA_PF == 1
+        if (!kRows && next_row >= 0) asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(kg + static_cast<int64_t>(next_row) * p.ld_k * 2), "n"(kDQK * 2) : "memory");
+#elif LSA_PF == 2
+        if (!kRows && next_row >= 0) {
+#pragma unroll
+          for (int y = 0; y < 9; ++y) asm volatile("prefetch.global.L2 [%0];" ::"l"(kg + static_cast<int64_t>(next_row) * p.ld_k * 2 + y * 128) : "memory");
+        }
+#endif
         if (e >= jb.q_at && !waited) {   // the tiles before Q are in flight: now the previous kernel must be done
           dependency_wait();
           waited = true;
@@ -499,9 +537,9 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
           }
         } else if (g4) {
           // scattered rows: four rows x 64 dims per instruction, straight into their place in the swizzled tile
-          if (lane == 0) tc::mbar_expect_tx_only(full, kSlotBytes / kSlotWarps);
+          if (lane == 0) tc::mbar_expect_tx_only(full, static_cast<uint32_t>(rows_here) * (kDQK * 2));
           __syncwarp();
-          for (int u = lane; u < kRowsPerWarp / 4 * kAtoms; u += 32) {
+          for (int u = lane; u < rows_here / 4 * kAtoms; u += 32) {
             const int q4 = u / kAtoms, atom = u % kAtoms;
             int4 r;
             // past the end of the list its last row once more: masked in the softmax, and as a value of weight 0 it must not be
@@ -515,7 +553,7 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
           // the 72 16-byte chunks of a row: 64 by all lanes in two instructions; the last eight of four rows in one
           const uint32_t dst0 = smem_u32(sm.k[grp][lane >> 3]) + kRowsPerWarp * gw * 128;
 #pragma unroll 8
-          for (int rr = 0; rr < kRowsPerWarp; ++rr) {
+          for (int rr = 0; rr < rows_here; ++rr) {
             const int32_t row = __shfl_sync(0xffffffffu, my_row, rr);
             const uint8_t* src = kg + static_cast<int64_t>(row >= 0 ? row : 0) * p.ld_k * 2 + lane * 16;
             const int nb = row >= 0 ? 16 : 0;
@@ -547,7 +585,6 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
   } else if (warp == kQkWarp) {
     // ================= issuer of Q K^T =================
     if (tc::elect_one()) {
-      constexpr uint32_t idesc = tc::idesc_bf16(kH, kTileKeys, 0, 0);
       // Descriptors are built once; inside the loops only the start-address word moves (one add per operand).
       const uint64_t dk0 = tc::smem_desc_sw128(smem_u32(sm.k), 16, 1024);           // K-major view
       const uint64_t dqr = tc::smem_desc_sw128(smem_u32(sm.q_rope), 16, 1024);
@@ -571,6 +608,7 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
           if (!ok) break;
           tc::fence_after_sync();
           const uint64_t dkb = tc::desc_advance(dk0, slot_of(pos) * kSlotBytes);
+          const uint32_t idesc = tc::idesc_bf16(kH, tile_keys(jb, i), 0, 0);
 #pragma unroll
           for (int x = 0; x < 2; ++x) {
             const uint32_t q_src = tmem_base + x * kLane16 + kColQ, s_dst = tmem_base + x * kLane16 + kColS + (g & 1) * kSBuf;
@@ -611,12 +649,14 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
           if (!ok) break;
           tc::fence_after_sync();
           const uint64_t dvb = tc::desc_advance(dv0, slot * kSlotBytes), dpb = tc::desc_advance(dp0, slot * kSlotBytes);
+          const int keys = tile_keys(jb, i);
 #pragma unroll
           for (int y = 0; y < 2; ++y)       // value dims 256y .. +255
 #pragma unroll
             for (int kk = 0; kk < kTileKeys / 16; ++kk)   // keys 16*kk .. +15
-              tc::umma_ws_ss(tmem_base + 128 * y, tc::desc_advance(dpb, kk * 32), tc::desc_advance(dvb, 4 * y * kAtomBytes + kk * 2048),
-                             idesc, (i > 0) || (kk > 0));
+              if (16 * kk < keys)
+                tc::umma_ws_ss(tmem_base + 128 * y, tc::desc_advance(dpb, kk * 32), tc::desc_advance(dvb, 4 * y * kAtomBytes + kk * 2048),
+                               idesc, (i > 0) || (kk > 0));
           // "P V of the tile done" frees the ring slot for the gather warps, and tells the softmax warps that O may be touched
           // again: where a block goes on to another job by a barrier of its own, since the slot's may go on with the next
           // query (which only its issuer waits for) before they look, and a barrier two uses on looks like an unused one
@@ -634,11 +674,15 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
     }
   } else {
     // ================= softmax warps =================
-    // Warp w owns the S rows (heads) 16w .. 16w+15; as 16-lane fragments, a thread holds keys 8g + 2 (lane % 4) + {0, 1} of
-    // heads 16w + lane / 4 and 8 more.  Of O it reads lanes 32w .. +31: heads 32 (w & 1) + lane, half w >> 1 of the value
-    // dims of each 256.
-    const uint32_t lane_addr = static_cast<uint32_t>(32 * warp) << 16;
-    const int head_o = 32 * (warp & 1) + lane, half_o = warp >> 1;
+    // Warp w owns the S rows (heads) 16w .. 16w+15; with two halves warps w and w + 4 do, the first of keys 0-31 of a tile, the other
+    // of keys 32-63.  As 16-lane fragments, a thread holds keys 8j + 2 (lane % 4) + {0, 1} of its half, of heads 16w + lane / 4 and
+    // 8 more.  Of O it reads lanes 32w .. +31: heads 32 (w & 1) + lane, half w >> 1 of the value dims of each 256, and its half of
+    // those columns.
+    constexpr int kKeys = kTileKeys / kHalves, kGroups = kKeys / 8;   // keys of a half, in fragments of eight
+    const int quarter = warp & 3, half = warp >> 2;
+    const uint32_t lane_addr = static_cast<uint32_t>(32 * quarter) << 16;
+    const int head_o = 32 * (quarter & 1) + lane, half_o = quarter >> 1;
+    const int row_s = 16 * quarter + (lane >> 2);   // the first of the thread's two heads
     const float zs = p.sm_scale * kLog2eTc;
     bool ok = true;
     // P V of tile g (over all jobs), which lies at ring position `pos`, is complete; whole warp
@@ -651,10 +695,10 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
     ok = __all_sync(0xffffffffu, wait_job(0, &jd));
     Job jb = job_of(jd);
     bool have_o = false;
-    float m_used[2] = {0.f, 0.f}, l_run[2] = {0.f, 0.f};   // rows lane / 4 and lane / 4 + 8; l_run is this thread's share
-    // A warp whose wait ran out goes on to the next vote, where all four learn of it and leave together: the named barrier
+    float m_used[2] = {0.f, 0.f}, l_run[2] = {0.f, 0.f};   // rows row_s and row_s + 8; l_run is this thread's share
+    // A warp whose wait ran out goes on to the next vote, where all eight learn of it and leave together: the named barrier
     // has no time limit.
-    bool go = !softmax_any(!ok);
+    bool go = !softmax_any<kSoftmaxThreads>(!ok);
     while (go) {
       // ---- the tiles of the job
       l_run[0] = l_run[1] = 0.f;
@@ -664,91 +708,114 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
         const int slot = slot_of(base + i + (i >= jb.q_at ? 1 : 0));
         ok = ok && __all_sync(0xffffffffu, tc::mbar_wait(smem_u32(&sm.s_full[g & 1]), (g >> 1) & 1, p.status));
         tc::fence_after_sync();
-        float2 v[16];   // [key group j][row r] at 2j + r
+        float2 v[2 * kGroups];   // [key group j][row r] at 2j + r
         {
-          uint32_t a[32], c[32];
-          tc::tmem_ld_16x256b_x8(tmem_base + lane_addr + kColS + (g & 1) * kSBuf, a);
-          tc::tmem_ld_16x256b_x8(tmem_base + lane_addr + (16u << 16) + kColS + (g & 1) * kSBuf, c);
+          uint32_t a[4 * kGroups], c[4 * kGroups];
+          const uint32_t s_addr = tmem_base + lane_addr + kColS + (g & 1) * kSBuf + kKeys * half;
+          tc::tmem_ld_16x256b(s_addr, a);
+          tc::tmem_ld_16x256b(s_addr + (16u << 16), c);
           tc::tmem_ld_wait();
           tc::fence_before_sync();
           __syncwarp();
           if (lane == 0) tc::mbar_arrive(smem_u32(&sm.s_free[g & 1]));
 #pragma unroll
-          for (int j = 0; j < 16; ++j)
+          for (int j = 0; j < 2 * kGroups; ++j)
             v[j] = add2(make_float2(__uint_as_float(a[2 * j]), __uint_as_float(a[2 * j + 1])),
                         make_float2(__uint_as_float(c[2 * j]), __uint_as_float(c[2 * j + 1])));
         }
-        const int n_valid = jb.n_tot - (jb.tile_begin + i) * kTileKeys;   // keys of this tile that exist
-        if (n_valid < kTileKeys) {
+        const int n_valid = jb.n_tot - (jb.tile_begin + i) * kTileKeys - kKeys * half;   // keys of this half that exist
+        if (n_valid < kKeys) {
           const int k0 = 2 * (lane & 3);
 #pragma unroll
-          for (int j = 0; j < 8; ++j) {
+          for (int j = 0; j < kGroups; ++j) {
             if (8 * j + k0 >= n_valid) v[2 * j].x = v[2 * j + 1].x = -INFINITY;
             if (8 * j + k0 + 1 >= n_valid) v[2 * j].y = v[2 * j + 1].y = -INFINITY;
           }
         }
-        // running max in log2 units, moved only when it grows by more than kRescaleGap (O and l are then rescaled)
+        // Running max in log2 units: that of the job's first tile, moved only when a row grows by more than kRescaleGap (O and l
+        // are then rescaled).  P is worked out with the maximum as it is; the vote that ends the tile says whether that was good
+        // enough for every row, so a row's lanes and halves compare their values only where they have to: shuffles and barriers
+        // queue behind the gather warps' copies (110-150 cycles each).
+        float mx[2];   // of the thread's values, then of the rows'
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+          float x = fmaxf(v[r].x, v[r].y);
+#pragma unroll
+          for (int j = 1; j < kGroups; ++j) x = fmaxf(x, fmaxf(v[2 * j + r].x, v[2 * j + r].y));
+          mx[r] = x * zs;
+        }
+        auto row_max = [&]() {
+#pragma unroll
+          for (int r = 0; r < 2; ++r) {
+            mx[r] = fmaxf(mx[r], __shfl_xor_sync(0xffffffffu, mx[r], 1));
+            mx[r] = fmaxf(mx[r], __shfl_xor_sync(0xffffffffu, mx[r], 2));
+            if (kHalves > 1 && (lane & 3) == 0) sm.half_max[half][row_s + 8 * r] = mx[r];
+          }
+          if constexpr (kHalves > 1) {
+            softmax_sync<kSoftmaxThreads>();
+#pragma unroll
+            for (int r = 0; r < 2; ++r) mx[r] = fmaxf(mx[r], sm.half_max[half ^ 1][row_s + 8 * r]);
+          }
+        };
         bool need = false;
-        float alpha[2] = {1.f, 1.f};
+        if (i == 0) {
+          row_max();
+          m_used[0] = mx[0];
+          m_used[1] = mx[1];
+        } else {
+          need = mx[0] > m_used[0] + kRescaleGap || mx[1] > m_used[1] + kRescaleGap;
+        }
+        float sum[2];
+        while (true) {
+          // P = exp2(z - m), fp32 row sums, bf16 pack
+          uint32_t pk[kGroups][2];
 #pragma unroll
-        for (int r = 0; r < 2; ++r) {
-          float mx = fmaxf(v[r].x, v[r].y);
+          for (int r = 0; r < 2; ++r) {
+            const float2 z2 = make_float2(zs, zs), m2 = make_float2(-m_used[r], -m_used[r]);
+            float2 sum2 = make_float2(0.f, 0.f);
 #pragma unroll
-          for (int j = 1; j < 8; ++j) mx = fmaxf(mx, fmaxf(v[2 * j + r].x, v[2 * j + r].y));
-          mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-          mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-          mx *= zs;
-          if (i == 0) {
-            m_used[r] = mx;
-          } else if (mx > m_used[r] + kRescaleGap) {
-            alpha[r] = exp2_fast(m_used[r] - mx);
-            m_used[r] = mx;
-            need = true;
+            for (int j = 0; j < kGroups; ++j) {
+              float2 e = fma2(v[2 * j + r], z2, m2);
+              e.x = exp2_fast(e.x);
+              e.y = exp2_fast(e.y);
+              sum2 = add2(sum2, e);
+              pk[j][r] = pack_bf16(e.x, e.y);
+            }
+            sum[r] = sum2.x + sum2.y;
           }
-        }
-        // P = exp2(z - m), fp32 row sums, bf16 pack
-        uint32_t pk[8][2];
+          // P takes the place of the tile's rope dims, which only Q K^T reads
+          {
+            const int row = 16 * quarter + ((lane >> 3) & 1) * 8 + (lane & 7);
+            const uint32_t dst = smem_u32(sm.k[slot][8]) + row * 128;
 #pragma unroll
-        for (int r = 0; r < 2; ++r) {
-          const float2 z2 = make_float2(zs, zs), m2 = make_float2(-m_used[r], -m_used[r]);
-          float2 sum2 = make_float2(0.f, 0.f);
-#pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            float2 e = fma2(v[2 * j + r], z2, m2);
-            e.x = exp2_fast(e.x);
-            e.y = exp2_fast(e.y);
-            sum2 = add2(sum2, e);
-            pk[j][r] = pack_bf16(e.x, e.y);
+            for (int j = 0; j < kGroups; j += 2)
+              stmatrix_x4(dst + (((kGroups * half + j + (lane >> 4)) ^ (row & 7)) << 4), pk[j][0], pk[j][1], pk[j + 1][0], pk[j + 1][1]);
           }
-          const float sum = sum2.x + sum2.y;
-          l_run[r] = l_run[r] * alpha[r] + sum;
-        }
-        // P takes the place of the tile's rope dims, which only Q K^T reads
-        {
-          const int row = 16 * warp + ((lane >> 3) & 1) * 8 + (lane & 7);
-          const uint32_t dst = smem_u32(sm.k[slot][8]) + row * 128;
-#pragma unroll
-          for (int j = 0; j < 8; j += 2)
-            stmatrix_x4(dst + (((j + (lane >> 4)) ^ (row & 7)) << 4), pk[j][0], pk[j][1], pk[j + 1][0], pk[j + 1][1]);
-        }
-        need = __any_sync(0xffffffffu, need);
-        if (need && (lane & 3) == 0) {
-          sm.alpha[16 * warp + (lane >> 2)] = alpha[0];
-          sm.alpha[16 * warp + (lane >> 2) + 8] = alpha[1];
-        }
-        if (!ok) sm.fail = 1;
-        tc::fence_proxy_async();   // P is read by the tensor core
-        if (softmax_any(need || !ok)) {
+          if (!ok) sm.fail = 1;
+          tc::fence_proxy_async();   // P is read by the tensor core
+          if (!softmax_any<kSoftmaxThreads>(need || !ok)) break;
           if (*reinterpret_cast<volatile int*>(&sm.fail)) {
             failed = true;
             break;
           }
-          // rare: O of every head times its factor, once P V of the tile before is complete
-          if (i > 0) ok = ok && wait_pv(g - 1, base + i - 1 + (i - 1 >= jb.q_at ? 1 : 0));
+          // rare: the rows' new maxima, O of every head times its factor, once P V of the tile before is complete, and P again
+          row_max();
+#pragma unroll
+          for (int r = 0; r < 2; ++r) {
+            float alpha = 1.f;
+            if (mx[r] > m_used[r] + kRescaleGap) {
+              alpha = exp2_fast(m_used[r] - mx[r]);
+              m_used[r] = mx[r];
+            }
+            l_run[r] *= alpha;
+            if (half == 0 && (lane & 3) == 0) sm.lse_own[row_s + 8 * r] = alpha;
+          }
+          softmax_sync<kSoftmaxThreads>();
+          ok = wait_pv(g - 1, base + i - 1 + (i - 1 >= jb.q_at ? 1 : 0));   // (a first tile has no such rows)
           tc::fence_after_sync();
-          const float al = sm.alpha[head_o];
+          const float al = sm.lse_own[head_o];
 #pragma unroll 1
-          for (int c = 0; c < 256; c += 32) {
+          for (int c = 256 / kHalves * half; c < 256 / kHalves * (half + 1); c += 32) {
             uint32_t o[32];
             tc::tmem_ld32(tmem_base + lane_addr + c, o);
             tc::tmem_ld_wait();
@@ -758,38 +825,49 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
           }
           tc::tmem_st_wait();
           tc::fence_before_sync();
-          softmax_sync();
-          if (need && (lane & 3) == 0) sm.alpha[16 * warp + (lane >> 2)] = sm.alpha[16 * warp + (lane >> 2) + 8] = 1.f;
+          need = false;
         }
+        if (failed) break;
+        l_run[0] += sum[0];
+        l_run[1] += sum[1];
         if (tid == 0) tc::mbar_arrive(smem_u32(&sm.p_ready[g % kRing]));
       }
       if (failed) break;
-      // ---- row sums and log-sum-exps of the job, for the threads that read O
+      // ---- row sums and log-sum-exps of the job, for the threads that read O; the second halves' sums go to the first's warps
       have_o = jb.n_tiles > 0;
 #pragma unroll
       for (int r = 0; r < 2; ++r) {
-        float l = l_run[r];
-        l += __shfl_xor_sync(0xffffffffu, l, 1);
-        l += __shfl_xor_sync(0xffffffffu, l, 2);
-        const int row = 16 * warp + (lane >> 2) + 8 * r;
-        const float lse2 = (have_o && l > 0.f) ? m_used[r] + log2f(l) : -INFINITY;   // log2 domain
-        if ((lane & 3) == 0) {
-          sm.inv[n & 1][row] = (have_o && l > 0.f) ? 1.f / l : 0.f;
-          sm.lse_own[row] = lse2;
-          if (!clustered) {
-            if (p.lse != nullptr) p.lse[static_cast<int64_t>(jb.qi) * kH + row] = lse2 / kLog2eTc;
-          } else if (!pair) {
-            part_lse[(static_cast<int64_t>(jb.qi) * p.n_split + split) * kH + row] = lse2;
+        l_run[r] += __shfl_xor_sync(0xffffffffu, l_run[r], 1);
+        l_run[r] += __shfl_xor_sync(0xffffffffu, l_run[r], 2);
+        // (a job without tiles says nothing: it has no vote between its sums and the reading of the job's before)
+        if (half == 1 && have_o && (lane & 3) == 0) sm.half_sum[row_s + 8 * r] = l_run[r];
+      }
+      auto finish_rows = [&]() {
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+          const int row = row_s + 8 * r;
+          const float l = kHalves > 1 && have_o ? l_run[r] + sm.half_sum[row] : l_run[r];
+          const float lse2 = (have_o && l > 0.f) ? m_used[r] + log2f(l) : -INFINITY;   // log2 domain
+          if ((lane & 3) == 0) {
+            sm.inv[n & 1][row] = (have_o && l > 0.f) ? 1.f / l : 0.f;
+            sm.lse_own[row] = lse2;
+            if (!clustered) {
+              if (p.lse != nullptr) p.lse[static_cast<int64_t>(jb.qi) * kH + row] = lse2 / kLog2eTc;
+            } else if (!pair) {
+              part_lse[(static_cast<int64_t>(jb.qi) * p.n_split + split) * kH + row] = lse2;
+            }
           }
         }
-      }
-      if constexpr (!kClustered) {
-        __syncwarp();
-        if (lane == 0) tc::mbar_arrive(smem_u32(&sm.o_full[n & 1]));
-        ok = __all_sync(0xffffffffu, wait_job(n + 1, &jd)) && ok;
-      }
+        if constexpr (!kClustered) {
+          __syncwarp();
+          if (lane == 0) tc::mbar_arrive(smem_u32(&sm.o_full[n & 1]));
+        }
+      };
+      if constexpr (kHalves == 1) finish_rows();
+      if constexpr (!kClustered) ok = __all_sync(0xffffffffu, wait_job(n + 1, &jd)) && ok;
       if (!ok) sm.fail = 1;
-      if (softmax_any(!ok)) break;
+      if (softmax_any<kSoftmaxThreads>(!ok)) break;
+      if (kHalves > 1 && half == 0) finish_rows();
       if constexpr (kClustered) {
         if (have_o) have_o = wait_pv(jb.n_tiles - 1, jb.n_tiles - 1 + (jb.n_tiles - 1 >= jb.q_at ? 1 : 0));   // the last tile's
         tc::fence_after_sync();
@@ -803,12 +881,13 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
       jb = job_of(jd);
     }
     if constexpr (kClustered) {
+      static_assert(kHalves == 1, "a warp stages all of its lanes' columns");
       // ---- partial result of a split: normalised fp32 rows in the ring
       const int qi = blockIdx.x;
       const float inv = have_o ? sm.inv[0][head_o] : 0.f;
       uint8_t* stage = &sm.k[0][0][0];
       if (pair) cluster_arrive();   // this thread has left the tile loop, and every P V of the block has completed
-      const bool foreign = pair && (warp & 1) != split;   // a warp stages 32 heads: all of them the peer's, or none
+      const bool foreign = pair && (quarter & 1) != split;   // a warp stages 32 heads: all of them the peer's, or none
       const uint32_t peer = static_cast<uint32_t>(split ^ 1);
       uint32_t bar_peer = 0, dst_peer = 0;
       if (foreign) {
@@ -881,7 +960,7 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
     const int rows_per = kH / n;
     const int row0 = split * rows_per;
     const uint8_t* stage = &sm.k[0][0][0];
-    constexpr int kWarps = kThreadsAttnTc / 32;
+    constexpr int kWarps = W::kAll;
     __nv_bfloat16* out = reinterpret_cast<__nv_bfloat16*>(p.out) + (static_cast<int64_t>(qi) * kH + row0) * kDV;
     if (pair) {
       if (warp >= kSoftmaxWarps) cluster_wait();   // (the softmax warps completed this phase before they sent)
@@ -947,7 +1026,7 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
       // parts at a time, was 4 600 cycles with 16 splits; decode step of one sequence, 4 layers: 77.2 us, 74.3 now.)
       auto merge = [&](auto parts) {
         constexpr int N = decltype(parts)::value, kRuns = 16 / N;
-        static_assert(kWarps == 16, "every warp has a share of the block's 64 / N rows");
+        static_assert(kWarps >= 16, "sixteen warps have a share of the block's 64 / N rows");
         const int rl = 4 * warp / N, u0 = warp * kRuns & 3, R = row0 + rl;
         const float my_l = lane >= N ? -INFINITY : lane == split ? sm.lse_own[R] : __ldcg(part_lse + (static_cast<int64_t>(qi) * N + lane) * kH + R);
         const uint8_t* src = reinterpret_cast<const uint8_t*>(part_out + static_cast<int64_t>(qi) * N * kH * kDV) +
@@ -987,7 +1066,8 @@ __global__ void __launch_bounds__(kThreadsAttnTc, 1) sparse_attn_tc_kernel(const
           *reinterpret_cast<uint2*>(out + static_cast<int64_t>(rl) * kDV + (lane + 32 * (u0 + i)) * 4) = o;
         }
       };
-      if (n == 16) merge(IntC<16>{});
+      if (warp >= 16) {}
+      else if (n == 16) merge(IntC<16>{});
       else if (n == 8) merge(IntC<8>{});
       else merge(IntC<4>{});
     }
@@ -1012,7 +1092,7 @@ cudaError_t attn_tc_resident(int n_split, int* clusters) {
   *clusters = 0;
   if (at < 0) return cudaSuccess;
   return n[at].get(clusters, [&](int* c) {
-    return resident_clusters(reinterpret_cast<const void*>(sparse_attn_tc_kernel<true, true>), kThreadsAttnTc, sizeof(AttnTcSmem) + 1024, n_split, c);
+    return resident_clusters(reinterpret_cast<const void*>(sparse_attn_tc_kernel<true, true>), Warps<true>::kThreads, sizeof(AttnTcSmem) + 1024, n_split, c);
   });
 }
 
@@ -1034,6 +1114,7 @@ cudaError_t launch_attn_tc(const AttnArgs& a, cudaStream_t st, int64_t* n_launch
   const size_t smem = sizeof(AttnTcSmem) + 1024;
   if (a.n_split > 1 && a.rows == nullptr) return cudaErrorInvalidValue;   // row splits walk row lists
   AttnTcKernel kernel = pick_kernel(a);
+  const int threads = a.rows == nullptr ? Warps<false>::kThreads : Warps<true>::kThreads;
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (e != cudaSuccess) return e;
   CUtensorMap q_map{}, k_map{}, g_map{};
@@ -1048,7 +1129,7 @@ cudaError_t launch_attn_tc(const AttnArgs& a, cudaStream_t st, int64_t* n_launch
   const int k_g4 = a.gather4 && a.ld_k % 8 == 0 && (reinterpret_cast<uintptr_t>(a.k) & 15u) == 0 &&
                    make_map_bf16_rows(&g_map, a.k, static_cast<uint64_t>(a.ld_k), g_rows, 1);
   if (a.n_split <= 1) {
-    if ((e = launch_pdl(kernel, dim3(a.n_query, 1, 1), dim3(kThreadsAttnTc), smem, st, q_map, q_tma, k_map, k_tma, g_map, k_g4, a)) != cudaSuccess) return e;
+    if ((e = launch_pdl(kernel, dim3(a.n_query, 1, 1), dim3(threads), smem, st, q_map, q_tma, k_map, k_tma, g_map, k_g4, a)) != cudaSuccess) return e;
   } else {
     bool ok = false;
     if ((e = attn_tc_split_ok(a.n_split, &ok)) != cudaSuccess) return e;
@@ -1056,7 +1137,7 @@ cudaError_t launch_attn_tc(const AttnArgs& a, cudaStream_t st, int64_t* n_launch
     if (a.n_split > 8 && (e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess) return e;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(a.n_query, a.n_split, 1);
-    cfg.blockDim = dim3(kThreadsAttnTc);
+    cfg.blockDim = dim3(threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cudaLaunchAttribute attr[2]{};
