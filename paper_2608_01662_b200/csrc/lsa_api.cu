@@ -177,16 +177,19 @@ WsLayout ws_layout(const lsa_params* p, int64_t n_query, int64_t n_key_max, int 
 
 int* status_word(lsa_ctx* c) { return c->ws ? reinterpret_cast<int*>(c->ws) : nullptr; }
 
-// Number of row splits per sequence in paged (decode) attention.  Blocks run one per SM in waves; a block costs its
-// share of the 64-key units plus a fixed part (Q load, tensor-memory set-up, fp32 partial output), taken as six
-// units' worth.  The split count with the smallest estimate wins; ties go to fewer splits (less merging).  The
-// tcgen05 kernel merges its splits inside a thread-block cluster and takes only the counts that allows; its waves are counted
-// in clusters that fit the chip together, not in SMs: 15 clusters of eight run at once, and a 16th sequence doubled the time
-// (decode step of 16 sequences, 4 layers: 190 us as 8 splits, 144 as 4; of 36: 255 as 4, 186 as 2; of one: 77.5 as 16, 82.7 as 8;
-// of 8: 153 and 99).
-cudaError_t pick_split(int sm_count, int batch, int max_rows, bool tc_kernel, int* split) {
+// Number of row splits per sequence in paged (decode) attention, and (tcgen05 kernel) the parts, 2^v_shift, that the value dims
+// of a split are taken in by clusters of their own.  Blocks run one per SM in waves; a block costs its share of the 64-key tiles
+// plus a fixed part: about two tiles' time for Q and its start, four for its fp32 rows to leave and be merged, less where it has
+// a part of the value dims.  The smallest estimate wins; ties go to fewer splits (less merging).  The tcgen05 kernel merges its
+// splits inside a thread-block cluster; its waves are counted in clusters that fit the chip together, not in SMs: 15 clusters
+// of eight run at once, and a 16th sequence doubled the time (decode step of 16 sequences, 4 layers: 190 us as 8 splits, 144 as 4;
+// of 36: 255 as 4, 186 as 2; of one: 77.5 as 16, 82.7 as 8; of 8: 153 and 99).  Three and six splits, and parts of the value dims,
+// where all of them run at once: attention of 16 sequences, 4 layers, 126 us as 4, 117 as 6; of 40 176 as 2, 168 as 3 (of 80, in two
+// waves, 303, and 263 undivided); of one, two, three sequences 83, 83, 84 us undivided, 73 in four parts, 76 and 78 in two.
+cudaError_t pick_split(int sm_count, int batch, int max_rows, bool tc_kernel, int* split, int* v_shift) {
   const int units = (max_rows + 63) / 64;
   *split = 1;
+  *v_shift = 0;
   long best_cost = -1;
   for (int s = 1; s <= kMaxSplit && s <= units; ++s) {
     int fit = 0;
@@ -195,11 +198,16 @@ cudaError_t pick_split(int sm_count, int batch, int max_rows, bool tc_kernel, in
       if (e != cudaSuccess) return e;
       if (fit == 0) continue;
     }
-    const long waves = fit > 0 ? (batch + fit - 1) / fit : (static_cast<long>(batch) * s + sm_count - 1) / sm_count;
-    const long cost = waves * ((units + s - 1) / s + 6);
-    if (best_cost < 0 || cost < best_cost) {
-      best_cost = cost;
-      *split = s;
+    for (int v = 0; v <= (tc_kernel && s == kMaxSplit ? 2 : 0); ++v) {
+      const long jobs = static_cast<long>(batch) << v;
+      const long waves = fit > 0 ? (jobs + fit - 1) / fit : (jobs * s + sm_count - 1) / sm_count;
+      if (fit > 0 && (v > 0 || !pow2(s)) && waves > 1) continue;
+      const long cost = waves * (2 * ((units + s - 1) / s + 2) + (8 >> v));
+      if (best_cost < 0 || cost < best_cost) {
+        best_cost = cost;
+        *split = s;
+        *v_shift = v;
+      }
     }
   }
   return cudaSuccess;
@@ -368,12 +376,13 @@ int run_attn(lsa_ctx* c, const lsa_params* p, const void* q, const void* k, cons
     bool split_ok = true;
     cudaError_t es = cudaSuccess;
     a.n_split = c->tune[LSA_TUNE_ATTN_SPLIT];
-    if (a.n_split <= 0) es = pick_split(c->sm_count, batch, a.rows_ld, use_tc, &a.n_split);
+    if (a.n_split <= 0) es = pick_split(c->sm_count, batch, a.rows_ld, use_tc, &a.n_split, &a.v_shift);
     else if (use_tc) es = lsa::attn_tc_split_ok(a.n_split, &split_ok);
     if (es != cudaSuccess) return cuda_fail(c, es);
     if (!split_ok) return LSA_ERR_ARG;
     a.part_out = reinterpret_cast<float*>(c->ws + l.part_out);
-    a.part_lse = reinterpret_cast<float*>(c->ws + l.part_lse);
+    // (parts of the value dims have log-sum-exps of their own, up to 64 x 64 of them: where the fine stage, which is over, keeps keys)
+    a.part_lse = reinterpret_cast<float*>(c->ws + (a.v_shift > 0 ? l.fine_keys : l.part_lse));
   }
   if (a.H == 64 && !(v == k && ld_v == ld_k)) return LSA_ERR_SHAPE;
   cudaError_t e = timed(c, LSA_K_ATTN, [&] {

@@ -43,8 +43,8 @@
 // 18 TB/s with 216 KB in flight on each, but only a slot or so is.  The hold is a chain of hand-overs of 200-500 cycles each beside
 // the MMAs, in a load/store pipe that the copies fill.  With four softmax warps that took a maximum over each row for every
 // tile, two gather warps a slot and the last tile worked on whole, holds were 4 500 and a gathered tile 2 264 (16384 rows; now
-// 2 110), but the clock gives half of it back under the power cap: 32768 queries, two layers, 24.4 ms -> 23.7 ms; 16384 of
-// 131072, four layers, 34.5 -> 33.5 ms; 4096 of a million, four layers, 11.4 -> 11.0 ms.
+// 2 110), but the clock gives half of it back and more under the power cap: 32768 queries, two layers, 24.3 ms -> 23.7 ms; 16384
+// of 131072, four layers, 34.8 -> 34.3 ms; 4096 of a million, four layers, 11.55 -> 11.45 ms; 1237 queries, four layers, 538 -> 527 us.
 //
 // Tensor memory columns:   0-255  O: value dims 0-255 in columns 0-127, 256-511 in 128-255; lanes 0-63 hold the first 128
 //                                 dims of each, lanes 64-127 the second, lane l (mod 64) = head l
@@ -190,14 +190,14 @@ __device__ __forceinline__ bool clc_answer(uint32_t answer, int* block_x) {
 
 // With n_split > 1 the kernel must be launched with clusters of (1, n_split, 1) blocks: the splits of one sequence
 // are co-scheduled and merge their partial results themselves (no second kernel).  Block s finishes heads
-// [s * 64 / n_split, (s + 1) * 64 / n_split): every block stages its rows (normalised, fp32) in shared memory and keeps
+// [64 s / n_split, 64 (s + 1) / n_split): every block stages its rows (normalised, fp32) in shared memory and keeps
 // its own share there.
 //   Two splits (the decode configuration): the other 32 rows and their log-sum-exps are pushed straight into the
 //   peer's shared memory, behind its staged rows, by bulk copies that count bytes on the peer's mbarrier.  The cluster
 //   barrier is used in halves: a thread arrives when it has left the tile loop and waits before the first copy (the
 //   peer's ring must be out of use before it receives), and once more around the end, so that no block leaves
 //   while the other may still write into it.  Nothing goes through global memory.
-//   Four, eight or 16 splits: the rows and all log-sum-exps go to the global scratch, where they stay in L2, as 16 bulk copies of
+//   More splits: the rows and all log-sum-exps go to the global scratch, where they stay in L2, as 16 bulk copies of
 //   8 KB; after one cluster barrier the owner of a row combines the parts.  (Loads from a peer's shared memory moved the
 //   same rows at about a quarter of the L2 path's rate; a bulk copy per row took 3 000 cycles longer to issue, stores
 //   straight from the registers 4 000.)
@@ -210,7 +210,8 @@ __device__ __forceinline__ bool clc_answer(uint32_t answer, int* block_x) {
 //   kRows       the caller's row lists are walked (else [window | sink | sparse] of a contiguous cache)
 //   kClustered  the blocks of a cluster are row splits of one sequence and merge their results; else the block goes on
 //               to further queries
-template <bool kRows, bool kClustered>
+//   kParts      (clustered) 16 splits whose value dims are taken in 2 or 4 parts
+template <bool kRows, bool kClustered, bool kParts>
 __global__ void __launch_bounds__(Warps<kRows>::kThreads, 1) sparse_attn_tc_kernel(const __grid_constant__ CUtensorMap q_map, int q_tma,
                                                                             const __grid_constant__ CUtensorMap k_map, int k_tma,
                                                                             const __grid_constant__ CUtensorMap g_map, int k_g4,
@@ -222,6 +223,8 @@ __global__ void __launch_bounds__(Warps<kRows>::kThreads, 1) sparse_attn_tc_kern
   AttnTcSmem& sm = *reinterpret_cast<AttnTcSmem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
   const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
   const int split = blockIdx.y;
+  // Few sequences (clusters): value dims of a split in 2^v_shift parts, each by a cluster of its own (512 >> v_shift dims from vpart on).
+  const int v_shift = kParts ? p.v_shift : 0, vpart = kParts ? static_cast<int>(blockIdx.z) : 0;
   float* const part_out = p.part_out;
   float* const part_lse = p.part_lse;
 
@@ -633,7 +636,9 @@ __global__ void __launch_bounds__(Warps<kRows>::kThreads, 1) sparse_attn_tc_kern
   } else if (warp == kPvWarp) {
     // ================= issuer of P V =================
     if (tc::elect_one()) {
-      constexpr uint32_t idesc = tc::idesc_bf16(kH, 256, 0, 1);   // B = V read MN-major
+      // B = V read MN-major; a cluster with a part of the value dims takes half as many, or one MMA of half the width, per step
+      const uint32_t idesc = v_shift == 2 ? tc::idesc_bf16(kH, 128, 0, 1) : tc::idesc_bf16(kH, 256, 0, 1);
+      const uint32_t v_block = static_cast<uint32_t>(vpart * (8 >> v_shift)) * kAtomBytes;
       const uint64_t dv0 = tc::smem_desc_sw128(smem_u32(sm.k), kAtomBytes, 1024);   // MN-major view of a tile
       const uint64_t dp0 = tc::smem_desc_sw128(smem_u32(sm.k[0][8]), 16, 1024);     // P in its rope block
       bool ok = true;
@@ -651,11 +656,11 @@ __global__ void __launch_bounds__(Warps<kRows>::kThreads, 1) sparse_attn_tc_kern
           const uint64_t dvb = tc::desc_advance(dv0, slot * kSlotBytes), dpb = tc::desc_advance(dp0, slot * kSlotBytes);
           const int keys = tile_keys(jb, i);
 #pragma unroll
-          for (int y = 0; y < 2; ++y)       // value dims 256y .. +255
+          for (int y = 0; y < 2; ++y)       // value dims 256y .. +255 (of the cluster's part)
 #pragma unroll
             for (int kk = 0; kk < kTileKeys / 16; ++kk)   // keys 16*kk .. +15
-              if (16 * kk < keys)
-                tc::umma_ws_ss(tmem_base + 128 * y, tc::desc_advance(dpb, kk * 32), tc::desc_advance(dvb, 4 * y * kAtomBytes + kk * 2048),
+              if (16 * kk < keys && (y == 0 || v_shift == 0))
+                tc::umma_ws_ss(tmem_base + 128 * y, tc::desc_advance(dpb, kk * 32), tc::desc_advance(dvb, v_block + 4 * y * kAtomBytes + kk * 2048),
                                idesc, (i > 0) || (kk > 0));
           // "P V of the tile done" frees the ring slot for the gather warps, and tells the softmax warps that O may be touched
           // again: where a block goes on to another job by a barrier of its own, since the slot's may go on with the next
@@ -815,7 +820,7 @@ __global__ void __launch_bounds__(Warps<kRows>::kThreads, 1) sparse_attn_tc_kern
           tc::fence_after_sync();
           const float al = sm.lse_own[head_o];
 #pragma unroll 1
-          for (int c = 256 / kHalves * half; c < 256 / kHalves * (half + 1); c += 32) {
+          for (int c = (256 / kHalves >> v_shift) * half; c < (256 / kHalves >> v_shift) * (half + 1); c += 32) {
             uint32_t o[32];
             tc::tmem_ld32(tmem_base + lane_addr + c, o);
             tc::tmem_ld_wait();
@@ -854,7 +859,7 @@ __global__ void __launch_bounds__(Warps<kRows>::kThreads, 1) sparse_attn_tc_kern
             if (!clustered) {
               if (p.lse != nullptr) p.lse[static_cast<int64_t>(jb.qi) * kH + row] = lse2 / kLog2eTc;
             } else if (!pair) {
-              part_lse[(static_cast<int64_t>(jb.qi) * p.n_split + split) * kH + row] = lse2;
+              part_lse[(((static_cast<int64_t>(jb.qi) << v_shift) + vpart) * p.n_split + split) * kH + row] = lse2;
             }
           }
         }
@@ -897,10 +902,11 @@ __global__ void __launch_bounds__(Warps<kRows>::kThreads, 1) sparse_attn_tc_kern
         bar_peer = peer_smem(smem_u32(&sm.recv_full), peer);
         dst_peer = peer_smem(smem_u32(stage + kRecvOffset + half_o * kWarpStage), peer);
       }
-      uint8_t* my_warp = stage + warp * kWarpStage;
-      uint8_t* dst_part = reinterpret_cast<uint8_t*>(part_out + (static_cast<int64_t>(qi) * p.n_split + split) * kH * kDV) + warp * kWarpStage;
+      uint8_t* my_warp = stage + quarter * (kWarpStage >> v_shift);
+      uint8_t* dst_part = reinterpret_cast<uint8_t*>(part_out + (((static_cast<int64_t>(qi) << v_shift) + vpart) * p.n_split + split) * (kH * kDV >> v_shift)) +
+                          quarter * (kWarpStage >> v_shift);
 #pragma unroll 1
-      for (int c = 0; c < 256; c += 64) {
+      for (int c = 0; c < 256 >> v_shift; c += 64) {
         uint32_t o[64];
         if (have_o) {
           tc::tmem_ld64(tmem_base + lane_addr + c, o);
@@ -1021,23 +1027,25 @@ __global__ void __launch_bounds__(Warps<kRows>::kThreads, 1) sparse_attn_tc_kern
       cluster_wait();   // (see the arrival above)
     } else {
       cluster_sync_all();   // every block of the cluster has written its rows
-      // A warp finishes 16 / n of the four 128-dim runs of one row: its 16 loads (n parts of each) and the log-sum-exps are
-      // asked for together, one trip to L2.  (A row per warp, four
-      // parts at a time, was 4 600 cycles with 16 splits; decode step of one sequence, 4 layers: 77.2 us, 74.3 now.)
-      auto merge = [&](auto parts) {
-        constexpr int N = decltype(parts)::value, kRuns = 16 / N;
-        static_assert(kWarps >= 16, "sixteen warps have a share of the block's 64 / N rows");
-        const int rl = 4 * warp / N, u0 = warp * kRuns & 3, R = row0 + rl;
-        const float my_l = lane >= N ? -INFINITY : lane == split ? sm.lse_own[R] : __ldcg(part_lse + (static_cast<int64_t>(qi) * N + lane) * kH + R);
-        const uint8_t* src = reinterpret_cast<const uint8_t*>(part_out + static_cast<int64_t>(qi) * N * kH * kDV) +
-                             (R >> 5) * kWarpStage + (lane >> 4) * 8192 + (R & 31) * 256 + (((lane & 15) ^ (R & 15)) << 4);
+      // A warp finishes kRuns of the four 128-dim runs of row R, from run u0 on: its loads (n parts of each run) and the log-sum-exps
+      // are asked for together, one trip to L2.  (A row per warp, four parts at a time, was 4 600 cycles with 16 splits; decode
+      // step of one sequence, 4 layers: 77.2 us, 74.3 so.  Runs of several rows per warp: 16 sequences 125 us, 138.)
+      auto merge = [&](auto parts, auto runs, int R, int u0) {
+        constexpr int N = decltype(parts)::value, kRuns = decltype(runs)::value;
+        // (value dims in parts, 16 splits only: a row is 4 >> v_shift runs, and of a quarter of the dims a run's second half lies with
+        // the rows that the warps of other lanes staged)
+        const int vs = N == 16 ? v_shift : 0, warp_stage = kWarpStage >> vs;   // (v_shift is 0 where the kernel is not built for parts)
+        const int64_t job = (static_cast<int64_t>(qi) << vs) + vpart;
+        const float my_l = lane >= N ? -INFINITY : lane == split ? sm.lse_own[R] : __ldcg(part_lse + (job * N + lane) * kH + R);
+        const uint8_t* src = reinterpret_cast<const uint8_t*>(part_out) + job * N * (kH * kDV * 4 >> vs) +
+                             (R >> 5) * warp_stage + (lane >> 4) * (vs == 2 ? 2 * warp_stage : 8192) + (R & 31) * 256 + (((lane & 15) ^ (R & 15)) << 4);
         float4 v[kRuns][N];
 #pragma unroll
         for (int i = 0; i < kRuns; ++i)
 #pragma unroll
           for (int j = 0; j < N; ++j) {   // dims 128u + 4 lane .. + 3 of part j: see the pair's version
             const int u = u0 + i;
-            v[i][j] = __ldcg(reinterpret_cast<const float4*>(src + j * (kH * kDV * 4) + (u & 1) * 2 * kWarpStage + (u >> 1) * 2 * 8192));
+            v[i][j] = __ldcg(reinterpret_cast<const float4*>(src + j * (kH * kDV * 4 >> vs) + (u & 1) * 2 * warp_stage + (u >> 1) * 2 * 8192));
           }
         float m = my_l;
 #pragma unroll
@@ -1047,7 +1055,7 @@ __global__ void __launch_bounds__(Warps<kRows>::kThreads, 1) sparse_attn_tc_kern
 #pragma unroll
         for (int d = 1; d < N; d <<= 1) den += __shfl_xor_sync(0xffffffffu, den, d);
         wgt = den > 0.f ? wgt / den : 0.f;
-        if (p.lse != nullptr && lane == 0 && u0 == 0)
+        if (p.lse != nullptr && lane == 0 && u0 == 0 && vpart == 0)
           p.lse[static_cast<int64_t>(qi) * kH + R] = den > 0.f ? (m + log2f(den)) / kLog2eTc : -INFINITY;
         float4 acc[kRuns] = {};
 #pragma unroll
@@ -1063,13 +1071,31 @@ __global__ void __launch_bounds__(Warps<kRows>::kThreads, 1) sparse_attn_tc_kern
           uint2 o;
           o.x = pack_bf16(acc[i].x, acc[i].y);
           o.y = pack_bf16(acc[i].z, acc[i].w);
-          *reinterpret_cast<uint2*>(out + static_cast<int64_t>(rl) * kDV + (lane + 32 * (u0 + i)) * 4) = o;
+          *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(p.out) + (static_cast<int64_t>(qi) * kH + R) * kDV +
+                                    (lane + 32 * (vpart * (4 >> vs) + u0 + i)) * 4) = o;
         }
       };
-      if (warp >= 16) {}
-      else if (n == 16) merge(IntC<16>{});
-      else if (n == 8) merge(IntC<8>{});
-      else merge(IntC<4>{});
+      static_assert(kWarps >= 16, "sixteen warps have a share of a block's rows");
+      // a number of splits that does not divide the rows: half a row at a time, dealt to all warps
+      [[maybe_unused]] auto merge_dealt = [&](auto parts) {
+        const int r0 = kH * split / n, halves = 2 * (kH * (split + 1) / n - r0);
+        for (int h = warp; h < halves; h += kWarps) merge(parts, IntC<2>{}, r0 + (h >> 1), 2 * (h & 1));
+      };
+      if constexpr (kParts) {
+        if (warp < 16 >> v_shift) merge(IntC<16>{}, IntC<1>{}, row0 + (warp >> (2 - v_shift)), warp & (3 >> v_shift));
+      } else {
+        if (n == 16) {
+          if (warp < 16) merge(IntC<16>{}, IntC<1>{}, row0 + (warp >> 2), warp & 3);
+        } else if (n == 8) {
+          if (warp < 16) merge(IntC<8>{}, IntC<2>{}, row0 + (warp >> 1), 2 * (warp & 1));
+        } else if (n == 4) {
+          if (warp < 16) merge(IntC<4>{}, IntC<4>{}, row0 + warp, 0);
+        } else if (n == 6) {
+          merge_dealt(IntC<6>{});
+        } else {
+          merge_dealt(IntC<3>{});
+        }
+      }
     }
   }
 }
@@ -1082,26 +1108,28 @@ using AttnTcKernel = void (*)(CUtensorMap, int, CUtensorMap, int, CUtensorMap, i
 
 // The instantiation that serves a call (see the kernel's template parameters).
 static AttnTcKernel pick_kernel(const AttnArgs& a) {
-  if (a.rows == nullptr) return sparse_attn_tc_kernel<false, false>;
-  return a.n_split > 1 ? sparse_attn_tc_kernel<true, true> : sparse_attn_tc_kernel<true, false>;
+  if (a.rows == nullptr) return sparse_attn_tc_kernel<false, false, false>;
+  if (a.n_split <= 1) return sparse_attn_tc_kernel<true, false, false>;
+  return a.v_shift > 0 ? sparse_attn_tc_kernel<true, true, true> : sparse_attn_tc_kernel<true, true, false>;
 }
 
+// (Clusters that run at once: 74 of 2 blocks, 45 of 3, 33 of 4, 26 of 5, 22 of 6, 15 of 7 to 9, 7 of 11 to 16.  Five gained nothing
+// over four: 24 sequences, four layers, 132 and 133 us.)
 cudaError_t attn_tc_resident(int n_split, int* clusters) {
-  static DeviceCount n[4];
-  const int at = n_split == 2 ? 0 : n_split == 4 ? 1 : n_split == 8 ? 2 : n_split == kMaxClusterSplit ? 3 : -1;
+  static DeviceCount n[kMaxClusterSplit + 1];
   *clusters = 0;
-  if (at < 0) return cudaSuccess;
-  return n[at].get(clusters, [&](int* c) {
-    return resident_clusters(reinterpret_cast<const void*>(sparse_attn_tc_kernel<true, true>), Warps<true>::kThreads, sizeof(AttnTcSmem) + 1024, n_split, c);
+  const bool merged = (n_split >= 2 && n_split <= 4) || n_split == 6 || n_split == 8 || n_split == kMaxClusterSplit;
+  if (!merged) return cudaSuccess;
+  return n[n_split].get(clusters, [&](int* c) {
+    return resident_clusters(reinterpret_cast<const void*>(sparse_attn_tc_kernel<true, true, false>), Warps<true>::kThreads, sizeof(AttnTcSmem) + 1024, n_split, c);
   });
 }
 
-// Row splits the tcgen05 kernel can merge inside a cluster: a power of two that divides the 64 heads, as many blocks as the
-// device can co-schedule.
+// Row splits that a caller may ask for: the powers of two, as many blocks as the device can co-schedule.
 cudaError_t attn_tc_split_ok(int n_split, bool* ok) {
   int n = 0;
   const cudaError_t e = attn_tc_resident(n_split, &n);
-  *ok = n_split == 1 || n > 0;
+  *ok = n_split == 1 || (n > 0 && (n_split & (n_split - 1)) == 0);
   return e;
 }
 
@@ -1131,12 +1159,12 @@ cudaError_t launch_attn_tc(const AttnArgs& a, cudaStream_t st, int64_t* n_launch
   if (a.n_split <= 1) {
     if ((e = launch_pdl(kernel, dim3(a.n_query, 1, 1), dim3(threads), smem, st, q_map, q_tma, k_map, k_tma, g_map, k_g4, a)) != cudaSuccess) return e;
   } else {
-    bool ok = false;
-    if ((e = attn_tc_split_ok(a.n_split, &ok)) != cudaSuccess) return e;
-    if (!ok) return cudaErrorInvalidValue;
+    int fit = 0;
+    if ((e = attn_tc_resident(a.n_split, &fit)) != cudaSuccess) return e;
+    if (fit == 0) return cudaErrorInvalidValue;
     if (a.n_split > 8 && (e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess) return e;
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(a.n_query, a.n_split, 1);
+    cfg.gridDim = dim3(a.n_query, a.n_split, 1 << a.v_shift);
     cfg.blockDim = dim3(threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;

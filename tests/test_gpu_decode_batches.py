@@ -38,3 +38,19 @@ def test_sixteen_splits(cuda_device, batch, lo, hi):
     assert wl.ctx.status() == 0
     m = pu.check_decode(wl, range(batch))
     m.assert_ok(pu.TOL_BF16)
+
+
+@pytest.mark.parametrize("batch,lo,hi", [(1, 20000, 20000), (1, 300, 300), (2, 700, 30000), (3, 1, 5000)])
+def test_parts_of_the_value_dims(cuda_device, batch, lo, hi):
+    """Few sequences: the value dims of a split in parts, each by a cluster of its own, give the bits of the undivided ones."""
+    cfg = CONFIGS["cfg4"].replace(batch=batch, ctx_lo=lo, ctx_hi=hi, R=2, seed=batch)
+    wl = DecodeWorkload(cfg, cuda_device)
+    wl.prepare()
+    wl.step()
+    parts = [t.clone() for t in wl.out + wl.lse]
+    m = pu.check_decode(wl, range(batch))
+    m.assert_ok(pu.TOL_BF16)
+    wl.ctx.tune(2, 16)             # LSA_TUNE_ATTN_SPLIT
+    wl.step()
+    assert wl.ctx.status() == 0
+    assert all(torch.equal(a, b) for a, b in zip(parts, wl.out + wl.lse))
