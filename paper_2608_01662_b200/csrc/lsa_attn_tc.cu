@@ -210,8 +210,10 @@ __device__ __forceinline__ bool clc_answer(uint32_t answer, int* block_x) {
 //   kRows       the caller's row lists are walked (else [window | sink | sparse] of a contiguous cache)
 //   kClustered  the blocks of a cluster are row splits of one sequence and merge their results; else the block goes on
 //               to further queries
-//   kParts      (clustered) 16 splits whose value dims are taken in 2 or 4 parts
-template <bool kRows, bool kClustered, bool kParts>
+//   kMerge      (clustered) how the splits' rows are put together: a kernel has the code of one way only, because it runs once per
+//               block, behind the fetch of its instructions (all in one kernel: 1 to 2 % of a step of 4 to 7 sequences)
+enum Merge { kPowers, kParts, kDealt };   // 2, 4, 8 or 16 splits; 16 with the value dims in 2 or 4 parts; 3 or 6
+template <bool kRows, bool kClustered, Merge kMerge>
 __global__ void __launch_bounds__(Warps<kRows>::kThreads, 1) sparse_attn_tc_kernel(const __grid_constant__ CUtensorMap q_map, int q_tma,
                                                                             const __grid_constant__ CUtensorMap k_map, int k_tma,
                                                                             const __grid_constant__ CUtensorMap g_map, int k_g4,
@@ -224,12 +226,12 @@ __global__ void __launch_bounds__(Warps<kRows>::kThreads, 1) sparse_attn_tc_kern
   const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
   const int split = blockIdx.y;
   // Few sequences (clusters): value dims of a split in 2^v_shift parts, each by a cluster of its own (512 >> v_shift dims from vpart on).
-  const int v_shift = kParts ? p.v_shift : 0, vpart = kParts ? static_cast<int>(blockIdx.z) : 0;
+  const int v_shift = kMerge == kParts ? p.v_shift : 0, vpart = kMerge == kParts ? static_cast<int>(blockIdx.z) : 0;
   float* const part_out = p.part_out;
   float* const part_lse = p.part_lse;
 
   constexpr bool clustered = kClustered;
-  const bool pair = kClustered && p.n_split == 2;   // two splits exchange their rows through shared memory
+  const bool pair = kClustered && kMerge == kPowers && p.n_split == 2;   // two splits exchange their rows through shared memory
   const bool raised = tc::status_raised(p.status);   // an earlier block of this launch (or an earlier launch) gave up on a wait
 
   // ---- set-up
@@ -1081,20 +1083,15 @@ __global__ void __launch_bounds__(Warps<kRows>::kThreads, 1) sparse_attn_tc_kern
         const int r0 = kH * split / n, halves = 2 * (kH * (split + 1) / n - r0);
         for (int h = warp; h < halves; h += kWarps) merge(parts, IntC<2>{}, r0 + (h >> 1), 2 * (h & 1));
       };
-      if constexpr (kParts) {
+      if constexpr (kMerge == kParts) {
         if (warp < 16 >> v_shift) merge(IntC<16>{}, IntC<1>{}, row0 + (warp >> (2 - v_shift)), warp & (3 >> v_shift));
-      } else {
-        if (n == 16) {
-          if (warp < 16) merge(IntC<16>{}, IntC<1>{}, row0 + (warp >> 2), warp & 3);
-        } else if (n == 8) {
-          if (warp < 16) merge(IntC<8>{}, IntC<2>{}, row0 + (warp >> 1), 2 * (warp & 1));
-        } else if (n == 4) {
-          if (warp < 16) merge(IntC<4>{}, IntC<4>{}, row0 + warp, 0);
-        } else if (n == 6) {
-          merge_dealt(IntC<6>{});
-        } else {
-          merge_dealt(IntC<3>{});
-        }
+      } else if constexpr (kMerge == kDealt) {
+        if (n == 6) merge_dealt(IntC<6>{});
+        else merge_dealt(IntC<3>{});
+      } else if (warp < 16) {
+        if (n == 16) merge(IntC<16>{}, IntC<1>{}, row0 + (warp >> 2), warp & 3);
+        else if (n == 8) merge(IntC<8>{}, IntC<2>{}, row0 + (warp >> 1), 2 * (warp & 1));
+        else merge(IntC<4>{}, IntC<4>{}, row0 + warp, 0);
       }
     }
   }
@@ -1108,9 +1105,10 @@ using AttnTcKernel = void (*)(CUtensorMap, int, CUtensorMap, int, CUtensorMap, i
 
 // The instantiation that serves a call (see the kernel's template parameters).
 static AttnTcKernel pick_kernel(const AttnArgs& a) {
-  if (a.rows == nullptr) return sparse_attn_tc_kernel<false, false, false>;
-  if (a.n_split <= 1) return sparse_attn_tc_kernel<true, false, false>;
-  return a.v_shift > 0 ? sparse_attn_tc_kernel<true, true, true> : sparse_attn_tc_kernel<true, true, false>;
+  if (a.rows == nullptr) return sparse_attn_tc_kernel<false, false, kPowers>;
+  if (a.n_split <= 1) return sparse_attn_tc_kernel<true, false, kPowers>;
+  if (a.v_shift > 0) return sparse_attn_tc_kernel<true, true, kParts>;
+  return a.n_split == 3 || a.n_split == 6 ? sparse_attn_tc_kernel<true, true, kDealt> : sparse_attn_tc_kernel<true, true, kPowers>;
 }
 
 // (Clusters that run at once: 74 of 2 blocks, 45 of 3, 33 of 4, 26 of 5, 22 of 6, 15 of 7 to 9, 7 of 11 to 16.  Five gained nothing
@@ -1121,7 +1119,7 @@ cudaError_t attn_tc_resident(int n_split, int* clusters) {
   const bool merged = (n_split >= 2 && n_split <= 4) || n_split == 6 || n_split == 8 || n_split == kMaxClusterSplit;
   if (!merged) return cudaSuccess;
   return n[n_split].get(clusters, [&](int* c) {
-    return resident_clusters(reinterpret_cast<const void*>(sparse_attn_tc_kernel<true, true, false>), Warps<true>::kThreads, sizeof(AttnTcSmem) + 1024, n_split, c);
+    return resident_clusters(reinterpret_cast<const void*>(sparse_attn_tc_kernel<true, true, kPowers>), Warps<true>::kThreads, sizeof(AttnTcSmem) + 1024, n_split, c);
   });
 }
 
