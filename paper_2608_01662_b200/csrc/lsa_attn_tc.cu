@@ -210,15 +210,17 @@ __device__ __forceinline__ bool clc_answer(uint32_t answer, int* block_x) {
 //   kRows       the caller's row lists are walked (else [window | sink | sparse] of a contiguous cache)
 //   kClustered  the blocks of a cluster are row splits of one sequence and merge their results; else the block goes on
 //               to further queries
-//   kMerge      (clustered) how the splits' rows are put together: a kernel has the code of one way only, because it runs once per
-//               block, behind the fetch of its instructions (all in one kernel: 1 to 2 % of a step of 4 to 7 sequences)
-enum Merge { kPowers, kParts, kDealt };   // 2, 4, 8 or 16 splits; 16 with the value dims in 2 or 4 parts; 3 or 6
-template <bool kRows, bool kClustered, Merge kMerge>
+//   kSplits     row splits of a sequence (1: no cluster).  A kernel has the code of one merge only, because it runs once per block,
+//               behind the fetch of its instructions (all in one kernel: 1 to 2 % of a decode step)
+//   kParts      16 splits whose value dims are taken in 2 or 4 parts
+template <bool kRows, int kSplits, bool kParts>
 __global__ void __launch_bounds__(Warps<kRows>::kThreads, 1) sparse_attn_tc_kernel(const __grid_constant__ CUtensorMap q_map, int q_tma,
                                                                             const __grid_constant__ CUtensorMap k_map, int k_tma,
                                                                             const __grid_constant__ CUtensorMap g_map, int k_g4,
                                                                             AttnArgs p) {
   using W = Warps<kRows>;
+  constexpr bool kClustered = kSplits > 1;
+  static_assert(kRows || !kClustered, "row splits walk row lists");
   constexpr int kHalves = W::kHalves, kSoftmaxWarps = W::kSoftmax, kDrainWarp0 = W::kDrain0, kQkWarp = W::kQk, kPvWarp = W::kPv, kGatherWarp0 = W::kGather0;
   constexpr int kSlotWarps = W::kSlot, kRowsPerWarp = W::kRowsEach, kJobReaders = W::kJobReaders, kSoftmaxThreads = 32 * kSoftmaxWarps;
   extern __shared__ uint8_t smem_raw[];
@@ -226,12 +228,12 @@ __global__ void __launch_bounds__(Warps<kRows>::kThreads, 1) sparse_attn_tc_kern
   const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
   const int split = blockIdx.y;
   // Few sequences (clusters): value dims of a split in 2^v_shift parts, each by a cluster of its own (512 >> v_shift dims from vpart on).
-  const int v_shift = kMerge == kParts ? p.v_shift : 0, vpart = kMerge == kParts ? static_cast<int>(blockIdx.z) : 0;
+  const int v_shift = kParts ? p.v_shift : 0, vpart = kParts ? static_cast<int>(blockIdx.z) : 0;
   float* const part_out = p.part_out;
   float* const part_lse = p.part_lse;
 
   constexpr bool clustered = kClustered;
-  const bool pair = kClustered && kMerge == kPowers && p.n_split == 2;   // two splits exchange their rows through shared memory
+  constexpr bool pair = kSplits == 2;   // two splits exchange their rows through shared memory
   const bool raised = tc::status_raised(p.status);   // an earlier block of this launch (or an earlier launch) gave up on a wait
 
   // ---- set-up
@@ -255,7 +257,7 @@ __global__ void __launch_bounds__(Warps<kRows>::kThreads, 1) sparse_attn_tc_kern
     tc::mbar_init(smem_u32(&sm.o_free), kDrainWarps);
     if constexpr (kClustered) {
       tc::mbar_init(smem_u32(&sm.recv_full), 1);
-      if (p.n_split == 2) tc::mbar_expect_tx(smem_u32(&sm.recv_full), kRecvBytes);   // armed once; used once per launch
+      if (pair) tc::mbar_expect_tx(smem_u32(&sm.recv_full), kRecvBytes);   // armed once; used once per launch
     }
     sm.fail = 0;
     tc::fence_mbar_init();
@@ -306,7 +308,7 @@ __global__ void __launch_bounds__(Warps<kRows>::kThreads, 1) sparse_attn_tc_kern
       b.n_win = static_cast<int>(max64(0, t - b.win0 + 1));
     }
     const int tiles_all = (b.n_tot + kTileKeys - 1) / kTileKeys;
-    const int tiles_per = kClustered ? (tiles_all + p.n_split - 1) / p.n_split : tiles_all;
+    const int tiles_per = kClustered ? (tiles_all + kSplits - 1) / kSplits : tiles_all;
     b.tile_begin = kClustered ? split * tiles_per : 0;
     b.n_tiles = max(0, min(tiles_all, b.tile_begin + tiles_per) - b.tile_begin);
     if (dead) b.n_tiles = 0;   // the peers of this cluster still expect this block at the cluster barrier
@@ -861,7 +863,7 @@ __global__ void __launch_bounds__(Warps<kRows>::kThreads, 1) sparse_attn_tc_kern
             if (!clustered) {
               if (p.lse != nullptr) p.lse[static_cast<int64_t>(jb.qi) * kH + row] = lse2 / kLog2eTc;
             } else if (!pair) {
-              part_lse[(((static_cast<int64_t>(jb.qi) << v_shift) + vpart) * p.n_split + split) * kH + row] = lse2;
+              part_lse[(((static_cast<int64_t>(jb.qi) << v_shift) + vpart) * kSplits + split) * kH + row] = lse2;
             }
           }
         }
@@ -905,7 +907,7 @@ __global__ void __launch_bounds__(Warps<kRows>::kThreads, 1) sparse_attn_tc_kern
         dst_peer = peer_smem(smem_u32(stage + kRecvOffset + half_o * kWarpStage), peer);
       }
       uint8_t* my_warp = stage + quarter * (kWarpStage >> v_shift);
-      uint8_t* dst_part = reinterpret_cast<uint8_t*>(part_out + (((static_cast<int64_t>(qi) << v_shift) + vpart) * p.n_split + split) * (kH * kDV >> v_shift)) +
+      uint8_t* dst_part = reinterpret_cast<uint8_t*>(part_out + (((static_cast<int64_t>(qi) << v_shift) + vpart) * kSplits + split) * (kH * kDV >> v_shift)) +
                           quarter * (kWarpStage >> v_shift);
 #pragma unroll 1
       for (int c = 0; c < 256 >> v_shift; c += 64) {
@@ -964,13 +966,13 @@ __global__ void __launch_bounds__(Warps<kRows>::kThreads, 1) sparse_attn_tc_kern
     // ---- merge of the splits (Sec. 4.1.1: online-softmax rescaling) for this block's heads: weights
     // 2^(lse_j - max) / sum, O = sum_j w_j O_j, bf16 to global.
     const int qi = blockIdx.x;
-    const int n = p.n_split;
-    const int rows_per = kH / n;
+    constexpr int n = kSplits;
+    constexpr int rows_per = kH / n;
     const int row0 = split * rows_per;
     const uint8_t* stage = &sm.k[0][0][0];
     constexpr int kWarps = W::kAll;
     __nv_bfloat16* out = reinterpret_cast<__nv_bfloat16*>(p.out) + (static_cast<int64_t>(qi) * kH + row0) * kDV;
-    if (pair) {
+    if constexpr (pair) {
       if (warp >= kSoftmaxWarps) cluster_wait();   // (the softmax warps completed this phase before they sent)
       // the peer's rows for this block's heads, and their log-sum-exps, are in shared memory when the byte count is met
       (void)tc::mbar_wait(smem_u32(&sm.recv_full), 0, p.status);
@@ -1083,15 +1085,12 @@ __global__ void __launch_bounds__(Warps<kRows>::kThreads, 1) sparse_attn_tc_kern
         const int r0 = kH * split / n, halves = 2 * (kH * (split + 1) / n - r0);
         for (int h = warp; h < halves; h += kWarps) merge(parts, IntC<2>{}, r0 + (h >> 1), 2 * (h & 1));
       };
-      if constexpr (kMerge == kParts) {
+      if constexpr (kParts) {
         if (warp < 16 >> v_shift) merge(IntC<16>{}, IntC<1>{}, row0 + (warp >> (2 - v_shift)), warp & (3 >> v_shift));
-      } else if constexpr (kMerge == kDealt) {
-        if (n == 6) merge_dealt(IntC<6>{});
-        else merge_dealt(IntC<3>{});
-      } else if (warp < 16) {
-        if (n == 16) merge(IntC<16>{}, IntC<1>{}, row0 + (warp >> 2), warp & 3);
-        else if (n == 8) merge(IntC<8>{}, IntC<2>{}, row0 + (warp >> 1), 2 * (warp & 1));
-        else merge(IntC<4>{}, IntC<4>{}, row0 + warp, 0);
+      } else if constexpr (n == 3 || n == 6) {
+        merge_dealt(IntC<n>{});
+      } else {   // a warp has 16 / n of the runs of one row
+        if (warp < 16) merge(IntC<n>{}, IntC<16 / n>{}, row0 + 4 * warp / n, warp * (16 / n) & 3);
       }
     }
   }
@@ -1105,10 +1104,16 @@ using AttnTcKernel = void (*)(CUtensorMap, int, CUtensorMap, int, CUtensorMap, i
 
 // The instantiation that serves a call (see the kernel's template parameters).
 static AttnTcKernel pick_kernel(const AttnArgs& a) {
-  if (a.rows == nullptr) return sparse_attn_tc_kernel<false, false, kPowers>;
-  if (a.n_split <= 1) return sparse_attn_tc_kernel<true, false, kPowers>;
-  if (a.v_shift > 0) return sparse_attn_tc_kernel<true, true, kParts>;
-  return a.n_split == 3 || a.n_split == 6 ? sparse_attn_tc_kernel<true, true, kDealt> : sparse_attn_tc_kernel<true, true, kPowers>;
+  if (a.rows == nullptr) return sparse_attn_tc_kernel<false, 1, false>;
+  switch (a.n_split) {
+    case 2: return sparse_attn_tc_kernel<true, 2, false>;
+    case 3: return sparse_attn_tc_kernel<true, 3, false>;
+    case 4: return sparse_attn_tc_kernel<true, 4, false>;
+    case 6: return sparse_attn_tc_kernel<true, 6, false>;
+    case 8: return sparse_attn_tc_kernel<true, 8, false>;
+    case kMaxClusterSplit: return a.v_shift > 0 ? sparse_attn_tc_kernel<true, kMaxClusterSplit, true> : sparse_attn_tc_kernel<true, kMaxClusterSplit, false>;
+    default: return sparse_attn_tc_kernel<true, 1, false>;
+  }
 }
 
 // (Clusters that run at once: 74 of 2 blocks, 45 of 3, 33 of 4, 26 of 5, 22 of 6, 15 of 7 to 9, 7 of 11 to 16.  Five gained nothing
@@ -1119,7 +1124,7 @@ cudaError_t attn_tc_resident(int n_split, int* clusters) {
   const bool merged = (n_split >= 2 && n_split <= 4) || n_split == 6 || n_split == 8 || n_split == kMaxClusterSplit;
   if (!merged) return cudaSuccess;
   return n[n_split].get(clusters, [&](int* c) {
-    return resident_clusters(reinterpret_cast<const void*>(sparse_attn_tc_kernel<true, true, kPowers>), Warps<true>::kThreads, sizeof(AttnTcSmem) + 1024, n_split, c);
+    return resident_clusters(reinterpret_cast<const void*>(sparse_attn_tc_kernel<true, kMaxClusterSplit, false>), Warps<true>::kThreads, sizeof(AttnTcSmem) + 1024, n_split, c);
   });
 }
 
