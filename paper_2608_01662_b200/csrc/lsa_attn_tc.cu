@@ -208,10 +208,9 @@ __device__ __forceinline__ bool clc_answer(uint32_t answer, int* block_x) {
 // describes the cache rows with a box one row high, and every other key tile is gathered four rows per instruction.
 //
 //   kRows       the caller's row lists are walked (else [window | sink | sparse] of a contiguous cache)
-//   kClustered  the blocks of a cluster are row splits of one sequence and merge their results; else the block goes on
-//               to further queries
-//   kSplits     row splits of a sequence (1: no cluster).  A kernel has the code of one merge only, because it runs once per block,
-//               behind the fetch of its instructions (all in one kernel: 1 to 2 % of a decode step)
+//   kSplits     row splits of a sequence: more than one are the blocks of a cluster and merge their results, with one the block goes
+//               on to further queries.  A kernel has the code of one merge only, because it runs once per block, behind the fetch
+//               of its instructions (all in one kernel: 1 to 3 % of a decode step; one sequence 68.1 us, 66.5 so, 24 137.1 and 134.6)
 //   kParts      16 splits whose value dims are taken in 2 or 4 parts
 template <bool kRows, int kSplits, bool kParts>
 __global__ void __launch_bounds__(Warps<kRows>::kThreads, 1) sparse_attn_tc_kernel(const __grid_constant__ CUtensorMap q_map, int q_tma,

@@ -54,3 +54,15 @@ def test_parts_of_the_value_dims(cuda_device, batch, lo, hi):
     wl.step()
     assert wl.ctx.status() == 0
     assert all(torch.equal(a, b) for a, b in zip(parts, wl.out + wl.lse))
+
+
+@pytest.mark.parametrize("batch,lo,hi", [(16, 700, 6000), (22, 1, 400), (34, 900, 3000), (45, 1, 2500)])
+def test_splits_that_do_not_divide_the_rows(cuda_device, batch, lo, hi):
+    """Six row splits (16 to 22 sequences) and three (34 to 45), also where some of them have no rows."""
+    cfg = CONFIGS["cfg4"].replace(batch=batch, ctx_lo=lo, ctx_hi=hi, R=2, seed=batch)
+    wl = DecodeWorkload(cfg, cuda_device)
+    wl.prepare()
+    wl.step()
+    assert wl.ctx.status() == 0
+    m = pu.check_decode(wl, range(0, batch, 3))
+    m.assert_ok(pu.TOL_BF16)
