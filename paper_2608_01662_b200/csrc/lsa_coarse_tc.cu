@@ -249,198 +249,6 @@ coarse_score_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
     score_again(p, q0, nq, static_cast<int64_t>(tile0) * kTileM >> spp_shift, static_cast<int64_t>(tile0 + n_tiles) * kTileM >> spp_shift);
 }
 
-// ---- page scores with the heads as rows of the accumulator ----
-//
-// Where a page is 8, 16 or 32 sub-blocks the product is taken the other way round: its rows are 32 heads of four queries (a
-// query's heads 0-31 in one unit, 32-63 in the next: M = 128), its columns the 128 mean keys of a tile.  A thread of the
-// epilogue then holds one head of one query and 32 mean keys: it sums their ReLUs over a page before it multiplies by its
-// head's weight, a register, and the lanes' sums meet by shuffles once per page and query.  Q lies in tensor memory (the rows
-// of a unit are 64 columns of packed bf16), so that shared memory feeds the MMAs one operand only, and the epilogue nothing.
-// With the mean keys as rows (above) 16 broadcast loads of weights per row and query and both operands of the MMAs share that pipe:
-// 4096 queries against a million keys 7.5 ms, 6.5 so; 16384 against 131072 3.57 and 3.16; a prompt of 32768 1.01 and 0.96.  An
-// accumulator comes back to the MMAs about 700 cycles after they finished it, of which the other one covers 512; units of 64 mean
-// keys in four accumulators 7.5 ms (an MMA reads its 128 rows of Q however many columns it has), the epilogue in two sets of eight
-// warps of 64 columns, one per four queries, 7.2.
-//   warp 0      TMA producer: mean-key tiles
-//   warp 1      issues tcgen05.mma (M128 N128 K16, Q from tensor memory): four units of a tile, two accumulators in turn
-//   warps 2-17  epilogue: lane quarter x quarter of the columns; at the start they move Q to tensor memory
-// Tensor memory: 0-255 Q of the four units, 256-511 the accumulators.
-constexpr int kPageQ = 8, kUnits = 4, kPageStages = 5;
-
-struct CoarsePageSmem {
-  alignas(1024) uint8_t a[kPageStages][kTileBytesA];
-  alignas(8) uint64_t full[kPageStages], empty[kPageStages], q_ready, acc_full[2], acc_empty[2];
-  uint32_t tmem_slot;
-  int again;   // a score is not finite
-};
-
-__global__ void __launch_bounds__(kThreadsTc, 1)
-coarse_page_scores_kernel(const __grid_constant__ CUtensorMap map_km, int parts, const __grid_constant__ IndexArgs p) {
-  extern __shared__ uint8_t smem_raw[];
-  CoarsePageSmem& sm = *reinterpret_cast<CoarsePageSmem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-  const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
-  pdl_wait();
-  pdl_launch_dependents();
-
-  // heavy blocks first: the first blocks take the last queries.  A query block's tiles are dealt to `parts` blocks.
-  const int qb = (gridDim.x - 1 - blockIdx.x) / parts, part = static_cast<int>(blockIdx.x) % parts;
-  const int q0 = qb * kPageQ;
-  const int nq = min(kPageQ, p.n_query - q0);
-  const int64_t t_max = p.q_pos0 + q0 + nq - 1;
-  const int64_t t_need = (static_cast<int64_t>(p.M) + p.S / p.P) * p.P + p.W;  // first query with more than M eligible pages
-  if (t_max < t_need) return;
-  if (tc::block_gives_up(p.status)) return;   // an earlier block of this launch gave up on a wait
-  const int spp = p.P / p.B;
-  const int spp_shift = 31 - __clz(spp);
-  const int tiles_all = static_cast<int>((t_max - p.W) / (static_cast<int64_t>(kTileM) * p.B)) + 1;
-  const int tile0 = static_cast<int>(static_cast<int64_t>(tiles_all) * part / parts);
-  const int n_tiles = static_cast<int>(static_cast<int64_t>(tiles_all) * (part + 1) / parts) - tile0;
-  if (n_tiles <= 0) return;
-
-  // ---- set-up
-  if (tid == 0) {
-    for (int s = 0; s < kPageStages; ++s) {
-      tc::mbar_init(smem_u32(&sm.full[s]), 1);
-      tc::mbar_init(smem_u32(&sm.empty[s]), 1);
-    }
-    tc::mbar_init(smem_u32(&sm.q_ready), kEpiWarps);
-    for (int b = 0; b < 2; ++b) {
-      tc::mbar_init(smem_u32(&sm.acc_full[b]), 1);
-      tc::mbar_init(smem_u32(&sm.acc_empty[b]), kEpiWarps);
-    }
-    sm.again = 0;
-    tc::fence_mbar_init();
-  }
-  if (warp == 1) {
-    tc::tmem_alloc(smem_u32(&sm.tmem_slot), kTmemCols);
-    tc::tmem_relinquish();
-  }
-  tc::fence_before_sync();
-  __syncthreads();
-  tc::fence_after_sync();
-  const uint32_t tmem_base = sm.tmem_slot, acc_base = tmem_base + kUnits * (kDI / 2);
-
-  if (warp == 0) {
-    // ================= producer =================
-    if (tc::elect_one()) {
-      for (int k = 0; k < n_tiles; ++k) {
-        const int s = k % kPageStages;
-        if (!tc::mbar_wait(smem_u32(&sm.empty[s]), ((k / kPageStages) & 1) ^ 1, p.status)) break;
-        tc::mbar_expect_tx(smem_u32(&sm.full[s]), kTileBytesA);
-        for (int a = 0; a < 2; ++a)
-          tc::tma_load_2d(smem_u32(sm.a[s]) + a * kAtomBytesA, &map_km, a * 64, (tile0 + k) * kTileM, smem_u32(&sm.full[s]));
-      }
-    }
-  } else if (warp == 1) {
-    // ================= MMA issuer =================
-    if (tc::elect_one()) {
-      constexpr uint32_t idesc = tc::idesc_bf16(128, kTileM, 0, 0);
-      const uint64_t d0 = tc::smem_desc_sw128(smem_u32(sm.a), 16, 1024);
-      bool ok = tc::mbar_wait(smem_u32(&sm.q_ready), 0, p.status);
-      for (int k = 0; k < n_tiles && ok; ++k) {
-        const int s = k % kPageStages;
-        ok = tc::mbar_wait(smem_u32(&sm.full[s]), (k / kPageStages) & 1, p.status);
-        const uint64_t dk = tc::desc_advance(d0, s * kTileBytesA);
-        for (int unit = 0; unit < kUnits && ok; ++unit) {
-          const int u = k * kUnits + unit, buf = u & 1;
-          ok = tc::mbar_wait(smem_u32(&sm.acc_empty[buf]), ((u >> 1) & 1) ^ 1, p.status);
-          if (!ok) break;
-          tc::fence_after_sync();
-#pragma unroll
-          for (int i = 0; i < kDI / 16; ++i)   // dims 16i .. +15: column block i / 4, 32-byte slice i % 4
-            tc::umma_ts(acc_base + buf * kTileM, tmem_base + unit * (kDI / 2) + 8 * i,
-                        tc::desc_advance(dk, (i >> 2) * kAtomBytesA + (i & 3) * 32), idesc, i != 0);
-          if (unit == kUnits - 1) tc::umma_commit(smem_u32(&sm.empty[s]));  // the stage is free once these MMAs are done
-          tc::umma_commit(smem_u32(&sm.acc_full[buf]));
-        }
-      }
-    }
-  } else {
-    // ================= epilogue =================
-    const int quarter = warp & 3, cols = (warp - 2) >> 2;   // TMEM lanes 32 quarter .. (query `quarter` of four); columns 32 cols ..
-    const uint32_t lane_addr = static_cast<uint32_t>(32 * quarter) << 16;
-    {
-      // Q: this warp moves the 32 rows of its lanes of unit `cols`, a row by one thread
-      const int q = 4 * (cols >> 1) + quarter, head = 32 * (cols & 1) + lane;
-      const uint4* src = reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(p.q_idx) +
-                                                        (static_cast<int64_t>(q0 + min(q, nq - 1)) * kHI + head) * kDI);
-#pragma unroll
-      for (int y = 0; y < 2; ++y) {
-        uint32_t w[32];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const uint4 x = src[8 * y + j];
-          w[4 * j] = x.x; w[4 * j + 1] = x.y; w[4 * j + 2] = x.z; w[4 * j + 3] = x.w;
-        }
-        tc::tmem_st32(tmem_base + lane_addr + cols * (kDI / 2) + 32 * y, w);
-      }
-      tc::tmem_st_wait();
-      tc::fence_before_sync();
-      __syncwarp();
-      if (lane == 0) tc::mbar_arrive(smem_u32(&sm.q_ready));
-    }
-    float wgt[kUnits];   // half of the weight: a ReLU is taken twice over (below)
-#pragma unroll
-    for (int unit = 0; unit < kUnits; ++unit) {
-      const int q = 4 * (unit >> 1) + quarter;
-      wgt[unit] = q < nq ? 0.5f * p.w[static_cast<int64_t>(q0 + q) * kHI + 32 * (unit & 1) + lane] : 0.f;
-    }
-    bool ok = true;
-    for (int k = 0; k < n_tiles && ok; ++k) {
-      float sum[4];
-#pragma unroll
-      for (int unit = 0; unit < kUnits; ++unit) {
-        const int u = k * kUnits + unit, buf = unit & 1;
-        ok = ok && __all_sync(0xffffffffu, tc::mbar_wait(smem_u32(&sm.acc_full[buf]), (u >> 1) & 1, p.status));
-        if (!ok) break;
-        tc::fence_after_sync();
-        uint32_t v[32];
-        tc::tmem_ld32(acc_base + lane_addr + buf * kTileM + 32 * cols, v);
-        tc::tmem_ld_wait();
-        tc::fence_before_sync();
-        __syncwarp();
-        if (lane == 0) tc::mbar_arrive(smem_u32(&sm.acc_empty[buf]));
-        // eight mean keys at a time: 2 max(v, 0) = v + |v|, the same number while it is finite (where it is not, score_again())
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          float2 a = make_float2(0.f, 0.f);
-#pragma unroll
-          for (int c = 0; c < 8; c += 2) {
-            const float x = __uint_as_float(v[8 * j + c]), y = __uint_as_float(v[8 * j + c + 1]);
-            a = add2(a, make_float2(x + fabsf(x), y + fabsf(y)));
-          }
-          const float s8 = wgt[unit] * (a.x + a.y);
-          sum[j] = (unit & 1) ? sum[j] + s8 : s8;
-        }
-        if (unit & 1) {
-          // over the 32 lanes: each ends up with the sum of group j = lane / 8
-          const bool hi = lane & 16, odd = lane & 8;
-          const float x0 = (hi ? sum[2] : sum[0]) + __shfl_xor_sync(0xffffffffu, hi ? sum[0] : sum[2], 16);
-          const float x1 = (hi ? sum[3] : sum[1]) + __shfl_xor_sync(0xffffffffu, hi ? sum[1] : sum[3], 16);
-          float r = (odd ? x1 : x0) + __shfl_xor_sync(0xffffffffu, odd ? x0 : x1, 8);
-          r += __shfl_xor_sync(0xffffffffu, r, 4);
-          r += __shfl_xor_sync(0xffffffffu, r, 2);
-          r += __shfl_xor_sync(0xffffffffu, r, 1);
-          // the groups of a page
-          if (spp > 8) r += __shfl_xor_sync(0xffffffffu, r, 8);
-          if (spp > 16) r += __shfl_xor_sync(0xffffffffu, r, 16);
-          const int ql = 4 * (unit >> 1) + quarter;
-          const int64_t page = (static_cast<int64_t>(tile0 + k) * kTileM + 32 * cols + lane) >> spp_shift;
-          if ((lane & (max(spp, 8) - 1)) == 0 && ql < nq && page * p.P <= p.q_pos0 + q0 + ql - p.W) {
-            p.page_scores[static_cast<int64_t>(q0 + ql) * p.ps_ld + page] = r;
-            if (!(fabsf(r) < INFINITY)) sm.again = 1;
-          }
-        }
-      }
-    }
-  }
-  tc::fence_before_sync();
-  __syncthreads();
-  if (warp == 1) tc::tmem_dealloc(tmem_base, kTmemCols);
-  if (sm.again)
-    score_again(p, q0, nq, static_cast<int64_t>(tile0) * kTileM >> spp_shift, static_cast<int64_t>(tile0 + n_tiles) * kTileM >> spp_shift);
-}
-
 }  // namespace
 
 // ---- host side: tensor maps -----------------------------------------------------------------------
@@ -514,17 +322,6 @@ bool make_map_bf16_tile(CUtensorMap* map, const void* base, uint64_t ld, uint64_
 
 namespace {
 
-// Blocks that the tiles of a query block are dealt to.  One block per SM, and a block's time is its tiles': with few query blocks
-// the last wave is mostly empty (512 blocks of 4096 queries against a million keys: 3.5 waves, 8.4 ms; in four parts each 13.8
-// waves, 7.7 ms).
-int tile_parts(const IndexArgs& a, int blocks) {
-  const int64_t tiles = (a.q_pos0 + a.n_query - a.W) / (static_cast<int64_t>(kTileM) * a.B) + 1;
-  const int sms = a.sm_count > 0 ? a.sm_count : 148;
-  int parts = 1;
-  while (parts < 8 && static_cast<int64_t>(blocks) * parts < kFullWaves * sms && tiles / (2 * parts) >= kMinTilesOfPart) parts *= 2;
-  return parts;
-}
-
 template <int NG>
 cudaError_t launch_tc(const IndexArgs& a, cudaStream_t st, int64_t* n_launch) {
   CUtensorMap map_q, map_km;
@@ -537,21 +334,14 @@ cudaError_t launch_tc(const IndexArgs& a, cudaStream_t st, int64_t* n_launch) {
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (e != cudaSuccess) return e;
   const int QB = NG * kGroupQ;
-  const int blocks = (a.n_query + QB - 1) / QB, parts = tile_parts(a, blocks);
+  const int blocks = (a.n_query + QB - 1) / QB;
+  // One block per SM, and a block's time is its tiles': with few query blocks the last wave is mostly empty (512 blocks of
+  // 4096 queries against a million keys: 3.5 waves, 8.4 ms; in four parts each 13.8 waves, 7.7 ms).
+  const int64_t tiles = (a.q_pos0 + a.n_query - a.W) / (static_cast<int64_t>(kTileM) * a.B) + 1;
+  const int sms = a.sm_count > 0 ? a.sm_count : 148;
+  int parts = 1;
+  while (parts < 8 && static_cast<int64_t>(blocks) * parts < kFullWaves * sms && tiles / (2 * parts) >= kMinTilesOfPart) parts *= 2;
   e = launch_pdl(kernel, dim3(blocks * parts), dim3(kThreadsTc), smem, st, map_q, map_km, parts, a);
-  ++*n_launch;
-  return e;
-}
-
-cudaError_t launch_page_scores(const IndexArgs& a, cudaStream_t st, int64_t* n_launch) {
-  CUtensorMap map_km;
-  const uint64_t n_sub = static_cast<uint64_t>((a.n_key + a.B - 1) / a.B);
-  if (!make_map_bf16_128(&map_km, a.kmean, n_sub, kTileM)) return cudaErrorInvalidValue;
-  const size_t smem = sizeof(CoarsePageSmem) + 1024;
-  cudaError_t e = cudaFuncSetAttribute(coarse_page_scores_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-  if (e != cudaSuccess) return e;
-  const int blocks = (a.n_query + kPageQ - 1) / kPageQ, parts = tile_parts(a, blocks);
-  e = launch_pdl(coarse_page_scores_kernel, dim3(blocks * parts), dim3(kThreadsTc), smem, st, map_km, parts, a);
   ++*n_launch;
   return e;
 }
@@ -565,9 +355,7 @@ bool coarse_tc_supported(const IndexArgs& a) {
 
 cudaError_t launch_coarse_tc(const IndexArgs& a, int groups, cudaStream_t st, int64_t* n_launch) {
   if (a.n_query == 0) return cudaSuccess;
-  if (groups != 2) return launch_tc<1>(a, st, n_launch);
-  const int spp = a.P / a.B;   // (1 where the "pages" are tokens: nothing to sum before the weights)
-  return spp == 8 || spp == 16 || spp == 32 ? launch_page_scores(a, st, n_launch) : launch_tc<2>(a, st, n_launch);
+  return groups == 2 ? launch_tc<2>(a, st, n_launch) : launch_tc<1>(a, st, n_launch);
 }
 
 }  // namespace lsa

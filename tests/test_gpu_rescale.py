@@ -7,6 +7,7 @@ import torch
 from oracle import reference_run as ref
 from paper_2608_01662_b200 import binding
 from paper_2608_01662_b200.configs import CONFIGS
+from paper_2608_01662_b200.workload import DecodeWorkload
 
 import parity_util as pu
 
@@ -43,3 +44,36 @@ def test_growing_rows(cuda_device, listed, gain):
         got = pu.to_np(out[i])
         assert np.linalg.norm(got - want[0]) <= 1e-2 * np.linalg.norm(want[0]), i
         assert np.abs(pu.to_np(lse[i]) - want_lse[0]).max() <= 1e-4 * max(1.0, np.abs(want_lse[0]).max()), i
+
+
+# one kernel for each number of row splits; several tiles a split
+@pytest.mark.parametrize("batch,split", [(2, 1), (150, 1), (2, 2), (2, 4), (2, 8), (2, 16),
+                                         (16, 0), (34, 0),         # six and three splits
+                                         (1, 0), (2, 0)])          # 16, the value dims in four and in two parts
+@pytest.mark.parametrize("gain", [0.01, 0.125])
+def test_growing_rows_of_a_row_list(cuda_device, batch, split, gain):
+    """Paged caches: a sequence attends all of its rows in order, and the scores' spread grows along them."""
+    cfg = CONFIGS["cfg4"].replace(batch=batch, ctx_lo=2050, ctx_hi=2300, R=2, seed=batch + split)
+    wl = DecodeWorkload(cfg, cuda_device)
+    assert cfg.ctx_hi <= cfg.S + cfg.Ksp + cfg.W
+    grow = torch.ones(wl.k[0].shape[0], device=cuda_device)
+    for row in wl.page_table.long():
+        pages = row[row >= 0]
+        place = torch.arange(pages.numel() * cfg.kv_page, device=cuda_device)
+        grow[pages[place // cfg.kv_page] * cfg.kv_page + place % cfg.kv_page] = 1.0 + gain * place
+    for k in wl.k:
+        k.mul_(grow[:, None])
+    wl.prepare()
+    wl.ctx.tune(2, split)          # LSA_TUNE_ATTN_SPLIT
+    wl.step()
+    assert wl.ctx.status() == 0
+    pools = (pu.to_np(wl.ctx_len), pu.to_np(wl.page_table), pu.to_np(wl.keys["k"]), pu.to_np(wl.keys["scale"]))
+    for b in sorted({0, 1, batch // 2, batch - 1} & set(range(batch))):
+        caches, t = pu.decode_caches(wl, b, pools)
+        chosen = pu.to_np(wl.sparse_idx[b])[:int(wl.n_sparse[b])]
+        assert len(chosen) == t + 1 - cfg.S - cfg.W
+        want, want_lse = ref.attend_query(t, [pu.to_np(q[b]) for q in wl.q], caches, chosen, S=cfg.S, W=cfg.W, sm_scale=cfg.sm_scale, d_v=cfg.d_v)
+        for r in range(cfg.R):      # the bounds of the test above
+            got = pu.to_np(wl.out[r][b])
+            assert np.linalg.norm(got - want[r]) <= 1e-2 * np.linalg.norm(want[r]), (b, r)
+            assert np.abs(pu.to_np(wl.lse[r][b]) - want_lse[r]).max() <= 1e-4 * max(1.0, np.abs(want_lse[r]).max()), (b, r)

@@ -1,5 +1,5 @@
-"""Indexer heads whose dot products leave the range of fp32, or come near its end (needs a B200): a head below it counts as 0 (the
-oracle's ReLU), whatever the form of the head sum."""
+"""Indexer scores at the ends of fp32 (needs a B200): heads whose dot products leave its range, or come near its end (a head below it
+counts as 0, the oracle's ReLU, whatever the form of the head sum), and heads that cancel but for its last bits."""
 import pytest
 import torch
 
@@ -62,3 +62,41 @@ def test_decode(cuda_device, key_dtype, change):
     m = pu.check_decode(wl, range(cfg.batch), check_attention=False)
     print(key_dtype, change, m.summary())
     m.assert_ok(pu.TOL_BF16)
+
+
+@pytest.mark.parametrize("groups", [1, 2])
+@pytest.mark.parametrize("base,B", [("cfg2", 4), ("cfg2", 8), ("cfg2", 16), ("cfg3", 8)])   # 32, 16 and 8 mean keys a page
+def test_pages_of_cancelling_heads(cuda_device, base, B, groups):
+    """Head dot products of 2^22 + e and 2^22 with weights 1 and -1: a mean key counts e, exact as long as its heads are added up before
+    it meets the page's other mean keys (a page's sum of one head, up to 2^27, is not).  Page scores are integers one apart."""
+    L, n_query = 9000, 3000
+    cfg = CONFIGS[base].replace(R=1, Ksp=256, W=130, seed=9, L=L, P=128, M=16, B=B)
+    wl = PrefillWorkload(cfg, cuda_device, q_pos0=L - n_query, n_query=n_query)
+    wl.ctx.tune(0, groups)             # LSA_TUNE_COARSE_GROUPS
+    n_pages, spp = -(-L // cfg.P), cfg.P // B
+    g = torch.Generator().manual_seed(B)
+    total = torch.randperm(n_pages, generator=g) + 2 * spp      # of a page: dealt to its mean keys, the last one takes the rest
+    e = torch.randint(0, 3, (n_pages, spp), generator=g)
+    e[:, -1] = total - e[:, :-1].sum(1)
+    code = torch.zeros((n_pages * spp, cfg.d_I))
+    code[:, 0] = 256.0                                          # e4m3 codes with a scale of 8, or their products: 2048, e
+    code[:, 1:17] = (e.reshape(-1, 1) - 16 * torch.arange(16)).clamp(0, 16)    # in parts of at most 16: exact in e4m3
+    code = code.repeat_interleave(B, 0)[:L]
+    if "scale" in wl.keys:
+        wl.keys["k"].copy_(code.to(torch.float8_e4m3fn).view(torch.uint8))
+        wl.keys["scale"].fill_(8.0)
+    else:
+        wl.keys["k"].copy_((8.0 * code).to(torch.bfloat16))
+    wl.q_idx.zero_()
+    wl.w.zero_()
+    for plus, minus in ((0, 1), (12, 45)):
+        wl.q_idx[:, [plus, minus], 0] = 2048.0
+        wl.q_idx[:, plus, 1:17] = 0.125
+        wl.w[:, plus], wl.w[:, minus] = 1.0, -1.0
+    wl.prepare()
+    pages = torch.empty((n_query, cfg.M), dtype=torch.int32, device=cuda_device)
+    wl.index(pages_out=pages)
+    assert wl.ctx.status() == 0
+    m = pu.check_prefill(wl, range(wl.q_pos0, wl.q_pos0 + n_query, 157), check_attention=False, pages=pages)
+    s = m.summary()
+    assert s["page_sets_differ"] == 0 and s["min_overlap"] == 1.0, s
