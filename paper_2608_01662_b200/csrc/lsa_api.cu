@@ -183,9 +183,9 @@ int* status_word(lsa_ctx* c) { return c->ws ? reinterpret_cast<int*>(c->ws) : nu
 // a part of the value dims.  The smallest estimate wins; ties go to fewer splits (less merging).  The tcgen05 kernel merges its
 // splits inside a thread-block cluster; its waves are counted in clusters that fit the chip together, not in SMs: 15 clusters
 // of eight run at once, and a 16th sequence doubled the time (decode step of 16 sequences, 4 layers: 190 us as 8 splits, 144 as 4;
-// of 36: 255 as 4, 186 as 2; of one: 77.5 as 16, 82.7 as 8; of 8: 153 and 99).  Three and six splits, and parts of the value dims,
-// where all of them run at once: attention of 16 sequences, 4 layers, 126 us as 4, 117 as 6; of 40 176 as 2, 168 as 3 (of 80, in two
-// waves, 303, and 263 undivided); of one, two, three sequences 83, 83, 84 us undivided, 73 in four parts, 76 and 78 in two.
+// of 36: 255 as 4, 186 as 2; of one: 77.5 as 16, 82.7 as 8; of 8: 153 and 99).  Parts of the value dims, where all of them run
+// at once (decode step, 4 layers, 16K to 24K tokens): one, two, three sequences 73, 73.5, 74.2 us undivided, 66 in four parts, 69 and
+// 73.8 in two.
 cudaError_t pick_split(int sm_count, int batch, int max_rows, bool tc_kernel, int* split, int* v_shift) {
   const int units = (max_rows + 63) / 64;
   *split = 1;
@@ -201,7 +201,7 @@ cudaError_t pick_split(int sm_count, int batch, int max_rows, bool tc_kernel, in
     for (int v = 0; v <= (tc_kernel && s == kMaxSplit ? 2 : 0); ++v) {
       const long jobs = static_cast<long>(batch) << v;
       const long waves = fit > 0 ? (jobs + fit - 1) / fit : (jobs * s + sm_count - 1) / sm_count;
-      if (fit > 0 && (v > 0 || !pow2(s)) && waves > 1) continue;
+      if (v > 0 && waves > 1) continue;
       const long cost = waves * (2 * ((units + s - 1) / s + 2) + (8 >> v));
       if (best_cost < 0 || cost < best_cost) {
         best_cost = cost;

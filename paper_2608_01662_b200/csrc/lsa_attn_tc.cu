@@ -190,14 +190,14 @@ __device__ __forceinline__ bool clc_answer(uint32_t answer, int* block_x) {
 
 // With n_split > 1 the kernel must be launched with clusters of (1, n_split, 1) blocks: the splits of one sequence
 // are co-scheduled and merge their partial results themselves (no second kernel).  Block s finishes heads
-// [64 s / n_split, 64 (s + 1) / n_split): every block stages its rows (normalised, fp32) in shared memory and keeps
+// [s * 64 / n_split, (s + 1) * 64 / n_split): every block stages its rows (normalised, fp32) in shared memory and keeps
 // its own share there.
 //   Two splits (the decode configuration): the other 32 rows and their log-sum-exps are pushed straight into the
 //   peer's shared memory, behind its staged rows, by bulk copies that count bytes on the peer's mbarrier.  The cluster
 //   barrier is used in halves: a thread arrives when it has left the tile loop and waits before the first copy (the
 //   peer's ring must be out of use before it receives), and once more around the end, so that no block leaves
 //   while the other may still write into it.  Nothing goes through global memory.
-//   More splits: the rows and all log-sum-exps go to the global scratch, where they stay in L2, as 16 bulk copies of
+//   Four, eight or 16 splits: the rows and all log-sum-exps go to the global scratch, where they stay in L2, as 16 bulk copies of
 //   8 KB; after one cluster barrier the owner of a row combines the parts.  (Loads from a peer's shared memory moved the
 //   same rows at about a quarter of the L2 path's rate; a bulk copy per row took 3 000 cycles longer to issue, stores
 //   straight from the registers 4 000.)
@@ -966,12 +966,11 @@ __global__ void __launch_bounds__(Warps<kRows>::kThreads, 1) sparse_attn_tc_kern
     // 2^(lse_j - max) / sum, O = sum_j w_j O_j, bf16 to global.
     const int qi = blockIdx.x;
     constexpr int n = kSplits;
-    constexpr int rows_per = kH / n;
-    const int row0 = split * rows_per;
+    const int row0 = split * (kH / n);
     const uint8_t* stage = &sm.k[0][0][0];
     constexpr int kWarps = W::kAll;
-    __nv_bfloat16* out = reinterpret_cast<__nv_bfloat16*>(p.out) + (static_cast<int64_t>(qi) * kH + row0) * kDV;
     if constexpr (pair) {
+      __nv_bfloat16* out = reinterpret_cast<__nv_bfloat16*>(p.out) + (static_cast<int64_t>(qi) * kH + row0) * kDV;
       if (warp >= kSoftmaxWarps) cluster_wait();   // (the softmax warps completed this phase before they sent)
       // the peer's rows for this block's heads, and their log-sum-exps, are in shared memory when the byte count is met
       (void)tc::mbar_wait(smem_u32(&sm.recv_full), 0, p.status);
@@ -1079,15 +1078,8 @@ __global__ void __launch_bounds__(Warps<kRows>::kThreads, 1) sparse_attn_tc_kern
         }
       };
       static_assert(kWarps >= 16, "sixteen warps have a share of a block's rows");
-      // a number of splits that does not divide the rows: half a row at a time, dealt to all warps
-      [[maybe_unused]] auto merge_dealt = [&](auto parts) {
-        const int r0 = kH * split / n, halves = 2 * (kH * (split + 1) / n - r0);
-        for (int h = warp; h < halves; h += kWarps) merge(parts, IntC<2>{}, r0 + (h >> 1), 2 * (h & 1));
-      };
       if constexpr (kParts) {
         if (warp < 16 >> v_shift) merge(IntC<16>{}, IntC<1>{}, row0 + (warp >> (2 - v_shift)), warp & (3 >> v_shift));
-      } else if constexpr (n == 3 || n == 6) {
-        merge_dealt(IntC<n>{});
       } else {   // a warp has 16 / n of the runs of one row
         if (warp < 16) merge(IntC<n>{}, IntC<16 / n>{}, row0 + 4 * warp / n, warp * (16 / n) & 3);
       }
@@ -1106,9 +1098,7 @@ static AttnTcKernel pick_kernel(const AttnArgs& a) {
   if (a.rows == nullptr) return sparse_attn_tc_kernel<false, 1, false>;
   switch (a.n_split) {
     case 2: return sparse_attn_tc_kernel<true, 2, false>;
-    case 3: return sparse_attn_tc_kernel<true, 3, false>;
     case 4: return sparse_attn_tc_kernel<true, 4, false>;
-    case 6: return sparse_attn_tc_kernel<true, 6, false>;
     case 8: return sparse_attn_tc_kernel<true, 8, false>;
     case kMaxClusterSplit: return a.v_shift > 0 ? sparse_attn_tc_kernel<true, kMaxClusterSplit, true> : sparse_attn_tc_kernel<true, kMaxClusterSplit, false>;
     default: return sparse_attn_tc_kernel<true, 1, false>;
@@ -1116,22 +1106,26 @@ static AttnTcKernel pick_kernel(const AttnArgs& a) {
 }
 
 // (Clusters that run at once: 74 of 2 blocks, 45 of 3, 33 of 4, 26 of 5, 22 of 6, 15 of 7 to 9, 7 of 11 to 16.  Five gained nothing
-// over four: 24 sequences, four layers, 132 and 133 us.)
+// over four: 24 sequences, four layers, 132 and 133 us.  Three and six, built and taken back; decode steps of four layers: sequences of
+// 16K to 24K tokens gain, 16 as six 116 us instead of 126 as four, 42 as three 172 instead of 184 as two, but 44 as three are 191
+// instead of 185 and 45 216, and contexts of 200 to 400 tokens 62.6 instead of 57.8 (16 as six; 61.5 with four of the six blocks at
+// work) and 79 instead of 67 (40 as three: two splits exchange their rows through shared memory); the host does not know the contexts.)
 cudaError_t attn_tc_resident(int n_split, int* clusters) {
   static DeviceCount n[kMaxClusterSplit + 1];
   *clusters = 0;
-  const bool merged = (n_split >= 2 && n_split <= 4) || n_split == 6 || n_split == 8 || n_split == kMaxClusterSplit;
+  const bool merged = n_split == 2 || n_split == 4 || n_split == 8 || n_split == kMaxClusterSplit;
   if (!merged) return cudaSuccess;
   return n[n_split].get(clusters, [&](int* c) {
     return resident_clusters(reinterpret_cast<const void*>(sparse_attn_tc_kernel<true, kMaxClusterSplit, false>), Warps<true>::kThreads, sizeof(AttnTcSmem) + 1024, n_split, c);
   });
 }
 
-// Row splits that a caller may ask for: the powers of two, as many blocks as the device can co-schedule.
+// Row splits the tcgen05 kernel can merge inside a cluster: a power of two that divides the 64 heads, as many blocks as the
+// device can co-schedule.
 cudaError_t attn_tc_split_ok(int n_split, bool* ok) {
   int n = 0;
   const cudaError_t e = attn_tc_resident(n_split, &n);
-  *ok = n_split == 1 || (n > 0 && (n_split & (n_split - 1)) == 0);
+  *ok = n_split == 1 || n > 0;
   return e;
 }
 

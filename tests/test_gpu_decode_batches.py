@@ -58,7 +58,7 @@ def test_parts_of_the_value_dims(cuda_device, batch, lo, hi):
 
 @pytest.mark.parametrize("batch,lo,hi", [(16, 700, 6000), (22, 1, 400), (34, 900, 3000), (45, 1, 2500)])
 def test_splits_that_do_not_divide_the_rows(cuda_device, batch, lo, hi):
-    """Six row splits (16 to 22 sequences) and three (34 to 45), also where some of them have no rows."""
+    """Batches between the numbers of clusters that run at once, which three or six splits would serve; some splits have no rows."""
     cfg = CONFIGS["cfg4"].replace(batch=batch, ctx_lo=lo, ctx_hi=hi, R=2, seed=batch)
     wl = DecodeWorkload(cfg, cuda_device)
     wl.prepare()
@@ -66,3 +66,16 @@ def test_splits_that_do_not_divide_the_rows(cuda_device, batch, lo, hi):
     assert wl.ctx.status() == 0
     m = pu.check_decode(wl, range(0, batch, 3))
     m.assert_ok(pu.TOL_BF16)
+
+
+@pytest.mark.parametrize("batch,lo,hi,split", [(16, 700, 6000, 4), (22, 1, 400, 4), (34, 900, 3000, 2), (45, 1, 2500, 2)])
+def test_splits_are_powers_of_two(cuda_device, batch, lo, hi, split):
+    """The bits of a call that asks for the number of splits (other numbers made short contexts and some batches slower)."""
+    wl = DecodeWorkload(CONFIGS["cfg4"].replace(batch=batch, ctx_lo=lo, ctx_hi=hi, R=2, seed=batch), cuda_device)
+    wl.prepare()
+    wl.step()
+    chosen = [t.clone() for t in wl.out + wl.lse]
+    wl.ctx.tune(2, split)          # LSA_TUNE_ATTN_SPLIT
+    wl.step()
+    assert wl.ctx.status() == 0
+    assert all(torch.equal(a, b) for a, b in zip(chosen, wl.out + wl.lse))
