@@ -741,9 +741,13 @@ __global__ void __launch_bounds__(Warps<kRows>::kThreads, 1) sparse_attn_tc_kern
           }
         }
         // Running max in log2 units: that of the job's first tile, moved only when a row grows by more than kRescaleGap (O and l
-        // are then rescaled).  P is worked out with the maximum as it is; the vote that ends the tile says whether that was good
-        // enough for every row, so a row's lanes and halves compare their values only where they have to: shuffles and barriers
-        // queue behind the gather warps' copies (110-150 cycles each).
+        // are then rescaled).  With two halves P is worked out with the maximum as it is, and the vote that ends the tile says whether
+        // that was good enough for every row, so a row's lanes and halves compare their values only where they have to: shuffles and
+        // barriers queue behind the gather warps' copies (110-150 cycles each).  If it was not, P is worked out again (300 queries of
+        // 3000 rows, two layers: 375 us with four warps that compare first, 366 so, 384 with eight that compare first; where the spread
+        // of the scores keeps growing along the rows, so that nearly every tile is rescaled, 409, 420 and 412).
+        // Where row lists are walked the lanes compare first: HBM paces those tiles, and a rescaling costs no second P (64 sequences
+        // whose last 300 rows score highest, as recent tokens do, three layers: 149.1 us, 151.4 with P first).
         float mx[2];   // of the thread's values, then of the rows'
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
@@ -765,16 +769,29 @@ __global__ void __launch_bounds__(Warps<kRows>::kThreads, 1) sparse_attn_tc_kern
             for (int r = 0; r < 2; ++r) mx[r] = fmaxf(mx[r], sm.half_max[half ^ 1][row_s + 8 * r]);
           }
         };
+        float alpha[2] = {1.f, 1.f};   // factors of the rows that have grown too far
+        auto move_max = [&]() {
+#pragma unroll
+          for (int r = 0; r < 2; ++r) {
+            alpha[r] = 1.f;
+            if (mx[r] > m_used[r] + kRescaleGap) {
+              alpha[r] = exp2_fast(m_used[r] - mx[r]);
+              m_used[r] = mx[r];
+            }
+            l_run[r] *= alpha[r];
+          }
+        };
         bool need = false;
+        if (i == 0 || kHalves == 1) row_max();
         if (i == 0) {
-          row_max();
           m_used[0] = mx[0];
           m_used[1] = mx[1];
         } else {
           need = mx[0] > m_used[0] + kRescaleGap || mx[1] > m_used[1] + kRescaleGap;
+          if constexpr (kHalves == 1) move_max();
         }
         float sum[2];
-        while (true) {
+        auto work_out_p = [&]() {
           // P = exp2(z - m), fp32 row sums, bf16 pack
           uint32_t pk[kGroups][2];
 #pragma unroll
@@ -792,13 +809,15 @@ __global__ void __launch_bounds__(Warps<kRows>::kThreads, 1) sparse_attn_tc_kern
             sum[r] = sum2.x + sum2.y;
           }
           // P takes the place of the tile's rope dims, which only Q K^T reads
-          {
-            const int row = 16 * quarter + ((lane >> 3) & 1) * 8 + (lane & 7);
-            const uint32_t dst = smem_u32(sm.k[slot][8]) + row * 128;
+          const int row = 16 * quarter + ((lane >> 3) & 1) * 8 + (lane & 7);
+          const uint32_t dst = smem_u32(sm.k[slot][8]) + row * 128;
 #pragma unroll
-            for (int j = 0; j < kGroups; j += 2)
-              stmatrix_x4(dst + (((kGroups * half + j + (lane >> 4)) ^ (row & 7)) << 4), pk[j][0], pk[j][1], pk[j + 1][0], pk[j + 1][1]);
-          }
+          for (int j = 0; j < kGroups; j += 2)
+            stmatrix_x4(dst + (((kGroups * half + j + (lane >> 4)) ^ (row & 7)) << 4), pk[j][0], pk[j][1], pk[j + 1][0], pk[j + 1][1]);
+        };
+        if constexpr (kHalves == 1) work_out_p();
+        while (true) {
+          if constexpr (kHalves > 1) work_out_p();
           if (!ok) sm.fail = 1;
           tc::fence_proxy_async();   // P is read by the tensor core
           if (!softmax_any<kSoftmaxThreads>(need || !ok)) break;
@@ -806,18 +825,14 @@ __global__ void __launch_bounds__(Warps<kRows>::kThreads, 1) sparse_attn_tc_kern
             failed = true;
             break;
           }
-          // rare: the rows' new maxima, O of every head times its factor, once P V of the tile before is complete, and P again
-          row_max();
-#pragma unroll
-          for (int r = 0; r < 2; ++r) {
-            float alpha = 1.f;
-            if (mx[r] > m_used[r] + kRescaleGap) {
-              alpha = exp2_fast(m_used[r] - mx[r]);
-              m_used[r] = mx[r];
-            }
-            l_run[r] *= alpha;
-            if (half == 0 && (lane & 3) == 0) sm.lse_own[row_s + 8 * r] = alpha;
+          // rare: O of every head times its factor, once P V of the tile before is complete
+          if constexpr (kHalves > 1) {
+            row_max();
+            move_max();
           }
+#pragma unroll
+          for (int r = 0; r < 2; ++r)
+            if (half == 0 && (lane & 3) == 0) sm.lse_own[row_s + 8 * r] = alpha[r];
           softmax_sync<kSoftmaxThreads>();
           ok = wait_pv(g - 1, base + i - 1 + (i - 1 >= jb.q_at ? 1 : 0));   // (a first tile has no such rows)
           tc::fence_after_sync();
