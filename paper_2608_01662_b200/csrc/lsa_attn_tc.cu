@@ -502,14 +502,6 @@ __global__ void __launch_bounds__(Warps<kRows>::kThreads, 1) sparse_attn_tc_kern
         const int i = tile_of(e);   // the tile (if this is not Q)
         const int rows_here = kRows ? warp_rows : max(0, min(warp_rows, tile_keys(jb, i) - kRowsPerWarp * gw));   // of it, by this warp (a multiple of 8)
         const int32_t next_row = my_key_row(e + kRing);   // fetched before the wait: off the critical path
-#if LSA_PF == 1
-        if (!kRows && next_row >= 0) asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(kg + static_cast<int64_t>(next_row) * p.ld_k * 2), "n"(kDQK * 2) : "memory");
-#elif LSA_PF == 2
-        if (!kRows && next_row >= 0) {
-#pragma unroll
-          for (int y = 0; y < 9; ++y) asm volatile("prefetch.global.L2 [%0];" ::"l"(kg + static_cast<int64_t>(next_row) * p.ld_k * 2 + y * 128) : "memory");
-        }
-#endif
         if (e >= jb.q_at && !waited) {   // the tiles before Q are in flight: now the previous kernel must be done
           dependency_wait();
           waited = true;
