@@ -1144,6 +1144,7 @@ cudaError_t launch_attn_tc(const AttnArgs& a, cudaStream_t st, int64_t* n_launch
   if (a.n_query == 0) return cudaSuccess;
   const size_t smem = sizeof(AttnTcSmem) + 1024;
   if (a.n_split > 1 && a.rows == nullptr) return cudaErrorInvalidValue;   // row splits walk row lists
+  if (a.v_shift != 0 && a.n_split != kMaxClusterSplit) return cudaErrorInvalidValue;   // (no other kernel knows of parts)
   AttnTcKernel kernel = pick_kernel(a);
   const int threads = a.rows == nullptr ? Warps<false>::kThreads : Warps<true>::kThreads;
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));

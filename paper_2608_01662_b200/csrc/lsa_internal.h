@@ -73,7 +73,7 @@ struct AttnArgs {
                           // stream started, so they may be read ahead of the programmatic dependency wait
   int sm_count;           // tcgen05 kernel: blocks that run at the same time
   int n_split;            // >1: partial results in part_out / part_lse, merged afterwards
-  int v_shift;            // tcgen05 kernel, n_split > 2: the value dims in 2^v_shift parts (0, 1 or 2)
+  int v_shift;            // tcgen05 kernel, 16 splits only: the value dims in 2^v_shift parts (0, 1 or 2)
   float* part_out;        // fp32 [n_query, n_split, H, DV]; with parts [n_query, part, n_split, H, DV >> v_shift]
   float* part_lse;        // fp32 [n_query, n_split, H]; with parts [n_query, part, n_split, H]
   int* status;
