@@ -131,7 +131,8 @@ LSA_API const char* lsa_last_cuda_error(lsa_ctx* ctx);
 /* Number of kernels this context has launched since creation (host counter). */
 LSA_API int64_t lsa_launch_count(lsa_ctx* ctx);
 
-/* Launch-shape knobs; results never depend on them.
+/* Launch-shape knobs.  Selections never depend on them; attention's results do by rounding where it is another kernel
+ * (LSA_TUNE_ATTN_TC) or another split of the rows (LSA_TUNE_ATTN_SPLIT: bf16 weights against other running maxima).
  *   LSA_TUNE_COARSE_GROUPS  4-query groups held per thread block of the coarse-score kernel (1 or 2; default 2)
  *   LSA_TUNE_ATTN_TC        1 (default): MLA-shape attention on tcgen05.mma; 0: the mma.sync kernel
  *   LSA_TUNE_ATTN_SPLIT     row splits per sequence in paged attention: 0 (default) = chosen by the wave cost model,

@@ -43,7 +43,7 @@
 // 18 TB/s with 216 KB in flight on each, but only a slot or so is.  The hold is a chain of hand-overs of 200-500 cycles each beside
 // the MMAs, in a load/store pipe that the copies fill.  With four softmax warps that took a maximum over each row for every
 // tile, two gather warps a slot and the last tile worked on whole, holds were 4 500 and a gathered tile 2 264 (16384 rows; now
-// 2 110), but the clock gives half of it back and more under the power cap: 32768 queries, two layers, 24.3 ms -> 23.7 ms; 16384
+// 2 110; struct Warps and tile_keys say what the last two gave alone), but the clock gives half of it back and more under the power cap: 32768 queries, two layers, 24.3 ms -> 23.7 ms; 16384
 // of 131072, four layers, 34.8 -> 34.3 ms; 4096 of a million, four layers, 11.55 -> 11.45 ms; 1237 queries, four layers, 538 -> 527 us.
 //
 // Tensor memory columns:   0-255  O: value dims 0-255 in columns 0-127, 256-511 in 128-255; lanes 0-63 hold the first 128
@@ -74,9 +74,12 @@ constexpr int kMaxClusterSplit = 16;         // row splits of one sequence = blo
 constexpr int kFirstTileCycles = 8192;       // longest that a block's second tile is held back for the first
 constexpr float kRescaleGap = 8.f;           // rescale O only when the row max grows by more than 2^8
 // Warps of a block.  Prefill: the softmax of a tile by two warps per lane quarter, each with half of its keys, and three gather
-// warps a ring slot (two issue a tile's 144 copies in 1 530 cycles, three in 1 430, which is about what the SM takes).  Where row
-// lists are walked one and two: HBM paces the tiles, and a layer's ends are shorter with fewer threads (64 sequences, four layers:
-// 189 us, 195 with the prefill's eight softmax warps).
+// warps a ring slot (two issue a tile's 144 copies in 1 530 cycles, three in 1 430, which is about what the SM takes: 300 queries of
+// 3000 rows 174 -> 171 us, 1000 of 9000 427 -> 420, a prompt of 32768, two layers, 24.8 -> 24.2 ms; 1237 queries of at most 1237 rows,
+// four layers, lose, 505 -> 512 us).  23 warps leave 80 registers a thread, and 24 bytes of the prefill kernel spill; none do in 20 warps,
+// with two gather warps a slot, which is the slower form all the same.  Where row lists are walked there are 16 warps, one softmax
+// warp per quarter and two gather warps a slot: HBM paces the tiles, and a layer's ends are shorter with fewer threads (64
+// sequences, four layers: 189 us, 195 with the prefill's eight softmax warps).
 template <bool kRows>
 struct Warps {
   static constexpr int kHalves = kRows ? 1 : 2, kSoftmax = 4 * kHalves;
@@ -314,8 +317,9 @@ __global__ void __launch_bounds__(Warps<kRows>::kThreads, 1) sparse_attn_tc_kern
     b.q_at = early_rows ? min(2, b.n_tiles) : 0;
     return b;
   };
-  // Keys of tile i that are worked on: the last tile's in whole MMA steps of 16 (3076 rows are 48 tiles and four rows).  Not where
-  // row lists are walked: HBM paces those tiles, and loops of a constant length are issued faster.
+  // Keys of tile i that are worked on: the last tile's in whole MMA steps of 16.  It shows where jobs are short (1237 queries of at
+  // most 1237 rows, four layers: 518 -> 512 us); 3076 rows are 48 tiles and four rows, and there it is within the noise.  Not where row
+  // lists are walked: HBM paces those tiles, and loops of a constant length are issued faster.
   auto tile_keys = [](const Job& b, int i) -> int {
     if constexpr (kRows) return kTileKeys;
     else return min(kTileKeys, (b.n_tot - (b.tile_begin + i) * kTileKeys + 15) & ~15);
@@ -696,7 +700,7 @@ __global__ void __launch_bounds__(Warps<kRows>::kThreads, 1) sparse_attn_tc_kern
     Job jb = job_of(jd);
     bool have_o = false;
     float m_used[2] = {0.f, 0.f}, l_run[2] = {0.f, 0.f};   // rows row_s and row_s + 8; l_run is this thread's share
-    // A warp whose wait ran out goes on to the next vote, where all eight learn of it and leave together: the named barrier
+    // A warp whose wait ran out goes on to the next vote, where all of them learn of it and leave together: the named barrier
     // has no time limit.
     bool go = !softmax_any<kSoftmaxThreads>(!ok);
     while (go) {

@@ -48,7 +48,7 @@ def test_growing_rows(cuda_device, listed, gain):
 
 # one kernel for each number of row splits; several tiles a split
 @pytest.mark.parametrize("batch,split", [(2, 1), (150, 1), (2, 2), (2, 4), (2, 8), (2, 16),
-                                         (16, 0), (34, 0),         # six and three splits
+                                         (16, 0), (34, 0),         # as many splits as the batch gets: four and two
                                          (1, 0), (2, 0)])          # 16, the value dims in four and in two parts
 @pytest.mark.parametrize("gain", [0.01, 0.125])
 def test_growing_rows_of_a_row_list(cuda_device, batch, split, gain):
